@@ -354,6 +354,9 @@ int sbi_step_launches(const sbi_ctx* ctx, int* launches);
  * each column's inputs arrive in shared memory by bulk copies (TMA,
  * cp.async.bulk), the next input in flight while the current one is
  * transformed; the arithmetic is the same.
+ * Two-dimensional FP32 groups (marked "packed") have two more choices: a row
+ * choice with "x<k>" runs at most k products of a pass per block, a column
+ * choice with "w<k>" transforms k inputs of the same columns at once.
  * (ms is -1 for a shape that was not timed: one candidate only, or a pass
  * that is not re-run because its outputs alias its inputs).
  * Writes at most cap bytes (NUL-terminated) into buf and the full length

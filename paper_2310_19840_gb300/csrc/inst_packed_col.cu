@@ -1,0 +1,35 @@
+// Column pass instantiations of packed groups (two-dimensional, FP32).
+#include "packed_kernels.cuh"
+
+namespace sbi {
+#define SBI_PACKED_NY(X) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
+#define SBI_SWITCH(N, F, BAD) switch (ny) { SBI_PACKED_NY(F) default: return BAD; }
+
+cudaError_t prepare_packed_col_kernels(int ny) {
+#define SBI_CASE(N) case N: return pk::prepare_packed_col_n<N>();
+  SBI_SWITCH(ny, SBI_CASE, cudaErrorInvalidValue)
+#undef SBI_CASE
+}
+cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st) {
+#define SBI_CASE(N) case N: return pk::launch_packed_col_n<N>(p, st);
+  SBI_SWITCH(ny, SBI_CASE, cudaErrorInvalidValue)
+#undef SBI_CASE
+}
+int packed_col_geometry(int ny, int* tpc, int* group) {
+  *tpc = *group = 0;
+#define SBI_CASE(N) case N: *tpc = pk::ColGeo<N>::T; *group = pk::ColGeo<N>::CI; return pk::ColGeo<N>::CPB;
+  SBI_SWITCH(ny, SBI_CASE, 0)
+#undef SBI_CASE
+}
+bool packed_col_stageable(int ny) {
+#define SBI_CASE(N) case N: return pk::ColGeo<N>::STAGEABLE;
+  SBI_SWITCH(ny, SBI_CASE, false)
+#undef SBI_CASE
+}
+int packed_col_most_wide(const ColParams& p) {
+  const int ny = p.ny;
+#define SBI_CASE(N) case N: return pk::col_most_wide<N>(p);
+  SBI_SWITCH(ny, SBI_CASE, 0)
+#undef SBI_CASE
+}
+}  // namespace sbi

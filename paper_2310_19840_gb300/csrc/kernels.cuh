@@ -1006,7 +1006,11 @@ __global__ void k_coef_table(T* __restrict__ out, const TableSpec s, int perm) {
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= (long long)s.W * s.ny) return;
   const int kx = (int)(idx / s.ny), n = (int)(idx % s.ny);
-  const long long at = (long long)kx * s.ny + (perm > 1 ? (n % perm) * 256 + n / perm : n);
+  long long at = (long long)kx * s.ny + (perm > 1 ? (n % perm) * 256 + n / perm : n);
+  if (s.packed) {   // tiles of four columns; the modes below ny / 2, then the others
+    const int ny2 = s.ny / 2;
+    at = (n < ny2 ? 0 : (long long)s.W * ny2) + ((long long)(kx >> 2) * ny2 + n % ny2) * 4 + (kx & 3);
+  }
   const int ns = (s.ny == 1) ? 0 : (n < s.ny / 2 ? n : n - s.ny);
   const double kxv = kx * s.two_pi_over_Lx, kyv = ns * s.two_pi_over_Ly;
   const double k = sqrt(kxv * kxv + kyv * kyv);
@@ -1057,6 +1061,7 @@ __global__ void k_coef_table(T* __restrict__ out, const TableSpec s, int perm) {
 // order of the modes of a column in the multiplier tables (k_coef_table)
 template <typename T>
 int col_table_perm(int ny) {
+  if (sizeof(T) == 4) return 1;   // one-dimensional, or the order of a packed group
   if (ny == 512 && ColCfg<T, 512>::SPLIT) return 2;
   if (ny == 1024 && ColCfg<T, 1024>::SPLIT) return 4;
   if (ny == 2048 && ColCfg<T, 2048>::SPLIT) return 8;
@@ -1176,6 +1181,10 @@ cudaError_t launch_col_n(const ColParams& p, cudaStream_t st) {
 
 #define SBI_FOR_NX(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096)
 #define SBI_FOR_NY(X) X(1) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
+// column lengths of the plain family: one-dimensional groups, and in FP64 all
+// (two-dimensional FP32 groups run on packed_kernels.cuh)
+template <typename T, int NY>
+inline constexpr bool kPlainCol = NY == 1 || sizeof(T) == 8;
 
 template <typename T>
 cudaError_t prepare_row_impl(int nx) {
@@ -1190,7 +1199,10 @@ cudaError_t prepare_row_impl(int nx) {
 template <typename T>
 cudaError_t prepare_col_impl(int ny) {
   switch (ny) {
-#define SBI_CASE(N) case N: return prepare_ny<T, N>();
+#define SBI_CASE(N) \
+  case N:           \
+    if constexpr (kPlainCol<T, N>) return prepare_ny<T, N>(); \
+    else return cudaErrorInvalidValue;
     SBI_FOR_NY(SBI_CASE)
 #undef SBI_CASE
     default: return cudaErrorInvalidValue;
@@ -1220,7 +1232,10 @@ cudaError_t launch_rk_impl(int nx, const RkParams& p, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_col_impl(int ny, const ColParams& p, cudaStream_t st) {
   switch (ny) {
-#define SBI_CASE(N) case N: return launch_col_n<T, N>(p, st);
+#define SBI_CASE(N) \
+  case N:           \
+    if constexpr (kPlainCol<T, N>) return launch_col_n<T, N>(p, st); \
+    else return cudaErrorInvalidValue;
     SBI_FOR_NY(SBI_CASE)
 #undef SBI_CASE
     default: return cudaErrorInvalidValue;

@@ -1,0 +1,1172 @@
+// packed_kernels.cuh - row, column and RK passes of two-dimensional FP32 groups.
+//
+// The passes of kernels.cuh in the packed arithmetic of packed.cuh.  Physical
+// fields and the state keep the row-major order.  A mixed field is stored
+// [member][kx / 4][y / 2][kx % 4][y % 2] (complex, the kept x-modes rounded up to
+// four columns Wp; the columns W <= kx < Wp hold zeros): the modes of a row pair
+// that neighbouring threads hold make up whole 32-byte sectors, so a row pass
+// reads and writes the transposed field straight from and to registers, and a
+// column pass reads two samples of four neighbouring columns as 64 bytes.
+//
+// In both passes a transform belongs to the threads of one warp wherever it
+// fits one, so that the kernels need no block barriers; rows of more than 1024
+// points and columns of more than 512 use the block.
+//
+// Against the scalar passes of kernels.cuh (GB300, 2.0 GHz): a 512-point row
+// takes 128 SM-cycles per transform instead of 312 and 336 instructions per
+// row instead of about 800; a 256-point column 137 instead of 312; the row pass
+// of a 4096 x 2048 grid 173 us per launch instead of 344; a step of 64 256^2 and
+// 32 512^2 members 4.42 ms instead of 6.03.
+#pragma once
+
+#include "kernels.cuh"
+#include "packed.cuh"
+
+namespace sbi {
+namespace pk {
+
+// ===========================================================================
+// Rows
+// ===========================================================================
+// 16 elements per thread from 256-point rows up.  128 registers (four blocks
+// of 128 threads per SM) hold a transform, the running product of a chain and
+// the field that multiplies it (32 registers each at 16 elements): the inner
+// loop reads no global memory, and shared memory only for the exchange and the
+// twiddles.  Shared-memory bandwidth is what bounds these passes.
+template <int NX>
+struct RowGeo {
+  static constexpr int n = NX / 2;
+  static constexpr int R = n >= 128 ? 16 : 8;
+  static constexpr int T = n / R;                       // threads per row
+  static constexpr bool WARP = T <= 32;
+  static constexpr int THREADS = 128;
+  static constexpr int MAXR = THREADS / T;              // rows per block
+  using F = PackedFft<One, n, R, WARP>;
+  using E = typename F::E;
+  // exchange elements per row; rows that share half a warp lie T 8-byte banks
+  // apart; rows of more than a warp also pass their upper half through it
+  static constexpr int XLEN = (F::xlen() + 15) / 16 * 16 + (T < 16 ? T : 0);
+  static constexpr bool TAB = n <= 256;                 // e^{-2 pi i k / NX}, k < n / 2, in shared memory
+  static constexpr int RTW = (F::TW + (TAB ? n / 2 : 0) + 1) / 2 * 2;   // twiddles of a block
+};
+template <int NX>
+__host__ __device__ constexpr size_t row_smem(int rows, int nslots) {
+  using G = RowGeo<NX>;
+  return 8 * ((size_t)G::RTW + (size_t)rows * (G::XLEN + nslots * G::n));
+}
+// The twiddles of a block's transforms and of the packed real transform: from
+// shared memory, or (long rows) products of the thread's own e^{-2 pi i j / NX}
+// by roots of unity.
+template <int NX>
+struct RowTwiddles {
+  using G = RowGeo<NX>;
+  const float2 *table, *tw;
+  int j;
+  float2 wj;
+  __device__ __forceinline__ RowTwiddles(const void* global, float2* shared, int j_)
+      : table(shared), tw(reinterpret_cast<const float2*>(global)), j(j_) {
+    G::F::fill_twiddles(shared, tw);
+    if constexpr (G::TAB) {
+      for (int k = threadIdx.x; k < G::n / 2; k += blockDim.x) shared[G::F::TW + k] = __ldg(tw + tw_off(NX) + k);
+    } else {
+      wj = __ldg(tw + tw_off(NX) + j);
+    }
+    __syncthreads();
+  }
+  __device__ __forceinline__ void run(One (&x)[G::R], typename G::E* xs) const {
+    G::F::run(x, xs, j, G::F::twiddles(table, j), tw);
+  }
+  // e^{-2 pi i (j + r T) / NX}; r < R / 2 with j < T, or r >= R / 2
+  __device__ __forceinline__ float2 lower(int r) const {
+    if constexpr (G::TAB) return table[G::F::TW + j + r * G::T];
+    else return r == 0 ? wj : wmul(wj, unit_root(r, 2 * G::R));
+  }
+  __device__ __forceinline__ float2 upper(int r) const {
+    if constexpr (G::TAB) {
+      // e(k) = -conj(e(n - k)), n - k = T - j + (R - 1 - r) T; the one k = n / 2
+      // (j = 0, r = R / 2) is multiplied by zero: any entry will do
+      const int kk = G::T - j + (G::R - 1 - r) * G::T;
+      const float2 e = table[G::F::TW + (r == G::R / 2 ? kk & (G::n / 2 - 1) : kk)];
+      return make_float2(-e.x, e.y);
+    } else {
+      return wmul(wj, unit_root(r, 2 * G::R));
+    }
+  }
+  // Products by roots of unity are formed where they are used: kept across a
+  // loop they would take more registers than there are.  Emits nothing.
+  __device__ __forceinline__ void renew() {
+    if constexpr (!G::TAB) asm volatile("" : "+f"(wj.x), "+f"(wj.y));
+  }
+};
+
+// the row of this thread's group; an absent or inactive row reads row 0 of
+// member 0 and stores nothing
+struct Row {
+  int member, y;
+  bool act;
+};
+template <int T>
+__device__ __forceinline__ Row row_of(int row_begin, int rows_total, int ny, const int* active, int member0) {
+  const int q = row_begin + (int)blockIdx.x * (int)(blockDim.x / T) + (int)threadIdx.x / T;
+  Row r;
+  r.act = q < rows_total;
+  r.member = r.act ? q / ny : 0;
+  r.y = r.act ? q - r.member * ny : 0;
+  if (r.act && active) r.act = active[member0 + r.member] != 0;
+  return r;
+}
+// mixed field at mode 0 of the row; mode k at + mode_at(k)
+__device__ __forceinline__ const unsigned long long* mixed_row(const BufRef& b, const Row& w) {
+  return reinterpret_cast<const unsigned long long*>(b.ptr) + (long long)w.member * b.stride + (w.y >> 1) * 8 + (w.y & 1);
+}
+__device__ __forceinline__ long long mode_at(int k, int ny) { return (long long)(k >> 2) * ny * 4 + (k & 3) * 2; }
+// physical row as complex pairs (x[2m], x[2m + 1])
+__device__ __forceinline__ float2* real_row(const BufRef& b, const Row& w, int n) {
+  return reinterpret_cast<float2*>(reinterpret_cast<float*>(b.ptr) + (long long)w.member * b.stride) + (long long)w.y * n;
+}
+
+// Input side of the packed inverse real transform of a row: Z[k] =
+// X[k] (1 + i w) for k < W, X[n - k]* (1 - i w) for k > n - W, w = e^{2 pi i k / NX}
+// (both terms where more than half of the modes are kept).  The inverse of Z
+// is taken as the conjugate of the transform of its conjugate: x = Z*.
+// EXACT: W = n / 2 (half of the modes, the default), every bound known at
+// compile time.  In that form load_modes runs ahead of the products.
+template <int NX, bool EXACT>
+inline constexpr bool kFastRow = EXACT && RowGeo<NX>::T >= 4;
+
+template <int NX>
+__device__ __forceinline__ void load_modes(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
+                                           int j) {
+  constexpr int R = RowGeo<NX>::R, T = RowGeo<NX>::T;
+  // k = j + r T: X[k] at lo + r step for r < R / 2; n - k = T - j + (R - 1 - r) T
+  const int step = T * ny;
+  const long long lo = mode_at(j, ny), hi = mode_at(T - j, ny);
+  const unsigned long long* src = mixed_row(bufs[0], w);
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    x[r].v = 0;
+    if (r < R / 2) x[r].v = src[lo + r * step];
+    else if (r > R / 2 || j != 0) x[r].v = src[hi + (R - 1 - r) * step];
+  }
+#pragma unroll 1
+  for (int q = 1; q < nb; ++q) {
+    src = mixed_row(bufs[q], w);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (r < R / 2) x[r] = add(x[r], One{src[lo + r * step]});
+      else if (r > R / 2 || j != 0) x[r] = add(x[r], One{src[hi + (R - 1 - r) * step]});
+    }
+  }
+}
+template <int NX>
+__device__ __forceinline__ void twist_modes(One (&x)[RowGeo<NX>::R], const RowTwiddles<NX>& t) {
+  constexpr int R = RowGeo<NX>::R;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (r < R / 2) {   // conj(X (1 + i w)), 1 + i w = (1 + e.y, e.x) with e = w*
+      const float2 e = t.lower(r);
+      const float f = 1.f + e.y;
+      x[r] = fma(both(-e.x), swp(x[r]), mul(f2(f, -f), x[r]));
+    } else {           // X (1 - i w)*, 1 - i w = (1 - e.y, -e.x)
+      const float2 e = t.upper(r);
+      x[r] = cmul(x[r], make_float2(1.f - e.y, e.x));
+    }
+  }
+}
+template <int NX, bool EXACT>
+__device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
+                                              int W, int j, const RowTwiddles<NX>& t) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  if constexpr (kFastRow<NX, EXACT>) {
+    const int step = T * ny;
+    const long long lo = mode_at(j, ny), hi = mode_at(T - j, ny);
+#pragma unroll 1
+    for (int q = 0; q < nb; ++q) {
+      const unsigned long long* src = mixed_row(bufs[q], w);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        One v = both(0.f);
+        if (r < R / 2) v.v = src[lo + r * step];
+        else if (r > R / 2 || j != 0) v.v = src[hi + (R - 1 - r) * step];
+        x[r] = q == 0 ? v : add(x[r], v);
+      }
+    }
+    twist_modes<NX>(x, t);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int k = j + r * T, kk = n - k;
+      One a = both(0.f), b = both(0.f);
+      for (int q = 0; q < nb; ++q) {
+        const unsigned long long* src = mixed_row(bufs[q], w);
+        if (k < W) a = add(a, One{src[mode_at(k, ny)]});
+        if (k > 0 && kk < W) b = add(b, One{src[mode_at(kk, ny)]});
+      }
+      const float2 e = __ldg(t.tw + tw_off(NX) + k);
+      const One o = cmul(sub_conj(a, b), make_float2(e.x, -e.y));
+      x[r] = conj(addi(add_conj(a, b), o));
+    }
+  }
+}
+
+// Output side of the packed forward real transform of a row, Z in x: stores
+// the kept modes X[k] = 1/2 (Z[k] + Z[n-k]*) - i/2 e^{-2 pi i k / NX} (Z[k] -
+// Z[n-k]*), k < W.  Z[n - k] sits in lane (T - j) mod T, register R - 1 - r
+// (thread 0: its own register (R - r) mod R): a shuffle, or, for rows of
+// several warps, a pass through the exchange buffer.
+template <int NX, bool EXACT>
+__device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const BufRef& dst, const Row& w, int ny,
+                                            int W, int j, typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  constexpr bool FAST = kFastRow<NX, EXACT>;
+  unsigned long long* out = const_cast<unsigned long long*>(mixed_row(dst, w));
+  const int step = T * ny;
+  if (FAST) out += mode_at(j, ny);
+  if constexpr (!G::WARP) {
+    // Z[n - k] of the kept modes: the elements above n - W, and Z[0]
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (r == 0 || (FAST ? r >= R / 2 : (r + 1) * T > n - W)) xs[j + r * T] = x[r].v;
+    __syncthreads();
+  }
+  One X[FAST ? R / 2 : R];
+#pragma unroll
+  for (int r = 0; r < (FAST ? R / 2 : R); ++r) {
+    if (!FAST && r * T >= W) break;
+    const int k = j + r * T;
+    One zc;
+    if constexpr (!G::WARP) {
+      zc.v = xs[(n - k) & (n - 1)];
+    } else {
+      zc = x[(R - r) & (R - 1)];
+      if constexpr (T > 1) {
+        const float2 a = parts(x[R - 1 - r]);
+        const int lane = (T - j) & (T - 1);
+        const One o = f2(__shfl_sync(0xffffffffu, a.x, lane, T), __shfl_sync(0xffffffffu, a.y, lane, T));
+        if (j != 0) zc = o;
+      }
+    }
+    const float2 e = FAST ? t.lower(r) : __ldg(t.tw + tw_off(NX) + k);
+    const One d = cmul(sub_conj(x[r], zc), e);
+    X[r] = scale(0.5f, subi(add_conj(x[r], zc), d));
+  }
+  if (w.act) {
+#pragma unroll
+    for (int r = 0; r < (FAST ? R / 2 : R); ++r) {
+      if (FAST) out[r * step] = X[r].v;
+      else if (j + r * T < W) out[mode_at(j + r * T, ny)] = X[r].v;
+    }
+  }
+  if constexpr (!G::WARP) __syncthreads();
+}
+
+// v *= f^p, one factor after the other
+template <int R>
+__device__ __forceinline__ void times_field(One (&v)[R], const One (&f)[R], int p) {
+#pragma unroll 1
+  for (int i = 0; i < p; ++i) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = mul(v[r], f[r]);
+  }
+}
+
+// Chains of one inverse transform and the products formed from it.  blockIdx.y
+// takes a segment of the operations: the whole list, or a few products of one
+// chain (the inverse transform and the products before them are then formed
+// again without being transformed, in the same order and so with the same
+// bits), which spreads a pass over few rows across the SMs.  Both directions
+// go through the one transform of the loop (instruction cache).
+template <int NX, bool EXACT>
+__global__ void __launch_bounds__(RowGeo<NX>::THREADS, 4)
+k_packed_row(const __grid_constant__ RowParams p) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + (threadIdx.x / T) * G::XLEN;
+  const int j = threadIdx.x % T;
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
+  const int ny = p.ny;
+  One run[R], x[R], f[R];
+  int held = 0;      // the field in f: 1 eta, 2 delta
+  auto hold = [&](int which) {
+    if (held == which) return;
+    const float2* src = real_row(which == 1 ? p.eta : p.delta, w, n) + j;
+#pragma unroll
+    for (int r = 0; r < R; ++r) f[r] = f2(__ldg(src + r * T));
+    held = which;
+  };
+  const int first = p.seg[blockIdx.y].first, end = p.seg[blockIdx.y].end, begin = p.seg[blockIdx.y].begin;
+  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+
+#pragma unroll 1
+  for (int o = begin; o < end; ++o) {
+    t.renew();
+    const RowOp op = p.ops[o];
+    const bool inverse = op.kind == ROP_C2R;
+    if (inverse) {
+      inverse_input<NX, EXACT>(x, p.buf + op.a, op.b, w, ny, p.W, j, t);
+    } else {
+      const bool running = (op.c & 2) != 0;
+      if (o < first && !running) continue;
+      if (!running) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = run[r];
+      }
+#pragma unroll 1
+      for (int q = 1; q <= 2; ++q) {
+        const int e = q == 1 ? op.a : op.b;
+        if (e == 0) continue;
+        hold(q);
+        if (running) times_field<R>(run, f, e);
+        else times_field<R>(x, f, e);
+      }
+      if (o < first) continue;
+      if (running) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = run[r];
+      }
+      if (op.coef_f != 1.f) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = scale(op.coef_f, x[r]);
+      }
+    }
+    t.run(x, xs);
+    if (inverse) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) run[r] = conj(x[r]);
+      if (op.dst != kNone && w.act) {
+        float2* out = real_row(p.buf[op.dst], w, n) + j;
+#pragma unroll
+        for (int r = 0; r < R; ++r) out[r * T] = parts(run[r]);
+      }
+    } else {
+      store_modes<NX, EXACT>(x, p.buf[op.dst], w, ny, p.W, j, xs, t);
+    }
+  }
+}
+
+// The pass that needs V, grad eta and grad phi~ of a row at once (ROP_N2,
+// ROP_VFW, ROP_WDOT).  grad eta . grad phi~, |grad eta|^2 and |grad phi~|^2 are
+// accumulated as the gradients come back from their transforms, in the
+// thread's own slots of shared memory; a derivative of eta waits in registers
+// for the one of phi~.  The modes of the next transform are loaded ahead of the
+// current one.  The quotient takes one residual correction (Newton) after an
+// approximate reciprocal of 1 + |grad eta|^2 >= 1: below one unit in the last
+// place, in five packed and two special operations for two values.
+struct RhsOps {
+  int8_t src[5];      // inverse transforms in the order eta_x, phi_x, eta_y, phi_y, V (indices into ops)
+  int8_t f, sx, sy;   // the operation; sponge products of phi_x and phi_y (-1: none)
+};
+__device__ __forceinline__ F2 quotient(F2 a, F2 d) {     // a / d, d >= 1 (or not finite)
+  const float2 p = parts(d);
+  const F2 r = f2(__fdividef(1.f, p.x), __fdividef(1.f, p.y));
+  const F2 q = mul(a, r);
+  return fma(fma(mul(both(-1.f), d), q, a), r, q);
+}
+template <int NX, bool EXACT>
+__global__ void __launch_bounds__(RowGeo<NX>::THREADS, 3)
+k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int rows = blockDim.x / T, nt = blockDim.x;
+  auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW;
+  unsigned long long* slot = xs + rows * G::XLEN + threadIdx.x;
+  xs += (threadIdx.x / T) * G::XLEN;
+  auto S = [&](int s, int r) -> F2& { return reinterpret_cast<F2*>(slot)[(s * R + r) * nt]; };
+  const int j = threadIdx.x % T;
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
+  const int ny = p.ny;
+  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+
+  One e[R], x[R];     // e: eta_x until phi_x is there, eta_y until phi_y
+#pragma unroll
+  for (int r = 0; r < R; ++r) e[r] = both(0.f);
+  // steps 0..4: the inverse transforms; the forward ones follow the step that
+  // forms their field.  One transform in the loop serves both.
+  constexpr bool AHEAD = kFastRow<NX, EXACT>;
+  One next[AHEAD ? R : 1];
+  auto load_ahead = [&](int step) {
+    if constexpr (AHEAD) load_modes<NX>(next, p.buf + p.ops[q.src[step]].a, p.ops[q.src[step]].b, w, ny, j);
+  };
+  load_ahead(0);
+  int s = 0, dst = -1;
+#pragma unroll 1
+  while (true) {
+    t.renew();
+    const bool forward = dst >= 0;
+    const RowOp c = p.ops[q.src[s < 5 ? s : 4]];
+    if (!forward) {
+      if constexpr (AHEAD) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = next[r];
+        twist_modes<NX>(x, t);
+        if (s < 4) load_ahead(s + 1);
+      } else {
+        inverse_input<NX, EXACT>(x, p.buf + c.a, c.b, w, ny, p.W, j, t);
+      }
+    }
+    t.run(x, xs);
+    if (forward) {
+      store_modes<NX, EXACT>(x, p.buf[dst], w, ny, p.W, j, xs, t);
+      dst = -1;
+      if (s == 5) return;
+      continue;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = conj(x[r]);
+    const int step = s++;
+    if (step == 0 || step == 2) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) e[r] = x[r];
+      continue;
+    }
+    if (step < 4) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const F2 h = x[r], g = e[r];
+        if (step == 1) {
+          S(0, r) = mul(g, g);
+          S(1, r) = mul(g, h);
+          S(2, r) = mul(h, h);
+        } else {
+          S(0, r) = fma(g, g, S(0, r));
+          S(1, r) = fma(g, h, S(1, r));
+          S(2, r) = fma(h, h, S(2, r));
+        }
+      }
+      const int so = step == 1 ? q.sx : q.sy;
+      if (so < 0) continue;
+      // w grad phi~ of the damping pressure
+      const float2* sponge = real_row(p.wgt, w, n) + j;
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = mul(x[r], f2(__ldg(sponge + r * T)));
+      dst = p.ops[so].dst;
+      continue;
+    }
+    if (c.dst != kNone && w.act) {   // physical V
+      float2* out = real_row(p.buf[c.dst], w, n) + j;
+#pragma unroll
+      for (int r = 0; r < R; ++r) out[r * T] = parts(x[r]);
+    }
+    const RowOp op = p.ops[q.f];
+    const float2* eta = p.eta.ptr ? real_row(p.eta, w, n) + j : nullptr;
+    const float2* pg = op.kind == ROP_N2 && p.pg ? reinterpret_cast<const float2*>(p.pg) + j : nullptr;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const F2 dot = S(1, r), den = add(both(1.f), S(0, r));
+      if (op.kind == ROP_VFW) {
+        x[r] = fma(x[r], den, mul(both(-1.f), dot));
+        continue;
+      }
+      const F2 num = add(x[r], dot);
+      if (op.kind == ROP_WDOT) {
+        x[r] = quotient(num, den);
+        continue;
+      }
+      x[r] = scale(0.5f, sub(quotient(mul(num, num), den), S(2, r)));
+      if (eta) x[r] = axpy(-op.coef_f, f2(__ldg(eta + r * T)), x[r]);
+      if (pg) x[r] = sub(x[r], f2(__ldg(pg + r * T)));
+    }
+    if (op.kind == ROP_WDOT) {
+      if (w.act) {
+        float2* out = real_row(p.buf[op.dst], w, n) + j;
+#pragma unroll
+        for (int r = 0; r < R; ++r) out[r * T] = parts(x[r]);
+      }
+      return;
+    }
+    dst = op.dst;
+  }
+}
+
+// ===========================================================================
+// RK pass.  blockIdx.y: the elevation (0) or the potential (1); the two need
+// nothing from each other, so a thread holds one transform at a time.
+// ===========================================================================
+template <int NX, bool EXACT, typename S>
+__global__ void __launch_bounds__(RowGeo<NX>::THREADS, 5)
+k_packed_rk(const __grid_constant__ RkParams p) {
+  using G = RowGeo<NX>;
+  using SP = StatePair<S>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + (threadIdx.x / T) * G::XLEN;
+  const int j = threadIdx.x % T;
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, 0);
+  const int ny = p.ny;
+  const bool potential = blockIdx.y != 0;
+  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+
+  const BufRef& st = potential ? p.phi0 : p.eta0;
+  const BufRef& sum = potential ? p.acc_phi : p.acc_eta;
+  const long long off = (long long)w.y * NX;
+  char* M = reinterpret_cast<char*>(st.ptr) + (w.member * st.stride + off) * 8;     // 8 bytes per value
+  char* A = reinterpret_cast<char*>(sum.ptr) + (w.member * sum.stride + off) * 8;
+  One x[R];
+  bool bad = false;
+  if (p.mode == RK_STAGE && !potential) {
+    const float2* v = real_row(p.V, w, n) + j;
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = f2(v[r * T]);
+  } else if (p.mode != RK_ENTRY) {
+    inverse_input<NX, EXACT>(x, potential && p.mode != RK_STAGE ? &p.corr_phi : &p.phit, 1, w, ny, p.W, j, t);
+    t.run(x, xs);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = conj(x[r]);
+  }
+  const float bw = (p.stage == 1 || p.stage == 4) ? 1.f : 2.f;
+  const RkScalar cdt = p.cdt, dt6 = p.dt6;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int m = j + r * T;
+    const float2 f = parts(x[r]);
+    SP e = w.act ? SP::load(M, m) : SP::zero();
+    if (p.mode == RK_STAGE) {
+      SP a = (w.act && p.stage > 1) ? SP::load(A, m) : SP::zero();
+      a.add(0, bw * f.x);
+      a.add(1, bw * f.y);
+      if (p.stage < 4) {
+        if (w.act) a.store(A, m);
+        x[r] = f2(e.template offset<float>(0, cdt, f.x), e.template offset<float>(1, cdt, f.y));
+      } else {
+        e.add_scaled(0, a, dt6);
+        e.add_scaled(1, a, dt6);
+        if (w.act) e.store(M, m);
+        bad |= !e.finite();
+        x[r] = f2(float(e.value(0)), float(e.value(1)));
+      }
+    } else {
+      if (p.mode != RK_ENTRY) {
+        e.add(0, f.x);
+        e.add(1, f.y);
+        if (p.mode == RK_CORRECT) {   // RK_OFFSET leaves the state unchanged
+          if (w.act) e.store(M, m);
+          bad |= !e.finite();
+        }
+      }
+      x[r] = f2(float(e.value(0)), float(e.value(1)));
+    }
+  }
+  if (bad && p.nonfinite) *p.nonfinite = 1;
+  if (!p.tail) return;
+  if (!potential && w.act) {
+    float2* ew = real_row(p.eta_w, w, n) + j;
+#pragma unroll
+    for (int r = 0; r < R; ++r) ew[r * T] = parts(x[r]);
+  }
+  t.run(x, xs);
+  store_modes<NX, EXACT>(x, potential ? p.phi_hat : p.eta_hat, w, ny, p.W, j, xs, t);
+}
+
+// ===========================================================================
+// Columns.  E[k] and O[k], the transforms of a column's even and odd samples
+// (one element holds both), give the modes k and k + ny2 as E +- w^k O, w =
+// e^{-2 pi i / ny}.
+// HALF: every output carries the dealias mask and at most half of the modes
+// are kept: of each pair k, k + ny2 only one can be kept, known at compile time
+// per register (r < R / 2: mode k), so only that one is formed, summed and
+// transformed back, and the sums of both accumulators stay in registers.
+// Otherwise the sums of both modes are kept in shared memory.
+// CI adjacent columns share a group of threads (lane = j CI + c), so that a
+// warp reads whole 64-byte (CI = 4) or 32-byte (CI = 2) runs.
+// Every input is copied ahead (cp.async) into the thread's own slots of shared
+// memory while the one before it is transformed, and the multipliers of an
+// input are loaded before its transform: with twelve warps per SM the loads
+// would otherwise take 40 % of the time.  No barrier is needed for either.
+// ===========================================================================
+template <int NY>
+struct ColGeo {
+  static constexpr int ny2 = NY / 2;
+  static constexpr int R = ny2 >= 128 ? 16 : (ny2 >= 8 ? 8 : 4);
+  static constexpr int T = ny2 / R;
+  static constexpr int CI = T == 16 || T == 64 ? 2 : 4;
+  static constexpr int GT = T * CI;                       // threads per group
+  static constexpr bool WARP = GT <= 32;
+  static constexpr int THREADS = 128;
+  static constexpr int MAXG = THREADS / GT;               // groups per block
+  static constexpr int CPB = CI * MAXG;                   // columns per block
+  static constexpr int SG = MAXG * CI >= 4 ? MAXG : 4 / CI;   // the same, staged form (whole tiles)
+  using F = PackedFft<Two, ny2, R, WARP, CI>;
+  using E = typename F::E;
+  static constexpr int XLEN = F::xlen() * CI + (GT < 8 ? GT : 0);   // exchange elements per group
+  static constexpr int CTW = (F::TW + 1) / 2;             // twiddles of a block, in elements of 16 bytes
+  static constexpr bool STAGEABLE = NY >= 32;
+  // whether the inputs are copied ahead: beside sums kept in shared memory the
+  // slots would cost resident blocks
+  __host__ __device__ static constexpr bool ahead(int nacc, bool half) {
+    return half;
+  }
+};
+template <int NY>
+__host__ __device__ constexpr size_t packed_col_smem(int groups, int nacc, bool half) {
+  using G = ColGeo<NY>;
+  return sizeof(typename G::E) *
+         ((size_t)G::CTW + (size_t)groups * G::XLEN + (half ? 0 : (size_t)nacc * G::R * groups * G::GT));
+}
+// the form that copies its inputs ahead
+template <int NY>
+__host__ __device__ constexpr size_t packed_col_smem_ahead(int groups, int nacc, bool half) {
+  using G = ColGeo<NY>;
+  return packed_col_smem<NY>(groups, nacc, half) +
+         (G::ahead(nacc, half) ? sizeof(typename G::E) * (size_t)G::R * groups * G::GT : 0);
+}
+// The staged form adds, 128-byte aligned, the block's tiles of four columns
+// and one mbarrier per tile.  Where that does not fit (2048 points, two sums
+// in shared memory) the tile lands in the exchange buffer instead, once the
+// transform of the input before it is done.
+template <int NY>
+__host__ __device__ constexpr bool col_stage_in_exchange(int nacc, bool half) {
+  using G = ColGeo<NY>;
+  return !G::WARP &&
+         (packed_col_smem<NY>(G::SG, nacc, half) + 127) / 128 * 128 + (size_t)(G::SG * G::CI / 4) * (NY * 32 + 8) > 227 * 1024;
+}
+template <int NY>
+__host__ __device__ constexpr size_t packed_col_smem_staged(int groups, int nacc, bool half) {
+  return (packed_col_smem<NY>(groups, nacc, half) + 127) / 128 * 128 +
+         (size_t)(groups * ColGeo<NY>::CI / 4) * ((col_stage_in_exchange<NY>(nacc, half) ? 0 : (size_t)NY * 32) + 8);
+}
+
+// a += v f i^q
+__device__ __forceinline__ F2 acc_term(F2 a, F2 v, float f, int q) {
+  const float g = q < 2 ? f : -f;
+  return (q & 1) ? fma(swp(v), f2(-g, g), a) : fma(both(g), v, a);
+}
+// (v f i^q)*
+__device__ __forceinline__ F2 conj_term(F2 v, float f, int q) {
+  const float g = q < 2 ? f : -f;
+  return (q & 1) ? mul(both(-g), swp(v)) : mul(f2(g, -g), v);
+}
+
+
+template <int NY, int NACC, bool HALF, bool STAGED>
+__global__ void __launch_bounds__(STAGED ? ColGeo<NY>::SG* ColGeo<NY>::GT : ColGeo<NY>::THREADS,
+                                  STAGED && ColGeo<NY>::SG > ColGeo<NY>::MAXG ? 1 : 3)
+k_packed_col(const __grid_constant__ ColParams p) {
+  using G = ColGeo<NY>;
+  using E = typename G::E;
+  using M = Mem<Two>;
+  constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int gave_up = (STAGED && p.err_flag) ? *(volatile int*)p.err_flag : 0;
+  float2* tab2 = reinterpret_cast<float2*>(smem_raw);
+  E* sm = reinterpret_cast<E*>(smem_raw) + G::CTW;
+  const int g = threadIdx.x / GT, l = threadIdx.x % GT, c = l % CI, j = l / CI;
+  const int groups = blockDim.x / GT;
+  E* xs = sm + g * G::XLEN + c;
+  E* sacc = sm + groups * G::XLEN + threadIdx.x;   // not HALF: [acc][r][thread]
+  constexpr bool AHEAD = !STAGED && G::ahead(NACC, HALF);
+  E* own = sacc + (HALF ? 0 : NACC) * R * blockDim.x;   // AHEAD: the next input, [r][thread]
+  const float2* tw = reinterpret_cast<const float2*>(p.tw);
+  const int col = p.col_begin + ((int)blockIdx.x * groups + g) * CI + c;
+  const bool valid = col < p.cols_total;
+  const int member = valid ? col / p.W : 0;
+  const int kx = valid ? col - member * p.W : 0;
+  const bool act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
+  const long long at0 = ((long long)(kx >> 2) * ny2 + j) * 4 + (kx & 3);   // element r at + 4 T r
+  auto field = [&](const BufRef& b) {
+    return reinterpret_cast<E*>(reinterpret_cast<float2*>(b.ptr) + (long long)member * b.stride) + at0;
+  };
+  const long long plane = (long long)p.W * ny2;   // table: modes k < ny2, then k + ny2
+  auto copy_ahead = [&](int i) {
+    if (act) {
+      const E* src = field(p.buf[i]);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        cp_async_elem(reinterpret_cast<double2*>(own + r * blockDim.x), reinterpret_cast<const double2*>(src + r * T * 4));
+    }
+    cp_async_commit();
+  };
+  if (AHEAD && p.nin > 0) copy_ahead(0);
+  G::F::fill_twiddles(tab2, tw);
+  const auto t = G::F::twiddles(tab2, j);
+  float2 wj = __ldg(tw + tw_off(NY) + j);   // w^j; w^{j + r T} = w^j e^{-2 pi i r / 2R}
+
+  // staged form: tiles of four columns (one contiguous run) and barriers
+  E* stg = nullptr;
+  unsigned long long* bar = nullptr;
+  constexpr unsigned kTileBytes = 32u * NY;
+  constexpr bool IN_EXCHANGE = STAGED && col_stage_in_exchange<NY>(NACC, HALF);
+  static_assert(!IN_EXCHANGE || sizeof(E) * G::XLEN * (4 / G::CI) >= kTileBytes, "a tile in the exchange buffer");
+  bool live = act, issuer = false;
+  auto issue = [&](int i) {
+    const char* src = reinterpret_cast<const char*>(reinterpret_cast<const float2*>(p.buf[i].ptr) +
+                                                    (long long)member * p.buf[i].stride) +
+                      (long long)(kx >> 2) * kTileBytes;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    mbar_expect_tx(bar, kTileBytes + (unsigned)p.stall_tx);
+    bulk_copy_g2s(stg, src, kTileBytes, bar);
+  };
+  if constexpr (STAGED) {
+    const int tile = (g * CI + c) / 4, tiles = groups * CI / 4;
+    unsigned char* st0 = smem_raw + (packed_col_smem<NY>(groups, NACC, HALF) + 127) / 128 * 128;
+    stg = IN_EXCHANGE ? sm + (size_t)(tile * 4 / CI) * G::XLEN : reinterpret_cast<E*>(st0 + (size_t)tile * kTileBytes);
+    bar = reinterpret_cast<unsigned long long*>(st0 + (IN_EXCHANGE ? 0 : (size_t)tiles * kTileBytes)) + tile;
+    if (gave_up) live = false;
+    issuer = (g * CI + c) % 4 == 0 && j == 0;
+    if (issuer) {
+      mbar_init(bar, 1);
+      mbar_init_fence();
+    }
+  }
+  __syncthreads();   // twiddles filled, barriers initialised
+  if constexpr (STAGED) {
+    if (issuer && live && p.nin > 0) issue(0);
+  }
+
+  F2 acc[HALF ? NACC : 1][HALF ? R : 1];
+  if constexpr (HALF) {
+#pragma unroll
+    for (int q = 0; q < NACC; ++q)
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[q][r] = both(0.f);
+  } else {
+    for (int q = 0; q < NACC; ++q)
+#pragma unroll
+      for (int r = 0; r < R; ++r) sacc[(q * R + r) * blockDim.x] = make_ulonglong2(0, 0);
+  }
+
+  float f[HALF ? R : 1];      // multipliers of a term (HALF)
+  auto load_factors = [&](const ColTerm& m) {
+    const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) f[r] = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+  };
+  // inputs, then outputs: both directions go through one transform
+#pragma unroll 1
+  for (int i = 0; i < p.nin + p.nouts; ++i) {
+    // the products of wj are formed where they are used, not kept in registers
+    asm volatile("" : "+f"(wj.x), "+f"(wj.y));
+    Two x[R];
+    const bool forward = i < p.nin;
+    if (forward) {
+      if constexpr (STAGED) {
+        if (live) live = mbar_wait_bounded(bar, (unsigned)(i & 1), p.err_flag);
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = M::from(live ? stg[(j + r * T) * 4 + (kx & 3)] : make_ulonglong2(0, 0));
+        __syncthreads();   // the staged tiles are read
+        if (!IN_EXCHANGE && issuer && live && i + 1 < p.nin) issue(i + 1);
+      } else if constexpr (AHEAD) {
+        cp_async_wait_all();
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = M::from(act ? own[r * blockDim.x] : make_ulonglong2(0, 0));
+        __syncwarp();      // the slots are read before they are filled again
+        if (i + 1 < p.nin) copy_ahead(i + 1);
+      } else {
+        const E* src = field(p.buf[i]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = M::from(act ? src[r * T * 4] : make_ulonglong2(0, 0));
+      }
+      if constexpr (HALF) {
+        if (p.term_begin[i] < p.term_begin[i + 1]) load_factors(p.terms[p.term_begin[i]]);
+      }
+    } else {
+      // even samples from the sums of the modes k and k + ny2, odd ones from
+      // their differences times w*; the inverse is the conjugate of the
+      // transform of the conjugates
+      const ColTerm m = p.outs[i - p.nin];
+      const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
+      const int ph = (m.gx + m.gy) & 3;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
+        if constexpr (HALF) {
+          const float f = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+          const F2 e = conj_term(NACC == 1 || m.acc == 0 ? acc[0][r] : acc[NACC - 1][r], f, ph);
+          x[r] = Two{e, cmul(e, r < R / 2 ? w : make_float2(-w.x, -w.y))};
+        } else {
+          const Two b = M::from(sacc[((m.acc ? R : 0) + r) * blockDim.x]);
+          const F2 y0 = conj_term(b.a, __ldg(tab + r * T * 4), ph);
+          const F2 y1 = conj_term(b.b, __ldg(tab + r * T * 4 + plane), ph);
+          x[r] = Two{add(y0, y1), cmul(sub(y0, y1), w)};
+        }
+      }
+    }
+    G::F::run(x, xs, j, t, tw);
+    if (forward) {
+      if constexpr (IN_EXCHANGE) {
+        if (issuer && live && i + 1 < p.nin) issue(i + 1);
+      }
+      F2 v[HALF ? R : 1];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
+        const F2 o = cmul(x[r].b, w);
+        if constexpr (HALF) v[r] = r < R / 2 ? add(x[r].a, o) : sub(x[r].a, o);
+        else x[r] = Two{add(x[r].a, o), sub(x[r].a, o)};   // modes (k, k + ny2)
+      }
+      for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
+        const ColTerm m = p.terms[q];
+        const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
+        const int ph = (m.gx + m.gy) & 3;
+        if constexpr (HALF) {
+          if (q > p.term_begin[i]) load_factors(m);
+          if (NACC == 1 || m.acc == 0) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[0][r] = acc_term(acc[0][r], v[r], f[r], ph);
+          } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[NACC - 1][r] = acc_term(acc[NACC - 1][r], v[r], f[r], ph);
+          }
+        } else {
+          E* a = sacc + (m.acc ? R : 0) * blockDim.x;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const Two b = M::from(a[r * blockDim.x]);
+            a[r * blockDim.x] = M::to(Two{acc_term(b.a, x[r].a, __ldg(tab + r * T * 4), ph),
+                                          acc_term(b.b, x[r].b, __ldg(tab + r * T * 4 + plane), ph)});
+          }
+        }
+      }
+      continue;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = Two{conj(x[r].a), conj(x[r].b)};
+    if (i == p.nin && act) {
+#pragma unroll 2
+      for (int q = 0; q < p.npass; ++q) {
+        const E* ps = field(p.pass[q]);
+        E v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = ps[r * T * 4];
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = add(x[r], M::from(v[r]));
+      }
+    }
+    if (act) {
+      E* dst = field(p.buf[p.outs[i - p.nin].in]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) dst[r * T * 4] = M::to(x[r]);
+    }
+  }
+}
+
+// Wide form of the HALF pass, for launches of few columns: the threads of a
+// set of columns (one warp, or the block's 128 threads where a transform needs
+// them) are there p.wide times, each copy transforms its share of the inputs,
+// leaves the kept modes in shared memory, and after one barrier every thread
+// sums some modes over all inputs, in the order of the other forms and with the
+// same operations (the same bits); the outputs are shared out the same way.
+// A pass of eight inputs and one output then takes the time of two transforms
+// instead of nine.
+template <int NY>
+struct WideGeo {
+  using G = ColGeo<NY>;
+  static constexpr int SET = G::WARP ? 32 : G::GT;      // threads of one copy
+  static constexpr int COLS = G::CI * (SET / G::GT);    // columns of a block
+  static constexpr int SX = G::XLEN * (SET / G::GT);    // exchange elements of one copy
+};
+template <int NY>
+__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nacc, int npass) {
+  using G = ColGeo<NY>;
+  using H = WideGeo<NY>;
+  const size_t modes = 8 * (size_t)nin * G::R * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
+  return 16 * ((size_t)G::CTW + (size_t)copies * H::SX) + 8 * (size_t)nacc * G::R * H::SET + (modes > pass ? modes : pass);
+}
+template <int NY>
+__global__ void __launch_bounds__(WideGeo<NY>::G::WARP ? 256 : 512)
+k_packed_col_wide(const __grid_constant__ ColParams p) {
+  using G = ColGeo<NY>;
+  using H = WideGeo<NY>;
+  using E = typename G::E;
+  using M = Mem<Two>;
+  constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2, SET = H::SET;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int copies = blockDim.x / SET, copy = threadIdx.x / SET, lane = threadIdx.x % SET;
+  const int g = lane / GT, l = lane % GT, c = l % CI, j = l / CI;
+  float2* tab2 = reinterpret_cast<float2*>(smem_raw);
+  E* xs0 = reinterpret_cast<E*>(smem_raw) + G::CTW;
+  E* xs = xs0 + (size_t)copy * H::SX + g * G::XLEN + c;
+  F2* sums = reinterpret_cast<F2*>(xs0 + (size_t)copies * H::SX);              // [acc][r][lane]
+  F2* modes = sums + (size_t)p.nacc * R * SET;                                 // [input][r][lane]
+  E* passed = reinterpret_cast<E*>(modes);                                     // later: [pass][r][lane]
+  const float2* tw = reinterpret_cast<const float2*>(p.tw);
+  const int col = p.col_begin + (int)blockIdx.x * H::COLS + g * CI + c;
+  const bool valid = col < p.cols_total;
+  const int member = valid ? col / p.W : 0;
+  const int kx = valid ? col - member * p.W : 0;
+  const bool act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
+  const long long at0 = ((long long)(kx >> 2) * ny2 + j) * 4 + (kx & 3);
+  auto field = [&](const BufRef& b) {
+    return reinterpret_cast<E*>(reinterpret_cast<float2*>(b.ptr) + (long long)member * b.stride) + at0;
+  };
+  const long long plane = (long long)p.W * ny2;
+  Two x[R];
+  auto load = [&](int i) {
+    const E* src = field(p.buf[i]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = M::from(act ? src[r * T * 4] : make_ulonglong2(0, 0));
+  };
+  if (copy < p.nin) load(copy);
+  G::F::fill_twiddles(tab2, tw);
+  const auto t = G::F::twiddles(tab2, j);
+  float2 wj = __ldg(tw + tw_off(NY) + j);
+  __syncthreads();
+#pragma unroll 1
+  for (int i0 = 0; i0 < p.nin; i0 += copies) {     // the same trips for every copy
+    asm volatile("" : "+f"(wj.x), "+f"(wj.y));
+    const int i = i0 + copy;
+    if (i0 > 0 && i < p.nin) load(i);
+    G::F::run(x, xs, j, t, tw);
+    if (i < p.nin) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
+        const F2 o = cmul(x[r].b, w);
+        modes[(i * R + r) * SET + lane] = r < R / 2 ? add(x[r].a, o) : sub(x[r].a, o);
+      }
+    }
+  }
+  __syncthreads();
+  // copy k sums the registers r = k, k + copies, ..
+  for (int r = copy; r < R; r += copies) {
+    const long long at = at0 + r * T * 4 + (r < R / 2 ? 0 : plane);
+    F2 a0 = both(0.f), a1 = a0;
+    for (int i = 0; i < p.nin; ++i) {
+      const F2 v = modes[(i * R + r) * SET + lane];
+      for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
+        const ColTerm m = p.terms[q];
+        const float f = __ldg(reinterpret_cast<const float*>(m.tab) + at);
+        const int ph = (m.gx + m.gy) & 3;
+        if (m.acc == 0) a0 = acc_term(a0, v, f, ph);
+        else a1 = acc_term(a1, v, f, ph);
+      }
+    }
+    sums[r * SET + lane] = a0;
+    if (p.nacc > 1) sums[(R + r) * SET + lane] = a1;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int o0 = 0; o0 < p.nouts; o0 += copies) {
+    asm volatile("" : "+f"(wj.x), "+f"(wj.y));
+    const int o = o0 + copy;
+    const ColTerm m = p.outs[o < p.nouts ? o : 0];
+    if (o == 0 && act) {
+      for (int q = 0; q < p.npass; ++q) {
+        const E* ps = field(p.pass[q]);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          cp_async_elem(reinterpret_cast<double2*>(passed + (q * R + r) * SET + lane),
+                        reinterpret_cast<const double2*>(ps + r * T * 4));
+      }
+      cp_async_commit();
+    }
+    if (o < p.nouts) {
+      const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
+      const int ph = (m.gx + m.gy) & 3;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
+        const float f = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+        const F2 e = conj_term(sums[((m.acc ? R : 0) + r) * SET + lane], f, ph);
+        x[r] = Two{e, cmul(e, r < R / 2 ? w : make_float2(-w.x, -w.y))};
+      }
+    }
+    G::F::run(x, xs, j, t, tw);
+    if (o < p.nouts && act) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = Two{conj(x[r].a), conj(x[r].b)};
+      if (o == 0) {
+        cp_async_wait_all();
+        for (int q = 0; q < p.npass; ++q) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) x[r] = add(x[r], M::from(passed[(q * R + r) * SET + lane]));
+        }
+      }
+      E* dst = field(p.buf[m.in]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) dst[r * T * 4] = M::to(x[r]);
+    }
+  }
+}
+
+// ===========================================================================
+// Launchers
+// ===========================================================================
+// Segments of a row pass: `per` products each, 0 keeps the operations of a row
+// in one block; returns their number (0: too many).
+inline int make_segments(RowParams& q, int per) {
+  if (per <= 0) {
+    q.seg[0] = RowSeg{0, 0, (uint8_t)q.nops};
+    return 1;
+  }
+  int ns = 0;
+  for (int o = 0; o < q.nops;) {
+    int e = o + 1;
+    while (e < q.nops && q.ops[e].kind != ROP_C2R) ++e;
+    int f = o + 1;
+    do {
+      if (ns == kMaxRowSegs) return 0;
+      const int last = f + per < e ? f + per : e;
+      q.seg[ns++] = RowSeg{(uint8_t)o, (uint8_t)f, (uint8_t)last};
+      f = last;
+    } while (f < e);
+    o = e;
+  }
+  return ns;
+}
+
+inline bool rhs_ops(const RowParams& p, RhsOps* q) {
+  int slot_op[kMaxSlots] = {-1, -1, -1, -1, -1};
+  *q = RhsOps{{-1, -1, -1, -1, -1}, -1, -1, -1};
+  for (int o = 0; o < p.nops; ++o) {
+    const RowOp& op = p.ops[o];
+    if (op.kind == ROP_C2R) slot_op[op.slot] = o;
+    else if (op.kind != ROP_PROD) q->f = (int8_t)o;
+    else if (op.slot == 3) q->sx = (int8_t)o;
+    else if (op.slot == 4) q->sy = (int8_t)o;
+  }
+  if (q->f < 0) return false;
+  const int s = p.ops[q->f].slot;
+  if (s != 0 || p.ops[q->f].a != 2) return false;
+  const int order[5] = {1, 3, 2, 4, 0};   // slots: V, eta_x, eta_y, phi_x, phi_y
+  for (int i = 0; i < 5; ++i) {
+    q->src[i] = (int8_t)slot_op[order[i]];
+    if (q->src[i] < 0) return false;
+  }
+  return true;
+}
+
+template <int NX>
+cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st) {
+  using G = RowGeo<NX>;
+  if (p.rpc < 1 || p.rpc > G::MAXR || (p.rpc * G::T) % 32 || p.row_begin < 0 || p.row_begin >= p.rows_total)
+    return cudaErrorInvalidValue;
+  const unsigned blocks = (unsigned)((p.rows_total - p.row_begin + p.rpc - 1) / p.rpc);
+  const int threads = p.rpc * G::T;
+  const bool exact = 2 * p.W == G::n;
+  RowParams q = p;
+  if (p.nslots > 1) {
+    RhsOps r;
+    if (!rhs_ops(q, &r)) return cudaErrorInvalidValue;
+    const size_t smem = row_smem<NX>(p.rpc, 3);
+    if (exact) k_packed_rhs<NX, true><<<blocks, threads, smem, st>>>(q, r);
+    else k_packed_rhs<NX, false><<<blocks, threads, smem, st>>>(q, r);
+  } else {
+    const int ns = q.nops > 0 && q.ops[0].kind == ROP_C2R ? make_segments(q, p.split) : 0;
+    if (ns == 0) return cudaErrorInvalidValue;
+    const size_t smem = row_smem<NX>(p.rpc, 0);
+    const dim3 grid(blocks, (unsigned)ns);
+    if (exact) k_packed_row<NX, true><<<grid, threads, smem, st>>>(q);
+    else k_packed_row<NX, false><<<grid, threads, smem, st>>>(q);
+  }
+  return cudaGetLastError();
+}
+
+template <int NX, bool EXACT>
+void launch_packed_rk_e(const RkParams& p, dim3 grid, size_t smem, cudaStream_t st) {
+  if (p.state64) k_packed_rk<NX, EXACT, double><<<grid, RowGeo<NX>::THREADS, smem, st>>>(p);
+  else k_packed_rk<NX, EXACT, float><<<grid, RowGeo<NX>::THREADS, smem, st>>>(p);
+}
+template <int NX>
+cudaError_t launch_packed_rk_n(const RkParams& p, cudaStream_t st) {
+  using G = RowGeo<NX>;
+  if (p.row_begin < 0 || p.row_begin >= p.rows_total) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)((p.rows_total - p.row_begin + G::MAXR - 1) / G::MAXR), 2);
+  const size_t smem = row_smem<NX>(G::MAXR, 0);
+  if (2 * p.W == G::n) launch_packed_rk_e<NX, true>(p, grid, smem, st);
+  else launch_packed_rk_e<NX, false>(p, grid, smem, st);
+  return cudaGetLastError();
+}
+
+// every output carries the dealias mask and at most half of the modes are kept
+inline bool col_half(const ColParams& p) {
+  bool half = p.ky_keep <= p.ny / 4;
+  for (int o = 0; o < p.nouts; ++o) half = half && p.outs[o].mask == 1;
+  return half;
+}
+// largest number of copies the wide form of a pass can take (0: none)
+template <int NY>
+int col_most_wide(const ColParams& p) {
+  if (!col_half(p) || p.staged) return 0;
+  const int most = (ColGeo<NY>::WARP ? 256 : 512) / WideGeo<NY>::SET;
+  for (int k = most; k >= 2; k /= 2)
+    if (packed_col_smem_wide<NY>(k, p.nin, p.nacc, p.npass) <= 227 * 1024) return k;
+  return 0;
+}
+
+template <int NY, int NACC, bool HALF>
+cudaError_t launch_packed_col_a(const ColParams& p, int groups, unsigned blocks, cudaStream_t st) {
+  using G = ColGeo<NY>;
+  if (p.staged) {
+    if constexpr (G::STAGEABLE)
+      k_packed_col<NY, NACC, HALF, true>
+          <<<blocks, groups * G::GT, packed_col_smem_staged<NY>(groups, NACC, HALF), st>>>(p);
+    else
+      return cudaErrorInvalidValue;
+  } else {
+    k_packed_col<NY, NACC, HALF, false>
+        <<<blocks, groups * G::GT, packed_col_smem_ahead<NY>(groups, NACC, HALF), st>>>(p);
+  }
+  return cudaGetLastError();
+}
+
+template <int NY>
+cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st) {
+  using G = ColGeo<NY>;
+  const int most = p.staged ? G::SG : G::MAXG;
+  const int cpb = p.cpb > 0 ? p.cpb : most * G::CI;
+  const int groups = cpb / G::CI;
+  if (cpb % G::CI || groups < 1 || groups > most || (groups * G::GT) % 32 || (p.staged && cpb % 4) ||
+      p.col_begin < 0 || p.col_begin % 4 || p.col_begin >= p.cols_total || p.W % 4 || p.nacc < 1 ||
+      p.nacc > kMaxColAcc)
+    return cudaErrorInvalidValue;
+  const unsigned blocks = (unsigned)((p.cols_total - p.col_begin + cpb - 1) / cpb);
+  const bool half = col_half(p);
+  if (p.wide > 0) {
+    using H = WideGeo<NY>;
+    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nacc, p.npass);
+    if (!half || p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
+    const unsigned wb = (unsigned)((p.cols_total - p.col_begin + H::COLS - 1) / H::COLS);
+    k_packed_col_wide<NY><<<wb, p.wide * H::SET, smem, st>>>(p);
+    return cudaGetLastError();
+  }
+  if (p.nacc == 1)
+    return half ? launch_packed_col_a<NY, 1, true>(p, groups, blocks, st)
+                : launch_packed_col_a<NY, 1, false>(p, groups, blocks, st);
+  return half ? launch_packed_col_a<NY, 2, true>(p, groups, blocks, st)
+              : launch_packed_col_a<NY, 2, false>(p, groups, blocks, st);
+}
+
+template <typename K>
+cudaError_t allow_smem(K k, size_t bytes) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <int NX, bool EXACT>
+cudaError_t prepare_packed_row_e() {
+  using G = RowGeo<NX>;
+  cudaError_t e = allow_smem(k_packed_row<NX, EXACT>, row_smem<NX>(G::MAXR, 0));
+  if (e == cudaSuccess) e = allow_smem(k_packed_rhs<NX, EXACT>, row_smem<NX>(G::MAXR, 3));
+  if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, float>, row_smem<NX>(G::MAXR, 0));
+  if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, double>, row_smem<NX>(G::MAXR, 0));
+  return e;
+}
+template <int NX>
+cudaError_t prepare_packed_row_n() {
+  const cudaError_t e = prepare_packed_row_e<NX, true>();
+  return e == cudaSuccess ? prepare_packed_row_e<NX, false>() : e;
+}
+template <int NY, int NACC, bool HALF>
+cudaError_t prepare_packed_col_a() {
+  using G = ColGeo<NY>;
+  cudaError_t e = allow_smem(k_packed_col<NY, NACC, HALF, false>, packed_col_smem_ahead<NY>(G::MAXG, NACC, HALF));
+  if constexpr (G::STAGEABLE) {
+    if (e == cudaSuccess)
+      e = allow_smem(k_packed_col<NY, NACC, HALF, true>, packed_col_smem_staged<NY>(G::SG, NACC, HALF));
+  }
+  return e;
+}
+template <int NY>
+cudaError_t prepare_packed_col_n() {
+  cudaError_t e = prepare_packed_col_a<NY, 1, true>();
+  if (e == cudaSuccess) e = prepare_packed_col_a<NY, 1, false>();
+  if (e == cudaSuccess) e = prepare_packed_col_a<NY, 2, true>();
+  if (e == cudaSuccess) e = prepare_packed_col_a<NY, 2, false>();
+  if (e == cudaSuccess) e = allow_smem(k_packed_col_wide<NY>, 227 * 1024);
+  return e;
+}
+
+}  // namespace pk
+}  // namespace sbi

@@ -68,6 +68,7 @@ struct NormParams {
   int W, ny, n;
   double* part;       // [n][kConvBlocks][4]
   double* out;        // [n][4]
+  int packed;           // fields of a packed group
 };
 
 // Device-side convergence test of the adaptive order (opt.adapt_tol > 0):
@@ -86,6 +87,7 @@ struct ConvParams {
   double tol2;
   int *conv, *orders, *notconv;
   double* red;          // [n][kConvBlocks][2]
+  int packed;             // fields of a packed group
 };
 // Pneumatic wavemaker: the surface pressure profile along x at one stage
 // time, out[x] = sum_j prof[j][x] sin(omega_j t_s + theta_j), t_s = *t + offset.
@@ -152,8 +154,11 @@ struct Group {
   double* d_crest = nullptr;    // crest position and height of one member (lazy)
   std::map<std::string, void*> mixed;
   std::map<std::string, void*> tables;   // multiplier tables by key
+  bool packed = false;            // runs on the packed kernels (packed_kernels.cuh): FP32, two-dimensional
   size_t phys_elems() const { return (size_t)nx * ny; }
-  size_t mixed_elems() const { return (size_t)ny * W; }
+  // stored columns of a mixed field (tiles of four in a packed group)
+  int columns() const { return packed ? (W + 3) / 4 * 4 : W; }
+  size_t mixed_elems() const { return (size_t)ny * columns(); }
 };
 
 // One branch of a step schedule is a Unit (schedule.h): the members [m0, m1)
@@ -290,6 +295,12 @@ RkScalar rk_scalar(double v) {
   return r;
 }
 
+// whether a column pass can take the staged (bulk-copy) form
+bool stageable(const sbi_ctx* c, const ColParams& p) {
+  if (p.packed) return packed_col_stageable(p.ny);
+  return c->fp64 ? col_stageable<double>(p.ny) : col_stageable<float>(p.ny);
+}
+
 struct Planner {
   sbi_ctx* c;
   Group& g;
@@ -345,6 +356,7 @@ struct Planner {
     r.p.ny = g.ny;
     r.p.W = g.W;
     r.p.tw = c->tw;
+    r.p.packed = g.packed;
     return r;
   }
   int add_buf(RowB& r, BufRef b) {
@@ -386,6 +398,7 @@ struct Planner {
     op.b = (uint8_t)db;
     op.c = (uint8_t)wc;
     op.coef = coef;
+    op.coef_f = (float)coef;
     op.dst = (uint8_t)add_buf(r, mref(dst));
     r.bytes += mixed_bytes();
     if (room(r)) r.p.ops[r.p.nops++] = op;
@@ -396,6 +409,7 @@ struct Planner {
     op.slot = (uint8_t)slot0;
     op.a = g.two_d ? 2 : 1;
     op.coef = if_stage > 0 ? 0.0 : c->gravity;   // the nonlinear part has no -g eta
+    op.coef_f = (float)op.coef;
     op.dst = (uint8_t)add_buf(r, mref(dst));
     r.bytes += mixed_bytes();
     if (room(r)) r.p.ops[r.p.nops++] = op;
@@ -419,6 +433,10 @@ struct Planner {
     if (room(r)) r.p.ops[r.p.nops++] = op;
   }
   int rpc_for(int nslots) {
+    if (g.packed) {
+      int tpr = 0;
+      return packed_row_geometry(g.nx, &tpr);
+    }
     const int r = c->fp64 ? row_rpc<double>(g.nx, g.W, nslots) : row_rpc<float>(g.nx, g.W, nslots);
     if (r <= 0) oom = true;
     return r > 0 ? r : 1;
@@ -438,6 +456,7 @@ struct Planner {
     }
     r.p.nslots = r.maxslot + 1;
     r.p.rpc = rpc_for(r.p.nslots);
+    if (g.packed) r.p.split = default_split(r.p);
     Pass ps{};
     ps.kind = PK_ROW;
     ps.nsize = g.nx;
@@ -449,7 +468,42 @@ struct Planner {
     return ps;
   }
 
+  // Products per segment of a packed group's row pass (0: the whole pass in one
+  // block): as few as it takes to give every SM twelve warps.
+  int default_split(const RowParams& p) const {
+    int tpr = 0;
+    packed_row_geometry(g.nx, &tpr);
+    const double warps = (double)p.rows_total * tpr / 32.0, want = 152.0 * 12.0;
+    if (p.nslots > 1 || warps >= want) return 0;
+    for (int per : {kMaxRowOps, 3, 2, 1})
+      if (per == 1 || warps * row_segments(p, per) >= want) return per;
+    return 1;
+  }
+  static int row_segments(const RowParams& p, int per) {
+    int ns = 0, prods = 0;
+    for (int o = 0; o <= p.nops; ++o)
+      if (o == p.nops || p.ops[o].kind == ROP_C2R) {
+        if (o > 0) ns += std::max(1, (prods + per - 1) / per);
+        prods = 0;
+      } else {
+        ++prods;
+      }
+    return ns;
+  }
+
   // --- column pass builder ---
+  // Copies of the wide form of a packed group's column pass (0: the plain
+  // form): doubled until every SM has eight warps, or each copy one transform.
+  int default_wide(const ColParams& p) const {
+    const int most = packed_col_most_wide(p);
+    int tpc = 0, group = 1;
+    packed_col_geometry(g.ny, &tpc, &group);
+    const double warps = (double)p.cols_total * tpc / 32.0;
+    if (most < 2 || warps * 2 > 152.0 * 8.0) return 0;
+    int k = 2;
+    while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < 152.0 * 8.0) k *= 2;
+    return k;
+  }
   struct ColIn {
     std::string name;
     std::vector<ColTerm> terms;
@@ -476,13 +530,14 @@ struct Planner {
              t.c, t.kpow, t.depth, t.gx, t.gy, t.mask, (dyn || t.depth >= 4) ? t.tau : 0.0);
     auto it = g.tables.find(key);
     if (it != g.tables.end()) return it->second;
-    void* p = dalloc(c, (size_t)g.W * g.ny * c->real_size);
+    void* p = dalloc(c, g.mixed_elems() * c->real_size);
     if (!p) {
       oom = true;
       return nullptr;
     }
     TableSpec s{};
-    s.W = g.W;
+    s.W = g.columns();
+    s.packed = g.packed;
     s.ny = g.ny;
     s.kx_keep = g.kx_keep;
     s.ky_keep = g.ky_keep;
@@ -514,10 +569,11 @@ struct Planner {
            int nacc, const std::vector<std::string>& passthrough = {}) {
     ColParams p;
     std::memset(&p, 0, sizeof(p));
-    p.W = g.W;
+    p.packed = g.packed;
+    p.W = g.columns();
     p.ny = g.ny;
     p.nx = g.nx;
-    p.cols_total = g.n * g.W;
+    p.cols_total = g.n * p.W;
     p.two_pi_over_Lx = 2.0 * M_PI / g.Lx;
     p.two_pi_over_Ly = g.two_d ? 2.0 * M_PI / g.Ly : 0.0;
     p.h0 = g.deep ? INFINITY : g.h0;
@@ -529,8 +585,7 @@ struct Planner {
     p.tw = c->tw;
     p.err_flag = c->d_flags + 1;
     p.stall_tx = c->stall_tx;
-    p.staged = (c->opt.col_staging == 1 &&
-                (c->fp64 ? col_stageable<double>(g.ny) : col_stageable<float>(g.ny))) ? 1 : 0;
+    p.staged = c->opt.col_staging == 1 && stageable(c, p) ? 1 : 0;
     const double scale = 1.0 / ((double)g.nx * g.ny);
     size_t total_terms = 0;
     for (auto& in : ins) total_terms += in.terms.size();
@@ -569,6 +624,7 @@ struct Planner {
       for (size_t q = 0; q < passthrough.size(); ++q) p.pass[q] = mref(passthrough[q]);
       p.npass = (int)passthrough.size();
     }
+    if (g.packed && !p.staged) p.wide = default_wide(p);
     Pass ps{};
     ps.kind = PK_COL;
     ps.nsize = g.ny;
@@ -709,8 +765,9 @@ struct Planner {
     for (int m = 1; m <= q.nlev && m <= 7; ++m) q.V[m - 1] = mixed(S("V%d", m));
     q.vsum = mixed("Vsum");
     q.stride = (long long)g.mixed_elems();
-    q.W = g.W;
+    q.W = g.columns();
     q.ny = g.ny;
+    q.packed = g.packed;
     q.n = g.n;
     q.level = l;
     q.last = l == c->opt.order;
@@ -865,10 +922,11 @@ struct Planner {
     p.mode = mode;
     p.stage = stage;
     p.tail = tail;
+    p.packed = g.packed;
     p.rows_total = g.n * g.ny;
     p.ny = g.ny;
     p.W = g.W;
-    {
+    if (!g.packed) {
       const int tpr = c->fp64 ? row_tpr<double>(g.nx) : row_tpr<float>(g.nx);
       p.rpc = std::max(1, kRkThreads / std::max(1, tpr));
     }
@@ -1056,7 +1114,8 @@ struct Planner {
     ps.kind = PK_NORM;
     ps.nsize = g.ny;
     ps.norm = NormParams{mixed("Ee"), mixed("Ep"), mixed("eta_m"), mixed("phi_m"),
-                         (long long)g.mixed_elems(), g.W, g.ny, g.n, g.d_part45, g.d_norm45};
+                         (long long)g.mixed_elems(), g.columns(), g.ny, g.n, g.d_part45, g.d_norm45,
+                         g.packed};
     ps.bytes = mixed_bytes() * 4;
     return ps;
   }
@@ -1323,7 +1382,12 @@ __global__ void k_conv_reset(ConvParams q, int order) {
 }
 
 // Parseval weights on the mixed layout: kx = 0 once, kx > 0 twice (the
-// conjugate modes); the common factor ny cancels in the ratio.
+// conjugate modes); the common factor ny cancels in the ratio.  A packed group
+// stores tiles of four columns, two samples of each in turn.
+__device__ __forceinline__ double parseval_weight(long long e, int ny, int packed) {
+  const bool first = packed ? e < 4LL * ny && ((e >> 1) & 3) == 0 : e < ny;
+  return first ? 1.0 : 2.0;
+}
 template <typename T>
 __global__ void k_conv_norms(ConvParams q) {
   using V = cx<T>;
@@ -1334,7 +1398,7 @@ __global__ void k_conv_norms(ConvParams q) {
     const long long ne = (long long)q.W * q.ny;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < ne;
          e += (long long)gridDim.x * blockDim.x) {
-      const double w = (e / q.ny) == 0 ? 1.0 : 2.0;
+      const double w = parseval_weight(e, q.ny, q.packed);
       double sr = 0.0, si = 0.0, lr = 0.0, li = 0.0;
       for (int l = 0; l < q.nlev; ++l) {
         const V v = reinterpret_cast<const V*>(q.V[l])[m * q.stride + e];
@@ -1435,7 +1499,7 @@ __global__ void k_norm45_partials(NormParams q) {
                      reinterpret_cast<const V*>(q.ue), reinterpret_cast<const V*>(q.up)};
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < ne;
        e += (long long)gridDim.x * blockDim.x) {
-    const double w = (e / q.ny) == 0 ? 1.0 : 2.0;
+    const double w = parseval_weight(e, q.ny, q.packed);
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const V v = src[f][m * q.stride + e];
@@ -1459,7 +1523,8 @@ __global__ void k_norm45_partials(NormParams q) {
 // once, kx > 0 twice), reduced in a fixed order.
 constexpr int kImplicitMaxIter = 64;
 template <typename T>
-__global__ void k_implicit_norms(const void* a, const void* b, long long stride, int W, int ny, double* out) {
+__global__ void k_implicit_norms(const void* a, const void* b, long long stride, int W, int ny, int packed,
+                                 double* out) {
   using V = cx<T>;
   __shared__ double sm[2][256];
   const int m = blockIdx.x;
@@ -1468,7 +1533,7 @@ __global__ void k_implicit_norms(const void* a, const void* b, long long stride,
   double d2 = 0.0, a2 = 0.0;
   const long long ne = (long long)W * ny;
   for (long long e = threadIdx.x; e < ne; e += blockDim.x) {
-    const double w = (e / ny) == 0 ? 1.0 : 2.0;
+    const double w = parseval_weight(e, ny, packed);
     const V u = pa[e], v = pb[e];
     const double dr = double(u.x) - double(v.x), di = double(u.y) - double(v.y);
     d2 += w * (dr * dr + di * di);
@@ -1591,7 +1656,10 @@ int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
     return SBI_OK;
   }
-  if (p.kind == PK_ROW) e = c->fp64 ? launch_row<double>(p.nsize, p.row, st) : launch_row<float>(p.nsize, p.row, st);
+  if (p.kind == PK_ROW && p.row.packed) e = launch_packed_row(p.nsize, p.row, st);
+  else if (p.kind == PK_COL && p.col.packed) e = launch_packed_col(p.nsize, p.col, st);
+  else if (p.kind == PK_RK && p.rk.packed) e = launch_packed_rk(p.nsize, p.rk, st);
+  else if (p.kind == PK_ROW) e = c->fp64 ? launch_row<double>(p.nsize, p.row, st) : launch_row<float>(p.nsize, p.row, st);
   else if (p.kind == PK_COL) e = c->fp64 ? launch_col<double>(p.nsize, p.col, st) : launch_col<float>(p.nsize, p.col, st);
   else e = c->fp64 ? launch_rk<double>(p.nsize, p.rk, st) : launch_rk<float>(p.nsize, p.rk, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
@@ -1656,25 +1724,30 @@ std::string pass_signature(const Pass& p) {
     for (int o = 0; o < p.row.nops; ++o) ops += "CPNWV"[p.row.ops[o].kind < 5 ? p.row.ops[o].kind : 0];
     snprintf(b, sizeof(b), "row nx=%d rows=%d slots=%d ops=%d ", p.nsize, p.row.rows_total - p.row.row_begin,
              p.row.nslots, p.row.nops);
-    return b + ops;
+    return b + ops + (p.row.packed ? " packed" : "");
   }
   snprintf(b, sizeof(b), "col ny=%d cols=%d in=%d terms=%d out=%d acc=%d pass=%d", p.nsize,
            p.col.cols_total - p.col.col_begin, p.col.nin, p.col.nterms, p.col.nouts, p.col.nacc, p.col.npass);
-  return b;
+  return p.col.packed ? std::string(b) + " packed" : std::string(b);
 }
 
 constexpr int kStagedTag = 1 << 16;
+constexpr int kWideTag = 1 << 18;
+constexpr int kSplitTag = 1 << 16;
 
 int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
   if (!c->opt.autotune || (p.kind != PK_ROW && p.kind != PK_COL)) return SBI_OK;
   // a column choice packs the columns per block and the staged form (bulk
-  // copies of the inputs into shared memory) as cpb + kStagedTag * staged
+  // copies of the inputs into shared memory) as cpb + kStagedTag * staged; a
+  // row choice the rows per block and, in packed groups, the products per segment
   auto apply = [&](Pass& q, int v) {
     if (q.kind == PK_ROW) {
-      q.row.rpc = v;
+      q.row.rpc = v % kSplitTag;
+      q.row.split = v / kSplitTag;
     } else {
       q.col.cpb = v % kStagedTag;
-      q.col.staged = v / kStagedTag;
+      q.col.staged = v % kWideTag / kStagedTag;
+      q.col.wide = v / kWideTag;
     }
   };
   const std::string key = pass_signature(p);
@@ -1685,26 +1758,44 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
   }
   std::vector<int> cand;
   int deflt = 0;
-  if (p.kind == PK_ROW) {
+  if (p.kind == PK_ROW && p.row.packed) {
+    int tpr = 0;
+    packed_row_geometry(p.nsize, &tpr);
+    deflt = p.row.rpc + kSplitTag * p.row.split;
+    for (int r = p.row.rpc; r >= 1 && cand.size() < 3; r /= 2)
+      if (r * tpr % 32 == 0) cand.push_back(r + kSplitTag * p.row.split);
+    if (p.row.nslots == 1)
+      for (int per : {0, kMaxRowOps, 3, 2, 1})
+        if (per != p.row.split) cand.push_back(p.row.rpc + kSplitTag * per);
+  } else if (p.kind == PK_ROW) {
     const int tpr = c->fp64 ? row_tpr<double>(p.nsize) : row_tpr<float>(p.nsize);
     deflt = p.row.rpc;
     for (int r = deflt; r >= 1 && cand.size() < 4; r /= 2)
       if (tpr > 0 && (r * tpr) % 32 == 0) cand.push_back(r);
   } else {
-    int tpc = 0;
-    const int cpb = c->fp64 ? col_geometry<double>(p.nsize, &tpc) : col_geometry<float>(p.nsize, &tpc);
-    const int base = p.col.cpb > 0 ? p.col.cpb : cpb;
-    deflt = base + kStagedTag * p.col.staged;
+    int tpc = 0, group = 1;
+    const int cpb = p.col.packed ? packed_col_geometry(p.nsize, &tpc, &group)
+                               : (c->fp64 ? col_geometry<double>(p.nsize, &tpc) : col_geometry<float>(p.nsize, &tpc));
+    // the staged form of a packed group takes whole tiles of four columns
+    auto base = [&](int staged) {
+      const int b = p.col.cpb > 0 ? p.col.cpb : cpb;
+      return staged && p.col.packed ? std::max(b, 4) : b;
+    };
+    deflt = base(p.col.staged) + kStagedTag * p.col.staged + kWideTag * p.col.wide;
     // the staged form is a candidate where the option leaves the choice open
-    const bool stg = c->opt.col_staging == 0 &&
-                     (c->fp64 ? col_stageable<double>(p.nsize) : col_stageable<float>(p.nsize));
+    const bool stg = c->opt.col_staging == 0 && stageable(c, p.col);
     for (int staged = p.col.staged; staged <= (stg ? 1 : p.col.staged); ++staged) {
       int k = 0;
-      for (int v = base; v >= 1 && k < 3; v /= 2)
-        if (tpc > 0 && (v * tpc) % 32 == 0) {
+      for (int v = base(staged); v >= 1 && k < 3; v /= 2)
+        if (tpc > 0 && (v * tpc) % 32 == 0 && v % group == 0 && !(staged && p.col.packed && v % 4)) {
           cand.push_back(v + kStagedTag * staged);
           ++k;
         }
+    }
+    if (p.col.packed && !p.col.staged) {   // copies of the wide form
+      const int most = packed_col_most_wide(p.col);
+      for (int k = 2; k <= most && k < 2 * std::max(p.col.nin, p.col.nouts); k *= 2)
+        cand.push_back(base(0) + kWideTag * k);
     }
   }
   int best = deflt;
@@ -1847,8 +1938,8 @@ Pass slice_pass(const Pass& p, const Group& g, int m0, int m1) {
     q.row.row_begin = m0 * g.ny;
     q.row.rows_total = m1 * g.ny;
   } else if (p.kind == PK_COL) {
-    q.col.col_begin = m0 * g.W;
-    q.col.cols_total = m1 * g.W;
+    q.col.col_begin = m0 * g.columns();
+    q.col.cols_total = m1 * g.columns();
   } else {
     q.rk.row_begin = m0 * g.ny;
     q.rk.rows_total = m1 * g.ny;
@@ -2552,6 +2643,7 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
       g.kx_keep = std::max(g.kx_keep, 1);
       g.ky_keep = std::max(g.ky_keep, 1);
       g.W = g.kx_keep;
+      g.packed = g.two_d && !c->fp64;
       c->groups.push_back(g);
     }
     Group& g = c->groups[sig[i]];
@@ -2580,8 +2672,11 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
   if (!c->d_flags) { c->err = "device allocation failed"; return bail(SBI_ENOMEM); }
 
   for (auto& g : c->groups) {
-    cudaError_t e = c->fp64 ? prepare_row_kernels<double>(g.nx) : prepare_row_kernels<float>(g.nx);
-    if (e == cudaSuccess) e = c->fp64 ? prepare_col_kernels<double>(g.ny) : prepare_col_kernels<float>(g.ny);
+    cudaError_t e = g.packed ? prepare_packed_row_kernels(g.nx)
+                           : (c->fp64 ? prepare_row_kernels<double>(g.nx) : prepare_row_kernels<float>(g.nx));
+    if (e == cudaSuccess)
+      e = g.packed ? prepare_packed_col_kernels(g.ny)
+                 : (c->fp64 ? prepare_col_kernels<double>(g.ny) : prepare_col_kernels<float>(g.ny));
     if (e != cudaSuccess) { cuda_fail(c, e, "kernel setup"); return bail(SBI_ECUDA); }
     int rc = init_group(c, g);
     if (rc) return bail(rc);
@@ -2965,8 +3060,8 @@ int sbi_vertical_velocity_implicit(sbi_ctx* c, int member, int iterations, doubl
     const void* dst = pl.mixed(it % 2 ? "IVb" : "IVa");
     const void* src = pl.mixed(it == 0 ? "V1" : (it % 2 ? "IVa" : "IVb"));
     double* out = g.d_implicit + (size_t)it * g.n * 2;
-    if (c->fp64) k_implicit_norms<double><<<g.n, 256, 0, c->stream>>>(dst, src, stride, g.W, g.ny, out);
-    else k_implicit_norms<float><<<g.n, 256, 0, c->stream>>>(dst, src, stride, g.W, g.ny, out);
+    if (c->fp64) k_implicit_norms<double><<<g.n, 256, 0, c->stream>>>(dst, src, stride, g.columns(), g.ny, g.packed, out);
+    else k_implicit_norms<float><<<g.n, 256, 0, c->stream>>>(dst, src, stride, g.columns(), g.ny, g.packed, out);
     CK(cudaGetLastError(), "implicit norms");
   }
   rc = run(fin);
@@ -3521,10 +3616,17 @@ int sbi_autotune_report(const sbi_ctx* cc, char* buf, size_t cap, size_t* needed
     const auto& t = cc->tuned.at(key);
     char line[96];
     const bool row = key.rfind("row", 0) == 0;
-    // column choices: "s" marks the staged form (inputs by bulk copies)
-    snprintf(line, sizeof(line), ": %s %d%s/%d%s %.4f ms\n", row ? "rpc" : "cpb",
-             row ? t.choice : t.choice % kStagedTag, (!row && t.choice >= kStagedTag) ? "s" : "",
-             row ? t.deflt : t.deflt % kStagedTag, (!row && t.deflt >= kStagedTag) ? "s" : "", t.ms);
+    // column choices: "s" marks the staged form (inputs by bulk copies), "w<k>"
+    // k copies of the wide form; row choices: "x<k>", k products per segment
+    auto shape = [&](int v) {
+      std::string o = std::to_string(v % kStagedTag);
+      if (row && v >= kSplitTag) o += "x" + std::to_string(v / kSplitTag);
+      if (!row && v % kWideTag >= kStagedTag) o += "s";
+      if (!row && v >= kWideTag) o += "w" + std::to_string(v / kWideTag);
+      return o;
+    };
+    snprintf(line, sizeof(line), ": %s %s/%s %.4f ms\n", row ? "rpc" : "cpb", shape(t.choice).c_str(),
+             shape(t.deflt).c_str(), t.ms);
     out += key + line;
   }
   *needed = out.size();

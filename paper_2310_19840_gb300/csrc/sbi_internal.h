@@ -15,6 +15,10 @@
 // multipliers k^p D(k) (i kx)^gx (i ky)^gy with D in {1, tanh(k h0),
 // sech(k h0), Lambda(k)} and sums them into accumulators, masks, and
 // transforms the outputs back along y.
+//
+// Two-dimensional FP32 groups ("packed" groups) run every pass in packed
+// arithmetic, on mixed fields in the order of packed_kernels.cuh; their columns
+// are counted up to W rounded to four.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -55,8 +59,16 @@ struct RowOp {
   uint8_t c;
   uint8_t dst;
   uint16_t pad_;
-  uint32_t pad2_;
+  float coef_f;   // coef in FP32 (packed groups)
   double coef;    // PROD: scalar coefficient; N2: gravity
+};
+
+// One segment of a packed group's row pass (the operations [begin, end) that a
+// block runs, begin an inverse transform; products before `first` are formed
+// but not transformed).
+constexpr int kMaxRowSegs = kMaxRowOps;
+struct RowSeg {
+  uint8_t begin, first, end;
 };
 
 struct BufRef {
@@ -81,6 +93,9 @@ struct RowParams {
   BufRef buf[kMaxRowBufs];
   RowOp ops[kMaxRowOps];
   const void* tw;
+  int packed;             // a packed group's pass
+  int split;            // packed groups: products per segment (0: all operations in one block)
+  RowSeg seg[kMaxRowSegs];   // set by the launcher
 };
 
 // One multiplier of a column pass: c k^p D(k) (i kx)^gx (i ky)^gy, times the
@@ -127,6 +142,8 @@ struct ColParams {
   ColTerm outs[kMaxColOuts];
   BufRef buf[kMaxColBufs];
   const void* tw;
+  int packed;               // a packed group's pass (W counts the padded columns)
+  int wide;                 // packed groups: copies of the wide form (0: one thread set per column)
   int stall_tx;             // test hook: bytes a staged copy's barrier expects beyond the copy
                             // (0; > 0 makes every wait run out, to test the timeout path)
 };
@@ -137,6 +154,7 @@ struct TableSpec {
   double two_pi_over_Lx, two_pi_over_Ly, h0, filt_kf, filt_beta2, c;
   double tau, gravity;  // propagator entries (depth 4..7)
   int kpow, depth, gx, gy, mask;
+  int packed;             // order of a packed group's table (W: padded columns)
 };
 
 // RK_ENTRY: working copies of the state; RK_STAGE: a classical RK4 stage;
@@ -175,6 +193,7 @@ struct RkParams {
   BufRef eta_hat, phi_hat;      // mixed working spectra (T complex)
   int* nonfinite;       // set to 1 when the new state holds NaN/Inf
   const void* tw;
+  int packed;             // a packed group's pass
 };
 
 // Launchers (one instantiation per real type and size, selected at run time).
@@ -200,5 +219,18 @@ template <typename T> int row_tpr(int nx);
 template <typename T> int col_geometry(int ny, int* tpc);
 // whether columns of ny points can take the staged (bulk-copy) form
 template <typename T> bool col_stageable(int ny);
+
+// The same for packed groups (packed_kernels.cuh).  packed_row_geometry: largest rows
+// per block and threads per row; packed_col_geometry: largest columns per
+// block, columns that share a group of threads and threads per column.
+cudaError_t prepare_packed_row_kernels(int nx);
+cudaError_t prepare_packed_col_kernels(int ny);
+cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st);
+cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st);
+cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st);
+int packed_row_geometry(int nx, int* threads);
+int packed_col_geometry(int ny, int* tpc, int* group);
+bool packed_col_stageable(int ny);
+int packed_col_most_wide(const ColParams& p);   // most copies of the wide form (0: not possible)
 
 }  // namespace sbi
