@@ -1,4 +1,5 @@
-// Column pass instantiations of packed groups (two-dimensional, FP32).
+// Column pass instantiations of packed groups (two-dimensional, FP32) and the
+// FP32 multiplier tables.
 #include "packed_kernels.cuh"
 
 namespace sbi {
@@ -31,5 +32,8 @@ int packed_col_most_wide(const ColParams& p) {
 #define SBI_CASE(N) case N: return pk::col_most_wide<N>(p);
   SBI_SWITCH(ny, SBI_CASE, 0)
 #undef SBI_CASE
+}
+template <> cudaError_t launch_coef_table<float>(void* out, const TableSpec& s, cudaStream_t st) {
+  return launch_coef_table_impl<float>(out, s, st);
 }
 }  // namespace sbi

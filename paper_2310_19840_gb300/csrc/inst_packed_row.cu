@@ -1,4 +1,5 @@
-// Row and RK pass instantiations of packed groups (two-dimensional, FP32).
+// Row and RK pass instantiations of packed groups (two-dimensional, FP32) and
+// the FP32 state conversions.
 #include "packed_kernels.cuh"
 
 namespace sbi {
@@ -32,5 +33,9 @@ int packed_row_geometry(int nx, int* threads) {
 #define SBI_CASE(N) case N: *threads = pk::RowGeo<N>::T; return pk::RowGeo<N>::MAXR;
   SBI_SWITCH(nx, SBI_CASE, 0)
 #undef SBI_CASE
+}
+template <> cudaError_t state_convert<float>(const void* src, void* dst, long long n, bool to_double,
+                                             cudaStream_t st) {
+  return state_convert_impl<float>(src, dst, n, to_double, st);
 }
 }  // namespace sbi

@@ -1181,10 +1181,6 @@ cudaError_t launch_col_n(const ColParams& p, cudaStream_t st) {
 
 #define SBI_FOR_NX(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096)
 #define SBI_FOR_NY(X) X(1) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
-// column lengths of the plain family: one-dimensional groups, and in FP64 all
-// (two-dimensional FP32 groups run on packed_kernels.cuh)
-template <typename T, int NY>
-inline constexpr bool kPlainCol = NY == 1 || sizeof(T) == 8;
 
 template <typename T>
 cudaError_t prepare_row_impl(int nx) {
@@ -1199,10 +1195,7 @@ cudaError_t prepare_row_impl(int nx) {
 template <typename T>
 cudaError_t prepare_col_impl(int ny) {
   switch (ny) {
-#define SBI_CASE(N) \
-  case N:           \
-    if constexpr (kPlainCol<T, N>) return prepare_ny<T, N>(); \
-    else return cudaErrorInvalidValue;
+#define SBI_CASE(N) case N: return prepare_ny<T, N>();
     SBI_FOR_NY(SBI_CASE)
 #undef SBI_CASE
     default: return cudaErrorInvalidValue;
@@ -1232,10 +1225,7 @@ cudaError_t launch_rk_impl(int nx, const RkParams& p, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_col_impl(int ny, const ColParams& p, cudaStream_t st) {
   switch (ny) {
-#define SBI_CASE(N) \
-  case N:           \
-    if constexpr (kPlainCol<T, N>) return launch_col_n<T, N>(p, st); \
-    else return cudaErrorInvalidValue;
+#define SBI_CASE(N) case N: return launch_col_n<T, N>(p, st);
     SBI_FOR_NY(SBI_CASE)
 #undef SBI_CASE
     default: return cudaErrorInvalidValue;

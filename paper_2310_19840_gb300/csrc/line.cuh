@@ -1,0 +1,273 @@
+// line.cuh - whole steps of one-dimensional FP32 members in one launch.
+//
+// A one-dimensional member is one row of 16 to 4096 points: a pass over it is
+// far below a launch in work, and a step of some 64 dependent launches took 7
+// to 15 us each.  Here one block per member runs the whole list of passes (a
+// program of phases, line.h), a block barrier between phases.  Every transform
+// of a phase goes to its own group of threads (packed.cuh), so the products of
+// a level are transformed side by side; physical fields stay in shared memory,
+// mixed fields (8 KB at most) in global memory, where the block finds them in
+// its L1 and L2.  What bounds it is the chain of dependent transforms: about 17
+// per right-hand side.
+// Measured (GB300, a step): 256 points 420 us in 64 launches -> see DESIGN's
+// table for the current figures.
+#pragma once
+
+#include "line.h"
+#include "packed_kernels.cuh"
+
+namespace sbi {
+namespace pk {
+
+constexpr int kLineThreads = 512;
+
+template <int NX>
+__host__ __device__ constexpr size_t line_smem(int program_bytes) {
+  using G = RowGeo<NX>;
+  return 8 * ((size_t)G::RTW + (size_t)(kLineThreads / G::T) * G::XLEN + (size_t)kLineSlots * G::n) +
+         (program_bytes + 15) / 16 * 16;
+}
+
+template <int NX, bool EXACT>
+__global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant__ LineParams p) {
+  using G = RowGeo<NX>;
+  using SP = StatePair<float>;
+  constexpr int n = G::n, R = G::R, T = G::T, GROUPS = kLineThreads / T;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  auto* xs0 = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW;
+  F2* slots = reinterpret_cast<F2*>(xs0 + GROUPS * G::XLEN);               // [slot][m]
+  unsigned char* prog = reinterpret_cast<unsigned char*>(slots + kLineSlots * n);
+  const int tid = threadIdx.x, g = tid / T, j = tid % T;
+  auto* xs = xs0 + g * G::XLEN;
+  const int member = p.member0 + (int)blockIdx.x;
+  for (int i = tid; i < (p.bytes + 15) / 16; i += kLineThreads)
+    reinterpret_cast<uint4*>(prog)[i] = reinterpret_cast<const uint4*>(p.program)[i];
+  const LineHeader& H = *reinterpret_cast<const LineHeader*>(prog);
+  __syncthreads();
+  RowTwiddles<NX> t(H.tw, reinterpret_cast<float2*>(smem_raw), j);
+  const LinePhase* phases = reinterpret_cast<const LinePhase*>(prog + H.phases);
+  const LineJob* jobs = reinterpret_cast<const LineJob*>(prog + H.jobs);
+  const LineTerm* terms = reinterpret_cast<const LineTerm*>(prog + H.terms);
+  const BufRef* bufs = reinterpret_cast<const BufRef*>(prog + H.bufs);
+  const int W = H.W;
+  auto mixed = [&](int b) { return reinterpret_cast<F2*>(bufs[b].ptr) + (long long)member * bufs[b].stride; };
+  auto real = [&](int b) {
+    return reinterpret_cast<F2*>(reinterpret_cast<float*>(bufs[b].ptr) + (long long)member * bufs[b].stride);
+  };
+
+#pragma unroll 1
+  for (int ip = 0; ip < H.nphases; ++ip) {
+    const LinePhase& P = phases[ip];
+    if (P.active && P.active[member] == 0) continue;      // the whole block
+    if (P.type == LP_INVERSE || P.type == LP_FORWARD) {
+      const bool inverse = P.type == LP_INVERSE;
+#pragma unroll 1
+      for (int first = P.begin; first < P.end; first += GROUPS) {
+        t.renew();
+        const bool valid = first + g < P.end;
+        if (G::WARP && first + (tid & ~31) / T >= P.end) break;   // a warp without a job
+        const LineJob job = jobs[valid ? first + g : P.begin];
+        One x[R];
+        if (inverse) {
+          // modes k < W and n - k < W of the sum of the sources (inverse_input)
+          if constexpr (kFastRow<NX, EXACT>) {
+#pragma unroll 1
+            for (int q = 0; q < job.nsrc; ++q) {
+              const F2* src = mixed(job.buf + q);
+#pragma unroll
+              for (int r = 0; r < R; ++r) {
+                const int k = j + r * T;
+                One v = both(0.f);
+                if (r < R / 2) v = src[k];
+                else if (r > R / 2 || j != 0) v = src[n - k];
+                x[r] = q == 0 ? v : add(x[r], v);
+              }
+            }
+            twist_modes<NX>(x, t);
+          } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int k = j + r * T, kk = n - k;
+              One a = both(0.f), b = both(0.f);
+              for (int q = 0; q < job.nsrc; ++q) {
+                const F2* src = mixed(job.buf + q);
+                if (k < W) a = add(a, src[k]);
+                if (k > 0 && kk < W) b = add(b, src[kk]);
+              }
+              const float2 e = __ldg(t.tw + tw_off(NX) + k);
+              const One o = cmul(sub_conj(a, b), make_float2(e.x, -e.y));
+              x[r] = conj(addi(add_conj(a, b), o));
+            }
+          }
+        } else {
+          const F2* s = slots + job.slot * n + j;
+          const F2* eta = P.eta >= 0 ? real(P.eta) + j : nullptr;
+          if (job.op == ROP_PROD) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) x[r] = s[r * T];
+            for (int f = 0; f < 3; ++f) {
+              const int e = f == 0 ? job.ea : (f == 1 ? job.eb : job.ew);
+              if (e == 0) continue;
+              const int b = f == 0 ? P.eta : (f == 1 ? P.delta : P.wgt);
+              const F2* src = real(b) + j;
+              One v[R];
+#pragma unroll
+              for (int r = 0; r < R; ++r) v[r] = src[r * T];
+              times_field<R>(x, v, e);
+            }
+            if (job.coef != 1.f) {
+#pragma unroll
+              for (int r = 0; r < R; ++r) x[r] = scale(job.coef, x[r]);
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const F2 v = s[r * T], ex = s[n + r * T], px = s[2 * n + r * T];
+              const F2 dot = mul(ex, px), den = fma(ex, ex, both(1.f));
+              if (job.op == ROP_VFW) {
+                x[r] = fma(v, den, mul(both(-1.f), dot));
+              } else {
+                const F2 num = add(v, dot);
+                x[r] = scale(0.5f, sub(quotient(mul(num, num), den), mul(px, px)));
+                if (eta) x[r] = axpy(-job.coef, eta[r * T], x[r]);
+                if (job.pg) x[r] = sub(x[r], slots[5 * n + j + r * T]);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        t.run(x, xs);
+        if (inverse) {
+          if (valid) {
+            F2* s = slots + job.slot * n + j;
+            F2* out = job.phys >= 0 ? real(job.phys) + j : nullptr;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const F2 v = conj(x[r]);
+              s[r * T] = v;
+              if (out) out[r * T] = v;
+            }
+          }
+        } else {
+          One X[kKept<NX, EXACT>];
+          kept_modes<NX, EXACT>(x, X, W, j, xs, t);
+          if (valid) {
+            F2* out = mixed(job.buf) + j;
+#pragma unroll
+            for (int r = 0; r < kKept<NX, EXACT>; ++r)
+              if (kFastRow<NX, EXACT> || j + r * T < W) out[r * T] = X[r];
+          }
+          if constexpr (!G::WARP) __syncthreads();
+        }
+      }
+    } else if (P.type == LP_COL) {
+      // outputs may overwrite inputs of the same mode: every load of a mode
+      // comes before its stores, by the same thread
+      for (int k = tid; k < W; k += kLineThreads) {
+        F2 a0 = both(0.f), a1 = a0;
+#pragma unroll 4
+        for (int q = P.begin; q < P.end; ++q) {
+          const LineTerm m = terms[q];
+          const F2 v = mixed(m.buf)[k];
+          const float f = __ldg(reinterpret_cast<const float*>(m.tab) + k);
+          if (m.acc == 0) a0 = acc_term(a0, v, f, m.ph);
+          else a1 = acc_term(a1, v, f, m.ph);
+        }
+        F2 extra = both(0.f);
+        for (int q = P.pass_begin; q < P.pass_end; ++q) extra = add(extra, mixed(q)[k]);
+        for (int q = P.out_begin; q < P.out_end; ++q) {
+          const LineTerm m = terms[q];
+          const float f = __ldg(reinterpret_cast<const float*>(m.tab) + k);
+          const F2 o = acc_term(both(0.f), m.acc == 0 ? a0 : a1, f, m.ph);
+          mixed(m.buf)[k] = q == P.out_begin && P.pass_begin < P.pass_end ? add(o, extra) : o;
+        }
+      }
+    } else if (P.type == LP_RK) {
+      const RkParams& q = reinterpret_cast<const RkParams*>(prog + H.rks)[P.out_begin];
+      bool bad = false;
+      const float bw = (q.stage == 1 || q.stage == 4) ? 1.f : 2.f;
+      const RkScalar cdt = q.cdt, dt6 = q.dt6;
+      for (int i = tid; i < 2 * n; i += kLineThreads) {
+        const bool potential = i >= n;
+        const int m = potential ? i - n : i;
+        const BufRef& st = potential ? q.phi0 : q.eta0;
+        const BufRef& sum = potential ? q.acc_phi : q.acc_eta;
+        char* M = reinterpret_cast<char*>(st.ptr) + (long long)member * st.stride * 8;      // 8 bytes per value
+        char* A = reinterpret_cast<char*>(sum.ptr) + (long long)member * sum.stride * 8;
+        float2 f = make_float2(0.f, 0.f);
+        if (q.mode == RK_STAGE && !potential)
+          f = parts(reinterpret_cast<const F2*>(reinterpret_cast<const float*>(q.V.ptr) + (long long)member * q.V.stride)[m]);
+        else if (q.mode != RK_ENTRY)
+          f = parts(slots[(potential ? 0 : 1) * n + m]);
+        float2 res;
+        auto update = [&](auto e) {
+          using S = decltype(e);
+          e = S::load(M, m);
+          if (q.mode == RK_STAGE) {
+            S a = q.stage > 1 ? S::load(A, m) : S::zero();
+            a.add(0, bw * f.x);
+            a.add(1, bw * f.y);
+            if (q.stage < 4) {
+              a.store(A, m);
+              res = make_float2(e.template offset<float>(0, cdt, f.x), e.template offset<float>(1, cdt, f.y));
+              return;
+            }
+            e.add_scaled(0, a, dt6);
+            e.add_scaled(1, a, dt6);
+            e.store(M, m);
+            bad |= !e.finite();
+          } else if (q.mode != RK_ENTRY) {
+            e.add(0, f.x);
+            e.add(1, f.y);
+            if (q.mode == RK_CORRECT) {   // RK_OFFSET leaves the state unchanged
+              e.store(M, m);
+              bad |= !e.finite();
+            }
+          }
+          res = make_float2(float(e.value(0)), float(e.value(1)));
+        };
+        if (q.state64) update(StatePair<double>::zero());
+        else update(SP::zero());
+        if (q.tail) {
+          slots[(potential ? 3 : 2) * n + m] = f2(res);
+          if (!potential)
+            reinterpret_cast<F2*>(reinterpret_cast<float*>(q.eta_w.ptr) + (long long)member * q.eta_w.stride)[m] = f2(res);
+        }
+      }
+      if (bad && q.nonfinite) *q.nonfinite = 1;
+    } else if (P.type == LP_WDOT) {
+      F2* out = real(P.dst);
+      for (int m = tid; m < n; m += kLineThreads) {
+        const F2 ex = slots[n + m];
+        out[m] = quotient(fma(ex, slots[2 * n + m], slots[m]), fma(ex, ex, both(1.f)));
+      }
+    } else {   // LP_WMK: FP64 sums and sines, rounded once
+      const LineWmk& q = reinterpret_cast<const LineWmk*>(prog + H.wmks)[P.out_begin];
+      const double time = *q.t + q.offset;
+      for (int x = tid; x < 2 * n; x += kLineThreads) {
+        double acc = 0.0;
+        for (int i = 0; i < q.J; ++i) acc += q.prof[(size_t)i * 2 * n + x] * sin(q.omega[i] * time + q.phase[i]);
+        reinterpret_cast<float*>(slots + 5 * n)[x] = float(acc);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <int NX>
+cudaError_t prepare_line_n() {
+  const cudaError_t e = allow_smem(k_line<NX, true>, line_smem<NX>(kLineMaxBytes));
+  return e == cudaSuccess ? allow_smem(k_line<NX, false>, line_smem<NX>(kLineMaxBytes)) : e;
+}
+template <int NX>
+cudaError_t launch_line_n(const LineParams& p, cudaStream_t st) {
+  if (p.member0 < 0 || p.member1 <= p.member0 || p.bytes > kLineMaxBytes) return cudaErrorInvalidValue;
+  const size_t smem = line_smem<NX>(p.bytes);
+  const unsigned blocks = (unsigned)(p.member1 - p.member0);
+  if (p.exact) k_line<NX, true><<<blocks, kLineThreads, smem, st>>>(p);
+  else k_line<NX, false><<<blocks, kLineThreads, smem, st>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace pk
+}  // namespace sbi

@@ -1,0 +1,70 @@
+// line.h - programs of the one-dimensional FP32 step (line.cuh): a list of
+// phases that one block runs for one member, a block barrier between them.
+#pragma once
+
+#include "sbi_internal.h"
+
+namespace sbi {
+
+constexpr int kLineSlots = 6;          // physical fields held in shared memory
+constexpr int kLineMaxBytes = 40960;   // largest program (it is copied into shared memory)
+
+enum LinePhaseType : uint8_t {
+  LP_INVERSE = 0,   // jobs: mixed sums -> slots, one transform each
+  LP_FORWARD = 1,   // jobs: products of slots -> mixed, one transform each
+  LP_COL = 2,       // per mode: sums of terms, outputs, pass-through sums
+  LP_RK = 3,        // state update; the new working values go to slots 2 (eta) and 3 (phi)
+  LP_WDOT = 4,      // physical dst <- (V + eta_x phi_x) / (1 + eta_x^2)
+  LP_WMK = 5,       // surface pressure profile -> slot 5
+};
+
+// One transform.  Inverse: slot <- inverse of the sum of bufs [buf, buf + nsrc),
+// also written to the physical bufs[phys] when phys >= 0.  Forward: bufs[buf] <-
+// transform of coef eta^ea delta^eb w^ew slot (op ROP_PROD), or of the
+// dynamic-condition / kinematic forms of slots slot, slot + 1, slot + 2 = V,
+// eta_x, phi_x (op ROP_N2, ROP_VFW).
+struct LineJob {
+  uint8_t op, slot, ea, eb, ew, nsrc;
+  uint8_t pg;            // ROP_N2: subtract the pressure of slot 5
+  uint8_t pad_;
+  int16_t buf, phys;
+  float coef;
+};
+// One multiplier of a column sum or output: src/dst is bufs[buf].
+struct LineTerm {
+  const void* tab;
+  int16_t buf;
+  uint8_t acc, ph;       // accumulator, power of i
+  int32_t pad_;
+};
+struct LinePhase {
+  uint8_t type;
+  int16_t begin, end;          // jobs; LP_COL: terms
+  int16_t out_begin, out_end;  // LP_COL: outputs (terms); LP_RK: index of the RkParams in out_begin
+  int16_t pass_begin, pass_end;  // LP_COL: pass-through bufs, added to the first output
+  int16_t eta, delta, wgt;     // physical bufs (-1: none)
+  int16_t dst;                 // LP_WDOT
+  const int* active;           // per-member flags (nullptr: every member runs the phase)
+};
+struct LineWmk {
+  const double *prof, *omega, *phase, *t;
+  double offset;
+  int J;
+};
+struct LineHeader {
+  int bytes;                   // of the whole program
+  int nphases, phases, jobs, terms, bufs, rks, wmks;   // byte offsets of the arrays
+  int W;
+  const void* tw;
+};
+struct LineParams {
+  const void* program;
+  int bytes;
+  int exact;                   // half of the modes kept
+  int member0, member1;        // members of this launch (one block each)
+};
+
+cudaError_t prepare_line_kernels(int nx);
+cudaError_t launch_line(int nx, const LineParams& p, cudaStream_t st);
+
+}  // namespace sbi

@@ -210,20 +210,20 @@ __device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const Buf
   }
 }
 
-// Output side of the packed forward real transform of a row, Z in x: stores
-// the kept modes X[k] = 1/2 (Z[k] + Z[n-k]*) - i/2 e^{-2 pi i k / NX} (Z[k] -
-// Z[n-k]*), k < W.  Z[n - k] sits in lane (T - j) mod T, register R - 1 - r
+// Output side of the packed forward real transform of a row, Z in x: the kept
+// modes X[k] = 1/2 (Z[k] + Z[n-k]*) - i/2 e^{-2 pi i k / NX} (Z[k] - Z[n-k]*),
+// k = j + r T < W.  Z[n - k] sits in lane (T - j) mod T, register R - 1 - r
 // (thread 0: its own register (R - r) mod R): a shuffle, or, for rows of
 // several warps, a pass through the exchange buffer.
 template <int NX, bool EXACT>
-__device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const BufRef& dst, const Row& w, int ny,
-                                            int W, int j, typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
+inline constexpr int kKept = kFastRow<NX, EXACT> ? RowGeo<NX>::R / 2 : RowGeo<NX>::R;
+
+template <int NX, bool EXACT>
+__device__ __forceinline__ void kept_modes(const One (&x)[RowGeo<NX>::R], One (&X)[kKept<NX, EXACT>], int W, int j,
+                                           typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
   using G = RowGeo<NX>;
   constexpr int n = G::n, R = G::R, T = G::T;
   constexpr bool FAST = kFastRow<NX, EXACT>;
-  unsigned long long* out = const_cast<unsigned long long*>(mixed_row(dst, w));
-  const int step = T * ny;
-  if (FAST) out += mode_at(j, ny);
   if constexpr (!G::WARP) {
     // Z[n - k] of the kept modes: the elements above n - W, and Z[0]
 #pragma unroll
@@ -231,9 +231,8 @@ __device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const
       if (r == 0 || (FAST ? r >= R / 2 : (r + 1) * T > n - W)) xs[j + r * T] = x[r].v;
     __syncthreads();
   }
-  One X[FAST ? R / 2 : R];
 #pragma unroll
-  for (int r = 0; r < (FAST ? R / 2 : R); ++r) {
+  for (int r = 0; r < kKept<NX, EXACT>; ++r) {
     if (!FAST && r * T >= W) break;
     const int k = j + r * T;
     One zc;
@@ -252,11 +251,22 @@ __device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const
     const One d = cmul(sub_conj(x[r], zc), e);
     X[r] = scale(0.5f, subi(add_conj(x[r], zc), d));
   }
+}
+template <int NX, bool EXACT>
+__device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const BufRef& dst, const Row& w, int ny,
+                                            int W, int j, typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
+  using G = RowGeo<NX>;
+  constexpr bool FAST = kFastRow<NX, EXACT>;
+  One X[kKept<NX, EXACT>];
+  kept_modes<NX, EXACT>(x, X, W, j, xs, t);
+  unsigned long long* out = const_cast<unsigned long long*>(mixed_row(dst, w));
+  const int step = G::T * ny;
+  if (FAST) out += mode_at(j, ny);
   if (w.act) {
 #pragma unroll
-    for (int r = 0; r < (FAST ? R / 2 : R); ++r) {
+    for (int r = 0; r < kKept<NX, EXACT>; ++r) {
       if (FAST) out[r * step] = X[r].v;
-      else if (j + r * T < W) out[mode_at(j + r * T, ny)] = X[r].v;
+      else if (j + r * G::T < W) out[mode_at(j + r * G::T, ny)] = X[r].v;
     }
   }
   if constexpr (!G::WARP) __syncthreads();

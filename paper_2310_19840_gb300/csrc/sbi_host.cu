@@ -35,6 +35,7 @@
 
 #include "../../include/sbi.h"
 #include "fft.cuh"
+#include "line.h"
 #include "sbi_internal.h"
 #include "schedule.h"
 
@@ -44,7 +45,8 @@ namespace {
 
 std::string g_create_error = "no error";
 
-enum PassKind { PK_ROW = 0, PK_COL = 1, PK_RK = 2, PK_CONV = 3, PK_WMK = 4, PK_NORM = 5 };
+// PK_LINE: a run of passes over one-dimensional FP32 members in one launch (line.h)
+enum PassKind { PK_ROW = 0, PK_COL = 1, PK_RK = 2, PK_CONV = 3, PK_WMK = 4, PK_NORM = 5, PK_LINE = 6 };
 
 // Cash-Karp 5(4) pair (the adaptive integrating factor): nodes, stage
 // weights, order-5 and order-4 solution weights
@@ -100,11 +102,12 @@ struct WmkParams {
   void* out;             // nx reals in the working precision
   int J, nx;
 };
-enum Family { FAM_COL = 0, FAM_ROW = 1, FAM_RK = 2, FAM_CONV = 3, FAM_WMK = 4, FAM_COUNT = 5 };
+enum Family { FAM_COL = 0, FAM_ROW = 1, FAM_RK = 2, FAM_CONV = 3, FAM_WMK = 4, FAM_LINE = 5, FAM_COUNT = 6 };
 const char* kFamilyNames[FAM_COUNT] = {"k_col (column FFT + spectral combine)",
                                        "k_row (row FFT + products)", "k_rk (RK4 stage)",
                                        "k_conv (adaptive-order test / step norms)",
-                                       "k_wavemaker (surface pressure profile)"};
+                                       "k_wavemaker (surface pressure profile)",
+                                       "k_line (passes of one-dimensional members)"};
 
 struct Pass {
   PassKind kind;
@@ -115,6 +118,8 @@ struct Pass {
   ConvParams conv;
   WmkParams wmk;
   NormParams norm;
+  LineParams line;
+  bool lined;     // runs inside a PK_LINE launch (set by the planner)
   double bytes;   // algorithmic device-memory traffic of the launch
   double xforms;  // 1-D transform passes over a whole field, times the field's points
 };
@@ -154,7 +159,8 @@ struct Group {
   double* d_crest = nullptr;    // crest position and height of one member (lazy)
   std::map<std::string, void*> mixed;
   std::map<std::string, void*> tables;   // multiplier tables by key
-  bool packed = false;            // runs on the packed kernels (packed_kernels.cuh): FP32, two-dimensional
+  bool packed = false;          // runs on the packed kernels (packed_kernels.cuh): FP32, two-dimensional
+  bool line = false;            // runs on k_line (line.cuh): FP32, one-dimensional
   size_t phys_elems() const { return (size_t)nx * ny; }
   // stored columns of a mixed field (tiles of four in a packed group)
   int columns() const { return packed ? (W + 3) / 4 * 4 : W; }
@@ -230,6 +236,7 @@ struct sbi_ctx {
     double ms;
   };
   std::map<std::string, Tuned> tuned;
+  std::map<std::string, void*> line_programs;   // device copies of k_line programs, by content
   std::vector<std::string> tune_order;  // signatures in the order they were tuned
   cudaEvent_t tune_ev[2] = {nullptr, nullptr};
   double dyn_h = NAN;   // the step the dynamic tables were last computed for
@@ -298,7 +305,7 @@ RkScalar rk_scalar(double v) {
 // whether a column pass can take the staged (bulk-copy) form
 bool stageable(const sbi_ctx* c, const ColParams& p) {
   if (p.packed) return packed_col_stageable(p.ny);
-  return c->fp64 ? col_stageable<double>(p.ny) : col_stageable<float>(p.ny);
+  return c->fp64 && col_stageable<double>(p.ny);
 }
 
 struct Planner {
@@ -433,11 +440,12 @@ struct Planner {
     if (room(r)) r.p.ops[r.p.nops++] = op;
   }
   int rpc_for(int nslots) {
+    if (g.line) return 1;
     if (g.packed) {
       int tpr = 0;
       return packed_row_geometry(g.nx, &tpr);
     }
-    const int r = c->fp64 ? row_rpc<double>(g.nx, g.W, nslots) : row_rpc<float>(g.nx, g.W, nslots);
+    const int r = row_rpc<double>(g.nx, g.W, nslots);
     if (r <= 0) oom = true;
     return r > 0 ? r : 1;
   }
@@ -926,8 +934,8 @@ struct Planner {
     p.rows_total = g.n * g.ny;
     p.ny = g.ny;
     p.W = g.W;
-    if (!g.packed) {
-      const int tpr = c->fp64 ? row_tpr<double>(g.nx) : row_tpr<float>(g.nx);
+    if (c->fp64) {
+      const int tpr = row_tpr<double>(g.nx);
       p.rpc = std::max(1, kRkThreads / std::max(1, tpr));
     }
     p.dt = dt;
@@ -1637,6 +1645,10 @@ int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st) {
     return e == cudaSuccess ? SBI_OK : cuda_fail(c, e, "kernel launch");
   }
   cudaError_t e = cudaSuccess;
+  if (p.kind == PK_LINE) {
+    e = launch_line(p.nsize, p.line, st);
+    return e == cudaSuccess ? SBI_OK : cuda_fail(c, e, "kernel launch");
+  }
   if (p.kind == PK_CONV) {
     const ConvParams& q = p.conv;
     const dim3 grid(kConvBlocks, q.n);
@@ -1656,13 +1668,305 @@ int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
     return SBI_OK;
   }
-  if (p.kind == PK_ROW && p.row.packed) e = launch_packed_row(p.nsize, p.row, st);
-  else if (p.kind == PK_COL && p.col.packed) e = launch_packed_col(p.nsize, p.col, st);
-  else if (p.kind == PK_RK && p.rk.packed) e = launch_packed_rk(p.nsize, p.rk, st);
-  else if (p.kind == PK_ROW) e = c->fp64 ? launch_row<double>(p.nsize, p.row, st) : launch_row<float>(p.nsize, p.row, st);
-  else if (p.kind == PK_COL) e = c->fp64 ? launch_col<double>(p.nsize, p.col, st) : launch_col<float>(p.nsize, p.col, st);
-  else e = c->fp64 ? launch_rk<double>(p.nsize, p.rk, st) : launch_rk<float>(p.nsize, p.rk, st);
+  if (p.kind == PK_ROW) e = p.row.packed ? launch_packed_row(p.nsize, p.row, st) : launch_row<double>(p.nsize, p.row, st);
+  else if (p.kind == PK_COL) e = p.col.packed ? launch_packed_col(p.nsize, p.col, st) : launch_col<double>(p.nsize, p.col, st);
+  else e = p.rk.packed ? launch_packed_rk(p.nsize, p.rk, st) : launch_rk<double>(p.nsize, p.rk, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
+  return SBI_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Programs of one-dimensional FP32 members: runs of passes become phases of
+// one launch (line.h).
+// ---------------------------------------------------------------------------
+bool lineable(const Pass& p) {
+  return p.kind == PK_ROW || p.kind == PK_COL || p.kind == PK_RK || p.kind == PK_WMK;
+}
+
+struct LineBuilder {
+  std::vector<LinePhase> phases;
+  std::vector<LineJob> jobs;
+  std::vector<LineTerm> terms;
+  std::vector<BufRef> bufs;
+  std::vector<RkParams> rks;
+  std::vector<LineWmk> wmks;
+  bool ok = true;
+
+  int16_t buf(const BufRef& b) {
+    if (!b.ptr) return -1;
+    for (size_t i = 0; i < bufs.size(); ++i)
+      if (bufs[i].ptr == b.ptr && bufs[i].stride == b.stride) return (int16_t)i;
+    bufs.push_back(b);
+    return (int16_t)(bufs.size() - 1);
+  }
+  // consecutive entries for a list
+  int16_t run(const BufRef* b, int n) {
+    if (n == 1) return buf(*b);
+    bufs.insert(bufs.end(), b, b + n);
+    return (int16_t)(bufs.size() - n);
+  }
+  LinePhase phase(LinePhaseType type, const int* active) {
+    LinePhase p;
+    std::memset(&p, 0, sizeof(p));
+    p.type = type;
+    p.active = active;
+    p.eta = p.delta = p.wgt = p.dst = -1;
+    p.begin = p.end = (int16_t)jobs.size();
+    return p;
+  }
+  void row(const RowParams& r) {
+    auto forward = [&]() {
+      LinePhase p = phase(LP_FORWARD, r.active);
+      p.eta = buf(r.eta);
+      p.delta = buf(r.delta);
+      p.wgt = buf(r.wgt);
+      return p;
+    };
+    auto inverse_job = [&](const RowOp& op, int slot) {
+      LineJob j;
+      std::memset(&j, 0, sizeof(j));
+      j.op = op.kind;
+      j.slot = (uint8_t)slot;
+      j.nsrc = op.b;
+      j.buf = run(r.buf + op.a, op.b);
+      j.phys = op.dst == kNone ? (int16_t)-1 : buf(r.buf[op.dst]);
+      jobs.push_back(j);
+    };
+    auto forward_job = [&](const RowOp& op, int slot, int ea, int eb) {
+      LineJob j;
+      std::memset(&j, 0, sizeof(j));
+      j.op = op.kind;
+      j.slot = (uint8_t)slot;
+      j.ea = (uint8_t)ea;
+      j.eb = (uint8_t)eb;
+      j.ew = op.kind == ROP_PROD ? op.c & 1 : 0;
+      j.pg = op.kind == ROP_N2 && r.pg ? 1 : 0;
+      j.coef = op.coef_f;
+      j.buf = buf(r.buf[op.dst]);
+      jobs.push_back(j);
+    };
+    if (r.nslots > 1) {   // every slot is needed at once
+      LinePhase in = phase(LP_INVERSE, r.active);
+      for (int o = 0; o < r.nops; ++o)
+        if (r.ops[o].kind == ROP_C2R) inverse_job(r.ops[o], r.ops[o].slot);
+      in.end = (int16_t)jobs.size();
+      phases.push_back(in);
+      LinePhase out = forward();
+      for (int o = 0; o < r.nops; ++o) {
+        const RowOp& op = r.ops[o];
+        if (op.kind == ROP_WDOT) {
+          LinePhase w = phase(LP_WDOT, r.active);
+          w.dst = buf(r.buf[op.dst]);
+          phases.push_back(w);
+        } else if (op.kind != ROP_C2R) {
+          forward_job(op, op.slot, op.kind == ROP_PROD ? op.a : 0, op.kind == ROP_PROD ? op.b : 0);
+        }
+        if (op.kind != ROP_C2R && op.kind != ROP_PROD && (op.a != 1 || op.slot != 0)) ok = false;
+      }
+      out.end = (int16_t)jobs.size();
+      if (out.end > out.begin) phases.push_back(out);
+      if (r.nslots > kLineSlots - 1) ok = false;
+      return;
+    }
+    // chains, up to kLineSlots - 1 at a time (the last slot holds the pressure)
+    for (int o = 0; o < r.nops;) {
+      std::vector<int> starts;
+      int e = o;
+      while (e < r.nops && !(r.ops[e].kind == ROP_C2R && (int)starts.size() == kLineSlots - 1)) {
+        if (r.ops[e].kind == ROP_C2R) starts.push_back(e);
+        ++e;
+      }
+      if (starts.empty() || starts[0] != o) {
+        ok = false;
+        return;
+      }
+      LinePhase in = phase(LP_INVERSE, r.active);
+      for (size_t i = 0; i < starts.size(); ++i) inverse_job(r.ops[starts[i]], (int)i);
+      in.end = (int16_t)jobs.size();
+      phases.push_back(in);
+      LinePhase out = forward();
+      int slot = -1, ea = 0, eb = 0;
+      for (int q = o; q < e; ++q) {
+        const RowOp& op = r.ops[q];
+        if (op.kind == ROP_C2R) {
+          ++slot;
+          ea = eb = 0;
+          continue;
+        }
+        if (op.kind != ROP_PROD) ok = false;
+        forward_job(op, slot, ea + op.a, eb + op.b);
+        if (op.c & 2) {   // the running product
+          ea += op.a;
+          eb += op.b;
+        }
+      }
+      out.end = (int16_t)jobs.size();
+      if (out.end > out.begin) phases.push_back(out);
+      o = e;
+    }
+  }
+  void col(const ColParams& c) {
+    LinePhase p = phase(LP_COL, c.active);
+    auto add = [&](const ColTerm& t) {
+      LineTerm u;
+      std::memset(&u, 0, sizeof(u));
+      u.tab = t.tab;
+      u.buf = buf(c.buf[t.in]);
+      u.acc = t.acc;
+      u.ph = (t.gx + t.gy) & 3;
+      terms.push_back(u);
+    };
+    p.begin = (int16_t)terms.size();
+    for (int q = 0; q < c.nterms; ++q) add(c.terms[q]);
+    p.end = p.out_begin = (int16_t)terms.size();
+    for (int q = 0; q < c.nouts; ++q) add(c.outs[q]);
+    p.out_end = (int16_t)terms.size();
+    if (c.npass > 0) {
+      bufs.insert(bufs.end(), c.pass, c.pass + c.npass);
+      p.pass_begin = (int16_t)(bufs.size() - c.npass);
+      p.pass_end = (int16_t)bufs.size();
+    }
+    phases.push_back(p);
+  }
+  void rk(const RkParams& k) {
+    if (k.mode != RK_ENTRY) {
+      LinePhase in = phase(LP_INVERSE, k.active);
+      auto job = [&](const BufRef& b, int slot) {
+        LineJob j;
+        std::memset(&j, 0, sizeof(j));
+        j.op = ROP_C2R;
+        j.slot = (uint8_t)slot;
+        j.nsrc = 1;
+        j.buf = buf(b);
+        j.phys = -1;
+        jobs.push_back(j);
+      };
+      if (k.mode == RK_STAGE) {
+        job(k.phit, 0);
+      } else {
+        job(k.corr_phi, 0);
+        job(k.phit, 1);
+      }
+      in.end = (int16_t)jobs.size();
+      phases.push_back(in);
+    }
+    LinePhase u = phase(LP_RK, k.active);
+    u.out_begin = (int16_t)rks.size();
+    rks.push_back(k);
+    phases.push_back(u);
+    if (!k.tail) return;
+    LinePhase out = phase(LP_FORWARD, k.active);
+    for (int q = 0; q < 2; ++q) {
+      LineJob j;
+      std::memset(&j, 0, sizeof(j));
+      j.op = ROP_PROD;
+      j.slot = (uint8_t)(2 + q);
+      j.coef = 1.f;
+      j.buf = buf(q ? k.phi_hat : k.eta_hat);
+      jobs.push_back(j);
+    }
+    out.end = (int16_t)jobs.size();
+    phases.push_back(out);
+  }
+  void add(const Pass& p) {
+    if (p.kind == PK_ROW) row(p.row);
+    else if (p.kind == PK_COL) col(p.col);
+    else if (p.kind == PK_RK) rk(p.rk);
+    else {
+      LinePhase w = phase(LP_WMK, nullptr);
+      w.out_begin = (int16_t)wmks.size();
+      wmks.push_back(LineWmk{p.wmk.prof, p.wmk.omega, p.wmk.phase, p.wmk.t, p.wmk.offset, p.wmk.J});
+      phases.push_back(w);
+    }
+  }
+  // the program as one block of bytes
+  std::string bytes(const Group& g, const void* tw) const {
+    LineHeader h;
+    std::memset(&h, 0, sizeof(h));
+    std::string out(sizeof(h), '\0');
+    auto put = [&](const void* d, size_t n) {
+      out.resize((out.size() + 15) / 16 * 16);
+      const int at = (int)out.size();
+      out.append(static_cast<const char*>(d), n);
+      return at;
+    };
+    h.nphases = (int)phases.size();
+    h.phases = put(phases.data(), phases.size() * sizeof(LinePhase));
+    h.jobs = put(jobs.data(), jobs.size() * sizeof(LineJob));
+    h.terms = put(terms.data(), terms.size() * sizeof(LineTerm));
+    h.bufs = put(bufs.data(), bufs.size() * sizeof(BufRef));
+    h.rks = put(rks.data(), rks.size() * sizeof(RkParams));
+    h.wmks = put(wmks.data(), wmks.size() * sizeof(LineWmk));
+    h.W = g.W;
+    h.tw = tw;
+    out.resize((out.size() + 15) / 16 * 16);
+    h.bytes = (int)out.size();
+    std::memcpy(&out[0], &h, sizeof(h));
+    return out;
+  }
+};
+
+// Replaces every run of lineable passes of a one-dimensional FP32 group by
+// PK_LINE passes over its members [m0, m1).  Uploads the programs (each distinct
+// one once per context); not to be called while a capture is running.
+int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1) {
+  if (!g.line) return SBI_OK;
+  std::vector<Pass> out;
+  LineBuilder lb;
+  double nbytes = 0.0, xforms = 0.0;
+  std::string ready;
+  auto emit = [&]() -> int {
+    if (ready.empty()) return SBI_OK;
+    void*& dev = c->line_programs[ready];
+    if (!dev) {
+      dev = dalloc(c, ready.size());
+      if (!dev) {
+        c->line_programs.erase(ready);
+        return fail(c, SBI_ENOMEM, "device allocation failed");
+      }
+      CK(cudaMemcpyAsync(dev, ready.data(), ready.size(), cudaMemcpyHostToDevice, c->cap), "upload program");
+      CK(cudaStreamSynchronize(c->cap), "upload program");
+    }
+    Pass p{};
+    p.kind = PK_LINE;
+    p.nsize = g.nx;
+    p.line = LineParams{dev, (int)ready.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1};
+    p.lined = true;
+    p.bytes = nbytes;
+    p.xforms = xforms;
+    out.push_back(p);
+    lb = LineBuilder();
+    ready.clear();
+    nbytes = xforms = 0.0;
+    return SBI_OK;
+  };
+  for (const Pass& p : ps) {
+    if (!lineable(p)) {
+      const int rc = emit();
+      if (rc) return rc;
+      out.push_back(p);
+      continue;
+    }
+    const LineBuilder before = lb;
+    lb.add(p);
+    std::string now = lb.bytes(g, c->tw);
+    if (now.size() > (size_t)kLineMaxBytes) {   // start another program
+      const int rc = before.phases.empty() ? fail(c, SBI_EINVAL, "a pass is too long") : emit();
+      if (rc) return rc;
+      lb = LineBuilder();
+      // the pressure profile lives in shared memory: formed again beside its reader
+      if (&p != &ps[0] && (&p)[-1].kind == PK_WMK) lb.add((&p)[-1]);
+      lb.add(p);
+      now = lb.bytes(g, c->tw);
+    }
+    if (!lb.ok) return fail(c, SBI_EINVAL, "a pass has no one-dimensional form");
+    ready = std::move(now);
+    nbytes += p.bytes;
+    xforms += p.xforms;
+  }
+  const int rc = emit();
+  if (rc) return rc;
+  ps = std::move(out);
   return SBI_OK;
 }
 
@@ -1768,14 +2072,14 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
       for (int per : {0, kMaxRowOps, 3, 2, 1})
         if (per != p.row.split) cand.push_back(p.row.rpc + kSplitTag * per);
   } else if (p.kind == PK_ROW) {
-    const int tpr = c->fp64 ? row_tpr<double>(p.nsize) : row_tpr<float>(p.nsize);
+    const int tpr = row_tpr<double>(p.nsize);
     deflt = p.row.rpc;
     for (int r = deflt; r >= 1 && cand.size() < 4; r /= 2)
       if (tpr > 0 && (r * tpr) % 32 == 0) cand.push_back(r);
   } else {
     int tpc = 0, group = 1;
     const int cpb = p.col.packed ? packed_col_geometry(p.nsize, &tpc, &group)
-                               : (c->fp64 ? col_geometry<double>(p.nsize, &tpc) : col_geometry<float>(p.nsize, &tpc));
+                               : col_geometry<double>(p.nsize, &tpc);
     // the staged form of a packed group takes whole tiles of four columns
     auto base = [&](int staged) {
       const int b = p.col.cpb > 0 ? p.col.cpb : cpb;
@@ -1910,6 +2214,9 @@ std::vector<std::vector<Pass>> plan_step_groups(sbi_ctx* c, double dt, bool* oom
     if (pl.oom) *oom = true;
     out.push_back(std::move(all));
   }
+  for (size_t gi = 0; gi < out.size(); ++gi)
+    if (c->groups[gi].line)
+      for (Pass& p : out[gi]) p.lined = lineable(p);
   return out;
 }
 
@@ -1928,7 +2235,9 @@ std::vector<std::vector<Pass>> plan_step_groups(sbi_ctx* c, double dt, bool* oom
 // the state saved before and restored after), and the fastest is kept; the
 // default stays unless another candidate is at least 3 % faster.
 // ---------------------------------------------------------------------------
-bool pass_sliceable(const Pass& p) { return p.kind == PK_ROW || p.kind == PK_COL || p.kind == PK_RK; }
+bool pass_sliceable(const Pass& p) {
+  return p.kind == PK_ROW || p.kind == PK_COL || p.kind == PK_RK || (p.kind == PK_WMK && p.lined);
+}
 
 // a group's pass restricted to its members [m0, m1)
 Pass slice_pass(const Pass& p, const Group& g, int m0, int m1) {
@@ -1940,7 +2249,7 @@ Pass slice_pass(const Pass& p, const Group& g, int m0, int m1) {
   } else if (p.kind == PK_COL) {
     q.col.col_begin = m0 * g.columns();
     q.col.cols_total = m1 * g.columns();
-  } else {
+  } else if (p.kind == PK_RK) {
     q.rk.row_begin = m0 * g.ny;
     q.rk.rows_total = m1 * g.ny;
   }
@@ -2069,6 +2378,7 @@ int update_dyn_tables(sbi_ctx* c, double h, cudaStream_t st) {
 }
 
 int family_of(const Pass& p) {
+  if (p.lined) return FAM_LINE;
   switch (p.kind) {
     case PK_COL: return FAM_COL;
     case PK_ROW: return FAM_ROW;
@@ -2104,6 +2414,11 @@ int build_step_graph(sbi_ctx* c, double dt, int kind, const Unit* only, GraphEnt
   if (oom) return fail(c, SBI_ENOMEM, "device allocation failed while planning the step");
   CK(cudaStreamSynchronize(c->cap), "sync before capture");
   CK(cudaStreamSynchronize(c->stream), "sync before capture");
+  for (size_t u = 0; u < gps.size(); ++u) {
+    const Unit& unit = only ? *only : c->units[u];
+    const int rc = lower_line(c, c->groups[unit.group], gps[u], unit.m0, unit.m1);
+    if (rc) return rc;
+  }
   // block shapes are tuned (or taken from earlier tuning) before capture
   for (auto& v : gps)
     for (auto& p : v) {
@@ -2459,6 +2774,8 @@ int run_diag(sbi_ctx* c, int gi, bool eulerian) {
   pl.plan_diag(ps);
   pl.plan_sum_v(ps, eulerian);
   if (pl.oom) return fail(c, SBI_ENOMEM, "device allocation failed");
+  const int low = lower_line(c, c->groups[gi], ps, 0, c->groups[gi].n);
+  if (low) return low;
   CK(cudaStreamSynchronize(c->cap), "sync");
   for (auto& p : ps) {
     int rc = tune_pass(c, p, c->stream);
@@ -2644,6 +2961,7 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
       g.ky_keep = std::max(g.ky_keep, 1);
       g.W = g.kx_keep;
       g.packed = g.two_d && !c->fp64;
+      g.line = !g.two_d && !c->fp64;
       c->groups.push_back(g);
     }
     Group& g = c->groups[sig[i]];
@@ -2673,10 +2991,9 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
 
   for (auto& g : c->groups) {
     cudaError_t e = g.packed ? prepare_packed_row_kernels(g.nx)
-                           : (c->fp64 ? prepare_row_kernels<double>(g.nx) : prepare_row_kernels<float>(g.nx));
-    if (e == cudaSuccess)
-      e = g.packed ? prepare_packed_col_kernels(g.ny)
-                 : (c->fp64 ? prepare_col_kernels<double>(g.ny) : prepare_col_kernels<float>(g.ny));
+                             : (g.line ? prepare_line_kernels(g.nx) : prepare_row_kernels<double>(g.nx));
+    if (e == cudaSuccess && !g.line)
+      e = g.packed ? prepare_packed_col_kernels(g.ny) : prepare_col_kernels<double>(g.ny);
     if (e != cudaSuccess) { cuda_fail(c, e, "kernel setup"); return bail(SBI_ECUDA); }
     int rc = init_group(c, g);
     if (rc) return bail(rc);
@@ -2708,6 +3025,8 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
     std::vector<Pass> ps;
     ps.push_back(pl.plan_rk(RK_ENTRY, 0, 0.0, 1));
     if (pl.oom) { c->err = "device allocation failed"; return bail(SBI_ENOMEM); }
+    const int rc = lower_line(c, g, ps, 0, g.n);
+    if (rc) return bail(rc);
     if (run_passes(c, ps, c->cap)) return bail(SBI_ECUDA);
   }
   if (cudaStreamSynchronize(c->cap) != cudaSuccess) {
@@ -2796,7 +3115,8 @@ int sbi_set_state(sbi_ctx* c, int member, const double* eta, const double* phi, 
     else if (p.kind == PK_COL) p.col.active = g.d_active;
     else p.rk.active = g.d_active;
   }
-  rc = run_passes(c, ps, c->cap);
+  rc = lower_line(c, g, ps, 0, g.n);
+  if (!rc) rc = run_passes(c, ps, c->cap);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->cap), "set_state");
   return SBI_OK;
@@ -2873,7 +3193,8 @@ int sbi_set_state_all(sbi_ctx* c, const double* eta, const double* phi, int on_d
     if (c->opt.set_state_dealias) pl.plan_project(ps, false);
     else ps.push_back(pl.plan_rk(RK_ENTRY, 0, 0.0, 1));
     if (pl.oom) return fail(c, SBI_ENOMEM, "device allocation failed");
-    const int rc = run_passes(c, ps, c->cap);
+    int rc = lower_line(c, g, ps, 0, g.n);
+    if (!rc) rc = run_passes(c, ps, c->cap);
     if (rc) return rc;
   }
   CK(cudaStreamSynchronize(c->cap), "set_state_all");
@@ -3042,6 +3363,10 @@ int sbi_vertical_velocity_implicit(sbi_ctx* c, int member, int iterations, doubl
   if (!g.d_implicit)
     g.d_implicit = (double*)dalloc(c, (size_t)kImplicitMaxIter * g.n * 2 * sizeof(double));
   if (pl.oom || !g.d_implicit) return fail(c, SBI_ENOMEM, "device allocation failed");
+  for (std::vector<Pass>* v : {&setup, &first, &ab, &ba, &fin}) {
+    rc = lower_line(c, g, *v, 0, g.n);
+    if (rc) return rc;
+  }
   CK(cudaStreamSynchronize(c->cap), "sync");
   auto run = [&](std::vector<Pass>& v) {
     for (auto& p : v) {
@@ -3157,6 +3482,8 @@ int streamed_run(sbi_ctx* c, const double* eta_in, const double* phi_in, double 
     else ps.push_back(pl.plan_rk(RK_ENTRY, 0, 0.0, 1));
     if (pl.oom) return fail(c, SBI_ENOMEM, "device allocation failed");
     for (const Pass& p : ps) entry[ui].push_back(slice_pass(p, g, u.m0, u.m1));
+    rc = lower_line(c, g, entry[ui], u.m0, u.m1);
+    if (rc) return rc;
   }
   int least = 0, greatest = 0;
   CK(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
@@ -3603,9 +3930,15 @@ int sbi_step_launches(const sbi_ctx* cc, int* launches) {
   sbi_ctx* c = const_cast<sbi_ctx*>(cc);
   if (!c || !launches) return SBI_EINVAL;
   bool oom = false;
-  std::vector<Pass> ps = plan_step(c, 1.0, &oom);
+  std::vector<int> kinds = {SK_STEP};
+  if (c->opt.integrator == SBI_IF_RK45) kinds = {SK_RK45_A, SK_RK45_B};
+  int count = c->wm_n > 0 ? 1 : 0;   // the time advance
+  for (int kind : kinds)
+    for (const auto& v : plan_step_units(c, 1.0, &oom, kind))
+      for (size_t i = 0; i < v.size(); ++i)   // a run of lined passes is one launch
+        count += !(v[i].lined && i > 0 && v[i - 1].lined);
   if (oom) return fail(c, SBI_ENOMEM, "device allocation failed");
-  *launches = (int)ps.size() + (c->wm_n > 0 ? 1 : 0);  // + the time advance
+  *launches = count;
   return SBI_OK;
 }
 
