@@ -3147,9 +3147,13 @@ double* device_view(void* p, int on_device) {
   return nullptr;
 }
 
+// A staging buffer's first use is on another stream than the one that zeroes it.
 int ensure_stage(sbi_ctx* c, Group& g) {
-  if (!g.stage64) g.stage64 = (double*)dalloc(c, g.phys_elems() * g.n * 8);
-  return g.stage64 ? SBI_OK : fail(c, SBI_ENOMEM, "device allocation failed");
+  if (g.stage64) return SBI_OK;
+  g.stage64 = (double*)dalloc(c, g.phys_elems() * g.n * 8);
+  if (!g.stage64) return fail(c, SBI_ENOMEM, "device allocation failed");
+  CK(cudaStreamSynchronize(c->cap), "sync");
+  return SBI_OK;
 }
 
 int sbi_set_state_all(sbi_ctx* c, const double* eta, const double* phi, int on_device) {
@@ -3474,8 +3478,11 @@ int streamed_run(sbi_ctx* c, const double* eta_in, const double* phi_in, double 
     }
     int rc = ensure_stage(c, g);
     if (rc) return rc;
-    if (!g.stage64b) g.stage64b = (double*)dalloc(c, g.phys_elems() * g.n * 8);
-    if (!g.stage64b) return fail(c, SBI_ENOMEM, "device allocation failed");
+    if (!g.stage64b) {
+      g.stage64b = (double*)dalloc(c, g.phys_elems() * g.n * 8);
+      if (!g.stage64b) return fail(c, SBI_ENOMEM, "device allocation failed");
+      CK(cudaStreamSynchronize(c->cap), "sync");
+    }
     Planner pl{c, g};
     std::vector<Pass> ps;
     if (c->opt.set_state_dealias) pl.plan_project(ps, false);
@@ -3748,6 +3755,7 @@ int sbi_invariants(sbi_ctx* c, int member, double* mass, double* energy) {
   if ((size_t)nchunks * 2 > c->partial_cap) {
     void* p = dalloc(c, (size_t)nchunks * 2 * 8);
     if (!p) return fail(c, SBI_ENOMEM, "device allocation failed");
+    CK(cudaStreamSynchronize(c->cap), "sync");
     c->d_partials = (double*)p;
     c->partial_cap = (size_t)nchunks * 2;
   }
