@@ -230,8 +230,9 @@ def measured_peaks():
 # the sources of the row, column and RK kernels whose DRAM traffic the
 # committed ncu summary records (host code and the other kernels live in
 # sbi_host.cu and sbi_noalloc.cu)
-KERNEL_SOURCES = ("bank_model.h", "fft.cuh", "kernels.cuh", "sbi_internal.h", "inst_col_f32.cu",
-                  "inst_col_f64.cu", "inst_row_f32.cu", "inst_row_f64.cu")
+KERNEL_SOURCES = ("bank_model.h", "fft.cuh", "kernels.cuh", "line.cuh", "line.h", "packed.cuh",
+                  "packed_kernels.cuh", "sbi_internal.h", "inst_col_f64.cu", "inst_line.cu",
+                  "inst_packed_col.cu", "inst_packed_row.cu", "inst_packed_row_long.cu", "inst_row_f64.cu")
 
 
 def source_sha():

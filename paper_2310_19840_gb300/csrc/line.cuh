@@ -2,15 +2,19 @@
 //
 // A one-dimensional member is one row of 16 to 4096 points: a pass over it is
 // far below a launch in work, and a step of some 64 dependent launches took 7
-// to 15 us each.  Here one block per member runs the whole list of passes (a
-// program of phases, line.h), a block barrier between phases.  Every transform
-// of a phase goes to its own group of threads (packed.cuh), so the products of
-// a level are transformed side by side; physical fields stay in shared memory,
-// mixed fields (8 KB at most) in global memory, where the block finds them in
-// its L1 and L2.  What bounds it is the chain of dependent transforms: about 17
-// per right-hand side.
-// Measured (GB300, a step): 256 points 420 us in 64 launches -> see DESIGN's
-// table for the current figures.
+// to 27 us each.  Here one launch runs the whole list of passes (a program of
+// phases, line.h) with a barrier between phases.  Every transform of a phase
+// goes to its own group of threads (packed.cuh), so the products of a level are
+// transformed side by side; physical fields stay in shared memory, mixed fields
+// (8 KB at most) in global memory, found in L1 and L2.  Rows of 2048 points and
+// more run on a cluster of 4 or 8 blocks: the inverse transforms and their
+// physical fields are formed in every block, the products and the modes are
+// shared out, and the cluster's barrier orders the phases that hand mixed
+// fields on.  The results do not depend on the number of blocks.
+// What bounds it is the chain of dependent phases, 25 per right-hand side of
+// about a microsecond each.
+// Measured (GB300, a step): 256 points 102 us (420 us as 64 launches); 4096
+// points over a bar 377 us (558 us in one block, 850 us as 64 launches).
 #pragma once
 
 #include "line.h"
@@ -39,7 +43,8 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
   unsigned char* prog = reinterpret_cast<unsigned char*>(slots + kLineSlots * n);
   const int tid = threadIdx.x, g = tid / T, j = tid % T;
   auto* xs = xs0 + g * G::XLEN;
-  const int member = p.member0 + (int)blockIdx.x;
+  const int C = p.cluster, rank = (int)blockIdx.x % C;
+  const int member = p.member0 + (int)blockIdx.x / C;
   for (int i = tid; i < (p.bytes + 15) / 16; i += kLineThreads)
     reinterpret_cast<uint4*>(prog)[i] = reinterpret_cast<const uint4*>(p.program)[i];
   const LineHeader& H = *reinterpret_cast<const LineHeader*>(prog);
@@ -58,15 +63,25 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
 #pragma unroll 1
   for (int ip = 0; ip < H.nphases; ++ip) {
     const LinePhase& P = phases[ip];
-    if (P.active && P.active[member] == 0) continue;      // the whole block
+    // also before a phase that this member skips: the next ones rely on it
+    if (C > 1 && P.sync) {
+      asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    } else {
+      __syncthreads();
+    }
+    if (P.active && P.active[member] == 0) continue;      // the whole cluster
     if (P.type == LP_INVERSE || P.type == LP_FORWARD) {
       const bool inverse = P.type == LP_INVERSE;
+      // every block runs all inverse transforms, and its share of the others
+      const int share = inverse ? 1 : C;
 #pragma unroll 1
-      for (int first = P.begin; first < P.end; first += GROUPS) {
+      for (int first = P.begin + (inverse ? 0 : rank); first < P.end; first += share * GROUPS) {
         t.renew();
-        const bool valid = first + g < P.end;
-        if (G::WARP && first + (tid & ~31) / T >= P.end) break;   // a warp without a job
-        const LineJob job = jobs[valid ? first + g : P.begin];
+        const int mine = first + share * g;
+        const bool valid = mine < P.end;
+        if (G::WARP && first + share * ((tid & ~31) / T) >= P.end) break;   // a warp without a job
+        const LineJob job = jobs[valid ? mine : P.begin];
         One x[R];
         if (inverse) {
           // modes k < W and n - k < W of the sum of the sources (inverse_input)
@@ -140,7 +155,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
         if (inverse) {
           if (valid) {
             F2* s = slots + job.slot * n + j;
-            F2* out = job.phys >= 0 ? real(job.phys) + j : nullptr;
+            F2* out = job.phys >= 0 && rank == 0 ? real(job.phys) + j : nullptr;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
               const F2 v = conj(x[r]);
@@ -163,9 +178,9 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
     } else if (P.type == LP_COL) {
       // outputs may overwrite inputs of the same mode: every load of a mode
       // comes before its stores, by the same thread
-      for (int k = tid; k < W; k += kLineThreads) {
+      for (int k = rank * kLineThreads + tid; k < W; k += C * kLineThreads) {
         F2 a0 = both(0.f), a1 = a0;
-#pragma unroll 4
+#pragma unroll 8
         for (int q = P.begin; q < P.end; ++q) {
           const LineTerm m = terms[q];
           const F2 v = mixed(m.buf)[k];
@@ -174,6 +189,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
           else a1 = acc_term(a1, v, f, m.ph);
         }
         F2 extra = both(0.f);
+#pragma unroll 4
         for (int q = P.pass_begin; q < P.pass_end; ++q) extra = add(extra, mixed(q)[k]);
         for (int q = P.out_begin; q < P.out_end; ++q) {
           const LineTerm m = terms[q];
@@ -187,7 +203,10 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
       bool bad = false;
       const float bw = (q.stage == 1 || q.stage == 4) ? 1.f : 2.f;
       const RkScalar cdt = q.cdt, dt6 = q.dt6;
-      for (int i = tid; i < 2 * n; i += kLineThreads) {
+      // the first block updates the elevation, the second (if there is one) the
+      // potential: the blocks that transform slots 2 and 3 (jobs 0 and 1)
+      for (int i = tid + (C > 1 ? rank * n : 0); i < (C > 1 ? (rank < 2 ? (rank + 1) * n : 0) : 2 * n);
+           i += kLineThreads) {
         const bool potential = i >= n;
         const int m = potential ? i - n : i;
         const BufRef& st = potential ? q.phi0 : q.eta0;
@@ -237,20 +256,22 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
       if (bad && q.nonfinite) *q.nonfinite = 1;
     } else if (P.type == LP_WDOT) {
       F2* out = real(P.dst);
-      for (int m = tid; m < n; m += kLineThreads) {
+      for (int m = rank * kLineThreads + tid; m < n; m += C * kLineThreads) {
         const F2 ex = slots[n + m];
         out[m] = quotient(fma(ex, slots[2 * n + m], slots[m]), fma(ex, ex, both(1.f)));
       }
-    } else {   // LP_WMK: FP64 sums and sines, rounded once
+    } else if (rank == 0) {   // LP_WMK: FP64 sums and sines, rounded once
       const LineWmk& q = reinterpret_cast<const LineWmk*>(prog + H.wmks)[P.out_begin];
       const double time = *q.t + q.offset;
+      double* sines = reinterpret_cast<double*>(xs0);       // the exchange buffer is free here
+      for (int i = tid; i < q.J; i += kLineThreads) sines[i] = sin(q.omega[i] * time + q.phase[i]);
+      __syncthreads();
       for (int x = tid; x < 2 * n; x += kLineThreads) {
         double acc = 0.0;
-        for (int i = 0; i < q.J; ++i) acc += q.prof[(size_t)i * 2 * n + x] * sin(q.omega[i] * time + q.phase[i]);
+        for (int i = 0; i < q.J; ++i) acc += q.prof[(size_t)i * 2 * n + x] * sines[i];
         reinterpret_cast<float*>(slots + 5 * n)[x] = float(acc);
       }
     }
-    __syncthreads();
   }
 }
 
@@ -261,12 +282,21 @@ cudaError_t prepare_line_n() {
 }
 template <int NX>
 cudaError_t launch_line_n(const LineParams& p, cudaStream_t st) {
-  if (p.member0 < 0 || p.member1 <= p.member0 || p.bytes > kLineMaxBytes) return cudaErrorInvalidValue;
-  const size_t smem = line_smem<NX>(p.bytes);
-  const unsigned blocks = (unsigned)(p.member1 - p.member0);
-  if (p.exact) k_line<NX, true><<<blocks, kLineThreads, smem, st>>>(p);
-  else k_line<NX, false><<<blocks, kLineThreads, smem, st>>>(p);
-  return cudaGetLastError();
+  if (p.member0 < 0 || p.member1 <= p.member0 || p.bytes > kLineMaxBytes || p.cluster < 1 ||
+      p.cluster > line_cluster(NX))
+    return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((p.member1 - p.member0) * p.cluster));
+  cfg.blockDim = dim3(kLineThreads);
+  cfg.dynamicSmemBytes = line_smem<NX>(p.bytes);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)p.cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = p.cluster > 1 ? 1 : 0;
+  return p.exact ? cudaLaunchKernelEx(&cfg, k_line<NX, true>, p) : cudaLaunchKernelEx(&cfg, k_line<NX, false>, p);
 }
 
 }  // namespace pk

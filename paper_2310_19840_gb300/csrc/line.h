@@ -1,5 +1,6 @@
 // line.h - programs of the one-dimensional FP32 step (line.cuh): a list of
-// phases that one block runs for one member, a block barrier between them.
+// phases that one block, or a cluster of blocks, runs for one member, with a
+// barrier between them.
 #pragma once
 
 #include "sbi_internal.h"
@@ -15,7 +16,7 @@ enum LinePhaseType : uint8_t {
   LP_COL = 2,       // per mode: sums of terms, outputs, pass-through sums
   LP_RK = 3,        // state update; the new working values go to slots 2 (eta) and 3 (phi)
   LP_WDOT = 4,      // physical dst <- (V + eta_x phi_x) / (1 + eta_x^2)
-  LP_WMK = 5,       // surface pressure profile -> slot 5
+  LP_WMK = 5,       // surface pressure profile -> slot 5 (of the first block, which runs job 0)
 };
 
 // One transform.  Inverse: slot <- inverse of the sum of bufs [buf, buf + nsrc),
@@ -39,6 +40,8 @@ struct LineTerm {
 };
 struct LinePhase {
   uint8_t type;
+  uint8_t sync;                // 1: what the phases before left in global memory, or still read there,
+                               // has to be ordered for every block of the cluster first
   int16_t begin, end;          // jobs; LP_COL: terms
   int16_t out_begin, out_end;  // LP_COL: outputs (terms); LP_RK: index of the RkParams in out_begin
   int16_t pass_begin, pass_end;  // LP_COL: pass-through bufs, added to the first output
@@ -61,8 +64,13 @@ struct LineParams {
   const void* program;
   int bytes;
   int exact;                   // half of the modes kept
-  int member0, member1;        // members of this launch (one block each)
+  int member0, member1;        // members of this launch (one cluster of blocks each)
+  int cluster;                 // blocks per member
 };
+// The most blocks per member: rows of 2048 points and more have too few groups
+// of threads in one block for the products of a level (at 1024 points two
+// blocks were 20 % slower than one).
+constexpr int line_cluster(int nx) { return nx >= 4096 ? 8 : (nx >= 2048 ? 4 : 1); }
 
 cudaError_t prepare_line_kernels(int nx);
 cudaError_t launch_line(int nx, const LineParams& p, cudaStream_t st);

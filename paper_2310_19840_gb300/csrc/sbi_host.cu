@@ -1879,8 +1879,55 @@ struct LineBuilder {
       phases.push_back(w);
     }
   }
+  // A phase is ordered for the whole cluster when it reads or overwrites, in
+  // global memory, what a phase since the last such point wrote, or overwrites
+  // what one of them read.
+  void order() {
+    std::vector<const void*> read, written;   // since the last point
+    for (LinePhase& p : phases) {
+      std::vector<const void*> in, out;
+      auto at = [&](int b) { if (b >= 0) in.push_back(bufs[b].ptr); };
+      if (p.type == LP_INVERSE || p.type == LP_FORWARD) {
+        at(p.eta);
+        at(p.delta);
+        at(p.wgt);
+        for (int i = p.begin; i < p.end; ++i) {
+          const LineJob& j = jobs[i];
+          if (p.type == LP_FORWARD) out.push_back(bufs[j.buf].ptr);
+          else for (int q = 0; q < j.nsrc; ++q) at(j.buf + q);
+          if (p.type == LP_INVERSE && j.phys >= 0) out.push_back(bufs[j.phys].ptr);
+          // slot 5 is the first block's, and so is a phase's first job
+          if (p.type == LP_FORWARD && j.pg && i != p.begin) ok = false;
+        }
+      } else if (p.type == LP_COL) {
+        for (int i = p.begin; i < p.end; ++i) at(terms[i].buf);
+        for (int i = p.pass_begin; i < p.pass_end; ++i) at(i);
+        for (int i = p.out_begin; i < p.out_end; ++i) out.push_back(bufs[terms[i].buf].ptr);
+      } else if (p.type == LP_RK) {
+        const RkParams& k = rks[p.out_begin];
+        in.push_back(k.V.ptr);
+        for (const BufRef* b : {&k.eta0, &k.phi0, &k.acc_eta, &k.acc_phi, &k.eta_w})
+          if (b->ptr) out.push_back(b->ptr);
+      } else if (p.type == LP_WDOT) {
+        out.push_back(bufs[p.dst].ptr);
+      }
+      auto meet = [](const std::vector<const void*>& a, const std::vector<const void*>& b) {
+        for (const void* x : a)
+          if (std::find(b.begin(), b.end(), x) != b.end()) return true;
+        return false;
+      };
+      p.sync = meet(in, written) || meet(out, written) || meet(out, read);
+      if (p.sync) {
+        read.clear();
+        written.clear();
+      }
+      read.insert(read.end(), in.begin(), in.end());
+      written.insert(written.end(), out.begin(), out.end());
+    }
+  }
   // the program as one block of bytes
-  std::string bytes(const Group& g, const void* tw) const {
+  std::string bytes(const Group& g, const void* tw) {
+    order();
     LineHeader h;
     std::memset(&h, 0, sizeof(h));
     std::string out(sizeof(h), '\0');
@@ -1930,7 +1977,11 @@ int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1
     Pass p{};
     p.kind = PK_LINE;
     p.nsize = g.nx;
-    p.line = LineParams{dev, (int)ready.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1};
+    // blocks per member: as many as the size can use, while every cluster has
+    // SMs of its own
+    int cluster = line_cluster(g.nx);
+    while (cluster > 1 && (m1 - m0) * cluster > 128) cluster /= 2;
+    p.line = LineParams{dev, (int)ready.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1, cluster};
     p.lined = true;
     p.bytes = nbytes;
     p.xforms = xforms;
