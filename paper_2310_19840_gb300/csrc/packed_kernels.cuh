@@ -492,6 +492,94 @@ k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
   }
 }
 
+// Wide form for launches of few rows: the five inverse transforms of a row at
+// once by five copies of its threads, the products by one copy each; the same
+// operations in the same order (the same bits).  A set of threads is a warp, or
+// the threads of a longer row.
+template <int NX>
+struct WideRow {
+  static constexpr int SET = RowGeo<NX>::WARP ? 32 : RowGeo<NX>::T;
+  static constexpr int ROWS = SET / RowGeo<NX>::T;
+};
+template <int NX>
+__host__ __device__ constexpr size_t row_smem_wide() {
+  using G = RowGeo<NX>;
+  using H = WideRow<NX>;
+  return 8 * ((size_t)G::RTW + 5 * (size_t)H::ROWS * (G::XLEN + G::n));
+}
+template <int NX, bool EXACT>
+__global__ void __launch_bounds__(5 * WideRow<NX>::SET)
+k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
+  using G = RowGeo<NX>;
+  using H = WideRow<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T, SET = H::SET;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int copy = threadIdx.x / SET, lane = threadIdx.x % SET;
+  const int j = lane % T;
+  auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + (threadIdx.x / T) * G::XLEN;
+  F2* slots = reinterpret_cast<F2*>(reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + 5 * H::ROWS * G::XLEN);
+  auto S = [&](int s, int r) -> F2& { return slots[(s * R + r) * SET + lane]; };
+  const int row = p.row_begin + (int)blockIdx.x * H::ROWS + lane / T;
+  Row w;
+  w.act = row < p.rows_total;
+  w.member = w.act ? row / p.ny : 0;
+  w.y = w.act ? row - w.member * p.ny : 0;
+  if (w.act && p.active) w.act = p.active[p.member0 + w.member] != 0;
+  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+  One x[R];
+  const RowOp c = p.ops[q.src[copy]];
+  inverse_input<NX, EXACT>(x, p.buf + c.a, c.b, w, p.ny, p.W, j, t);
+  t.run(x, xs);
+#pragma unroll
+  for (int r = 0; r < R; ++r) S(copy, r) = x[r] = conj(x[r]);
+  if (c.dst != kNone && w.act) {   // physical V
+    float2* out = real_row(p.buf[c.dst], w, n) + j;
+#pragma unroll
+    for (int r = 0; r < R; ++r) out[r * T] = parts(x[r]);
+  }
+  __syncthreads();
+  // slots in the order of q.src: eta_x, phi_x, eta_y, phi_y, V
+  const RowOp op = p.ops[q.f];
+  int dst = -1;
+  if (copy == 0) {
+    const float2* eta = p.eta.ptr ? real_row(p.eta, w, n) + j : nullptr;
+    const float2* pg = op.kind == ROP_N2 && p.pg ? reinterpret_cast<const float2*>(p.pg) + j : nullptr;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const F2 ex = S(0, r), px = S(1, r), ey = S(2, r), py = S(3, r), v = S(4, r);
+      const F2 dot = fma(ey, py, mul(ex, px)), den = add(both(1.f), fma(ey, ey, mul(ex, ex)));
+      if (op.kind == ROP_VFW) {
+        x[r] = fma(v, den, mul(both(-1.f), dot));
+        continue;
+      }
+      const F2 num = add(v, dot);
+      if (op.kind == ROP_WDOT) {
+        x[r] = quotient(num, den);
+        continue;
+      }
+      x[r] = scale(0.5f, sub(quotient(mul(num, num), den), fma(py, py, mul(px, px))));
+      if (eta) x[r] = axpy(-op.coef_f, f2(__ldg(eta + r * T)), x[r]);
+      if (pg) x[r] = sub(x[r], f2(__ldg(pg + r * T)));
+    }
+    dst = op.dst;
+    if (op.kind == ROP_WDOT && w.act) {
+      float2* out = real_row(p.buf[op.dst], w, n) + j;
+#pragma unroll
+      for (int r = 0; r < R; ++r) out[r * T] = parts(x[r]);
+    }
+  } else if ((copy == 1 || copy == 3) && (copy == 1 ? q.sx : q.sy) >= 0) {
+    const float2* sponge = real_row(p.wgt, w, n) + j;
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = mul(x[r], f2(__ldg(sponge + r * T)));
+    dst = p.ops[copy == 1 ? q.sx : q.sy].dst;
+  }
+  if (op.kind == ROP_WDOT) return;           // the whole block
+  if (G::WARP && dst < 0) return;            // the whole warp
+  t.run(x, xs);
+  if (dst < 0) w.act = false;
+  store_modes<NX, EXACT>(x, p.buf[dst < 0 ? 0 : dst], w, p.ny, p.W, j, xs, t);
+}
+
 // ===========================================================================
 // RK pass.  blockIdx.y: the elevation (0) or the potential (1); the two need
 // nothing from each other, so a thread holds one transform at a time.
@@ -529,35 +617,49 @@ k_packed_rk(const __grid_constant__ RkParams p) {
   }
   const float bw = (p.stage == 1 || p.stage == 4) ? 1.f : 2.f;
   const RkScalar cdt = p.cdt, dt6 = p.dt6;
+  const bool sums = p.mode == RK_STAGE && p.stage > 1;
+  // the state (and sums) of four elements are loaded before any of them is used
+  constexpr int B = R < 4 ? R : 4;
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int m = j + r * T;
-    const float2 f = parts(x[r]);
-    SP e = w.act ? SP::load(M, m) : SP::zero();
-    if (p.mode == RK_STAGE) {
-      SP a = (w.act && p.stage > 1) ? SP::load(A, m) : SP::zero();
-      a.add(0, bw * f.x);
-      a.add(1, bw * f.y);
-      if (p.stage < 4) {
-        if (w.act) a.store(A, m);
-        x[r] = f2(e.template offset<float>(0, cdt, f.x), e.template offset<float>(1, cdt, f.y));
+  for (int r0 = 0; r0 < R; r0 += B) {
+    SP st4[B], sum4[B];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      st4[i] = SP::load(M, j + (r0 + i) * T);
+      sum4[i] = sums ? SP::load(A, j + (r0 + i) * T) : SP::zero();
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const int r = r0 + i, m = j + r * T;
+      const float2 f = parts(x[r]);
+      SP e = st4[i];
+      if (p.mode == RK_STAGE) {
+        SP a = sum4[i];
+        a.add(0, bw * f.x);
+        a.add(1, bw * f.y);
+        if (p.stage < 4) {
+          if (w.act) a.store(A, m);
+          x[r] = f2(e.template offset<float>(0, cdt, f.x), e.template offset<float>(1, cdt, f.y));
+        } else {
+          e.add_scaled(0, a, dt6);
+          e.add_scaled(1, a, dt6);
+          if (w.act) {
+            e.store(M, m);
+            bad |= !e.finite();
+          }
+          x[r] = f2(float(e.value(0)), float(e.value(1)));
+        }
       } else {
-        e.add_scaled(0, a, dt6);
-        e.add_scaled(1, a, dt6);
-        if (w.act) e.store(M, m);
-        bad |= !e.finite();
+        if (p.mode != RK_ENTRY) {
+          e.add(0, f.x);
+          e.add(1, f.y);
+          if (p.mode == RK_CORRECT && w.act) {   // RK_OFFSET leaves the state unchanged
+            e.store(M, m);
+            bad |= !e.finite();
+          }
+        }
         x[r] = f2(float(e.value(0)), float(e.value(1)));
       }
-    } else {
-      if (p.mode != RK_ENTRY) {
-        e.add(0, f.x);
-        e.add(1, f.y);
-        if (p.mode == RK_CORRECT) {   // RK_OFFSET leaves the state unchanged
-          if (w.act) e.store(M, m);
-          bad |= !e.finite();
-        }
-      }
-      x[r] = f2(float(e.value(0)), float(e.value(1)));
     }
   }
   if (bad && p.nonfinite) *p.nonfinite = 1;
@@ -853,6 +955,9 @@ k_packed_col(const __grid_constant__ ColParams p) {
   }
 }
 
+__device__ __forceinline__ void copy_float_ahead(float* dst_smem, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
 // Wide form of the HALF pass, for launches of few columns: the threads of a
 // set of columns (one warp, or the block's 128 threads where a transform needs
 // them) are there p.wide times, each copy transforms its share of the inputs,
@@ -869,10 +974,10 @@ struct WideGeo {
   static constexpr int SX = G::XLEN * (SET / G::GT);    // exchange elements of one copy
 };
 template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nacc, int npass) {
+__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nterms, int nacc, int npass) {
   using G = ColGeo<NY>;
   using H = WideGeo<NY>;
-  const size_t modes = 8 * (size_t)nin * G::R * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
+  const size_t modes = (8 * (size_t)nin + 4 * (size_t)nterms) * G::R * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
   return 16 * ((size_t)G::CTW + (size_t)copies * H::SX) + 8 * (size_t)nacc * G::R * H::SET + (modes > pass ? modes : pass);
 }
 template <int NY>
@@ -891,6 +996,7 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   E* xs = xs0 + (size_t)copy * H::SX + g * G::XLEN + c;
   F2* sums = reinterpret_cast<F2*>(xs0 + (size_t)copies * H::SX);              // [acc][r][lane]
   F2* modes = sums + (size_t)p.nacc * R * SET;                                 // [input][r][lane]
+  float* factors = reinterpret_cast<float*>(modes + (size_t)p.nin * R * SET);  // [term][r][lane]
   E* passed = reinterpret_cast<E*>(modes);                                     // later: [pass][r][lane]
   const float2* tw = reinterpret_cast<const float2*>(p.tw);
   const int col = p.col_begin + (int)blockIdx.x * H::COLS + g * CI + c;
@@ -919,6 +1025,16 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
     asm volatile("" : "+f"(wj.x), "+f"(wj.y));
     const int i = i0 + copy;
     if (i0 > 0 && i < p.nin) load(i);
+    // the multipliers of this input's terms, for the sums
+    if (i < p.nin) {
+      for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
+        const float* tab = reinterpret_cast<const float*>(p.terms[q].tab) + at0;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          copy_float_ahead(factors + (q * R + r) * SET + lane, tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+      }
+      cp_async_commit();
+    }
     G::F::run(x, xs, j, t, tw);
     if (i < p.nin) {
 #pragma unroll
@@ -929,16 +1045,23 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
       }
     }
   }
+  // the multipliers of this copy's first output
+  float fo[R];
+  if (copy < p.nouts) {
+    const float* tab = reinterpret_cast<const float*>(p.outs[copy].tab) + at0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) fo[r] = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+  }
+  cp_async_wait_all();
   __syncthreads();
   // copy k sums the registers r = k, k + copies, ..
   for (int r = copy; r < R; r += copies) {
-    const long long at = at0 + r * T * 4 + (r < R / 2 ? 0 : plane);
     F2 a0 = both(0.f), a1 = a0;
     for (int i = 0; i < p.nin; ++i) {
       const F2 v = modes[(i * R + r) * SET + lane];
       for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
         const ColTerm m = p.terms[q];
-        const float f = __ldg(reinterpret_cast<const float*>(m.tab) + at);
+        const float f = factors[(q * R + r) * SET + lane];
         const int ph = (m.gx + m.gy) & 3;
         if (m.acc == 0) a0 = acc_term(a0, v, f, ph);
         else a1 = acc_term(a1, v, f, ph);
@@ -969,7 +1092,7 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
-        const float f = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+        const float f = o0 == 0 ? fo[r] : __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
         const F2 e = conj_term(sums[((m.acc ? R : 0) + r) * SET + lane], f, ph);
         x[r] = Two{e, cmul(e, r < R / 2 ? w : make_float2(-w.x, -w.y))};
       }
@@ -1051,6 +1174,13 @@ cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st) {
   if (p.nslots > 1) {
     RhsOps r;
     if (!rhs_ops(q, &r)) return cudaErrorInvalidValue;
+    if (p.split > 0) {
+      const unsigned wb = (unsigned)((p.rows_total - p.row_begin + WideRow<NX>::ROWS - 1) / WideRow<NX>::ROWS);
+      const int wt = 5 * WideRow<NX>::SET;
+      if (exact) k_packed_rhs_wide<NX, true><<<wb, wt, row_smem_wide<NX>(), st>>>(q, r);
+      else k_packed_rhs_wide<NX, false><<<wb, wt, row_smem_wide<NX>(), st>>>(q, r);
+      return cudaGetLastError();
+    }
     const size_t smem = row_smem<NX>(p.rpc, 3);
     if (exact) k_packed_rhs<NX, true><<<blocks, threads, smem, st>>>(q, r);
     else k_packed_rhs<NX, false><<<blocks, threads, smem, st>>>(q, r);
@@ -1093,7 +1223,7 @@ int col_most_wide(const ColParams& p) {
   if (!col_half(p) || p.staged) return 0;
   const int most = (ColGeo<NY>::WARP ? 256 : 512) / WideGeo<NY>::SET;
   for (int k = most; k >= 2; k /= 2)
-    if (packed_col_smem_wide<NY>(k, p.nin, p.nacc, p.npass) <= 227 * 1024) return k;
+    if (packed_col_smem_wide<NY>(k, p.nin, p.nterms, p.nacc, p.npass) <= 227 * 1024) return k;
   return 0;
 }
 
@@ -1127,7 +1257,7 @@ cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st) {
   const bool half = col_half(p);
   if (p.wide > 0) {
     using H = WideGeo<NY>;
-    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nacc, p.npass);
+    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nterms, p.nacc, p.npass);
     if (!half || p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
     const unsigned wb = (unsigned)((p.cols_total - p.col_begin + H::COLS - 1) / H::COLS);
     k_packed_col_wide<NY><<<wb, p.wide * H::SET, smem, st>>>(p);
@@ -1149,6 +1279,7 @@ cudaError_t prepare_packed_row_e() {
   using G = RowGeo<NX>;
   cudaError_t e = allow_smem(k_packed_row<NX, EXACT>, row_smem<NX>(G::MAXR, 0));
   if (e == cudaSuccess) e = allow_smem(k_packed_rhs<NX, EXACT>, row_smem<NX>(G::MAXR, 3));
+  if (e == cudaSuccess) e = allow_smem(k_packed_rhs_wide<NX, EXACT>, row_smem_wide<NX>());
   if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, float>, row_smem<NX>(G::MAXR, 0));
   if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, double>, row_smem<NX>(G::MAXR, 0));
   return e;

@@ -482,7 +482,8 @@ struct Planner {
     int tpr = 0;
     packed_row_geometry(g.nx, &tpr);
     const double warps = (double)p.rows_total * tpr / 32.0, want = 152.0 * 12.0;
-    if (p.nslots > 1 || warps >= want) return 0;
+    if (warps >= want) return 0;
+    if (p.nslots > 1) return 1;
     for (int per : {kMaxRowOps, 3, 2, 1})
       if (per == 1 || warps * row_segments(p, per) >= want) return per;
     return 1;
@@ -2119,9 +2120,8 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     deflt = p.row.rpc + kSplitTag * p.row.split;
     for (int r = p.row.rpc; r >= 1 && cand.size() < 3; r /= 2)
       if (r * tpr % 32 == 0) cand.push_back(r + kSplitTag * p.row.split);
-    if (p.row.nslots == 1)
-      for (int per : {0, kMaxRowOps, 3, 2, 1})
-        if (per != p.row.split) cand.push_back(p.row.rpc + kSplitTag * per);
+    for (int per : {0, kMaxRowOps, 3, 2, 1})
+      if (per != p.row.split && (p.row.nslots == 1 || per < 2)) cand.push_back(p.row.rpc + kSplitTag * per);
   } else if (p.kind == PK_ROW) {
     const int tpr = row_tpr<double>(p.nsize);
     deflt = p.row.rpc;

@@ -94,7 +94,8 @@ struct RowParams {
   RowOp ops[kMaxRowOps];
   const void* tw;
   int packed;             // a packed group's pass
-  int split;            // packed groups: products per segment (0: all operations in one block)
+  int split;            // packed groups: products per segment (0: all operations in one block); with
+                        // several slots, 1: a row's inverse transforms at once
   RowSeg seg[kMaxRowSegs];   // set by the launcher
 };
 
