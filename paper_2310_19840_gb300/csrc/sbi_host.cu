@@ -489,6 +489,7 @@ struct Planner {
     return 1;
   }
   static int row_segments(const RowParams& p, int per) {
+    if (per == 0) return 1;
     int ns = 0, prods = 0;
     for (int o = 0; o <= p.nops; ++o)
       if (o == p.nops || p.ops[o].kind == ROP_C2R) {
@@ -2120,8 +2121,18 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     deflt = p.row.rpc + kSplitTag * p.row.split;
     for (int r = p.row.rpc; r >= 1 && cand.size() < 3; r /= 2)
       if (r * tpr % 32 == 0) cand.push_back(r + kSplitTag * p.row.split);
-    for (int per : {0, kMaxRowOps, 3, 2, 1})
-      if (per != p.row.split && (p.row.nslots == 1 || per < 2)) cand.push_back(p.row.rpc + kSplitTag * per);
+    // split forms that differ in their number of blocks, while the rows alone
+    // are less than a few waves
+    std::vector<int> counts{Planner::row_segments(p.row, p.row.split)};
+    if ((double)p.row.rows_total * tpr < 32.0 * 152 * 12 * 4)
+      for (int per : {0, kMaxRowOps, 3, 2, 1}) {
+        const int n = Planner::row_segments(p.row, per);
+        if (p.row.nslots > 1 ? per < 2 && per != p.row.split
+                             : std::find(counts.begin(), counts.end(), n) == counts.end()) {
+          cand.push_back(p.row.rpc + kSplitTag * per);
+          counts.push_back(n);
+        }
+      }
   } else if (p.kind == PK_ROW) {
     const int tpr = row_tpr<double>(p.nsize);
     deflt = p.row.rpc;
@@ -2149,8 +2160,9 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     }
     if (p.col.packed && !p.col.staged) {   // copies of the wide form
       const int most = packed_col_most_wide(p.col);
-      for (int k = 2; k <= most && k < 2 * std::max(p.col.nin, p.col.nouts); k *= 2)
-        cand.push_back(base(0) + kWideTag * k);
+      const double warps = (double)p.col.cols_total * tpc / 32.0;
+      for (int k = 2; k <= most && k < 2 * std::max(p.col.nin, p.col.nouts) && warps * k < 152.0 * 8.0 * 4; k *= 2)
+        if (2 * k >= p.col.wide) cand.push_back(base(0) + kWideTag * k);
     }
   }
   int best = deflt;
