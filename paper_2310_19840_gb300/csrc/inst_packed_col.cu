@@ -11,8 +11,8 @@ cudaError_t prepare_packed_col_kernels(int ny) {
   SBI_SWITCH(ny, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }
-cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st) {
-#define SBI_CASE(N) case N: return pk::launch_packed_col_n<N>(p, st);
+cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st, bool chained) {
+#define SBI_CASE(N) case N: return pk::launch_packed_col_n<N>(p, st, chained);
   SBI_SWITCH(ny, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }

@@ -6,8 +6,8 @@ namespace sbi {
 // the long rows are compiled in inst_packed_row_long.cu
 #define SBI_LONG_ROWS(N)                                                                    \
   extern template cudaError_t pk::prepare_packed_row_n<N>();                                  \
-  extern template cudaError_t pk::launch_packed_row_n<N>(const RowParams&, cudaStream_t);     \
-  extern template cudaError_t pk::launch_packed_rk_n<N>(const RkParams&, cudaStream_t);
+  extern template cudaError_t pk::launch_packed_row_n<N>(const RowParams&, cudaStream_t, bool);     \
+  extern template cudaError_t pk::launch_packed_rk_n<N>(const RkParams&, cudaStream_t, bool);
 SBI_LONG_ROWS(512) SBI_LONG_ROWS(1024) SBI_LONG_ROWS(2048) SBI_LONG_ROWS(4096)
 
 #define SBI_PACKED_NX(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096)
@@ -18,13 +18,13 @@ cudaError_t prepare_packed_row_kernels(int nx) {
   SBI_SWITCH(nx, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }
-cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st) {
-#define SBI_CASE(N) case N: return pk::launch_packed_row_n<N>(p, st);
+cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st, bool chained) {
+#define SBI_CASE(N) case N: return pk::launch_packed_row_n<N>(p, st, chained);
   SBI_SWITCH(nx, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }
-cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st) {
-#define SBI_CASE(N) case N: return pk::launch_packed_rk_n<N>(p, st);
+cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st, bool chained) {
+#define SBI_CASE(N) case N: return pk::launch_packed_rk_n<N>(p, st, chained);
   SBI_SWITCH(nx, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }

@@ -57,6 +57,16 @@ __host__ __device__ constexpr size_t row_smem(int rows, int nslots) {
 // The twiddles of a block's transforms and of the packed real transform: from
 // shared memory, or (long rows) products of the thread's own e^{-2 pi i j / NX}
 // by roots of unity.
+// Passes are launched so that the blocks of one may start, and form what
+// depends on constants alone (twiddle tables, multipliers), while the blocks of
+// the pass before still run; nothing a pass wrote may be read, and nothing it
+// reads written, before this.  Every thread of every block waits: a pass that is
+// complete then has all the earlier ones behind it.
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
 template <int NX>
 struct RowTwiddles {
   using G = RowGeo<NX>;
@@ -296,19 +306,20 @@ k_packed_row(const __grid_constant__ RowParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + (threadIdx.x / T) * G::XLEN;
   const int j = threadIdx.x % T;
-  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
   const int ny = p.ny;
+  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+  wait_for_previous();
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
   One run[R], x[R], f[R];
   int held = 0;      // the field in f: 1 eta, 2 delta
   auto hold = [&](int which) {
     if (held == which) return;
     const float2* src = real_row(which == 1 ? p.eta : p.delta, w, n) + j;
 #pragma unroll
-    for (int r = 0; r < R; ++r) f[r] = f2(__ldg(src + r * T));
+    for (int r = 0; r < R; ++r) f[r] = f2(src[r * T]);
     held = which;
   };
   const int first = p.seg[blockIdx.y].first, end = p.seg[blockIdx.y].end, begin = p.seg[blockIdx.y].begin;
-  RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
 
 #pragma unroll 1
   for (int o = begin; o < end; ++o) {
@@ -387,9 +398,10 @@ k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
   xs += (threadIdx.x / T) * G::XLEN;
   auto S = [&](int s, int r) -> F2& { return reinterpret_cast<F2*>(slot)[(s * R + r) * nt]; };
   const int j = threadIdx.x % T;
-  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
   const int ny = p.ny;
   RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+  wait_for_previous();
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, p.member0);
 
   One e[R], x[R];     // e: eta_x until phi_x is there, eta_y until phi_y
 #pragma unroll
@@ -477,8 +489,8 @@ k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
         continue;
       }
       x[r] = scale(0.5f, sub(quotient(mul(num, num), den), S(2, r)));
-      if (eta) x[r] = axpy(-op.coef_f, f2(__ldg(eta + r * T)), x[r]);
-      if (pg) x[r] = sub(x[r], f2(__ldg(pg + r * T)));
+      if (eta) x[r] = axpy(-op.coef_f, f2(eta[r * T]), x[r]);
+      if (pg) x[r] = sub(x[r], f2(pg[r * T]));
     }
     if (op.kind == ROP_WDOT) {
       if (w.act) {
@@ -524,8 +536,9 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
   w.act = row < p.rows_total;
   w.member = w.act ? row / p.ny : 0;
   w.y = w.act ? row - w.member * p.ny : 0;
-  if (w.act && p.active) w.act = p.active[p.member0 + w.member] != 0;
   RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+  wait_for_previous();
+  if (w.act && p.active) w.act = p.active[p.member0 + w.member] != 0;
   One x[R];
   const RowOp c = p.ops[q.src[copy]];
   inverse_input<NX, EXACT>(x, p.buf + c.a, c.b, w, p.ny, p.W, j, t);
@@ -558,8 +571,8 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
         continue;
       }
       x[r] = scale(0.5f, sub(quotient(mul(num, num), den), fma(py, py, mul(px, px))));
-      if (eta) x[r] = axpy(-op.coef_f, f2(__ldg(eta + r * T)), x[r]);
-      if (pg) x[r] = sub(x[r], f2(__ldg(pg + r * T)));
+      if (eta) x[r] = axpy(-op.coef_f, f2(eta[r * T]), x[r]);
+      if (pg) x[r] = sub(x[r], f2(pg[r * T]));
     }
     dst = op.dst;
     if (op.kind == ROP_WDOT && w.act) {
@@ -593,10 +606,11 @@ k_packed_rk(const __grid_constant__ RkParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   auto* xs = reinterpret_cast<typename G::E*>(smem_raw) + G::RTW + (threadIdx.x / T) * G::XLEN;
   const int j = threadIdx.x % T;
-  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, 0);
   const int ny = p.ny;
   const bool potential = blockIdx.y != 0;
   RowTwiddles<NX> t(p.tw, reinterpret_cast<float2*>(smem_raw), j);
+  wait_for_previous();
+  const Row w = row_of<T>(p.row_begin, p.rows_total, p.ny, p.active, 0);
 
   const BufRef& st = potential ? p.phi0 : p.eta0;
   const BufRef& sum = potential ? p.acc_phi : p.acc_eta;
@@ -762,7 +776,6 @@ k_packed_col(const __grid_constant__ ColParams p) {
   using M = Mem<Two>;
   constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int gave_up = (STAGED && p.err_flag) ? *(volatile int*)p.err_flag : 0;
   float2* tab2 = reinterpret_cast<float2*>(smem_raw);
   E* sm = reinterpret_cast<E*>(smem_raw) + G::CTW;
   const int g = threadIdx.x / GT, l = threadIdx.x % GT, c = l % CI, j = l / CI;
@@ -776,8 +789,13 @@ k_packed_col(const __grid_constant__ ColParams p) {
   const bool valid = col < p.cols_total;
   const int member = valid ? col / p.W : 0;
   const int kx = valid ? col - member * p.W : 0;
-  const bool act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
   const long long at0 = ((long long)(kx >> 2) * ny2 + j) * 4 + (kx & 3);   // element r at + 4 T r
+  G::F::fill_twiddles(tab2, tw);
+  const auto t = G::F::twiddles(tab2, j);
+  float2 wj = __ldg(tw + tw_off(NY) + j);   // w^j; w^{j + r T} = w^j e^{-2 pi i r / 2R}
+  wait_for_previous();
+  const int gave_up = (STAGED && p.err_flag) ? *(volatile int*)p.err_flag : 0;
+  const bool act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
   auto field = [&](const BufRef& b) {
     return reinterpret_cast<E*>(reinterpret_cast<float2*>(b.ptr) + (long long)member * b.stride) + at0;
   };
@@ -792,9 +810,6 @@ k_packed_col(const __grid_constant__ ColParams p) {
     cp_async_commit();
   };
   if (AHEAD && p.nin > 0) copy_ahead(0);
-  G::F::fill_twiddles(tab2, tw);
-  const auto t = G::F::twiddles(tab2, j);
-  float2 wj = __ldg(tw + tw_off(NY) + j);   // w^j; w^{j + r T} = w^j e^{-2 pi i r / 2R}
 
   // staged form: tiles of four columns (one contiguous run) and barriers
   E* stg = nullptr;
@@ -1003,8 +1018,8 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   const bool valid = col < p.cols_total;
   const int member = valid ? col / p.W : 0;
   const int kx = valid ? col - member * p.W : 0;
-  const bool act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
   const long long at0 = ((long long)(kx >> 2) * ny2 + j) * 4 + (kx & 3);
+  bool act = valid;
   auto field = [&](const BufRef& b) {
     return reinterpret_cast<E*>(reinterpret_cast<float2*>(b.ptr) + (long long)member * b.stride) + at0;
   };
@@ -1015,25 +1030,31 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = M::from(act ? src[r * T * 4] : make_ulonglong2(0, 0));
   };
-  if (copy < p.nin) load(copy);
+  // the multipliers of an input's terms, for the sums
+  auto load_factors = [&](int i) {
+    for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
+      const float* tab = reinterpret_cast<const float*>(p.terms[q].tab) + at0;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        copy_float_ahead(factors + (q * R + r) * SET + lane, tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+    }
+    cp_async_commit();
+  };
+  if (copy < p.nin) load_factors(copy);
   G::F::fill_twiddles(tab2, tw);
   const auto t = G::F::twiddles(tab2, j);
   float2 wj = __ldg(tw + tw_off(NY) + j);
+  wait_for_previous();
+  act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
+  if (copy < p.nin) load(copy);
   __syncthreads();
 #pragma unroll 1
   for (int i0 = 0; i0 < p.nin; i0 += copies) {     // the same trips for every copy
     asm volatile("" : "+f"(wj.x), "+f"(wj.y));
     const int i = i0 + copy;
-    if (i0 > 0 && i < p.nin) load(i);
-    // the multipliers of this input's terms, for the sums
-    if (i < p.nin) {
-      for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
-        const float* tab = reinterpret_cast<const float*>(p.terms[q].tab) + at0;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          copy_float_ahead(factors + (q * R + r) * SET + lane, tab + r * T * 4 + (r < R / 2 ? 0 : plane));
-      }
-      cp_async_commit();
+    if (i0 > 0 && i < p.nin) {
+      load(i);
+      load_factors(i);
     }
     G::F::run(x, xs, j, t, tw);
     if (i < p.nin) {
@@ -1141,6 +1162,23 @@ inline int make_segments(RowParams& q, int per) {
   return ns;
 }
 
+// Launches a pass; chained: behind another pass of the same stream, which it may
+// overlap up to its wait_for_previous().
+template <typename... P, typename... A>
+cudaError_t launch(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 inline bool rhs_ops(const RowParams& p, RhsOps* q) {
   int slot_op[kMaxSlots] = {-1, -1, -1, -1, -1};
   *q = RhsOps{{-1, -1, -1, -1, -1}, -1, -1, -1};
@@ -1163,7 +1201,7 @@ inline bool rhs_ops(const RowParams& p, RhsOps* q) {
 }
 
 template <int NX>
-cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st) {
+cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st, bool chained) {
   using G = RowGeo<NX>;
   if (p.rpc < 1 || p.rpc > G::MAXR || (p.rpc * G::T) % 32 || p.row_begin < 0 || p.row_begin >= p.rows_total)
     return cudaErrorInvalidValue;
@@ -1177,38 +1215,32 @@ cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st) {
     if (p.split > 0) {
       const unsigned wb = (unsigned)((p.rows_total - p.row_begin + WideRow<NX>::ROWS - 1) / WideRow<NX>::ROWS);
       const int wt = 5 * WideRow<NX>::SET;
-      if (exact) k_packed_rhs_wide<NX, true><<<wb, wt, row_smem_wide<NX>(), st>>>(q, r);
-      else k_packed_rhs_wide<NX, false><<<wb, wt, row_smem_wide<NX>(), st>>>(q, r);
-      return cudaGetLastError();
+      return launch(exact ? k_packed_rhs_wide<NX, true> : k_packed_rhs_wide<NX, false>, wb, wt, row_smem_wide<NX>(), st,
+                    chained, q, r);
     }
-    const size_t smem = row_smem<NX>(p.rpc, 3);
-    if (exact) k_packed_rhs<NX, true><<<blocks, threads, smem, st>>>(q, r);
-    else k_packed_rhs<NX, false><<<blocks, threads, smem, st>>>(q, r);
+    return launch(exact ? k_packed_rhs<NX, true> : k_packed_rhs<NX, false>, blocks, threads, row_smem<NX>(p.rpc, 3), st,
+                  chained, q, r);
   } else {
     const int ns = q.nops > 0 && q.ops[0].kind == ROP_C2R ? make_segments(q, p.split) : 0;
     if (ns == 0) return cudaErrorInvalidValue;
-    const size_t smem = row_smem<NX>(p.rpc, 0);
-    const dim3 grid(blocks, (unsigned)ns);
-    if (exact) k_packed_row<NX, true><<<grid, threads, smem, st>>>(q);
-    else k_packed_row<NX, false><<<grid, threads, smem, st>>>(q);
+    return launch(exact ? k_packed_row<NX, true> : k_packed_row<NX, false>, dim3(blocks, (unsigned)ns), threads,
+                  row_smem<NX>(p.rpc, 0), st, chained, q);
   }
-  return cudaGetLastError();
 }
 
 template <int NX, bool EXACT>
-void launch_packed_rk_e(const RkParams& p, dim3 grid, size_t smem, cudaStream_t st) {
-  if (p.state64) k_packed_rk<NX, EXACT, double><<<grid, RowGeo<NX>::THREADS, smem, st>>>(p);
-  else k_packed_rk<NX, EXACT, float><<<grid, RowGeo<NX>::THREADS, smem, st>>>(p);
+cudaError_t launch_packed_rk_e(const RkParams& p, dim3 grid, cudaStream_t st, bool chained) {
+  using G = RowGeo<NX>;
+  return launch(p.state64 ? k_packed_rk<NX, EXACT, double> : k_packed_rk<NX, EXACT, float>, grid, G::THREADS,
+                row_smem<NX>(G::MAXR, 0), st, chained, p);
 }
 template <int NX>
-cudaError_t launch_packed_rk_n(const RkParams& p, cudaStream_t st) {
+cudaError_t launch_packed_rk_n(const RkParams& p, cudaStream_t st, bool chained) {
   using G = RowGeo<NX>;
   if (p.row_begin < 0 || p.row_begin >= p.rows_total) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)((p.rows_total - p.row_begin + G::MAXR - 1) / G::MAXR), 2);
-  const size_t smem = row_smem<NX>(G::MAXR, 0);
-  if (2 * p.W == G::n) launch_packed_rk_e<NX, true>(p, grid, smem, st);
-  else launch_packed_rk_e<NX, false>(p, grid, smem, st);
-  return cudaGetLastError();
+  return 2 * p.W == G::n ? launch_packed_rk_e<NX, true>(p, grid, st, chained)
+                         : launch_packed_rk_e<NX, false>(p, grid, st, chained);
 }
 
 // every output carries the dealias mask and at most half of the modes are kept
@@ -1228,23 +1260,19 @@ int col_most_wide(const ColParams& p) {
 }
 
 template <int NY, int NACC, bool HALF>
-cudaError_t launch_packed_col_a(const ColParams& p, int groups, unsigned blocks, cudaStream_t st) {
+cudaError_t launch_packed_col_a(const ColParams& p, int groups, unsigned blocks, cudaStream_t st, bool chained) {
   using G = ColGeo<NY>;
-  if (p.staged) {
-    if constexpr (G::STAGEABLE)
-      k_packed_col<NY, NACC, HALF, true>
-          <<<blocks, groups * G::GT, packed_col_smem_staged<NY>(groups, NACC, HALF), st>>>(p);
-    else
-      return cudaErrorInvalidValue;
-  } else {
-    k_packed_col<NY, NACC, HALF, false>
-        <<<blocks, groups * G::GT, packed_col_smem_ahead<NY>(groups, NACC, HALF), st>>>(p);
-  }
-  return cudaGetLastError();
+  if (!p.staged)
+    return launch(k_packed_col<NY, NACC, HALF, false>, blocks, groups * G::GT,
+                  packed_col_smem_ahead<NY>(groups, NACC, HALF), st, chained, p);
+  if constexpr (G::STAGEABLE)
+    return launch(k_packed_col<NY, NACC, HALF, true>, blocks, groups * G::GT,
+                  packed_col_smem_staged<NY>(groups, NACC, HALF), st, chained, p);
+  return cudaErrorInvalidValue;
 }
 
 template <int NY>
-cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st) {
+cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st, bool chained) {
   using G = ColGeo<NY>;
   const int most = p.staged ? G::SG : G::MAXG;
   const int cpb = p.cpb > 0 ? p.cpb : most * G::CI;
@@ -1260,14 +1288,13 @@ cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st) {
     const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nterms, p.nacc, p.npass);
     if (!half || p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
     const unsigned wb = (unsigned)((p.cols_total - p.col_begin + H::COLS - 1) / H::COLS);
-    k_packed_col_wide<NY><<<wb, p.wide * H::SET, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(k_packed_col_wide<NY>, wb, p.wide * H::SET, smem, st, chained, p);
   }
   if (p.nacc == 1)
-    return half ? launch_packed_col_a<NY, 1, true>(p, groups, blocks, st)
-                : launch_packed_col_a<NY, 1, false>(p, groups, blocks, st);
-  return half ? launch_packed_col_a<NY, 2, true>(p, groups, blocks, st)
-              : launch_packed_col_a<NY, 2, false>(p, groups, blocks, st);
+    return half ? launch_packed_col_a<NY, 1, true>(p, groups, blocks, st, chained)
+                : launch_packed_col_a<NY, 1, false>(p, groups, blocks, st, chained);
+  return half ? launch_packed_col_a<NY, 2, true>(p, groups, blocks, st, chained)
+              : launch_packed_col_a<NY, 2, false>(p, groups, blocks, st, chained);
 }
 
 template <typename K>

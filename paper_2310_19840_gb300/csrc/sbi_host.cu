@@ -1630,7 +1630,32 @@ __global__ void k_norm45_finish(NormParams q) {
 // ---------------------------------------------------------------------------
 // Execution
 // ---------------------------------------------------------------------------
-int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st) {
+// Whether a pass may start its blocks beside the pass before it: its blocks are
+// at most about one wave (16 warps on every SM).  Larger ones, and those of the
+// streamed step's branches, would hold SMs that other work could use: 48 members
+// streamed from the host took 4.19 ms with every pass chained, 3.91 ms with the
+// small ones and 3.55 ms with none; one 512^2 member takes 1.89 and 1.98.
+bool chainable(const Pass& p) {
+  int t = 0, group = 1;
+  double threads = 0.0;
+  if (p.kind == PK_ROW && p.row.packed) {
+    packed_row_geometry(p.nsize, &t);
+    threads = (double)(p.row.rows_total - p.row.row_begin) * t *
+              (p.row.nslots > 1 ? (p.row.split ? 5 : 1) : Planner::row_segments(p.row, p.row.split));
+  } else if (p.kind == PK_RK && p.rk.packed) {
+    packed_row_geometry(p.nsize, &t);
+    threads = 2.0 * (p.rk.rows_total - p.rk.row_begin) * t;
+  } else if (p.kind == PK_COL && p.col.packed) {
+    packed_col_geometry(p.nsize, &t, &group);
+    threads = (double)(p.col.cols_total - p.col.col_begin) * t * std::max(p.col.wide, 1);
+  } else {
+    return false;
+  }
+  return threads <= 152.0 * 16 * 32;
+}
+
+// chained: another pass was launched on st just before
+int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st, bool chained = false) {
   if (p.kind == PK_NORM) {
     const NormParams& q = p.norm;
     if (c->fp64) k_norm45_partials<double><<<dim3(kConvBlocks, q.n), 256, 0, st>>>(q);
@@ -1670,9 +1695,9 @@ int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
     return SBI_OK;
   }
-  if (p.kind == PK_ROW) e = p.row.packed ? launch_packed_row(p.nsize, p.row, st) : launch_row<double>(p.nsize, p.row, st);
-  else if (p.kind == PK_COL) e = p.col.packed ? launch_packed_col(p.nsize, p.col, st) : launch_col<double>(p.nsize, p.col, st);
-  else e = p.rk.packed ? launch_packed_rk(p.nsize, p.rk, st) : launch_rk<double>(p.nsize, p.rk, st);
+  if (p.kind == PK_ROW) e = p.row.packed ? launch_packed_row(p.nsize, p.row, st, chained) : launch_row<double>(p.nsize, p.row, st);
+  else if (p.kind == PK_COL) e = p.col.packed ? launch_packed_col(p.nsize, p.col, st, chained) : launch_col<double>(p.nsize, p.col, st);
+  else e = p.rk.packed ? launch_packed_rk(p.nsize, p.rk, st, chained) : launch_rk<double>(p.nsize, p.rk, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
   return SBI_OK;
 }
@@ -2532,7 +2557,7 @@ int build_step_graph(sbi_ctx* c, double dt, int kind, const Unit* only, GraphEnt
     for (size_t i = 0; i < gps[gi].size() && rc == SBI_OK; ++i, ++evi) {
       // external event records become timing nodes of the graph
       if (c->prof) cudaEventRecordWithFlags(ge.ev[2 * evi], st, cudaEventRecordExternal);
-      rc = launch_pass(c, gps[gi][i], st);
+      rc = launch_pass(c, gps[gi][i], st, i > 0 && !c->prof && !only && chainable(gps[gi][i]));
       if (c->prof) cudaEventRecordWithFlags(ge.ev[2 * evi + 1], st, cudaEventRecordExternal);
     }
     if (branch) {

@@ -226,9 +226,9 @@ template <typename T> bool col_stageable(int ny);
 // block, columns that share a group of threads and threads per column.
 cudaError_t prepare_packed_row_kernels(int nx);
 cudaError_t prepare_packed_col_kernels(int ny);
-cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st);
-cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st);
-cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st);
+cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st, bool chained);
+cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st, bool chained);
+cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st, bool chained);
 int packed_row_geometry(int nx, int* threads);
 int packed_col_geometry(int ny, int* tpc, int* group);
 bool packed_col_stageable(int ny);
