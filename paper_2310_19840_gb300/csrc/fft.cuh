@@ -33,7 +33,25 @@ template <typename T> using cx = typename cplx<T>::type;
 template <typename V> __device__ __forceinline__ V mk(decltype(V::x) a, decltype(V::x) b) { V v; v.x = a; v.y = b; return v; }
 template <typename V> __device__ __forceinline__ V cadd(V a, V b) { return mk<V>(a.x + b.x, a.y + b.y); }
 template <typename V> __device__ __forceinline__ V csub(V a, V b) { return mk<V>(a.x - b.x, a.y - b.y); }
-template <typename V> __device__ __forceinline__ V cmul(V a, V b) { return mk<V>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+// A complex product is two products and two fused multiply-adds, spelled out so
+// that every instantiation rounds alike.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
+  return mk<V>(fma(a.x, b.x, -mul_rn(a.y, b.y)), fma(a.x, b.y, mul_rn(a.y, b.x)));
+}
+// s + w z in four fused multiply-adds
+template <typename V> __device__ __forceinline__ V cfma(V w, V z, V s) {
+  return mk<V>(fma(w.x, z.x, fma(-w.y, z.y, s.x)), fma(w.x, z.y, fma(w.y, z.x, s.y)));
+}
+// a, b <- a + w b, a - w b.  The difference is 2 a - (a + w b): six fused
+// multiply-adds where the product and the two sums take eight operations.
+template <typename V> __device__ __forceinline__ void butterfly(V& a, V& b, V w) {
+  using S = decltype(V::x);
+  const V s = cfma(w, b, a);
+  b = mk<V>(fma(S(2), a.x, -s.x), fma(S(2), a.y, -s.y));
+  a = s;
+}
 template <typename V> __device__ __forceinline__ V cconj(V a) { return mk<V>(a.x, -a.y); }
 template <typename V, typename S> __device__ __forceinline__ V cscale(V a, S s) { return mk<V>(a.x * s, a.y * s); }
 // multiply by SIGN * i
@@ -51,22 +69,8 @@ __host__ __device__ constexpr int padded_len(int n) { return n + (n >> 4) + 1; }
 __host__ __device__ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// exp(SIGN 2 pi i q / 16) for q = 0..7 (q a compile-time constant after
-// unrolling)
-template <int SIGN, typename V>
-__device__ __forceinline__ V root16(int q) {
-  using S = decltype(V::x);
-  constexpr double c[8] = {1.0, 0.92387953251128675613, 0.70710678118654752440,
-                           0.38268343236508977173, 0.0, -0.38268343236508977173,
-                           -0.70710678118654752440, -0.92387953251128675613};
-  constexpr double s[8] = {0.0, 0.38268343236508977173, 0.70710678118654752440,
-                           0.92387953251128675613, 1.0, 0.92387953251128675613,
-                           0.70710678118654752440, 0.38268343236508977173};
-  return mk<V>(S(c[q]), SIGN > 0 ? S(s[q]) : S(-s[q]));
-}
-
 // ---------------------------------------------------------------------------
-// Radix-R DFT in registers, R in {1, 2, 4, 8, 16}, y_q = sum_r x_r w_R^{r q}.
+// Radix-R DFT in registers, R in {1, 2, 4, 8}, y_q = sum_r x_r w_R^{r q}.
 // ---------------------------------------------------------------------------
 template <int R, int SIGN, typename V> struct Dft;
 
@@ -93,43 +97,39 @@ template <int SIGN, typename V> struct Dft<4, SIGN, V> {
   }
 };
 
-// Split radix-2 step: DFT of length R from two DFTs of length R/2 of the even
-// and odd elements, y_q = E_q + w_R^q O_q, y_{q+R/2} = E_q - w_R^q O_q.
+// Split radix-2 step: DFT of length 8 from two DFTs of length 4 of the even and
+// odd elements, y_q = E_q + w_8^q O_q, y_{q+4} = E_q - w_8^q O_q; the factor
+// sqrt(1/2) of w_8 and w_8^3 enters by fused multiply-adds.
+template <int SIGN, typename V>
+__device__ __forceinline__ void dft8_join(V* x, const V* e, const V* o) {
+  using S = decltype(V::x);
+  const S h = S(0.70710678118654752440);
+  // w8^1 = h (1 + SIGN i), w8^2 = SIGN i, w8^3 = h (-1 + SIGN i)
+  const V u = cadd(o[1], rot<SIGN>(o[1])), v = csub(rot<SIGN>(o[3]), o[3]), o2 = rot<SIGN>(o[2]);
+  x[0] = cadd(e[0], o[0]); x[4] = csub(e[0], o[0]);
+  x[2] = cadd(e[2], o2);   x[6] = csub(e[2], o2);
+  x[1] = mk<V>(fma(h, u.x, e[1].x), fma(h, u.y, e[1].y));
+  x[5] = mk<V>(fma(-h, u.x, e[1].x), fma(-h, u.y, e[1].y));
+  x[3] = mk<V>(fma(h, v.x, e[3].x), fma(h, v.y, e[3].y));
+  x[7] = mk<V>(fma(-h, v.x, e[3].x), fma(-h, v.y, e[3].y));
+}
 template <int SIGN, typename V> struct Dft<8, SIGN, V> {
   __device__ __forceinline__ static void run(V* x) {
-    using S = decltype(V::x);
     V e[4] = {x[0], x[2], x[4], x[6]};
     V o[4] = {x[1], x[3], x[5], x[7]};
     Dft<4, SIGN, V>::run(e);
     Dft<4, SIGN, V>::run(o);
-    const S h = S(0.70710678118654752440);
-    // w8^1 = h (1 + SIGN i), w8^2 = SIGN i, w8^3 = h (-1 + SIGN i)
-    V o1 = cscale(cadd(o[1], rot<SIGN>(o[1])), h);
-    V o2 = rot<SIGN>(o[2]);
-    V o3 = cscale(csub(rot<SIGN>(o[3]), o[3]), h);
-    x[0] = cadd(e[0], o[0]); x[4] = csub(e[0], o[0]);
-    x[1] = cadd(e[1], o1);   x[5] = csub(e[1], o1);
-    x[2] = cadd(e[2], o2);   x[6] = csub(e[2], o2);
-    x[3] = cadd(e[3], o3);   x[7] = csub(e[3], o3);
+    dft8_join<SIGN>(x, e, o);
   }
 };
-
-template <int SIGN, typename V> struct Dft<16, SIGN, V> {
-  __device__ __forceinline__ static void run(V* x) {
-    using S = decltype(V::x);
-    V e[8], o[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { e[i] = x[2 * i]; o[i] = x[2 * i + 1]; }
-    Dft<8, SIGN, V>::run(e);
-    Dft<8, SIGN, V>::run(o);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      V t = q == 0 ? o[0] : cmul(o[q], root16<SIGN, V>(q));
-      x[q] = cadd(e[q], t);
-      x[q + 8] = csub(e[q], t);
-    }
-  }
-};
+// the same with x[2] .. x[5] = 0 (not read)
+template <int SIGN, typename V>
+__device__ __forceinline__ void dft8_outer(V* x) {
+  const V t = rot<SIGN>(x[6]), u = rot<SIGN>(x[7]);
+  const V e[4] = {cadd(x[0], x[6]), csub(x[0], t), csub(x[0], x[6]), cadd(x[0], t)};
+  const V o[4] = {cadd(x[1], x[7]), csub(x[1], u), csub(x[1], x[7]), cadd(x[1], u)};
+  dft8_join<SIGN>(x, e, o);
+}
 
 // ---------------------------------------------------------------------------
 // Twiddle tables: tw[off(N) + j] = exp(-2 pi i j / N), j < N, N = 2^q >= 2,
@@ -137,16 +137,52 @@ template <int SIGN, typename V> struct Dft<16, SIGN, V> {
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int tw_off(int n) { return n - 2; }
 
-// FP32 transforms form most twiddle powers by complex products of a few
-// table entries, which trades load/store-pipe work for FMA work; FP64
-// transforms load every power, because FP64 arithmetic is the scarcer
-// resource on this part.
-template <typename V> inline constexpr bool kProductTwiddles = sizeof(V) == 8;
-
 template <int SIGN, typename V>
 __device__ __forceinline__ V twiddle(const V* __restrict__ tw, int N, int idx) {
   V w = __ldg(tw + tw_off(N) + idx);
   return SIGN > 0 ? cconj(w) : w;
+}
+
+// DFT of length R of x[r] w^r, w = w_N^idx (idx < N / R): the twiddles of a
+// Stockham pass enter the butterflies, (a + w b, a - w b) at six fused
+// multiply-adds each, and only the powers w, w^2, w^4 and w w_8 are loaded.  A
+// radix-8 pass takes 72 FP64 operations (84 with the products first), a radix-4
+// pass 24 (28).
+template <int SIGN, typename V>
+__device__ __forceinline__ void dft4_twiddled(V& x0, V& x1, V& x2, V& x3, V w, V w2) {
+  butterfly(x0, x2, w2);
+  butterfly(x1, x3, w2);             // x0 + w^2 x2, x1 + w^2 x3 and the differences
+  butterfly(x0, x1, w);              // y0, y2
+  butterfly(x2, x3, rot<SIGN>(w));   // y1, y3
+  const V y2 = x1;
+  x1 = x2;
+  x2 = y2;
+}
+template <int R, int SIGN, typename V>
+__device__ __forceinline__ void dft_twiddled(V* x, const V* __restrict__ tw, int N, int idx) {
+  static_assert(R == 1 || R == 2 || R == 4 || R == 8, "radix");
+  if constexpr (R == 1) return;
+  const V w = twiddle<SIGN>(tw, N, idx);
+  if constexpr (R == 2) {
+    butterfly(x[0], x[1], w);
+  } else if constexpr (R == 4) {
+    dft4_twiddled<SIGN>(x[0], x[1], x[2], x[3], w, twiddle<SIGN>(tw, N, 2 * idx));
+  } else if constexpr (R == 8) {
+    const V w2 = twiddle<SIGN>(tw, N, 2 * idx), w4 = twiddle<SIGN>(tw, N, 4 * idx);
+    const V wr = twiddle<SIGN>(tw, N, idx + N / 8);
+    dft4_twiddled<SIGN>(x[0], x[2], x[4], x[6], w2, w4);   // E_q in x[2 q]
+    dft4_twiddled<SIGN>(x[1], x[3], x[5], x[7], w2, w4);   // O_q in x[2 q + 1]
+    butterfly(x[0], x[1], w);
+    butterfly(x[2], x[3], wr);
+    butterfly(x[4], x[5], rot<SIGN>(w));
+    butterfly(x[6], x[7], rot<SIGN>(wr));
+    const V y[4] = {x[1], x[3], x[5], x[7]};
+    x[1] = x[2];
+    x[2] = x[4];
+    x[3] = x[6];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[4 + q] = y[q];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -234,16 +270,7 @@ __device__ __forceinline__ void last_pass_by_shuffles(V (&x)[8], V* s, int j, co
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int b = j + q * T;
-    if constexpr (RP == 4 && kProductTwiddles<V>) {
-      const V w1 = twiddle<SIGN>(tw, N, b), w2 = cmul(w1, w1);
-      v[q][1] = cmul(v[q][1], w1);
-      v[q][2] = cmul(v[q][2], w2);
-      v[q][3] = cmul(v[q][3], cmul(w1, w2));
-    } else {
-#pragma unroll
-      for (int m = 1; m < RP; ++m) v[q][m] = cmul(v[q][m], twiddle<SIGN>(tw, N, m * b));
-    }
-    Dft<RP, SIGN, V>::run(v[q]);
+    dft_twiddled<RP, SIGN>(v[q], tw, N, b);
 #pragma unroll
     for (int m = 0; m < RP; ++m) {
       if constexpr (REGS) x[q + Q * m] = v[q][m];
@@ -257,7 +284,8 @@ __device__ __forceinline__ void last_pass_by_shuffles(V (&x)[8], V* s, int j, co
 template <int N, int R>
 inline constexpr bool kShuffleFft = kShuffleLastExchange && R == 8 && (N == 128 || N == 256);
 
-template <int N, int R, int Ls, int SIGN, typename V, bool REGS = false>
+// OUTER (first pass, R = 8): x[2] .. x[5] are zero and not read.
+template <int N, int R, int Ls, int SIGN, typename V, bool REGS = false, bool OUTER = false>
 struct StockhamPass {
   static constexpr bool WARP = (N / R) <= 32;
   __device__ __forceinline__ static void run(V (&x)[R], V* s, int j, const V* __restrict__ tw) {
@@ -266,47 +294,16 @@ struct StockhamPass {
       // the Ls = 8 pass, then the last pass fed by shuffles
       const int k = j & (Ls - 1);
       const int base = k * (N / (Ls * R));
-      if constexpr (kProductTwiddles<V>) {
-        const V w1 = twiddle<SIGN>(tw, N, base), w4 = twiddle<SIGN>(tw, N, 4 * base);
-        const V w2 = cmul(w1, w1), w3 = cmul(w1, w2);
-        x[1] = cmul(x[1], w1);
-        x[2] = cmul(x[2], w2);
-        x[3] = cmul(x[3], w3);
-        x[4] = cmul(x[4], w4);
-        x[5] = cmul(x[5], cmul(w4, w1));
-        x[6] = cmul(x[6], cmul(w4, w2));
-        x[7] = cmul(x[7], cmul(w4, w3));
-      } else {
-#pragma unroll
-        for (int r = 1; r < R; ++r) x[r] = cmul(x[r], twiddle<SIGN>(tw, N, r * base));
-      }
-      Dft<R, SIGN, V>::run(x);
+      dft_twiddled<R, SIGN>(x, tw, N, base);
       last_pass_by_shuffles<N, SIGN, REGS, V>(x, s, j, tw);
       return;
     }
     if constexpr (N / Ls >= R) {
       // full pass of radix R
       const int k = j & (Ls - 1);
-      if constexpr (Ls > 1) {
-        const int base = k * (N / (Ls * R));
-        if constexpr (R == 8 && kProductTwiddles<V>) {
-          // w^1 and w^4 from the table, the other powers by products (at most
-          // three roundings each): 2 loads instead of 7
-          const V w1 = twiddle<SIGN>(tw, N, base), w4 = twiddle<SIGN>(tw, N, 4 * base);
-          const V w2 = cmul(w1, w1), w3 = cmul(w1, w2);
-          x[1] = cmul(x[1], w1);
-          x[2] = cmul(x[2], w2);
-          x[3] = cmul(x[3], w3);
-          x[4] = cmul(x[4], w4);
-          x[5] = cmul(x[5], cmul(w4, w1));
-          x[6] = cmul(x[6], cmul(w4, w2));
-          x[7] = cmul(x[7], cmul(w4, w3));
-        } else {
-#pragma unroll
-          for (int r = 1; r < R; ++r) x[r] = cmul(x[r], twiddle<SIGN>(tw, N, r * base));
-        }
-      }
-      Dft<R, SIGN, V>::run(x);
+      if constexpr (Ls > 1) dft_twiddled<R, SIGN>(x, tw, N, k * (N / (Ls * R)));
+      else if constexpr (OUTER && R == 8) dft8_outer<SIGN>(x);
+      else Dft<R, SIGN, V>::run(x);
       const int sb = pad((j - k) * R) + pad(k);   // pad((j - k) R + k + r Ls) - pad(r Ls)
 #pragma unroll
       for (int r = 0; r < R; ++r) s[sb + pad(r * Ls)] = x[r];
@@ -329,17 +326,7 @@ struct StockhamPass {
         const int b = j + q * T;
 #pragma unroll
         for (int m = 0; m < RP; ++m) v[m] = x[q + m * Q];
-        if constexpr (RP == 4 && kProductTwiddles<V>) {
-          // w^b from the table, w^2b and w^3b by products
-          const V w1 = twiddle<SIGN>(tw, N, b), w2 = cmul(w1, w1);
-          v[1] = cmul(v[1], w1);
-          v[2] = cmul(v[2], w2);
-          v[3] = cmul(v[3], cmul(w1, w2));
-        } else {
-#pragma unroll
-          for (int m = 1; m < RP; ++m) v[m] = cmul(v[m], twiddle<SIGN>(tw, N, m * b));
-        }
-        Dft<RP, SIGN, V>::run(v);
+        dft_twiddled<RP, SIGN>(v, tw, N, b);
 #pragma unroll
         for (int m = 0; m < RP; ++m) s[pad(j) + pad(q * T) + pad(m * Ls)] = v[m];
       }
@@ -348,7 +335,7 @@ struct StockhamPass {
   }
 };
 
-template <int N, int R, int SIGN, typename V>
+template <int N, int R, int SIGN, typename V, bool OUTER = false>
 __device__ __forceinline__ void fft_block(V (&x)[R], V* s, int j, const V* __restrict__ tw) {
   static_assert((N & (N - 1)) == 0 && N >= 1, "N must be a power of two");
   static_assert(R >= 1 && R <= N && (R & (R - 1)) == 0, "R must be a power of two <= N");
@@ -356,7 +343,7 @@ __device__ __forceinline__ void fft_block(V (&x)[R], V* s, int j, const V* __res
     s[0] = x[0];
     __syncwarp();
   } else {
-    StockhamPass<N, R, 1, SIGN, V>::run(x, s, j, tw);
+    StockhamPass<N, R, 1, SIGN, V, false, OUTER>::run(x, s, j, tw);
   }
 }
 
@@ -364,13 +351,13 @@ __device__ __forceinline__ void fft_block(V (&x)[R], V* s, int j, const V* __res
 // registers on exit: x[r] = X[j + r N/R].  Where the last pass is fed by
 // shuffles it ends there (no final scatter and read-back); otherwise the
 // result is read back from s.  s has no live data on exit either way.
-template <int N, int R, int SIGN, typename V>
+template <int N, int R, int SIGN, bool OUTER = false, typename V>
 __device__ __forceinline__ void fft_block_regs(V (&x)[R], V* s, int j, const V* __restrict__ tw) {
   if constexpr (kShuffleFft<N, R>) {
-    StockhamPass<N, R, 1, SIGN, V, true>::run(x, s, j, tw);
+    StockhamPass<N, R, 1, SIGN, V, true, OUTER>::run(x, s, j, tw);
   } else {
     constexpr int T = N / R;
-    fft_block<N, R, SIGN>(x, s, j, tw);
+    fft_block<N, R, SIGN, V, OUTER>(x, s, j, tw);
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = s[pad(j) + pad(r * T)];
   }
@@ -407,32 +394,11 @@ __host__ __device__ constexpr int fft_scratch_len() {
   return kSplitFft<N, R> ? (N / 256) * padded_len(256) : padded_len(N);
 }
 
-// v[k] *= w_N^{k m} for k = 1 .. S - 1 (FP32: powers by products, at most
-// three roundings each; FP64: every power from the table)
+// v[k] *= w_N^{k m} for k = 1 .. S - 1
 template <int S, int SIGN, typename V>
 __device__ __forceinline__ void twiddle_run(V (&v)[S], const V* __restrict__ tw, int N, int m) {
-  if constexpr (S == 1) {
-    return;
-  } else if constexpr (kProductTwiddles<V>) {
-    const V w1 = twiddle<SIGN>(tw, N, m);
-    const V w2 = cmul(w1, w1);
-    v[1] = cmul(v[1], w1);
-    if constexpr (S >= 4) {
-      const V w3 = cmul(w1, w2);
-      v[2] = cmul(v[2], w2);
-      v[3] = cmul(v[3], w3);
-      if constexpr (S == 8) {
-        const V w4 = twiddle<SIGN>(tw, N, 4 * m);
-        v[4] = cmul(v[4], w4);
-        v[5] = cmul(v[5], cmul(w4, w1));
-        v[6] = cmul(v[6], cmul(w4, w2));
-        v[7] = cmul(v[7], cmul(w4, w3));
-      }
-    }
-  } else {
 #pragma unroll
-    for (int k = 1; k < S; ++k) v[k] = cmul(v[k], twiddle<SIGN>(tw, N, k * m));
-  }
+  for (int k = 1; k < S; ++k) v[k] = cmul(v[k], twiddle<SIGN>(tw, N, k * m));
 }
 
 template <int N, int SIGN, typename V>
@@ -458,23 +424,12 @@ __device__ __forceinline__ void fft_split_dif(V (&x)[8], V* s, int j, const V* _
   fft_block_regs<256, 8, SIGN>(x, row, l, tw);
 }
 
-template <int N, int SIGN, typename V>
+template <int N, int SIGN, bool OUTER = false, typename V>
 __device__ __forceinline__ void fft_split_dit(V (&x)[8], V* s, int j, const V* __restrict__ tw) {
   constexpr int S = N / 256, P = 8 / S, T = N / 8, PP = padded_len(256);
   const int q = j >> 5, l = j & 31;
   V* row = s + q * PP;
-  fft_block_regs<256, 8, SIGN>(x, row, l, tw);   // x[r] = Y_q[l + 32 r]; row free again
-  if (q > 0) {
-    // w_N^{q (l + 32 r)} = w_N^{q l} w_N^{32 q r}
-    if constexpr (kProductTwiddles<V>) {
-      const V wl = twiddle<SIGN>(tw, N, q * l);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) x[r] = cmul(x[r], r == 0 ? wl : cmul(wl, twiddle<SIGN>(tw, N, 32 * q * r)));
-    } else {
-#pragma unroll
-      for (int r = 0; r < 8; ++r) x[r] = cmul(x[r], twiddle<SIGN>(tw, N, q * (l + 32 * r)));
-    }
-  }
+  fft_block_regs<256, 8, SIGN, OUTER>(x, row, l, tw);   // x[r] = Y_q[l + 32 r]; row free again
 #pragma unroll
   for (int r = 0; r < 8; ++r) row[pad(l) + pad(32 * r)] = x[r];
   __syncthreads();
@@ -484,7 +439,7 @@ __device__ __forceinline__ void fft_split_dit(V (&x)[8], V* s, int j, const V* _
     V v[S];
 #pragma unroll
     for (int k = 0; k < S; ++k) v[k] = s[k * PP + pad(m)];
-    Dft<S, SIGN, V>::run(v);
+    dft_twiddled<S, SIGN>(v, tw, N, m);
 #pragma unroll
     for (int w = 0; w < S; ++w) x[p + P * w] = v[w];
   }

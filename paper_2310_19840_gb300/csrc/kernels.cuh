@@ -235,23 +235,17 @@ __device__ __forceinline__ void c2r_input(cx<T> (&x)[RowCfg<NX>::R], const cx<T>
                                           const cx<T>* __restrict__ tw) {
   using V = cx<T>;
   using C = RowCfg<NX>;
-  // e^{+2 pi i k / NX} = e^{+2 pi i j / NX} e^{+pi i r / R}: in FP32 with
-  // R = 8 one table load and products by the 16th roots of unity
-  constexpr bool kProd = C::R == 8 && kProductTwiddles<V>;
-  const V wj = kProd ? cconj(__ldg(tw + tw_off(NX) + j)) : mk<V>(T(1), T(0));
   if (2 * W <= C::n) {
     // At most half the packed modes are kept: X[k] and X[n-k] are never both
-    // nonzero, so Z[k] = X[k] (1 + i w) for k < W, conj(X[n-k]) (1 - i w) for
-    // k > n - W and 0 in between (one load and one product per element).
+    // nonzero, so Z[k] = X[k] + i w X[k] for k < W, Y - i w Y with Y = conj(X[n-k])
+    // for k > n - W and 0 in between (four fused multiply-adds).
 #pragma unroll
     for (int r = 0; r < C::R; ++r) {
       const int k = j + r * C::TPR;
-      V w;
-      if constexpr (kProd) w = r == 0 ? wj : cmul(wj, root16<1, V>(r));
-      else w = cconj(__ldg(tw + tw_off(NX) + k));
+      const V w = cconj(__ldg(tw + tw_off(NX) + k));
       V z = mk<V>(T(0), T(0));
-      if (k < W) z = cmul(stg[k], mk<V>(T(1) - w.y, w.x));                       // (1 + i w)
-      else if (k > C::n - W) z = cmul(cconj(stg[C::n - k]), mk<V>(T(1) + w.y, -w.x));  // (1 - i w)
+      if (k < W) z = cfma(rot<1>(w), stg[k], stg[k]);
+      else if (k > C::n - W) z = cfma(rot<-1>(w), cconj(stg[C::n - k]), cconj(stg[C::n - k]));
       x[r] = cconj(z);
     }
     return;
@@ -263,22 +257,19 @@ __device__ __forceinline__ void c2r_input(cx<T> (&x)[RowCfg<NX>::R], const cx<T>
     const V a = (k < W) ? stg[k] : mk<V>(T(0), T(0));
     const V b = (k > 0 && kk < W) ? stg[kk] : mk<V>(T(0), T(0));
     const V bc = cconj(b);
-    const V E = cadd(a, bc);
-    V w;
-    if constexpr (kProd) w = r == 0 ? wj : cmul(wj, root16<1, V>(r));
-    else w = cconj(__ldg(tw + tw_off(NX) + k));
-    const V O = cmul(csub(a, bc), w);
-    x[r] = cconj(cadd(E, rot<1>(O)));
+    const V w = cconj(__ldg(tw + tw_off(NX) + k));
+    x[r] = cconj(cfma(rot<1>(w), csub(a, bc), cadd(a, bc)));
   }
 }
 
 // Packed forward real FFT, output side, block-cooperative: each row's
 // natural-order Z is in fb[rl]; the kept modes
 // X[k] = 1/2 (Z[k] + Z*[n-k]) - i/2 e^{-2 pi i k / NX} (Z[k] - Z*[n-k]), k < W,
-// are written to the transposed mixed field dst.
+// are written to the transposed mixed field dst.  halved: the transform's input
+// carried the factor 1/2 already.
 template <typename T, int NX>
 __device__ __forceinline__ void r2c_store(const cx<T>* fb_all, int fbs, const BufRef& dst, const RowIO& io,
-                                          const cx<T>* __restrict__ tw) {
+                                          const cx<T>* __restrict__ tw, bool halved) {
   using V = cx<T>;
   using C = RowCfg<NX>;
   if (!io.ok) return;
@@ -287,9 +278,8 @@ __device__ __forceinline__ void r2c_store(const cx<T>* fb_all, int fbs, const Bu
   for (int k = io.k0; k < io.W; k += io.kstep) {
     const V zk = fb[pad(k)];
     const V zc = cconj(fb[pad((C::n - k) & (C::n - 1))]);
-    const V s = cadd(zk, zc);
-    const V d = cmul(csub(zk, zc), __ldg(tw + tw_off(NX) + k));
-    out[io.at(dst, k)] = cscale(csub(s, rot<1>(d)), T(0.5));
+    const V s = cfma(rot<-1>(__ldg(tw + tw_off(NX) + k)), csub(zk, zc), cadd(zk, zc));
+    out[io.at(dst, k)] = halved ? s : cscale(s, T(0.5));
   }
 }
 
@@ -298,18 +288,14 @@ __device__ __forceinline__ void r2c_store(const cx<T>* fb_all, int fbs, const Bu
 // X[k] = 1/2 (Z[k] + Z*[n-k]) - i/2 e^{-2 pi i k / NX} (Z[k] - Z*[n-k]) for its
 // own k = j + r TPR < W, writing it to the row's buffer xrow[k].  Z[n-k] sits
 // in lane (TPR - j) mod TPR of the row, register R-1-r (thread 0: its own
-// register (R - r) mod R), so one shuffle per kept register fetches it.  The
-// twiddle is e^{-2 pi i j / NX} times e^{-2 pi i r / 16} (TPR / NX = 1/16)
-// in FP32, the table entry in FP64.
+// register (R - r) mod R), so one shuffle per kept register fetches it.
 template <typename T, int NX>
 __device__ __forceinline__ void r2c_regs(const cx<T> (&x)[RowCfg<NX>::R], cx<T>* xrow, int W, int j,
-                                         const cx<T>* __restrict__ tw) {
+                                         const cx<T>* __restrict__ tw, bool halved) {
   using V = cx<T>;
   using C = RowCfg<NX>;
   constexpr int R = C::R, TPR = C::TPR;
   static_assert(R == 8 && 2 * R * TPR == NX, "rows of the shuffle-fed transforms only");
-  constexpr bool kProd = kProductTwiddles<V>;     // FP64: every twiddle from the table
-  const V wj = __ldg(tw + tw_off(NX) + j);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     if (r * TPR >= W) break;                       // no thread keeps a mode here
@@ -318,14 +304,9 @@ __device__ __forceinline__ void r2c_regs(const cx<T> (&x)[RowCfg<NX>::R], cx<T>*
     zc.y = __shfl_sync(0xffffffffu, x[R - 1 - r].y, (TPR - j) & (TPR - 1), TPR);
     if (j == 0) zc = x[(R - r) & (R - 1)];
     zc = cconj(zc);
-    const V zk = x[r];
     const int k = j + r * TPR;
-    V w;
-    if constexpr (kProd) w = r == 0 ? wj : cmul(wj, root16<-1, V>(r));
-    else w = __ldg(tw + tw_off(NX) + k);
-    const V sum = cadd(zk, zc);
-    const V d = cmul(csub(zk, zc), w);
-    if (k < W) xrow[k] = cscale(csub(sum, rot<1>(d)), T(0.5));
+    const V s = cfma(rot<-1>(__ldg(tw + tw_off(NX) + k)), csub(x[r], zc), cadd(x[r], zc));
+    if (k < W) xrow[k] = halved ? s : cscale(s, T(0.5));
   }
 }
 
@@ -381,6 +362,7 @@ k_row(const __grid_constant__ RowParams p) {
   for (int o = 0; o < p.nops; ++o) {
     const RowOp op = p.ops[o];
     V x[R];
+    bool halved = false;
     if (op.kind == ROP_C2R) {
       if (o == pending) {
         cp_async_wait_all();
@@ -397,7 +379,9 @@ k_row(const __grid_constant__ RowParams p) {
       if (pending >= 0) stage_async<T>(stg_all, sw, p.buf[p.ops[pending].a], io);
     } else if (op.kind == ROP_PROD) {
       V* slot = op.slot == kNone ? nullptr : slot_base + (op.slot * rpc + rloc) * n;
-      const T cf = T(op.coef);
+      // the factor 1/2 of the packed transform's output goes with the product's own
+      halved = op.coef != 1.0;
+      const T cf = T(0.5 * op.coef);
       const bool running = (op.c & 2) != 0;
       const V* drow = (act && op.b > 0 && p.delta.ptr) ? phys_row<T>(p.delta, member, y, NX) : nullptr;
       const V* wrow = (act && (op.c & 1) && p.wgt.ptr) ? phys_row<T>(p.wgt, member, y, NX) : nullptr;
@@ -411,7 +395,7 @@ k_row(const __grid_constant__ RowParams p) {
           V v = slot[m];
           v = mk<V>(v.x * e.x, v.y * e.y);
           slot[m] = v;
-          x[r] = mk<V>(cf * v.x, cf * v.y);
+          x[r] = halved ? cscale(v, cf) : v;
         }
       } else {
 #pragma unroll
@@ -435,7 +419,7 @@ k_row(const __grid_constant__ RowParams p) {
           const V w = __ldg(wrow + m);
           v = mk<V>(v.x * w.x, v.y * w.y);
         }
-        x[r] = mk<V>(cf * v.x, cf * v.y);
+        x[r] = halved ? cscale(v, cf) : v;
       }
       }
     } else {
@@ -498,13 +482,13 @@ k_row(const __grid_constant__ RowParams p) {
     if constexpr (kShuffleFft<n, R>) {
       // spectrum in registers, kept modes formed in the row's own threads
       fft_block_regs<n, R, -1>(x, fb, j, tw);
-      r2c_regs<T, NX>(x, fb, p.W, j, tw);
+      r2c_regs<T, NX>(x, fb, p.W, j, tw, halved);
       __syncthreads();  // every row's kept modes ready
       store_modes<T>(fb_all, fbs, p.buf[op.dst], io);
     } else {
       fft_to_smem<n, R, -1>(x, fb, j, tw);
       __syncthreads();  // every row's spectrum ready
-      r2c_store<T, NX>(fb_all, fbs, p.buf[op.dst], io, tw);
+      r2c_store<T, NX>(fb_all, fbs, p.buf[op.dst], io, tw, halved);
     }
   }
 }
@@ -757,11 +741,11 @@ k_rk(const __grid_constant__ RkParams p) {
   __syncthreads();
   fft_to_smem<n, R, -1>(xe, fb, j, tw);
   __syncthreads();
-  r2c_store<T, NX>(fb_all, fbs, p.eta_hat, io, tw);
+  r2c_store<T, NX>(fb_all, fbs, p.eta_hat, io, tw, false);
   __syncthreads();
   fft_to_smem<n, R, -1>(xp, fb, j, tw);
   __syncthreads();
-  r2c_store<T, NX>(fb_all, fbs, p.phi_hat, io, tw);
+  r2c_store<T, NX>(fb_all, fbs, p.phi_hat, io, tw, false);
 }
 
 // ===========================================================================
@@ -828,22 +812,35 @@ __host__ __device__ constexpr bool col_cpb_ok(int cpb) {
   return cpb >= 1 && cpb <= C::CPB && (cpb * C::TPC) % 32 == 0;
 }
 
+// a + x f i^q
 template <typename V, typename S>
-__device__ __forceinline__ V cmul_ipow(V x, S f, int q) {   // x f i^q
-  const S re = x.x * f, im = x.y * f;
-  S r2 = (q & 1) ? -im : re;
-  S i2 = (q & 1) ? re : im;
-  if (q & 2) {
-    r2 = -r2;
-    i2 = -i2;
-  }
-  return mk<V>(r2, i2);
+__device__ __forceinline__ V acc_ipow(V a, V x, S f, int q) {
+  const S u = (q & 1) ? x.y : x.x, v = (q & 1) ? x.x : x.y;
+  return mk<V>(fma(q == 1 || q == 2 ? -f : f, u, a.x), fma(q & 2 ? -f : f, v, a.y));
+}
+// (x f i^q)*
+template <typename V, typename S>
+__device__ __forceinline__ V conj_ipow(V x, S f, int q) {
+  const S u = (q & 1) ? x.y : x.x, v = (q & 1) ? x.x : x.y;
+  return mk<V>((q == 1 || q == 2 ? -f : f) * u, (q & 2 ? f : -f) * v);
+}
+
+// every output carries the dealias mask and at most half of the modes are kept
+inline bool col_outer(const ColParams& p) {
+  bool outer = p.ky_keep <= p.ny / 4;
+  for (int o = 0; o < p.nouts; ++o) outer = outer && p.outs[o].mask == 1;
+  return outer;
 }
 
 // STAGED: each column's inputs arrive by bulk copies (TMA) into a staging
 // column in shared memory, the next input in flight while the current one is
 // transformed and accumulated; the arithmetic is that of the direct form.
-template <typename T, int NY, bool STAGED>
+// OUTER (col_outer): of a thread's eight modes only slots 0, 1, 6 and 7 can be
+// kept, so their sums stay in registers and the others are neither formed by
+// the forward transform's last pass nor read by the inverse one's first.
+// FP64 issue bounds the pass (two lanes per cycle and SM): per column element
+// and transform it took some 30 FP64 operations, and takes 21 to 22.
+template <typename T, int NY, bool OUTER, bool STAGED>
 __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS, ColCfg<T, NY>::MIN_BLOCKS)
 k_col(const __grid_constant__ ColParams p) {
   using V = cx<T>;
@@ -876,12 +873,20 @@ k_col(const __grid_constant__ ColParams p) {
   auto nat = [&](int r) { return j + r * TPC; };
   auto fwd = [&](int r) { return SPLIT ? jd + r * TPC : nat(r); };
   auto acc_at = [&](int m) { return SPLIT ? pad(m) : m; };
+  auto outer_slot = [](int r) { return r < 2 ? r : r + 4; };
   // table position of slot r's mode m (split: the table's decimated order)
   auto tab_at = [&](int r, int m) { return SPLIT ? 256 * (j >> 5) + (j & 31) + 32 * r : m; };
+  V sum[OUTER ? kMaxColAcc : 1][OUTER ? 4 : 1];   // OUTER: slots 0, 1, 6, 7
+  if constexpr (OUTER) {
+    static_assert(RC == 8 && kMaxColAcc == 2, "two accumulators of eight slots");
 #pragma unroll
-  for (int r = 0; r < RC; ++r) {
-    acc0[acc_at(fwd(r))] = mk<V>(T(0), T(0));
-    acc1[acc_at(fwd(r))] = mk<V>(T(0), T(0));
+    for (int r = 0; r < 4; ++r) sum[0][r] = sum[1][r] = mk<V>(T(0), T(0));
+  } else {
+#pragma unroll
+    for (int r = 0; r < RC; ++r) {
+      acc0[acc_at(fwd(r))] = mk<V>(T(0), T(0));
+      acc1[acc_at(fwd(r))] = mk<V>(T(0), T(0));
+    }
   }
   // staged form: the column's staging run and barrier; thread j = 0 of the
   // column arms the barrier and issues the copy of input i (16-byte aligned:
@@ -943,12 +948,24 @@ k_col(const __grid_constant__ ColParams p) {
       const ColTerm t = p.terms[q];
       const T* tab = reinterpret_cast<const T*>(t.tab) + col_off;
       const int ph = (t.gx + t.gy) & 3;
-      V* acc = (t.acc == 0) ? acc0 : acc1;
+      if constexpr (OUTER) {
+        T f[4];
 #pragma unroll
-      for (int r = 0; r < RC; ++r) {
-        const int ni = fwd(r);
-        const V v = x[r];
-        acc[acc_at(ni)] = cadd(acc[acc_at(ni)], cmul_ipow(v, __ldg(tab + tab_at(r, ni)), ph));
+        for (int r = 0; r < 4; ++r) f[r] = __ldg(tab + tab_at(outer_slot(r), fwd(outer_slot(r))));
+        if (t.acc == 0) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) sum[0][r] = acc_ipow(sum[0][r], x[outer_slot(r)], f[r], ph);
+        } else {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) sum[1][r] = acc_ipow(sum[1][r], x[outer_slot(r)], f[r], ph);
+        }
+      } else {
+        V* acc = (t.acc == 0) ? acc0 : acc1;
+#pragma unroll
+        for (int r = 0; r < RC; ++r) {
+          const int ni = fwd(r);
+          acc[acc_at(ni)] = acc_ipow(acc[acc_at(ni)], x[r], __ldg(tab + tab_at(r, ni)), ph);
+        }
       }
     }
   }
@@ -957,22 +974,30 @@ k_col(const __grid_constant__ ColParams p) {
     const ColTerm t = p.outs[o];
     const T* tab = reinterpret_cast<const T*>(t.tab) + col_off;
     const int ph = (t.gx + t.gy) & 3;
-    const V* acc = (t.acc == 0) ? acc0 : acc1;
     V x[RC];
     // conjugated input: the forward FFT of conj(X) is the conjugate of F^{-1}(X)
+    if constexpr (OUTER) {
 #pragma unroll
-    for (int r = 0; r < RC; ++r) {
-      const int ni = fwd(r);
-      x[r] = cconj(cmul_ipow(acc[acc_at(ni)], __ldg(tab + tab_at(r, ni)), ph));
+      for (int r = 0; r < 4; ++r) {
+        const V a = t.acc == 0 ? sum[0][r] : sum[1][r];
+        x[outer_slot(r)] = conj_ipow(a, __ldg(tab + tab_at(outer_slot(r), fwd(outer_slot(r)))), ph);
+      }
+    } else {
+      const V* acc = (t.acc == 0) ? acc0 : acc1;
+#pragma unroll
+      for (int r = 0; r < RC; ++r) {
+        const int ni = fwd(r);
+        x[r] = conj_ipow(acc[acc_at(ni)], __ldg(tab + tab_at(r, ni)), ph);
+      }
     }
     if constexpr (SPLIT) {
       __syncthreads();
-      fft_split_dit<NY, -1>(x, sc, j, tw);         // x[r]: element nat(r)
+      fft_split_dit<NY, -1, OUTER>(x, sc, j, tw);  // x[r]: element nat(r)
 #pragma unroll
       for (int r = 0; r < RC; ++r) x[r] = cconj(x[r]);
     } else if constexpr (NY > 1) {
       group_sync<C::WARP>();
-      fft_block_regs<NY, RC, -1>(x, sc, j, tw);
+      fft_block_regs<NY, RC, -1, OUTER>(x, sc, j, tw);
 #pragma unroll
       for (int r = 0; r < RC; ++r) x[r] = cconj(x[r]);
     } else {
@@ -1123,11 +1148,17 @@ cudaError_t prepare_nx() {
 
 template <typename T, int NY>
 cudaError_t prepare_ny() {
-  cudaError_t e = cudaFuncSetAttribute(k_col<T, NY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)col_smem<T, NY>(kMaxColAcc, ColCfg<T, NY>::CPB));
-  if (e != cudaSuccess || !kColStageable<T, NY>) return e;
-  return cudaFuncSetAttribute(k_col<T, NY, kColStageable<T, NY>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)col_smem_staged<T, NY>(kMaxColAcc, ColCfg<T, NY>::CPB));
+  constexpr bool O = NY >= 8, S = kColStageable<T, NY>;
+  auto allow = [](auto k, size_t bytes) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  const size_t plain = col_smem<T, NY>(kMaxColAcc, ColCfg<T, NY>::CPB);
+  const size_t staged = col_smem_staged<T, NY>(kMaxColAcc, ColCfg<T, NY>::CPB);
+  cudaError_t e = allow(k_col<T, NY, false, false>, plain);
+  if (e == cudaSuccess) e = allow(k_col<T, NY, O, false>, plain);
+  if (e == cudaSuccess && S) e = allow(k_col<T, NY, false, S>, staged);
+  if (e == cudaSuccess && S) e = allow(k_col<T, NY, O, S>, staged);
+  return e;
 }
 
 template <typename T, int NX>
@@ -1168,13 +1199,22 @@ cudaError_t launch_col_n(const ColParams& p, cudaStream_t st) {
   const int cpb = col_cpb<T, NY>(p.cpb);
   if (!col_cpb_ok<T, NY>(cpb) || p.col_begin < 0 || p.col_begin >= p.cols_total) return cudaErrorInvalidValue;
   const int blocks = (p.cols_total - p.col_begin + cpb - 1) / cpb;
+  constexpr bool O = NY >= 8;
+  const bool outer = O && col_outer(p);
+  // OUTER: the sums are in registers, no accumulators in shared memory
+  const int nacc = outer ? 0 : p.nacc;
   if (p.staged) {
-    if constexpr (kColStageable<T, NY>)
-      k_col<T, NY, true><<<blocks, C::TPC * cpb, col_smem_staged<T, NY>(p.nacc, cpb), st>>>(p);
-    else
+    if constexpr (kColStageable<T, NY>) {
+      const size_t smem = col_smem_staged<T, NY>(p.nacc, cpb);
+      if (outer) k_col<T, NY, O, true><<<blocks, C::TPC * cpb, smem, st>>>(p);
+      else k_col<T, NY, false, true><<<blocks, C::TPC * cpb, smem, st>>>(p);
+    } else {
       return cudaErrorInvalidValue;
+    }
   } else {
-    k_col<T, NY, false><<<blocks, C::TPC * cpb, col_smem<T, NY>(p.nacc, cpb), st>>>(p);
+    const size_t smem = col_smem<T, NY>(nacc, cpb);
+    if (outer) k_col<T, NY, O, false><<<blocks, C::TPC * cpb, smem, st>>>(p);
+    else k_col<T, NY, false, false><<<blocks, C::TPC * cpb, smem, st>>>(p);
   }
   return cudaGetLastError();
 }
