@@ -218,8 +218,8 @@ __device__ __forceinline__ void stage_async(cx<T>* stg_all, int sw, const BufRef
 // inputs are staged asynchronously, ahead of time), else -1.  A C2R that sums
 // several buffers is staged synchronously, so nothing may be in flight into
 // the staging rows before it.
-__device__ __forceinline__ int next_async_c2r(const RowParams& p, int o) {
-  for (; o < p.nops; ++o)
+__device__ __forceinline__ int next_async_c2r(const RowParams& p, int o, int end) {
+  for (; o < end; ++o)
     if (p.ops[o].kind == ROP_C2R) return p.ops[o].b == 1 ? o : -1;
   return -1;
 }
@@ -328,6 +328,9 @@ __device__ __forceinline__ T ipow(T v, int p) {
   return r;
 }
 
+// blockIdx.y takes a segment of the operations: the whole list, or one inverse
+// transform and the products formed from it.  A pass over few rows then has
+// several times the blocks, and every SM's FP64 lanes the same share of them.
 template <typename T, int NX>
 __global__ void __launch_bounds__(RowCfg<NX>::MAX_THREADS, RowCfg<NX>::template min_blocks<T>())
 k_row(const __grid_constant__ RowParams p) {
@@ -356,10 +359,11 @@ k_row(const __grid_constant__ RowParams p) {
   const V* eta = (act && p.eta.ptr) ? phys_row<T>(p.eta, member, y, NX) : nullptr;
 
   // the first single-buffer input is in flight from the start
-  int pending = next_async_c2r(p, 0);
+  const int end = p.seg[blockIdx.y].end;
+  int pending = next_async_c2r(p, p.seg[blockIdx.y].begin, end);
   if (pending >= 0) stage_async<T>(stg_all, sw, p.buf[p.ops[pending].a], io);
 
-  for (int o = 0; o < p.nops; ++o) {
+  for (int o = p.seg[blockIdx.y].begin; o < end; ++o) {
     const RowOp op = p.ops[o];
     V x[R];
     bool halved = false;
@@ -375,7 +379,7 @@ k_row(const __grid_constant__ RowParams p) {
       c2r_input<T, NX>(x, stg_all + rloc * sw, p.W, fft_in_index<n, R>(j), tw);
       __syncthreads();  // every row has read its staging row; scratch free
       // the next single-buffer input lands while this one is transformed
-      pending = next_async_c2r(p, o + 1);
+      pending = next_async_c2r(p, o + 1, end);
       if (pending >= 0) stage_async<T>(stg_all, sw, p.buf[p.ops[pending].a], io);
     } else if (op.kind == ROP_PROD) {
       V* slot = op.slot == kNone ? nullptr : slot_base + (op.slot * rpc + rloc) * n;
@@ -1161,6 +1165,29 @@ cudaError_t prepare_ny() {
   return e;
 }
 
+// Segments of a row pass: `per` products each, 0 keeps the operations of a row
+// in one block; returns their number (0: too many).
+inline int make_segments(RowParams& q, int per) {
+  if (per <= 0) {
+    q.seg[0] = RowSeg{0, 0, (uint8_t)q.nops};
+    return 1;
+  }
+  int ns = 0;
+  for (int o = 0; o < q.nops;) {
+    int e = o + 1;
+    while (e < q.nops && q.ops[e].kind != ROP_C2R) ++e;
+    int f = o + 1;
+    do {
+      if (ns == kMaxRowSegs) return 0;
+      const int last = f + per < e ? f + per : e;
+      q.seg[ns++] = RowSeg{(uint8_t)o, (uint8_t)f, (uint8_t)last};
+      f = last;
+    } while (f < e);
+    o = e;
+  }
+  return ns;
+}
+
 template <typename T, int NX>
 cudaError_t launch_row_n(const RowParams& p, cudaStream_t st) {
   using C = RowCfg<NX>;
@@ -1174,7 +1201,9 @@ cudaError_t launch_row_n(const RowParams& p, cudaStream_t st) {
   q.sws = rs.sws;
   const size_t smem = row_smem<T, NX>(q.rpc, q.fbs, q.sws, q.nslots);
   if (smem > row_smem_bound<T, NX>(q.W, q.nslots) * (size_t)q.rpc) return cudaErrorInvalidValue;
-  k_row<T, NX><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
+  const int ns = make_segments(q, p.split);
+  if (ns < 1 || (p.split > 0 && (p.nslots > 1 || p.split < kMaxRowOps))) return cudaErrorInvalidValue;
+  k_row<T, NX><<<dim3((unsigned)blocks, (unsigned)ns), C::TPR * q.rpc, smem, st>>>(q);
   return cudaGetLastError();
 }
 

@@ -1139,29 +1139,6 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
 // ===========================================================================
 // Launchers
 // ===========================================================================
-// Segments of a row pass: `per` products each, 0 keeps the operations of a row
-// in one block; returns their number (0: too many).
-inline int make_segments(RowParams& q, int per) {
-  if (per <= 0) {
-    q.seg[0] = RowSeg{0, 0, (uint8_t)q.nops};
-    return 1;
-  }
-  int ns = 0;
-  for (int o = 0; o < q.nops;) {
-    int e = o + 1;
-    while (e < q.nops && q.ops[e].kind != ROP_C2R) ++e;
-    int f = o + 1;
-    do {
-      if (ns == kMaxRowSegs) return 0;
-      const int last = f + per < e ? f + per : e;
-      q.seg[ns++] = RowSeg{(uint8_t)o, (uint8_t)f, (uint8_t)last};
-      f = last;
-    } while (f < e);
-    o = e;
-  }
-  return ns;
-}
-
 // Launches a pass; chained: behind another pass of the same stream, which it may
 // overlap up to its wait_for_previous().
 template <typename... P, typename... A>

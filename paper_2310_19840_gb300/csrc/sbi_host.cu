@@ -464,7 +464,7 @@ struct Planner {
     }
     r.p.nslots = r.maxslot + 1;
     r.p.rpc = rpc_for(r.p.nslots);
-    if (g.packed) r.p.split = default_split(r.p);
+    r.p.split = g.packed ? default_split(r.p) : default_split64(r.p);
     Pass ps{};
     ps.kind = PK_ROW;
     ps.nsize = g.nx;
@@ -487,6 +487,12 @@ struct Planner {
     for (int per : {kMaxRowOps, 3, 2, 1})
       if (per == 1 || warps * row_segments(p, per) >= want) return per;
     return 1;
+  }
+  // FP64 passes: one chain per block while the rows are fewer than sixteen warps
+  // an SM (a pass of rows alone leaves most SMs idle or unevenly loaded).
+  int default_split64(const RowParams& p) const {
+    const double warps = (double)p.rows_total * row_tpr<double>(g.nx) / 32.0;
+    return p.nslots == 1 && p.ops[0].kind == ROP_C2R && warps < 152.0 * 16 ? kMaxRowOps : 0;
   }
   static int row_segments(const RowParams& p, int per) {
     if (per == 0) return 1;
@@ -2160,9 +2166,10 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
       }
   } else if (p.kind == PK_ROW) {
     const int tpr = row_tpr<double>(p.nsize);
-    deflt = p.row.rpc;
-    for (int r = deflt; r >= 1 && cand.size() < 4; r /= 2)
-      if (tpr > 0 && (r * tpr) % 32 == 0) cand.push_back(r);
+    deflt = p.row.rpc + kSplitTag * p.row.split;
+    for (int r = p.row.rpc; r >= 1 && cand.size() < 4; r /= 2)
+      if (tpr > 0 && (r * tpr) % 32 == 0) cand.push_back(r + kSplitTag * p.row.split);
+    if (p.row.split) cand.push_back(p.row.rpc);
   } else {
     int tpc = 0, group = 1;
     const int cpb = p.col.packed ? packed_col_geometry(p.nsize, &tpc, &group)
