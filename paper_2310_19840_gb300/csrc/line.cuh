@@ -32,7 +32,9 @@ __host__ __device__ constexpr size_t line_smem(int program_bytes) {
          (program_bytes + 15) / 16 * 16;
 }
 
-template <int NX, bool EXACT>
+// MULTI: a cluster of p.cluster blocks per member (else one block, whose code
+// then has no shares to work out: 7 % of a 256-point step)
+template <int NX, bool EXACT, bool MULTI>
 __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant__ LineParams p) {
   using G = RowGeo<NX>;
   using SP = StatePair<float>;
@@ -43,7 +45,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
   unsigned char* prog = reinterpret_cast<unsigned char*>(slots + kLineSlots * n);
   const int tid = threadIdx.x, g = tid / T, j = tid % T;
   auto* xs = xs0 + g * G::XLEN;
-  const int C = p.cluster, rank = (int)blockIdx.x % C;
+  const int C = MULTI ? p.cluster : 1, rank = MULTI ? (int)blockIdx.x % C : 0;
   const int member = p.member0 + (int)blockIdx.x / C;
   for (int i = tid; i < (p.bytes + 15) / 16; i += kLineThreads)
     reinterpret_cast<uint4*>(prog)[i] = reinterpret_cast<const uint4*>(p.program)[i];
@@ -64,7 +66,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
   for (int ip = 0; ip < H.nphases; ++ip) {
     const LinePhase& P = phases[ip];
     // also before a phase that this member skips: the next ones rely on it
-    if (C > 1 && P.sync) {
+    if (MULTI && P.sync) {
       asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
       asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     } else {
@@ -277,11 +279,17 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
 
 template <int NX>
 cudaError_t prepare_line_n() {
-  const cudaError_t e = allow_smem(k_line<NX, true>, line_smem<NX>(kLineMaxBytes));
-  return e == cudaSuccess ? allow_smem(k_line<NX, false>, line_smem<NX>(kLineMaxBytes)) : e;
+  constexpr bool M = line_cluster(NX) > 1;
+  constexpr size_t bytes = line_smem<NX>(kLineMaxBytes);
+  cudaError_t e = allow_smem(k_line<NX, true, false>, bytes);
+  if (e == cudaSuccess) e = allow_smem(k_line<NX, false, false>, bytes);
+  if (e == cudaSuccess) e = allow_smem(k_line<NX, true, M>, bytes);
+  if (e == cudaSuccess) e = allow_smem(k_line<NX, false, M>, bytes);
+  return e;
 }
 template <int NX>
 cudaError_t launch_line_n(const LineParams& p, cudaStream_t st) {
+  constexpr bool M = line_cluster(NX) > 1;
   if (p.member0 < 0 || p.member1 <= p.member0 || p.bytes > kLineMaxBytes || p.cluster < 1 ||
       p.cluster > line_cluster(NX))
     return cudaErrorInvalidValue;
@@ -290,13 +298,16 @@ cudaError_t launch_line_n(const LineParams& p, cudaStream_t st) {
   cfg.blockDim = dim3(kLineThreads);
   cfg.dynamicSmemBytes = line_smem<NX>(p.bytes);
   cfg.stream = st;
+  if (p.cluster == 1)
+    return p.exact ? cudaLaunchKernelEx(&cfg, k_line<NX, true, false>, p)
+                   : cudaLaunchKernelEx(&cfg, k_line<NX, false, false>, p);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)p.cluster;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = p.cluster > 1 ? 1 : 0;
-  return p.exact ? cudaLaunchKernelEx(&cfg, k_line<NX, true>, p) : cudaLaunchKernelEx(&cfg, k_line<NX, false>, p);
+  cfg.numAttrs = 1;
+  return p.exact ? cudaLaunchKernelEx(&cfg, k_line<NX, true, M>, p) : cudaLaunchKernelEx(&cfg, k_line<NX, false, M>, p);
 }
 
 }  // namespace pk
