@@ -1,4 +1,6 @@
-// kernels.cuh - row, column and RK4 passes of the ESBI step (templates).
+// kernels.cuh - row, column and RK4 passes of FP64 groups (packed_kernels.cuh has
+// those of two-dimensional FP32 groups, line.cuh the one-dimensional ones), the
+// state formats, the multiplier tables and the copy helpers of all of them.
 //
 // Layouts (see sbi_internal.h): physical fields are [member][y][x]; mixed
 // fields (x-spectral, y-physical, only the W kept x-modes) are stored
@@ -24,11 +26,7 @@ namespace sbi {
 // ===========================================================================
 // Row-pass geometry: 8 elements per thread (radix-8 Stockham passes).  Up to
 // n = 256 a row is transformed by one warp or less (warp-synchronous), longer
-// rows by several warps with block barriers; a block holds up to 512
-// threads.  In FP32 the blocks are compiled for two resident blocks per SM
-// (64 registers per thread, no spills): measured against 16 elements per
-// thread this doubles the warps per SM and runs the row passes faster at
-// every size.
+// rows by several warps with block barriers; a block holds up to 512 threads.
 template <int NX>
 struct RowCfg {
   static constexpr int n = NX / 2;                         // packed complex length
@@ -38,9 +36,6 @@ struct RowCfg {
   static constexpr int RPC_MAX = cmin(256, WARP ? cmax(16, 512 / TPR) : cmax(1, 512 / TPR));
   static constexpr int MAX_THREADS = TPR * RPC_MAX;
   static constexpr int FBUF = fft_scratch_len<n, R>();    // FFT scratch per row
-  template <typename T>
-  // 0: no minimum, the register count is left to the compiler
-  static constexpr int min_blocks() { return sizeof(T) == 4 ? 2 : 0; }
 };
 
 // shared memory of a row block: per row the FFT scratch (row stride fbs), the
@@ -332,7 +327,7 @@ __device__ __forceinline__ T ipow(T v, int p) {
 // transform and the products formed from it.  A pass over few rows then has
 // several times the blocks, and every SM's FP64 lanes the same share of them.
 template <typename T, int NX>
-__global__ void __launch_bounds__(RowCfg<NX>::MAX_THREADS, RowCfg<NX>::template min_blocks<T>())
+__global__ void __launch_bounds__(RowCfg<NX>::MAX_THREADS)
 k_row(const __grid_constant__ RowParams p) {
   using V = cx<T>;
   using C = RowCfg<NX>;
@@ -600,20 +595,15 @@ template <> struct StatePair<float> {
 // RK4 stage pass (row layout).  State and sums in StatePair<T> storage.
 // ===========================================================================
 // RK stage geometry: blocks of kRkThreads threads (a whole row when a row
-// needs more); three resident blocks per SM in FP32 (at most 85 registers),
-// two in FP64 (128).
+// needs more); two resident blocks per SM (at most 128 registers).
 template <int NX>
 struct RkCfg {
   static constexpr int RPC = cmax(1, kRkThreads / RowCfg<NX>::TPR);
   static constexpr int THREADS = RowCfg<NX>::TPR * RPC;
-  template <typename T>
-  static constexpr int min_blocks() { return sizeof(T) == 4 ? 3 : 2; }
 };
 
-// S: the state storage format (T itself, or double for the FP32 path with an
-// FP64 state)
-template <typename T, int NX, typename S>
-__global__ void __launch_bounds__(RkCfg<NX>::THREADS, RkCfg<NX>::template min_blocks<T>())
+template <typename T, int NX>
+__global__ void __launch_bounds__(RkCfg<NX>::THREADS, 2)
 k_rk(const __grid_constant__ RkParams p) {
   using V = cx<T>;
   using C = RowCfg<NX>;
@@ -635,7 +625,7 @@ k_rk(const __grid_constant__ RkParams p) {
   const long long off = (long long)y * NX;
 
   // new state in the working precision (the FFT inputs of the tail)
-  using SP = StatePair<S>;
+  using SP = StatePair<T>;
   V xe[R], xp[R];
   const long long eoff = member * p.eta0.stride + off, poff = member * p.phi0.stride + off;
   char* E0 = reinterpret_cast<char*>(p.eta0.ptr) + eoff * 8;   // 8 bytes per value
@@ -762,16 +752,14 @@ k_rk(const __grid_constant__ RkParams p) {
 // instantiation serves both directions.
 // ===========================================================================
 // Column-pass geometry: 8 elements per thread (one warp per column at 256,
-// two at 512, ...).  In FP32 columns of at least a warp are compiled for four
-// resident blocks per SM (64 registers).
+// two at 512, ...).
 
 template <typename T, int NY>
 struct ColCfg {
   static constexpr int RC = NY == 1 ? 1 : cmin(8, NY);
   static constexpr int TPC = NY / RC;
   static constexpr bool WARP = TPC <= 32;
-  // 8-byte elements: 256 threads per block; 16-byte elements: half the columns
-  static constexpr int CPB = NY == 1 ? 256 : cmax(1, 256 / TPC / (int)(sizeof(T) / 4));
+  static constexpr int CPB = NY == 1 ? 256 : cmax(1, 128 / TPC);
   static constexpr int THREADS = TPC * CPB;
   // 512- to 2048-point columns by the split transforms of fft.cuh: forward
   // by decimation in frequency (natural loads, spectrum in decimated order),
@@ -781,7 +769,6 @@ struct ColCfg {
   // accumulator length per column (padded where the modes are held with
   // stride NY / 256, so that those accesses spread over the banks)
   static constexpr int ACC = SPLIT ? padded_len(NY) : NY;
-  static constexpr int MIN_BLOCKS = (sizeof(T) == 4 && RC == 8 && TPC >= 32) ? 4 : 0;  // 0: no minimum
 };
 
 template <typename T, int NY>
@@ -845,7 +832,7 @@ inline bool col_outer(const ColParams& p) {
 // FP64 issue bounds the pass (two lanes per cycle and SM): per column element
 // and transform it took some 30 FP64 operations, and takes 21 to 22.
 template <typename T, int NY, bool OUTER, bool STAGED>
-__global__ void __launch_bounds__(ColCfg<T, NY>::THREADS, ColCfg<T, NY>::MIN_BLOCKS)
+__global__ void __launch_bounds__(ColCfg<T, NY>::THREADS)
 k_col(const __grid_constant__ ColParams p) {
   using V = cx<T>;
   using C = ColCfg<T, NY>;
@@ -1145,9 +1132,7 @@ cudaError_t prepare_nx() {
   const int maxb = 227 * 1024;
   cudaError_t e = cudaFuncSetAttribute(k_row<T, NX>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_rk<T, NX, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
-  if (e != cudaSuccess || sizeof(T) == 8) return e;
-  return cudaFuncSetAttribute(k_rk<T, NX, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
+  return cudaFuncSetAttribute(k_rk<T, NX>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
 }
 
 template <typename T, int NY>
@@ -1216,8 +1201,7 @@ cudaError_t launch_rk_n(const RkParams& p, cudaStream_t st) {
   RkParams q = p;
   q.fbs = bank::choose(C::n, C::R, C::TPR, p.rpc, p.W, (int)sizeof(cx<T>), true, false, C::FBUF).fbs;
   const size_t smem = sizeof(cx<T>) * (size_t)q.rpc * q.fbs;
-  if (q.state64 && sizeof(T) == 4) k_rk<T, NX, double><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
-  else k_rk<T, NX, T><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
+  k_rk<T, NX><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
   return cudaGetLastError();
 }
 
@@ -1302,12 +1286,10 @@ cudaError_t launch_col_impl(int ny, const ColParams& p, cudaStream_t st) {
 }
 
 // Largest rows-per-block (power of two, <= the kernel's maximum) whose shared
-// memory stays within 200 KB; 0 if even one row does not fit.
+// memory fits a block; 0 if even one row does not fit.
 template <typename T>
 int row_rpc_impl(int nx, int W, int nslots) {
-  // one block may take the whole 227 KB; blocks compiled for two per SM get
-  // half of the SM's 228 KB less the 1 KB each block reserves
-  size_t budget = 227 * 1024;
+  const size_t budget = 227 * 1024;
   int maxr = 0;
   size_t per = 0;
   switch (nx) {
@@ -1315,7 +1297,6 @@ int row_rpc_impl(int nx, int W, int nslots) {
   case N:                                                                   \
     maxr = RowCfg<N>::RPC_MAX;                                              \
     per = row_smem_bound<T, N>(W, nslots);                                  \
-    if (RowCfg<N>::template min_blocks<T>() == 2) budget = 113 * 1024;      \
     break;
     SBI_FOR_NX(SBI_CASE)
 #undef SBI_CASE
