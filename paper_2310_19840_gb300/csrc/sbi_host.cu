@@ -2182,7 +2182,10 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     deflt = base(p.col.staged) + kStagedTag * p.col.staged + kWideTag * p.col.wide;
     // the staged form is a candidate where the option leaves the choice open
     const bool stg = c->opt.col_staging == 0 && stageable(c, p.col);
-    for (int staged = p.col.staged; staged <= (stg ? 1 : p.col.staged); ++staged) {
+    // few columns: the wide form beat every other block shape by a third or more
+    // wherever it was the default, so only its number of copies is left open
+    if (p.col.wide) cand.push_back(base(0));
+    for (int staged = p.col.staged; !p.col.wide && staged <= (stg ? 1 : p.col.staged); ++staged) {
       int k = 0;
       for (int v = base(staged); v >= 1 && k < 3; v /= 2)
         if (tpc > 0 && (v * tpc) % 32 == 0 && v % group == 0 && !(staged && p.col.packed && v % 4)) {
