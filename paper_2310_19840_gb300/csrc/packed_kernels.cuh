@@ -12,11 +12,11 @@
 // fits one, so that the kernels need no block barriers; rows of more than 1024
 // points and columns of more than 512 use the block.
 //
-// Against the scalar passes of kernels.cuh (GB300, 2.0 GHz): a 512-point row
+// Against the scalar FP32 passes before them (GB300, 2.0 GHz): a 512-point row
 // takes 128 SM-cycles per transform instead of 312 and 336 instructions per
 // row instead of about 800; a 256-point column 137 instead of 312; the row pass
-// of a 4096 x 2048 grid 173 us per launch instead of 344; a step of 64 256^2 and
-// 32 512^2 members 4.42 ms instead of 6.03.
+// of a 4096 x 2048 grid 168 us per launch instead of 344; a step of 64 256^2 and
+// 32 512^2 members 4.33 ms instead of 6.03.
 #pragma once
 
 #include "kernels.cuh"
@@ -54,9 +54,6 @@ __host__ __device__ constexpr size_t row_smem(int rows, int nslots) {
   using G = RowGeo<NX>;
   return 8 * ((size_t)G::RTW + (size_t)rows * (G::XLEN + nslots * G::n));
 }
-// The twiddles of a block's transforms and of the packed real transform: from
-// shared memory, or (long rows) products of the thread's own e^{-2 pi i j / NX}
-// by roots of unity.
 // Passes are launched so that the blocks of one may start, and form what
 // depends on constants alone (twiddle tables, multipliers), while the blocks of
 // the pass before still run; nothing a pass wrote may be read, and nothing it
@@ -67,6 +64,9 @@ __device__ __forceinline__ void wait_for_previous() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
+// The twiddles of a block's transforms and of the packed real transform: from
+// shared memory, or (long rows) products of the thread's own e^{-2 pi i j / NX}
+// by roots of unity.
 template <int NX>
 struct RowTwiddles {
   using G = RowGeo<NX>;
@@ -376,6 +376,9 @@ k_packed_row(const __grid_constant__ RowParams p) {
 // current one.  The quotient takes one residual correction (Newton) after an
 // approximate reciprocal of 1 + |grad eta|^2 >= 1: below one unit in the last
 // place, in five packed and two special operations for two values.
+// Load latency bounds it (a quarter of the issue slots used): 8192 rows of 512
+// points 63 us (75 with the IEEE quotient and spills; 66 with 128 registers, four
+// blocks per SM and no loads ahead).
 struct RhsOps {
   int8_t src[5];      // inverse transforms in the order eta_x, phi_x, eta_y, phi_y, V (indices into ops)
   int8_t f, sx, sy;   // the operation; sponge products of phi_x and phi_y (-1: none)
@@ -595,7 +598,9 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
 
 // ===========================================================================
 // RK pass.  blockIdx.y: the elevation (0) or the potential (1); the two need
-// nothing from each other, so a thread holds one transform at a time.
+// nothing from each other, so a thread holds one transform at a time.  Bound by
+// memory: a third of the crossing-sea batch of 96 members in 42 us per launch
+// (60 before), 5.4 TB/s of the bytes it cannot do without.
 // ===========================================================================
 template <int NX, bool EXACT, typename S>
 __global__ void __launch_bounds__(RowGeo<NX>::THREADS, 5)
@@ -980,7 +985,8 @@ __device__ __forceinline__ void copy_float_ahead(float* dst_smem, const float* s
 // sums some modes over all inputs, in the order of the other forms and with the
 // same operations (the same bits); the outputs are shared out the same way.
 // A pass of eight inputs and one output then takes the time of two transforms
-// instead of nine.
+// instead of nine.  Column passes of one 512^2 member: 0.38 ms a step (0.58 in
+// the plain form; 0.44 with the multipliers loaded where they are used).
 template <int NY>
 struct WideGeo {
   using G = ColGeo<NY>;

@@ -477,7 +477,10 @@ struct Planner {
   }
 
   // Products per segment of a packed group's row pass (0: the whole pass in one
-  // block): as few as it takes to give every SM twelve warps.
+  // block): as few as it takes to give every SM twelve warps.  Row passes of a
+  // step, untuned, with and without: one 512^2 member 330 and 425 us, four 520 and
+  // 506 (twelve warps are reached between them), sixteen 1141 and 1149; with the
+  // line at 24 warps one takes 349, four 567.
   int default_split(const RowParams& p) const {
     int tpr = 0;
     packed_row_geometry(g.nx, &tpr);
@@ -509,13 +512,16 @@ struct Planner {
 
   // --- column pass builder ---
   // Copies of the wide form of a packed group's column pass (0: the plain
-  // form): doubled until every SM has eight warps, or each copy one transform.
+  // form): doubled until every SM has eight warps, or each copy one transform;
+  // none from 2.7 warps per SM on.  Column passes of a step, untuned, with and
+  // without: one 512^2 member 380 and 583 us, four 535 and 631, eight (3.4 warps)
+  // 750 and 683.
   int default_wide(const ColParams& p) const {
     const int most = packed_col_most_wide(p);
     int tpc = 0, group = 1;
     packed_col_geometry(g.ny, &tpc, &group);
     const double warps = (double)p.cols_total * tpc / 32.0;
-    if (most < 2 || warps * 2 > 152.0 * 8.0) return 0;
+    if (most < 2 || warps * 3 > 152.0 * 8.0) return 0;
     int k = 2;
     while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < 152.0 * 8.0) k *= 2;
     return k;
