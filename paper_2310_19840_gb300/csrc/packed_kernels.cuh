@@ -102,6 +102,10 @@ struct RowTwiddles {
       return wmul(wj, unit_root(r, 2 * G::R));
     }
   }
+  __device__ __forceinline__ float2 any(int r) const {
+    if (r == G::R / 2 && j == 0) return make_float2(0.f, -1.f);
+    return r < G::R / 2 ? lower(r) : upper(r);
+  }
   // Products by roots of unity are formed where they are used: kept across a
   // loop they would take more registers than there are.  Emits nothing.
   __device__ __forceinline__ void renew() {
@@ -204,18 +208,37 @@ __device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const Buf
     }
     twist_modes<NX>(x, t);
   } else {
+    // four elements at a time: eight loads without a branch between them (one
+    // after the other they made this form two to three times as slow)
+    constexpr int B = R < 4 ? R : 4;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int k = j + r * T, kk = n - k;
-      One a = both(0.f), b = both(0.f);
+    for (int r0 = 0; r0 < R; r0 += B) {
+      One a[B], b[B];
+#pragma unroll
+      for (int i = 0; i < B; ++i) a[i] = b[i] = both(0.f);
+#pragma unroll 1
       for (int q = 0; q < nb; ++q) {
         const unsigned long long* src = mixed_row(bufs[q], w);
-        if (k < W) a = add(a, One{src[mode_at(k, ny)]});
-        if (k > 0 && kk < W) b = add(b, One{src[mode_at(kk, ny)]});
+        One va[B], vb[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          const int k = j + (r0 + i) * T, kk = n - k;
+          va[i].v = k < W ? src[mode_at(k, ny)] : 0ull;
+          vb[i].v = k > 0 && kk < W ? src[mode_at(kk, ny)] : 0ull;
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          a[i] = add(a[i], va[i]);
+          b[i] = add(b[i], vb[i]);
+        }
       }
-      const float2 e = __ldg(t.tw + tw_off(NX) + k);
-      const One o = cmul(sub_conj(a, b), make_float2(e.x, -e.y));
-      x[r] = conj(addi(add_conj(a, b), o));
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        const int r = r0 + i;
+        const float2 e = t.any(r);
+        const One o = cmul(sub_conj(a[i], b[i]), make_float2(e.x, -e.y));
+        x[r] = conj(addi(add_conj(a[i], b[i]), o));
+      }
     }
   }
 }
@@ -257,7 +280,7 @@ __device__ __forceinline__ void kept_modes(const One (&x)[RowGeo<NX>::R], One (&
         if (j != 0) zc = o;
       }
     }
-    const float2 e = FAST ? t.lower(r) : __ldg(t.tw + tw_off(NX) + k);
+    const float2 e = FAST ? t.lower(r) : t.any(r);
     const One d = cmul(sub_conj(x[r], zc), e);
     X[r] = scale(0.5f, subi(add_conj(x[r], zc), d));
   }
@@ -978,10 +1001,10 @@ k_packed_col(const __grid_constant__ ColParams p) {
 __device__ __forceinline__ void copy_float_ahead(float* dst_smem, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
-// Wide form of the HALF pass, for launches of few columns: the threads of a
+// Wide form, for launches of few columns: the threads of a
 // set of columns (one warp, or the block's 128 threads where a transform needs
 // them) are there p.wide times, each copy transforms its share of the inputs,
-// leaves the kept modes in shared memory, and after one barrier every thread
+// leaves their modes in shared memory, and after one barrier every thread
 // sums some modes over all inputs, in the order of the other forms and with the
 // same operations (the same bits); the outputs are shared out the same way.
 // A pass of eight inputs and one output then takes the time of two transforms
@@ -995,13 +1018,17 @@ struct WideGeo {
   static constexpr int SX = G::XLEN * (SET / G::GT);    // exchange elements of one copy
 };
 template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nterms, int nacc, int npass) {
+__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nterms, int nacc, int npass,
+                                                          bool half) {
   using G = ColGeo<NY>;
   using H = WideGeo<NY>;
-  const size_t modes = (8 * (size_t)nin + 4 * (size_t)nterms) * G::R * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
-  return 16 * ((size_t)G::CTW + (size_t)copies * H::SX) + 8 * (size_t)nacc * G::R * H::SET + (modes > pass ? modes : pass);
+  const size_t NM = (half ? 1 : 2) * G::R;
+  const size_t modes = (8 * (size_t)nin + 4 * (size_t)nterms) * NM * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
+  return 16 * ((size_t)G::CTW + (size_t)copies * H::SX) + 8 * (size_t)nacc * NM * H::SET + (modes > pass ? modes : pass);
 }
-template <int NY>
+// A thread's modes: HALF the R that can be kept (j + r T, from r = R / 2 on plus
+// NY / 2), else j + r T and, from R on, those plus NY / 2.
+template <int NY, bool HALF>
 __global__ void __launch_bounds__(WideGeo<NY>::G::WARP ? 256 : 512)
 k_packed_col_wide(const __grid_constant__ ColParams p) {
   using G = ColGeo<NY>;
@@ -1009,6 +1036,7 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   using E = typename G::E;
   using M = Mem<Two>;
   constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2, SET = H::SET;
+  constexpr int NM = HALF ? R : 2 * R, UP = HALF ? R / 2 : R;   // modes, the first one of the upper plane
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int copies = blockDim.x / SET, copy = threadIdx.x / SET, lane = threadIdx.x % SET;
   const int g = lane / GT, l = lane % GT, c = l % CI, j = l / CI;
@@ -1016,8 +1044,8 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   E* xs0 = reinterpret_cast<E*>(smem_raw) + G::CTW;
   E* xs = xs0 + (size_t)copy * H::SX + g * G::XLEN + c;
   F2* sums = reinterpret_cast<F2*>(xs0 + (size_t)copies * H::SX);              // [acc][r][lane]
-  F2* modes = sums + (size_t)p.nacc * R * SET;                                 // [input][r][lane]
-  float* factors = reinterpret_cast<float*>(modes + (size_t)p.nin * R * SET);  // [term][r][lane]
+  F2* modes = sums + (size_t)p.nacc * NM * SET;                                 // [input][r][lane]
+  float* factors = reinterpret_cast<float*>(modes + (size_t)p.nin * NM * SET);  // [term][r][lane]
   E* passed = reinterpret_cast<E*>(modes);                                     // later: [pass][r][lane]
   const float2* tw = reinterpret_cast<const float2*>(p.tw);
   const int col = p.col_begin + (int)blockIdx.x * H::COLS + g * CI + c;
@@ -1041,8 +1069,8 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
     for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
       const float* tab = reinterpret_cast<const float*>(p.terms[q].tab) + at0;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        copy_float_ahead(factors + (q * R + r) * SET + lane, tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+      for (int r = 0; r < NM; ++r)
+        copy_float_ahead(factors + (q * NM + r) * SET + lane, tab + r % R * T * 4 + (r < UP ? 0 : plane));
     }
     cp_async_commit();
   };
@@ -1068,34 +1096,39 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
       for (int r = 0; r < R; ++r) {
         const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
         const F2 o = cmul(x[r].b, w);
-        modes[(i * R + r) * SET + lane] = r < R / 2 ? add(x[r].a, o) : sub(x[r].a, o);
+        if (HALF) {
+          modes[(i * NM + r) * SET + lane] = r < UP ? add(x[r].a, o) : sub(x[r].a, o);
+        } else {
+          modes[(i * NM + r) * SET + lane] = add(x[r].a, o);
+          modes[(i * NM + R + r) * SET + lane] = sub(x[r].a, o);
+        }
       }
     }
   }
   // the multipliers of this copy's first output
-  float fo[R];
+  float fo[NM];
   if (copy < p.nouts) {
     const float* tab = reinterpret_cast<const float*>(p.outs[copy].tab) + at0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) fo[r] = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+    for (int r = 0; r < NM; ++r) fo[r] = __ldg(tab + r % R * T * 4 + (r < UP ? 0 : plane));
   }
   cp_async_wait_all();
   __syncthreads();
-  // copy k sums the registers r = k, k + copies, ..
-  for (int r = copy; r < R; r += copies) {
+  // copy k sums the modes r = k, k + copies, ..
+  for (int r = copy; r < NM; r += copies) {
     F2 a0 = both(0.f), a1 = a0;
     for (int i = 0; i < p.nin; ++i) {
-      const F2 v = modes[(i * R + r) * SET + lane];
+      const F2 v = modes[(i * NM + r) * SET + lane];
       for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
         const ColTerm m = p.terms[q];
-        const float f = factors[(q * R + r) * SET + lane];
+        const float f = factors[(q * NM + r) * SET + lane];
         const int ph = (m.gx + m.gy) & 3;
         if (m.acc == 0) a0 = acc_term(a0, v, f, ph);
         else a1 = acc_term(a1, v, f, ph);
       }
     }
     sums[r * SET + lane] = a0;
-    if (p.nacc > 1) sums[(R + r) * SET + lane] = a1;
+    if (p.nacc > 1) sums[(NM + r) * SET + lane] = a1;
   }
   __syncthreads();
 #pragma unroll 1
@@ -1119,9 +1152,16 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const float2 w = r == 0 ? wj : wmul(wj, unit_root(r, 2 * R));
-        const float f = o0 == 0 ? fo[r] : __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
-        const F2 e = conj_term(sums[((m.acc ? R : 0) + r) * SET + lane], f, ph);
-        x[r] = Two{e, cmul(e, r < R / 2 ? w : make_float2(-w.x, -w.y))};
+        const F2* sum = sums + ((m.acc ? NM : 0) + r) * SET + lane;
+        if (HALF) {
+          const float f = o0 == 0 ? fo[r] : __ldg(tab + r * T * 4 + (r < UP ? 0 : plane));
+          const F2 e = conj_term(*sum, f, ph);
+          x[r] = Two{e, cmul(e, r < UP ? w : make_float2(-w.x, -w.y))};
+        } else {
+          const F2 y0 = conj_term(*sum, o0 == 0 ? fo[r] : __ldg(tab + r * T * 4), ph);
+          const F2 y1 = conj_term(sum[R * SET], o0 == 0 ? fo[NM - R + r] : __ldg(tab + r * T * 4 + plane), ph);
+          x[r] = Two{add(y0, y1), cmul(sub(y0, y1), w)};
+        }
       }
     }
     G::F::run(x, xs, j, t, tw);
@@ -1235,10 +1275,11 @@ inline bool col_half(const ColParams& p) {
 // largest number of copies the wide form of a pass can take (0: none)
 template <int NY>
 int col_most_wide(const ColParams& p) {
-  if (!col_half(p) || p.staged) return 0;
+  if (p.staged) return 0;
+  const bool half = col_half(p);
   const int most = (ColGeo<NY>::WARP ? 256 : 512) / WideGeo<NY>::SET;
   for (int k = most; k >= 2; k /= 2)
-    if (packed_col_smem_wide<NY>(k, p.nin, p.nterms, p.nacc, p.npass) <= 227 * 1024) return k;
+    if (packed_col_smem_wide<NY>(k, p.nin, p.nterms, p.nacc, p.npass, half) <= 227 * 1024) return k;
   return 0;
 }
 
@@ -1268,10 +1309,10 @@ cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st, bool chaine
   const bool half = col_half(p);
   if (p.wide > 0) {
     using H = WideGeo<NY>;
-    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nterms, p.nacc, p.npass);
-    if (!half || p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
+    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nterms, p.nacc, p.npass, half);
+    if (p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
     const unsigned wb = (unsigned)((p.cols_total - p.col_begin + H::COLS - 1) / H::COLS);
-    return launch(k_packed_col_wide<NY>, wb, p.wide * H::SET, smem, st, chained, p);
+    return launch(half ? k_packed_col_wide<NY, true> : k_packed_col_wide<NY, false>, wb, p.wide * H::SET, smem, st, chained, p);
   }
   if (p.nacc == 1)
     return half ? launch_packed_col_a<NY, 1, true>(p, groups, blocks, st, chained)
@@ -1315,7 +1356,8 @@ cudaError_t prepare_packed_col_n() {
   if (e == cudaSuccess) e = prepare_packed_col_a<NY, 1, false>();
   if (e == cudaSuccess) e = prepare_packed_col_a<NY, 2, true>();
   if (e == cudaSuccess) e = prepare_packed_col_a<NY, 2, false>();
-  if (e == cudaSuccess) e = allow_smem(k_packed_col_wide<NY>, 227 * 1024);
+  if (e == cudaSuccess) e = allow_smem(k_packed_col_wide<NY, true>, 227 * 1024);
+  if (e == cudaSuccess) e = allow_smem(k_packed_col_wide<NY, false>, 227 * 1024);
   return e;
 }
 

@@ -85,3 +85,24 @@ def test_a_member_alone_equals_it_in_a_batch(sbi, nx, ny, n):
         ctx.close()
     for key in ((n, 0), (n, 1)):
         assert np.array_equal(out[key][0], out[1, 0][0]) and np.array_equal(out[key][1], out[1, 0][1]), key
+
+
+@pytest.mark.parametrize("alpha", [1.0 / 3.0, 0.75])
+@pytest.mark.parametrize("nx, ny, n", [(64, 32, 70), (256, 128, 33), (512, 512, 6), (64, 1024, 12)])
+def test_other_widths_alone_equal_the_batch(sbi, nx, ny, n, alpha):
+    # the same for more and fewer than half of the modes: the wide column form of
+    # every mode of a column, the rows' general form
+    spec = (nx, ny, 0.1 * nx, 0.1 * ny)
+    eta = np.concatenate([W.random_field(nx, ny, 100 + i, amplitude=0.004).ravel() for i in range(n)])
+    phi = np.concatenate([W.random_field(nx, ny, 200 + i, amplitude=0.02).ravel() for i in range(n)])
+    out = {}
+    for count, tune in ((1, 0), (n, 0), (n, 1)):
+        ctx = sbi.Context([spec] * count, 9.81, None, h0=0.7, order=4, alias_frac=alpha, autotune=tune)
+        k = count * nx * ny
+        ctx.set_state_all(eta[:k], phi[:k])
+        ctx.step(0.005, 2)
+        e, p = ctx.get_state_all()
+        out[count, tune] = e[:nx * ny], p[:nx * ny]
+        ctx.close()
+    for key in ((n, 0), (n, 1)):
+        assert np.array_equal(out[key][0], out[1, 0][0]) and np.array_equal(out[key][1], out[1, 0][1]), key
