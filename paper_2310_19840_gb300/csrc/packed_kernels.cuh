@@ -208,28 +208,28 @@ __device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const Buf
     }
     twist_modes<NX>(x, t);
   } else {
-    // four elements at a time: eight loads without a branch between them (one
+    // eight elements at a time: sixteen loads without a branch between them (one
     // after the other they made this form two to three times as slow)
-    constexpr int B = R < 4 ? R : 4;
+    constexpr int B = R < 8 ? R : 8;
 #pragma unroll
     for (int r0 = 0; r0 < R; r0 += B) {
       One a[B], b[B];
-#pragma unroll
-      for (int i = 0; i < B; ++i) a[i] = b[i] = both(0.f);
-#pragma unroll 1
-      for (int q = 0; q < nb; ++q) {
+      auto load = [&](int q, int i, One& va, One& vb) {
         const unsigned long long* src = mixed_row(bufs[q], w);
-        One va[B], vb[B];
+        const int k = j + (r0 + i) * T, kk = n - k;
+        va.v = k < W ? src[mode_at(k, ny)] : 0ull;
+        vb.v = k > 0 && kk < W ? src[mode_at(kk, ny)] : 0ull;
+      };
+#pragma unroll
+      for (int i = 0; i < B; ++i) load(0, i, a[i], b[i]);
+#pragma unroll 1
+      for (int q = 1; q < nb; ++q) {
 #pragma unroll
         for (int i = 0; i < B; ++i) {
-          const int k = j + (r0 + i) * T, kk = n - k;
-          va[i].v = k < W ? src[mode_at(k, ny)] : 0ull;
-          vb[i].v = k > 0 && kk < W ? src[mode_at(kk, ny)] : 0ull;
-        }
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-          a[i] = add(a[i], va[i]);
-          b[i] = add(b[i], vb[i]);
+          One va, vb;
+          load(q, i, va, vb);
+          a[i] = add(a[i], va);
+          b[i] = add(b[i], vb);
         }
       }
 #pragma unroll
