@@ -1114,21 +1114,37 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   }
   cp_async_wait_all();
   __syncthreads();
-  // copy k sums the modes r = k, k + copies, ..
-  for (int r = copy; r < NM; r += copies) {
-    F2 a0 = both(0.f), a1 = a0;
+  // copy k sums the modes r = k, k + copies, .., four at a time: their loads
+  // from shared memory overlap
+  for (int r0 = copy; r0 < NM; r0 += 4 * copies) {
+    F2 a0[4], a1[4];
+#pragma unroll
+    for (int c4 = 0; c4 < 4; ++c4) a0[c4] = a1[c4] = both(0.f);
     for (int i = 0; i < p.nin; ++i) {
-      const F2 v = modes[(i * NM + r) * SET + lane];
+      F2 v[4];
+#pragma unroll
+      for (int c4 = 0; c4 < 4; ++c4) v[c4] = modes[(i * NM + min(r0 + c4 * copies, NM - 1)) * SET + lane];
       for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
         const ColTerm m = p.terms[q];
-        const float f = factors[(q * NM + r) * SET + lane];
         const int ph = (m.gx + m.gy) & 3;
-        if (m.acc == 0) a0 = acc_term(a0, v, f, ph);
-        else a1 = acc_term(a1, v, f, ph);
+        float f[4];
+#pragma unroll
+        for (int c4 = 0; c4 < 4; ++c4) f[c4] = factors[(q * NM + min(r0 + c4 * copies, NM - 1)) * SET + lane];
+#pragma unroll
+        for (int c4 = 0; c4 < 4; ++c4) {
+          if (m.acc == 0) a0[c4] = acc_term(a0[c4], v[c4], f[c4], ph);
+          else a1[c4] = acc_term(a1[c4], v[c4], f[c4], ph);
+        }
       }
     }
-    sums[r * SET + lane] = a0;
-    if (p.nacc > 1) sums[(NM + r) * SET + lane] = a1;
+#pragma unroll
+    for (int c4 = 0; c4 < 4; ++c4) {
+      const int r = r0 + c4 * copies;
+      if (r < NM) {
+        sums[r * SET + lane] = a0[c4];
+        if (p.nacc > 1) sums[(NM + r) * SET + lane] = a1[c4];
+      }
+    }
   }
   __syncthreads();
 #pragma unroll 1
