@@ -286,6 +286,7 @@ void* dalloc(sbi_ctx* c, size_t bytes) {
   if (p) {
     c->allocs.push_back(p);
     cudaMemsetAsync(p, 0, bytes, c->cap);
+    cudaStreamSynchronize(c->cap);   // the first use may be on any stream
   }
   return p;
 }
@@ -3251,13 +3252,9 @@ double* device_view(void* p, int on_device) {
   return nullptr;
 }
 
-// A staging buffer's first use is on another stream than the one that zeroes it.
 int ensure_stage(sbi_ctx* c, Group& g) {
-  if (g.stage64) return SBI_OK;
-  g.stage64 = (double*)dalloc(c, g.phys_elems() * g.n * 8);
-  if (!g.stage64) return fail(c, SBI_ENOMEM, "device allocation failed");
-  CK(cudaStreamSynchronize(c->cap), "sync");
-  return SBI_OK;
+  if (!g.stage64) g.stage64 = (double*)dalloc(c, g.phys_elems() * g.n * 8);
+  return g.stage64 ? SBI_OK : fail(c, SBI_ENOMEM, "device allocation failed");
 }
 
 int sbi_set_state_all(sbi_ctx* c, const double* eta, const double* phi, int on_device) {
@@ -3582,11 +3579,8 @@ int streamed_run(sbi_ctx* c, const double* eta_in, const double* phi_in, double 
     }
     int rc = ensure_stage(c, g);
     if (rc) return rc;
-    if (!g.stage64b) {
-      g.stage64b = (double*)dalloc(c, g.phys_elems() * g.n * 8);
-      if (!g.stage64b) return fail(c, SBI_ENOMEM, "device allocation failed");
-      CK(cudaStreamSynchronize(c->cap), "sync");
-    }
+    if (!g.stage64b) g.stage64b = (double*)dalloc(c, g.phys_elems() * g.n * 8);
+    if (!g.stage64b) return fail(c, SBI_ENOMEM, "device allocation failed");
     Planner pl{c, g};
     std::vector<Pass> ps;
     if (c->opt.set_state_dealias) pl.plan_project(ps, false);
@@ -3859,7 +3853,6 @@ int sbi_invariants(sbi_ctx* c, int member, double* mass, double* energy) {
   if ((size_t)nchunks * 2 > c->partial_cap) {
     void* p = dalloc(c, (size_t)nchunks * 2 * 8);
     if (!p) return fail(c, SBI_ENOMEM, "device allocation failed");
-    CK(cudaStreamSynchronize(c->cap), "sync");
     c->d_partials = (double*)p;
     c->partial_cap = (size_t)nchunks * 2;
   }
@@ -3881,14 +3874,22 @@ int sbi_invariants(sbi_ctx* c, int member, double* mass, double* energy) {
   return SBI_OK;
 }
 
+// Host values to device memory that kernels of any stream read next.  A plain
+// cudaMemcpy would be on the legacy stream, which the library's streams (created
+// non-blocking) do not wait for, and may return before its copy has landed.
+int upload_bytes(sbi_ctx* c, void* dst, const void* src, size_t bytes) {
+  CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->cap), "upload");
+  CK(cudaStreamSynchronize(c->cap), "upload");
+  return SBI_OK;
+}
+
 int ensure_time(sbi_ctx* c) {
   if (!c->d_time) {
     c->d_time = (double*)dalloc(c, sizeof(double));
     if (!c->d_time) return fail(c, SBI_ENOMEM, "device allocation failed");
   }
   CK(cudaStreamSynchronize(c->stream), "sync");
-  CK(cudaMemcpy(c->d_time, &c->t_host, sizeof(double), cudaMemcpyHostToDevice), "copy time");
-  return SBI_OK;
+  return upload_bytes(c, c->d_time, &c->t_host, sizeof(double));
 }
 
 int sbi_set_time(sbi_ctx* c, double t) {
@@ -3932,7 +3933,8 @@ int sbi_set_wavemaker(sbi_ctx* c, int ncomp, const double* amp, const double* om
     par[j] = omega[j];
     par[ncomp + j] = phase[j];
   }
-  CK(cudaMemcpy(c->wm_params, par.data(), par.size() * sizeof(double), cudaMemcpyHostToDevice), "copy");
+  rc = upload_bytes(c, c->wm_params, par.data(), par.size() * sizeof(double));
+  if (rc) return rc;
   const double bell = std::sqrt(std::exp(1.0) / (2.0 * M_PI));
   for (auto& g : c->groups) {
     if (ncomp > g.wm_cap) {
@@ -3968,7 +3970,8 @@ int sbi_set_wavemaker(sbi_ctx* c, int ncomp, const double* amp, const double* om
         prof[(size_t)j * g.nx + x] = A * std::exp(-0.5 * (k * d) * (k * d));
       }
     }
-    CK(cudaMemcpy(g.wm_prof, prof.data(), prof.size() * sizeof(double), cudaMemcpyHostToDevice), "copy");
+    rc = upload_bytes(c, g.wm_prof, prof.data(), prof.size() * sizeof(double));
+    if (rc) return rc;
   }
   c->wm_n = ncomp;
   return SBI_OK;

@@ -1,0 +1,69 @@
+"""The library's host code on a CUDA runtime that only keeps books (fake_cudart.cpp):
+a stream's copies and fills happen when that stream is synchronised, no kernel
+runs.  What a call leaves to chance on a GPU is then certain to go wrong here.
+"""
+import ctypes as C
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
+    cxx, nvcc = shutil.which("g++"), shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not cxx or not os.path.exists(nvcc):
+        pytest.skip("no compiler")
+    import __graft_entry__ as g
+    from paper_2310_19840_gb300 import build as b
+    g.build()
+    objs = [os.path.join(b.BUILD, os.path.splitext(s)[0] + ".o") for s in b.SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        b.build(force=True)
+    out = str(tmp_path_factory.mktemp("fake") / "libsbi_host.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", cuda,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp"), *objs, "-Wl,-Bsymbolic", "-o", out], check=True)
+    return out
+
+
+@pytest.fixture
+def host(built, monkeypatch):
+    from paper_2310_19840_gb300 import sbi
+    lib = C.CDLL(built)
+    for name, (res, args) in sbi.EXPORTS.items():
+        f = getattr(lib, name)
+        f.restype, f.argtypes = res, args
+    lib.fake_made_at.restype, lib.fake_made_at.argtypes = C.c_void_p, [C.c_int, C.POINTER(C.c_size_t)]
+    lib.fake_live_bytes.restype = C.c_size_t
+    monkeypatch.setattr(sbi, "_lib", lib)
+    sbi.fake = lib
+    yield sbi
+    del sbi.fake
+
+
+def doubles(lib, since):
+    """The device allocations made from number `since` on, as float64 arrays."""
+    out, n = [], C.c_size_t()
+    for i in range(since, lib.fake_made()):
+        p = lib.fake_made_at(i, C.byref(n))
+        out.append(np.ctypeslib.as_array(C.cast(p, C.POINTER(C.c_double)), (n.value // 8,)).copy())
+    return out
+
+
+def test_time_and_wavemaker_outlast_the_zeroing_of_their_buffers(host):
+    ctx = host.Context([(64, 1, 6.4, 1.0)], 9.81, None, h0=0.7)
+    before = host.fake.fake_made()
+    ctx.set_time(2.5)
+    ctx.set_wavemaker([0.01, 0.02], [3.0, 4.0], [0.1, 0.2], 0.3)
+    host.fake.fake_drain()
+    time, params, profiles = doubles(host.fake, before)[:3]
+    assert time[0] == 2.5
+    assert list(params) == [3.0, 4.0, 0.1, 0.2]
+    assert profiles.size == 128 and profiles.reshape(2, 64).max(axis=1).min() > 0
+    ctx.close()
