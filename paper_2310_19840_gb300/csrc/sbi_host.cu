@@ -584,6 +584,7 @@ struct Planner {
       return p;
     }
     cudaError_t e = c->fp64 ? launch_coef_table<double>(p, s, c->cap) : launch_coef_table<float>(p, s, c->cap);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap);   // the passes that read it run on any stream
     if (e != cudaSuccess) oom = true;
     return p;
   }

@@ -67,3 +67,17 @@ def test_time_and_wavemaker_outlast_the_zeroing_of_their_buffers(host):
     assert list(params) == [3.0, 4.0, 0.1, 0.2]
     assert profiles.size == 128 and profiles.reshape(2, 64).max(axis=1).min() > 0
     ctx.close()
+
+
+def test_streamed_passes_wait_for_their_tables(host):
+    # a filtered step needs the table of Lambda only, the entry of the streamed
+    # call the one of the mask
+    grids = [(32, 16, 3.2, 1.6), (64, 32, 6.4, 3.2)]
+    n = sum(g[0] * g[1] for g in grids)
+    ctx = host.Context(grids, 9.81, None, h0=0.7, filt_beta1=8.0, filt_beta2=30.0, k_ref=1.0, autotune=0)
+    a = np.zeros(n)
+    ctx.step(0.01, 1)
+    before = host.fake.fake_overtaken()
+    ctx.step_streamed(a, a, 0.01, 1)
+    assert host.fake.fake_overtaken() == before
+    ctx.close()
