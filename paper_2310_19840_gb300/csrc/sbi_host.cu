@@ -1994,25 +1994,30 @@ struct LineBuilder {
   }
 };
 
-// Replaces every run of lineable passes of a one-dimensional FP32 group by
-// PK_LINE passes over its members [m0, m1).  Uploads the programs (each distinct
-// one once per context); not to be called while a capture is running.
+// Replaces every run of lineable passes of a one-dimensional FP32 group by one
+// PK_LINE pass over its members [m0, m1).  Uploads the programs (each distinct
+// one once per context); not to be called while a capture is running.  The
+// longest program that the options allow, both halves of the adaptive pair over
+// a variable bottom or with the HOS diagnostic at order 7, has 28 KB of the 40.
 int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1) {
   if (!g.line) return SBI_OK;
   std::vector<Pass> out;
   LineBuilder lb;
   double nbytes = 0.0, xforms = 0.0;
-  std::string ready;
   auto emit = [&]() -> int {
-    if (ready.empty()) return SBI_OK;
-    void*& dev = c->line_programs[ready];
+    if (lb.phases.empty()) return SBI_OK;
+    if (!lb.ok) return fail(c, SBI_EINVAL, "a pass has no one-dimensional form");
+    const std::string program = lb.bytes(g, c->tw);
+    if (!lb.ok || program.size() > (size_t)kLineMaxBytes)
+      return fail(c, SBI_EINVAL, "the passes have no one-dimensional form");
+    void*& dev = c->line_programs[program];
     if (!dev) {
-      dev = dalloc(c, ready.size());
+      dev = dalloc(c, program.size());
       if (!dev) {
-        c->line_programs.erase(ready);
+        c->line_programs.erase(program);
         return fail(c, SBI_ENOMEM, "device allocation failed");
       }
-      CK(cudaMemcpyAsync(dev, ready.data(), ready.size(), cudaMemcpyHostToDevice, c->cap), "upload program");
+      CK(cudaMemcpyAsync(dev, program.data(), program.size(), cudaMemcpyHostToDevice, c->cap), "upload program");
       CK(cudaStreamSynchronize(c->cap), "upload program");
     }
     Pass p{};
@@ -2022,39 +2027,25 @@ int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1
     // SMs of its own
     int cluster = line_cluster(g.nx);
     while (cluster > 1 && (m1 - m0) * cluster > 128) cluster /= 2;
-    p.line = LineParams{dev, (int)ready.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1, cluster};
+    p.line = LineParams{dev, (int)program.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1, cluster};
     p.lined = true;
     p.bytes = nbytes;
     p.xforms = xforms;
     out.push_back(p);
     lb = LineBuilder();
-    ready.clear();
     nbytes = xforms = 0.0;
     return SBI_OK;
   };
   for (const Pass& p : ps) {
-    if (!lineable(p)) {
-      const int rc = emit();
-      if (rc) return rc;
-      out.push_back(p);
+    if (lineable(p)) {
+      lb.add(p);
+      nbytes += p.bytes;
+      xforms += p.xforms;
       continue;
     }
-    const LineBuilder before = lb;
-    lb.add(p);
-    std::string now = lb.bytes(g, c->tw);
-    if (now.size() > (size_t)kLineMaxBytes) {   // start another program
-      const int rc = before.phases.empty() ? fail(c, SBI_EINVAL, "a pass is too long") : emit();
-      if (rc) return rc;
-      lb = LineBuilder();
-      // the pressure profile lives in shared memory: formed again beside its reader
-      if (&p != &ps[0] && (&p)[-1].kind == PK_WMK) lb.add((&p)[-1]);
-      lb.add(p);
-      now = lb.bytes(g, c->tw);
-    }
-    if (!lb.ok) return fail(c, SBI_EINVAL, "a pass has no one-dimensional form");
-    ready = std::move(now);
-    nbytes += p.bytes;
-    xforms += p.xforms;
+    const int rc = emit();
+    if (rc) return rc;
+    out.push_back(p);
   }
   const int rc = emit();
   if (rc) return rc;

@@ -81,3 +81,24 @@ def test_streamed_passes_wait_for_their_tables(host):
     ctx.step_streamed(a, a, 0.01, 1)
     assert host.fake.fake_overtaken() == before
     ctx.close()
+
+
+@pytest.mark.parametrize("integrator", [0, 1, 2])
+@pytest.mark.parametrize("diagnostic, bar, adapt", [(0, 0, 0.0), (0, 1, 0.0), (1, 0, 0.0), (0, 0, 1e-6), (0, 1, 1e-6)])
+def test_a_one_dimensional_step_is_one_launch_between_adaptive_tests(host, integrator, diagnostic, bar, adapt):
+    # at the highest order and with every term: the longest programs there are
+    if integrator and adapt:
+        pytest.skip("refused: the integrating factor takes no adapt_tol")
+    nx = 64
+    depth = np.full(nx, 0.7) - 0.1 * np.cos(2 * np.pi * np.arange(nx) / nx)
+    ctx = host.Context([(nx, 1, 6.4, 1.0)], 9.81, [depth] if bar else None, h0=0.7, order=7, integrator=integrator,
+                       diagnostic=diagnostic, adapt_tol=adapt, sponge_w=np.ones(nx), sponge_nu=0.3, filt_beta1=8.0,
+                       filt_beta2=30.0, autotune=0)
+    if integrator < 2:
+        ctx.set_wavemaker([0.1] * 256, [1.0] * 256, [0.0] * 256, 0.0)
+        ctx.step(0.01, 1)
+        assert host.fake.fake_captured() == ctx.step_launches()
+        assert adapt or ctx.step_launches() == 2       # with the time advance
+    else:
+        ctx.step_adaptive(0.001, 1e-3, 0.001)
+    ctx.close()
