@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
       const RkParams& q = reinterpret_cast<const RkParams*>(prog + H.rks)[P.out_begin];
       bool bad = false;
       const float bw = (q.stage == 1 || q.stage == 4) ? 1.f : 2.f;
-      const RkScalar cdt = q.cdt, dt6 = q.dt6;
+      const RkScalar cdt = p.cdt[q.mode == RK_STAGE ? q.stage - 1 : 0], dt6 = p.dt6;
       // the first block updates the elevation, the second (if there is one) the
       // potential: the blocks that transform slots 2 and 3 (jobs 0 and 1)
       for (int i = tid + (C > 1 ? rank * n : 0); i < (C > 1 ? (rank < 2 ? (rank + 1) * n : 0) : 2 * n);
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
       }
     } else if (rank == 0) {   // LP_WMK: FP64 sums and sines, rounded once
       const LineWmk& q = reinterpret_cast<const LineWmk*>(prog + H.wmks)[P.out_begin];
-      const double time = *q.t + q.offset;
+      const double time = *q.t + p.offset[q.stage];
       double* sines = reinterpret_cast<double*>(xs0);       // the exchange buffer is free here
       for (int i = tid; i < q.J; i += kLineThreads) sines[i] = sin(q.omega[i] * time + q.phase[i]);
       __syncthreads();

@@ -9,6 +9,7 @@ namespace sbi {
 
 constexpr int kLineSlots = 6;          // physical fields held in shared memory
 constexpr int kLineMaxBytes = 40960;   // largest program (it is copied into shared memory)
+constexpr int kLineStages = 4;         // RK4 stages of a program
 
 enum LinePhaseType : uint8_t {
   LP_INVERSE = 0,   // jobs: mixed sums -> slots, one transform each
@@ -51,8 +52,7 @@ struct LinePhase {
 };
 struct LineWmk {
   const double *prof, *omega, *phase, *t;
-  double offset;
-  int J;
+  int J, stage;                // stage: of LineParams::offset
 };
 struct LineHeader {
   int bytes;                   // of the whole program
@@ -60,12 +60,16 @@ struct LineHeader {
   int W;
   const void* tw;
 };
+// What depends on the step size is handed over with the launch: a program is the
+// same for every step (of a scheme whose tables are).
 struct LineParams {
   const void* program;
   int bytes;
   int exact;                   // half of the modes kept
   int member0, member1;        // members of this launch (one cluster of blocks each)
   int cluster;                 // blocks per member
+  RkScalar cdt[kLineStages], dt6;   // RK_STAGE phases, by stage - 1
+  double offset[kLineStages];       // stage time minus step start, by LineWmk::stage
 };
 // The most blocks per member: rows of 2048 points and more have too few groups
 // of threads in one block for the products of a level (at 1024 points two

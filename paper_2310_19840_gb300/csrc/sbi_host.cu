@@ -30,6 +30,7 @@
 #include <functional>
 #include <list>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -122,6 +123,7 @@ struct Pass {
   bool lined;     // runs inside a PK_LINE launch (set by the planner)
   double bytes;   // algorithmic device-memory traffic of the launch
   double xforms;  // 1-D transform passes over a whole field, times the field's points
+  std::shared_ptr<void> program;   // PK_LINE: keeps the device copy
 };
 
 // A table whose values depend on the step h: tau = r h, coefficient c0 h^p.
@@ -184,6 +186,7 @@ struct GraphEntry {
   int launches = 0;
   std::vector<cudaEvent_t> ev;       // profiled graphs: event pair per pass
   std::vector<int> ev_family;
+  std::vector<std::shared_ptr<void>> programs;   // of its PK_LINE launches
 };
 
 // What a captured graph runs: a whole step of a fixed-step scheme; or, for
@@ -236,7 +239,9 @@ struct sbi_ctx {
     double ms;
   };
   std::map<std::string, Tuned> tuned;
-  std::map<std::string, void*> line_programs;   // device copies of k_line programs, by content
+  // device copies of k_line programs, by content; the ones that no graph and no
+  // list of passes uses any more are given back when there are kLinePrograms
+  std::map<std::string, std::shared_ptr<void>> line_programs;
   std::vector<std::string> tune_order;  // signatures in the order they were tuned
   cudaEvent_t tune_ev[2] = {nullptr, nullptr};
   double dyn_h = NAN;   // the step the dynamic tables were last computed for
@@ -289,6 +294,12 @@ void* dalloc(sbi_ctx* c, size_t bytes) {
     cudaStreamSynchronize(c->cap);   // the first use may be on any stream
   }
   return p;
+}
+
+void dfree(sbi_ctx* c, void* p) {
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+  if (c->opt.dev_free) c->opt.dev_free(p, c->opt.alloc_user);
+  else cudaFree(p);
 }
 
 // ---------------------------------------------------------------------------
@@ -1724,6 +1735,8 @@ bool lineable(const Pass& p) {
   return p.kind == PK_ROW || p.kind == PK_COL || p.kind == PK_RK || p.kind == PK_WMK;
 }
 
+constexpr size_t kLinePrograms = 32;
+
 struct LineBuilder {
   std::vector<LinePhase> phases;
   std::vector<LineJob> jobs;
@@ -1731,6 +1744,7 @@ struct LineBuilder {
   std::vector<BufRef> bufs;
   std::vector<RkParams> rks;
   std::vector<LineWmk> wmks;
+  LineParams launch{};   // its step sizes
   bool ok = true;
 
   int16_t buf(const BufRef& b) {
@@ -1894,6 +1908,15 @@ struct LineBuilder {
     LinePhase u = phase(LP_RK, k.active);
     u.out_begin = (int16_t)rks.size();
     rks.push_back(k);
+    RkParams& q = rks.back();   // without the step size and the member range
+    q.dt = 0.0;
+    q.cdt = q.dt6 = rk_scalar(0.0);
+    q.row_begin = q.rows_total = 0;
+    if (k.mode == RK_STAGE) {
+      if (k.stage < 1 || k.stage > kLineStages) ok = false;
+      else launch.cdt[k.stage - 1] = k.cdt;
+      launch.dt6 = k.dt6;
+    }
     phases.push_back(u);
     if (!k.tail) return;
     LinePhase out = phase(LP_FORWARD, k.active);
@@ -1916,7 +1939,9 @@ struct LineBuilder {
     else {
       LinePhase w = phase(LP_WMK, nullptr);
       w.out_begin = (int16_t)wmks.size();
-      wmks.push_back(LineWmk{p.wmk.prof, p.wmk.omega, p.wmk.phase, p.wmk.t, p.wmk.offset, p.wmk.J});
+      if (wmks.size() == kLineStages) ok = false;
+      else launch.offset[wmks.size()] = p.wmk.offset;
+      wmks.push_back(LineWmk{p.wmk.prof, p.wmk.omega, p.wmk.phase, p.wmk.t, p.wmk.J, (int)wmks.size()});
       phases.push_back(w);
     }
   }
@@ -1995,8 +2020,8 @@ struct LineBuilder {
 };
 
 // Replaces every run of lineable passes of a one-dimensional FP32 group by one
-// PK_LINE pass over its members [m0, m1).  Uploads the programs (each distinct
-// one once per context); not to be called while a capture is running.  The
+// PK_LINE pass over its members [m0, m1).  Uploads the programs that the context
+// does not hold already; not to be called while a capture is running.  The
 // longest program that the options allow, both halves of the adaptive pair over
 // a variable bottom or with the HOS diagnostic at order 7, has 28 KB of the 40.
 int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1) {
@@ -2010,13 +2035,23 @@ int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1
     const std::string program = lb.bytes(g, c->tw);
     if (!lb.ok || program.size() > (size_t)kLineMaxBytes)
       return fail(c, SBI_EINVAL, "the passes have no one-dimensional form");
-    void*& dev = c->line_programs[program];
-    if (!dev) {
-      dev = dalloc(c, program.size());
-      if (!dev) {
-        c->line_programs.erase(program);
-        return fail(c, SBI_ENOMEM, "device allocation failed");
+    auto held = c->line_programs.find(program);
+    if (held == c->line_programs.end()) {
+      if (c->line_programs.size() >= kLinePrograms) {
+        CK(cudaStreamSynchronize(c->cap), "sync");      // launches of the ones given back
+        CK(cudaStreamSynchronize(c->stream), "sync");
+        for (auto it = c->line_programs.begin(); it != c->line_programs.end();) {
+          if (it->second.use_count() > 1) {
+            ++it;
+            continue;
+          }
+          dfree(c, it->second.get());
+          it = c->line_programs.erase(it);
+        }
       }
+      void* dev = dalloc(c, program.size());
+      if (!dev) return fail(c, SBI_ENOMEM, "device allocation failed");
+      held = c->line_programs.emplace(program, std::shared_ptr<void>(dev, [](void*) {})).first;
       CK(cudaMemcpyAsync(dev, program.data(), program.size(), cudaMemcpyHostToDevice, c->cap), "upload program");
       CK(cudaStreamSynchronize(c->cap), "upload program");
     }
@@ -2027,7 +2062,14 @@ int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1
     // SMs of its own
     int cluster = line_cluster(g.nx);
     while (cluster > 1 && (m1 - m0) * cluster > 128) cluster /= 2;
-    p.line = LineParams{dev, (int)program.size(), 4 * g.W == g.nx ? 1 : 0, m0, m1, cluster};
+    p.line = lb.launch;
+    p.line.program = held->second.get();
+    p.line.bytes = (int)program.size();
+    p.line.exact = 4 * g.W == g.nx ? 1 : 0;
+    p.line.member0 = m0;
+    p.line.member1 = m1;
+    p.line.cluster = cluster;
+    p.program = held->second;
     p.lined = true;
     p.bytes = nbytes;
     p.xforms = xforms;
@@ -2602,6 +2644,9 @@ int build_step_graph(sbi_ctx* c, double dt, int kind, const Unit* only, GraphEnt
     return cuda_fail(c, e, "graph instantiate");
   }
   ge.launches = (int)npasses;
+  for (auto& v : gps)
+    for (auto& p : v)
+      if (p.program) ge.programs.push_back(p.program);
   return SBI_OK;
 }
 

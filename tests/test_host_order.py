@@ -102,3 +102,27 @@ def test_a_one_dimensional_step_is_one_launch_between_adaptive_tests(host, integ
     else:
         ctx.step_adaptive(0.001, 1e-3, 0.001)
     ctx.close()
+
+
+@pytest.mark.parametrize("schemes", ["rk4", "wavemaker"])
+def test_step_sizes_and_wavemakers_leave_no_programs_behind(host, schemes):
+    # a program does not hold the step size; of those of earlier wavemakers at
+    # most 32, and the one in use, are kept (40 KB each)
+    nx = 64
+    ctx = host.Context([(nx, 1, 6.4, 1.0)], 9.81, None, h0=0.7, autotune=0)
+    ctx.set_wavemaker([0.1] * 256, [1.0] * 256, [0.0] * 256, 0.0)
+    ctx.step(0.01, 1)
+    held, made = host.fake.fake_live_bytes(), host.fake.fake_made()
+    for k in range(100):
+        if schemes == "rk4":
+            ctx.step(0.01 + 1e-4 * (k + 1), 1)
+        else:
+            n = 1 + k
+            ctx.set_wavemaker([0.1] * n, [1.0] * n, [0.0] * n, 0.0)
+            ctx.step(0.01, 1)
+    if schemes == "rk4":
+        assert host.fake.fake_made() == made
+    else:
+        assert host.fake.fake_live_bytes() < held + 34 * 40960
+    ctx.close()
+    assert host.fake.fake_live_bytes() == 0
