@@ -533,9 +533,10 @@ struct Planner {
     int tpc = 0, group = 1;
     packed_col_geometry(g.ny, &tpc, &group);
     const double warps = (double)p.cols_total * tpc / 32.0;
-    if (most < 2 || warps * 3 > 152.0 * 8.0) return 0;
+    const int useful = std::max(p.nin, p.nouts);   // copies beyond these have nothing to transform
+    if (most < 2 || useful < 2 || warps * 3 > 152.0 * 8.0) return 0;
     int k = 2;
-    while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < 152.0 * 8.0) k *= 2;
+    while (2 * k <= most && k < useful && warps * k < 152.0 * 8.0) k *= 2;
     return k;
   }
   struct ColIn {
