@@ -396,21 +396,17 @@ k_packed_row(const __grid_constant__ RowParams p) {
 // accumulated as the gradients come back from their transforms, in the
 // thread's own slots of shared memory; a derivative of eta waits in registers
 // for the one of phi~.  The modes of the next transform are loaded ahead of the
-// current one.  The quotient takes one residual correction (Newton) after an
-// approximate reciprocal of 1 + |grad eta|^2 >= 1: below one unit in the last
-// place, in five packed and two special operations for two values.
-// Load latency bounds it (a quarter of the issue slots used): 8192 rows of 512
-// points 63 us (75 with the IEEE quotient and spills; 66 with 128 registers, four
-// blocks per SM and no loads ahead).
+// current one.  The quotients are IEEE divisions, correct to half a unit in the
+// last place for every operand.  Load latency bounds the pass (a quarter of the
+// issue slots used): 8192 rows of 512 points 65 us, 128 of the 168 registers
+// (four blocks per SM and no loads ahead) 66.
 struct RhsOps {
   int8_t src[5];      // inverse transforms in the order eta_x, phi_x, eta_y, phi_y, V (indices into ops)
   int8_t f, sx, sy;   // the operation; sponge products of phi_x and phi_y (-1: none)
 };
-__device__ __forceinline__ F2 quotient(F2 a, F2 d) {     // a / d, d >= 1 (or not finite)
-  const float2 p = parts(d);
-  const F2 r = f2(__fdividef(1.f, p.x), __fdividef(1.f, p.y));
-  const F2 q = mul(a, r);
-  return fma(fma(mul(both(-1.f), d), q, a), r, q);
+__device__ __forceinline__ F2 quotient(F2 a, F2 d) {
+  const float2 p = parts(a), q = parts(d);
+  return f2(__fdiv_rn(p.x, q.x), __fdiv_rn(p.y, q.y));
 }
 template <int NX, bool EXACT>
 __global__ void __launch_bounds__(RowGeo<NX>::THREADS, 3)
