@@ -257,16 +257,13 @@ struct PackedFft {
     return Twiddles{t + (N <= R * R ? j : j & (R - 1))};
   }
   // Butterflies b = j + q T (q < Q) of radix RP on elements v[m] = x[q + m Q].
-  // A third pass forms its twiddles from the thread's own w_N^j (and w_N^{4j}):
-  // w_N^{qT} = e^{-2 pi i q / R}.
+  // A third pass (512 elements and more) loads w_N^b and w_N^{4b} and forms the
+  // other powers by products.  With w_N^b itself a product, w_N^j e^{-2 pi i q / R},
+  // the powers carried its error up to three times: a step of a 4096 x 2048 sea
+  // was 1.39e-7 from the 64-bit one, and is 1.24e-7.
   template <int RP, bool SECOND>
   __device__ __forceinline__ static void last_pass(V (&x)[R], int j, Twiddles t, const float2* __restrict__ tw) {
     constexpr int Q = R / RP;
-    float2 wj = make_float2(1.f, 0.f), wj4 = wj;
-    if constexpr (!SECOND) {
-      wj = __ldg(tw + tw_off(N) + j);
-      if constexpr (RP >= 8) wj4 = __ldg(tw + tw_off(N) + 4 * j);
-    }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       V v[RP];
@@ -276,7 +273,7 @@ struct PackedFft {
 #pragma unroll
         for (int m = 1; m < RP; ++m) v[m] = cmul(v[m], t(m, q));
       } else {
-        const float2 w1 = q == 0 ? wj : wmul(wj, unit_root(q, R));
+        const float2 w1 = __ldg(tw + tw_off(N) + j + q * T);
         v[1] = cmul(v[1], w1);
         if constexpr (RP >= 4) {
           const float2 w2 = wmul(w1, w1), w3 = wmul(w1, w2);
@@ -284,7 +281,7 @@ struct PackedFft {
           v[3] = cmul(v[3], w3);
           if constexpr (RP >= 8) {
             static_assert(RP == 8, "third passes of radix 2, 4 and 8");
-            const float2 w4 = q == 0 ? wj4 : wmul(wj4, unit_root(4 * q, R));
+            const float2 w4 = __ldg(tw + tw_off(N) + 4 * (j + q * T));
             v[4] = cmul(v[4], w4);
             v[5] = cmul(v[5], wmul(w4, w1));
             v[6] = cmul(v[6], wmul(w4, w2));
