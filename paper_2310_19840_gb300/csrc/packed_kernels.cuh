@@ -1076,7 +1076,12 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
   float2 wj = __ldg(tw + tw_off(NY) + j);
   wait_for_previous();
   act = valid && (p.active == nullptr || p.active[p.member0 + member] != 0);
-  if (copy < p.nin) load(copy);
+  if (copy < p.nin) {
+    load(copy);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = Two{both(0.f), both(0.f)};
+  }
   __syncthreads();
 #pragma unroll 1
   for (int i0 = 0; i0 < p.nin; i0 += copies) {     // the same trips for every copy
@@ -1086,7 +1091,7 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
       load(i);
       load_factors(i);
     }
-    G::F::run(x, xs, j, t, tw);
+    if (!G::WARP || i < p.nin) G::F::run(x, xs, j, t, tw);   // a set of several warps has block barriers in it
     if (i < p.nin) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -1176,7 +1181,7 @@ k_packed_col_wide(const __grid_constant__ ColParams p) {
         }
       }
     }
-    G::F::run(x, xs, j, t, tw);
+    if (!G::WARP || o < p.nouts) G::F::run(x, xs, j, t, tw);
     if (o < p.nouts && act) {
 #pragma unroll
       for (int r = 0; r < R; ++r) x[r] = Two{conj(x[r].a), conj(x[r].b)};

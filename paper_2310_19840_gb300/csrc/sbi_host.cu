@@ -527,16 +527,17 @@ struct Planner {
   // form): doubled until every SM has eight warps, or each copy one transform;
   // none from 2.7 warps per SM on.  Column passes of a step, untuned, with and
   // without: one 512^2 member 380 and 583 us, four 535 and 631, eight (3.4 warps)
-  // 750 and 683.
+  // 750 and 683.  Passes of one input and one output take two copies as well:
+  // the second sums half of the modes (four steps of one 512^2 member 1.91 ms, and
+  // 2.00 with the plain form there).
   int default_wide(const ColParams& p) const {
     const int most = packed_col_most_wide(p);
     int tpc = 0, group = 1;
     packed_col_geometry(g.ny, &tpc, &group);
     const double warps = (double)p.cols_total * tpc / 32.0;
-    const int useful = std::max(p.nin, p.nouts);   // copies beyond these have nothing to transform
-    if (most < 2 || useful < 2 || warps * 3 > 152.0 * 8.0) return 0;
+    if (most < 2 || warps * 3 > 152.0 * 8.0) return 0;
     int k = 2;
-    while (2 * k <= most && k < useful && warps * k < 152.0 * 8.0) k *= 2;
+    while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < 152.0 * 8.0) k *= 2;
     return k;
   }
   struct ColIn {
@@ -2238,7 +2239,8 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     if (p.col.packed && !p.col.staged) {   // copies of the wide form
       const int most = packed_col_most_wide(p.col);
       const double warps = (double)p.col.cols_total * tpc / 32.0;
-      for (int k = 2; k <= most && k < 2 * std::max(p.col.nin, p.col.nouts) && warps * k < 152.0 * 8.0 * 4; k *= 2)
+      const int useful = std::max({2, p.col.nin, p.col.nouts});
+      for (int k = 2; k <= most && k < 2 * useful && warps * k < 152.0 * 8.0 * 4; k *= 2)
         if (2 * k >= p.col.wide) cand.push_back(base(0) + kWideTag * k);
     }
   }

@@ -128,19 +128,18 @@ def test_step_sizes_and_wavemakers_leave_no_programs_behind(host, schemes):
     assert host.fake.fake_live_bytes() == 0
 
 
-def test_column_passes_of_one_transform_take_no_idle_copies(host):
-    # the tuner lists chosen/default; the wide form has at most one power of two
-    # more copies than the pass has transforms to share out
+def test_the_wide_default_of_a_column_pass_is_among_the_timed_shapes(host):
+    # the report gives chosen/default and the time of the chosen one (-1: none was
+    # timed); at most one power of two more copies than transforms to share out
     import re
     ctx = host.Context([(64, 64, 6.4, 6.4)], 9.81, None, h0=0.7, order=4)
     ctx.step(0.01, 1)
     seen = set()
     for line in ctx.autotune_report().splitlines():
-        m = re.match(r"col .* in=(\d+) .* out=(\d+) .*: cpb \S+/(\S+) ", line)
+        m = re.match(r"col .* in=(\d+) .* out=(\d+) .*: cpb \S+/\S+w(\d+) (\S+) ms", line)
         if m:
-            share = max(int(m[1]), int(m[2]))
-            wide = re.search(r"w(\d+)$", m[3])
-            assert (int(wide[1]) if wide else 1) < 2 * share, line
+            share = max(2, int(m[1]), int(m[2]))
+            assert int(m[3]) < 2 * share and float(m[4]) > 0.0, line
             seen.add(share)
-    assert 1 in seen and max(seen) > 2
+    assert 2 in seen and max(seen) > 2
     ctx.close()
