@@ -222,6 +222,7 @@ struct sbi_ctx {
   int stream_k = 0;   // streamed step: each schedule unit cut into stream_k member ranges (0: not chosen)
   int stall_tx = 0;   // test hook of the staged column pass (sbi_test_stall_staged_copies)
   std::vector<void*> allocs;
+  bool fresh = false;  // buffers or tables are made that nothing has waited for (settle)
   void* tw = nullptr;
   void* wgt = nullptr;  // shared sponge weight (working precision) or null
   int* d_flags = nullptr;  // [0]: non-finite state; [1]: a bounded wait gave up
@@ -291,9 +292,17 @@ void* dalloc(sbi_ctx* c, size_t bytes) {
   if (p) {
     c->allocs.push_back(p);
     cudaMemsetAsync(p, 0, bytes, c->cap);
-    cudaStreamSynchronize(c->cap);   // the first use may be on any stream
+    c->fresh = true;
   }
   return p;
+}
+
+// New buffers are zeroed, and new tables filled, on c->cap.  Before work on
+// another stream (that nothing else orders behind c->cap) can use them:
+cudaError_t settle(sbi_ctx* c) {
+  if (!c->fresh) return cudaSuccess;
+  c->fresh = false;
+  return cudaStreamSynchronize(c->cap);
 }
 
 void dfree(sbi_ctx* c, void* p) {
@@ -597,7 +606,7 @@ struct Planner {
       return p;
     }
     cudaError_t e = c->fp64 ? launch_coef_table<double>(p, s, c->cap) : launch_coef_table<float>(p, s, c->cap);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->cap);   // the passes that read it run on any stream
+    c->fresh = true;
     if (e != cudaSuccess) oom = true;
     return p;
   }
@@ -3294,7 +3303,9 @@ double* device_view(void* p, int on_device) {
 
 int ensure_stage(sbi_ctx* c, Group& g) {
   if (!g.stage64) g.stage64 = (double*)dalloc(c, g.phys_elems() * g.n * 8);
-  return g.stage64 ? SBI_OK : fail(c, SBI_ENOMEM, "device allocation failed");
+  if (!g.stage64) return fail(c, SBI_ENOMEM, "device allocation failed");
+  CK(settle(c), "sync");
+  return SBI_OK;
 }
 
 int sbi_set_state_all(sbi_ctx* c, const double* eta, const double* phi, int on_device) {
@@ -3630,6 +3641,7 @@ int streamed_run(sbi_ctx* c, const double* eta_in, const double* phi_in, double 
     rc = lower_line(c, g, entry[ui], u.m0, u.m1);
     if (rc) return rc;
   }
+  CK(settle(c), "sync");
   int least = 0, greatest = 0;
   CK(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
   while (c->pstreams.size() < U) {
@@ -3893,6 +3905,7 @@ int sbi_invariants(sbi_ctx* c, int member, double* mass, double* energy) {
   if ((size_t)nchunks * 2 > c->partial_cap) {
     void* p = dalloc(c, (size_t)nchunks * 2 * 8);
     if (!p) return fail(c, SBI_ENOMEM, "device allocation failed");
+    CK(settle(c), "sync");
     c->d_partials = (double*)p;
     c->partial_cap = (size_t)nchunks * 2;
   }
