@@ -231,7 +231,7 @@ def measured_peaks():
 # committed ncu summary records (host code and the other kernels live in
 # sbi_host.cu and sbi_noalloc.cu)
 KERNEL_SOURCES = ("bank_model.h", "fft.cuh", "kernels.cuh", "line.cuh", "line.h", "packed.cuh",
-                  "packed_kernels.cuh", "sbi_internal.h", "inst_col_f64.cu", "inst_line.cu",
+                  "packed_kernels.cuh", "sbi_internal.h", "inst_batch_f32.cu", "inst_col_f64.cu", "inst_line.cu",
                   "inst_packed_col.cu", "inst_packed_row.cu", "inst_packed_row_long.cu", "inst_row_f64.cu")
 
 

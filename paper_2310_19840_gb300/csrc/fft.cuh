@@ -143,11 +143,25 @@ __device__ __forceinline__ V twiddle(const V* __restrict__ tw, int N, int idx) {
   return SIGN > 0 ? cconj(w) : w;
 }
 
+template <typename V> inline constexpr bool kProductTwiddles = sizeof(V) == 8;   // FP32
+// exp(-2 pi i q / 16), q = 0 .. 7 (a constant after unrolling)
+template <typename V>
+__device__ __forceinline__ V root16(int q) {
+  using S = decltype(V::x);
+  constexpr double c[8] = {1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173,
+                           0.0, -0.38268343236508977173, -0.70710678118654752440, -0.92387953251128675613};
+  constexpr double s[8] = {0.0, 0.38268343236508977173, 0.70710678118654752440, 0.92387953251128675613,
+                           1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173};
+  return mk<V>(S(c[q]), S(-s[q]));
+}
+
 // DFT of length R of x[r] w^r, w = w_N^idx (idx < N / R): the twiddles of a
 // Stockham pass enter the butterflies, (a + w b, a - w b) at six fused
 // multiply-adds each, and only the powers w, w^2, w^4 and w w_8 are loaded.  A
 // radix-8 pass takes 72 FP64 operations (84 with the products first), a radix-4
-// pass 24 (28).
+// pass 24 (28).  In FP32, where loads are the scarcer resource, w^2 and w w_8 are
+// products of w (one rounding each): a step of 2432 members of 2048 points 2.29 ->
+// 2.10 ms.
 template <int SIGN, typename V>
 __device__ __forceinline__ void dft4_twiddled(V& x0, V& x1, V& x2, V& x3, V w, V w2) {
   butterfly(x0, x2, w2);
@@ -166,10 +180,21 @@ __device__ __forceinline__ void dft_twiddled(V* x, const V* __restrict__ tw, int
   if constexpr (R == 2) {
     butterfly(x[0], x[1], w);
   } else if constexpr (R == 4) {
-    dft4_twiddled<SIGN>(x[0], x[1], x[2], x[3], w, twiddle<SIGN>(tw, N, 2 * idx));
+    V w2;
+    if constexpr (kProductTwiddles<V>) w2 = cmul(w, w);
+    else w2 = twiddle<SIGN>(tw, N, 2 * idx);
+    dft4_twiddled<SIGN>(x[0], x[1], x[2], x[3], w, w2);
   } else if constexpr (R == 8) {
-    const V w2 = twiddle<SIGN>(tw, N, 2 * idx), w4 = twiddle<SIGN>(tw, N, 4 * idx);
-    const V wr = twiddle<SIGN>(tw, N, idx + N / 8);
+    const V w4 = twiddle<SIGN>(tw, N, 4 * idx);
+    V w2, wr;
+    if constexpr (kProductTwiddles<V>) {
+      using S = decltype(V::x);
+      w2 = cmul(w, w);
+      wr = cmul(w, mk<V>(S(0.70710678118654752440), S(SIGN * 0.70710678118654752440)));
+    } else {
+      w2 = twiddle<SIGN>(tw, N, 2 * idx);
+      wr = twiddle<SIGN>(tw, N, idx + N / 8);
+    }
     dft4_twiddled<SIGN>(x[0], x[2], x[4], x[6], w2, w4);   // E_q in x[2 q]
     dft4_twiddled<SIGN>(x[1], x[3], x[5], x[7], w2, w4);   // O_q in x[2 q + 1]
     butterfly(x[0], x[1], w);

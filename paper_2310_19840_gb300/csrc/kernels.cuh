@@ -1,6 +1,7 @@
-// kernels.cuh - row, column and RK4 passes of FP64 groups (packed_kernels.cuh has
-// those of two-dimensional FP32 groups, line.cuh the one-dimensional ones), the
-// state formats, the multiplier tables and the copy helpers of all of them.
+// kernels.cuh - row, column and RK4 passes of FP64 groups and of large ensembles of
+// one-dimensional FP32 members (packed_kernels.cuh has those of two-dimensional
+// FP32 groups, line.cuh those of fewer one-dimensional members), the state
+// formats, the multiplier tables and the copy helpers of all of them.
 //
 // Layouts (see sbi_internal.h): physical fields are [member][y][x]; mixed
 // fields (x-spectral, y-physical, only the W kept x-modes) are stored
@@ -36,6 +37,10 @@ struct RowCfg {
   static constexpr int RPC_MAX = cmin(256, WARP ? cmax(16, 512 / TPR) : cmax(1, 512 / TPR));
   static constexpr int MAX_THREADS = TPR * RPC_MAX;
   static constexpr int FBUF = fft_scratch_len<n, R>();    // FFT scratch per row
+  // resident blocks per SM that a row pass is compiled for (0: no minimum); in
+  // FP32 two, 64 registers per thread
+  template <typename T>
+  static constexpr int min_blocks() { return sizeof(T) == 4 ? 2 : 0; }
 };
 
 // shared memory of a row block: per row the FFT scratch (row stride fbs), the
@@ -230,6 +235,13 @@ __device__ __forceinline__ void c2r_input(cx<T> (&x)[RowCfg<NX>::R], const cx<T>
                                           const cx<T>* __restrict__ tw) {
   using V = cx<T>;
   using C = RowCfg<NX>;
+  // e^{2 pi i (j + r TPR) / NX}; in FP32 a product by a 16th root of unity
+  constexpr bool kProd = C::R == 8 && kProductTwiddles<V>;
+  const V wj = __ldg(tw + tw_off(NX) + j);
+  auto factor = [&](int r) {
+    if constexpr (kProd) return cconj(r == 0 ? wj : cmul(wj, root16<V>(r)));
+    else return cconj(__ldg(tw + tw_off(NX) + j + r * C::TPR));
+  };
   if (2 * W <= C::n) {
     // At most half the packed modes are kept: X[k] and X[n-k] are never both
     // nonzero, so Z[k] = X[k] + i w X[k] for k < W, Y - i w Y with Y = conj(X[n-k])
@@ -237,7 +249,7 @@ __device__ __forceinline__ void c2r_input(cx<T> (&x)[RowCfg<NX>::R], const cx<T>
 #pragma unroll
     for (int r = 0; r < C::R; ++r) {
       const int k = j + r * C::TPR;
-      const V w = cconj(__ldg(tw + tw_off(NX) + k));
+      const V w = factor(r);
       V z = mk<V>(T(0), T(0));
       if (k < W) z = cfma(rot<1>(w), stg[k], stg[k]);
       else if (k > C::n - W) z = cfma(rot<-1>(w), cconj(stg[C::n - k]), cconj(stg[C::n - k]));
@@ -252,7 +264,7 @@ __device__ __forceinline__ void c2r_input(cx<T> (&x)[RowCfg<NX>::R], const cx<T>
     const V a = (k < W) ? stg[k] : mk<V>(T(0), T(0));
     const V b = (k > 0 && kk < W) ? stg[kk] : mk<V>(T(0), T(0));
     const V bc = cconj(b);
-    const V w = cconj(__ldg(tw + tw_off(NX) + k));
+    const V w = factor(r);
     x[r] = cconj(cfma(rot<1>(w), csub(a, bc), cadd(a, bc)));
   }
 }
@@ -328,7 +340,7 @@ __device__ __forceinline__ T ipow(T v, int p) {
 // several times the blocks, and every SM's FP64 lanes the same share of them:
 // six mixed members 6.14 -> 5.80 ms of row passes a step.
 template <typename T, int NX>
-__global__ void __launch_bounds__(RowCfg<NX>::MAX_THREADS)
+__global__ void __launch_bounds__(RowCfg<NX>::MAX_THREADS, RowCfg<NX>::template min_blocks<T>())
 k_row(const __grid_constant__ RowParams p) {
   using V = cx<T>;
   using C = RowCfg<NX>;
@@ -596,15 +608,20 @@ template <> struct StatePair<float> {
 // RK4 stage pass (row layout).  State and sums in StatePair<T> storage.
 // ===========================================================================
 // RK stage geometry: blocks of kRkThreads threads (a whole row when a row
-// needs more); two resident blocks per SM (at most 128 registers).
+// needs more); two resident blocks per SM (at most 128 registers) in FP64, three
+// in FP32 (85).
 template <int NX>
 struct RkCfg {
   static constexpr int RPC = cmax(1, kRkThreads / RowCfg<NX>::TPR);
   static constexpr int THREADS = RowCfg<NX>::TPR * RPC;
+  template <typename T>
+  static constexpr int min_blocks() { return sizeof(T) == 4 ? 3 : 2; }
 };
 
-template <typename T, int NX>
-__global__ void __launch_bounds__(RkCfg<NX>::THREADS, 2)
+// S: the state storage format (T itself, or double for the FP32 path with an
+// FP64 state)
+template <typename T, int NX, typename S>
+__global__ void __launch_bounds__(RkCfg<NX>::THREADS, RkCfg<NX>::template min_blocks<T>())
 k_rk(const __grid_constant__ RkParams p) {
   using V = cx<T>;
   using C = RowCfg<NX>;
@@ -626,7 +643,7 @@ k_rk(const __grid_constant__ RkParams p) {
   const long long off = (long long)y * NX;
 
   // new state in the working precision (the FFT inputs of the tail)
-  using SP = StatePair<T>;
+  using SP = StatePair<S>;
   V xe[R], xp[R];
   const long long eoff = member * p.eta0.stride + off, poff = member * p.phi0.stride + off;
   char* E0 = reinterpret_cast<char*>(p.eta0.ptr) + eoff * 8;   // 8 bytes per value
@@ -1134,7 +1151,9 @@ cudaError_t prepare_nx() {
   const int maxb = 227 * 1024;
   cudaError_t e = cudaFuncSetAttribute(k_row<T, NX>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_rk<T, NX>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
+  e = cudaFuncSetAttribute(k_rk<T, NX, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
+  if (e != cudaSuccess || sizeof(T) == 8) return e;
+  return cudaFuncSetAttribute(k_rk<T, NX, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
 }
 
 template <typename T, int NY>
@@ -1203,7 +1222,8 @@ cudaError_t launch_rk_n(const RkParams& p, cudaStream_t st) {
   RkParams q = p;
   q.fbs = bank::choose(C::n, C::R, C::TPR, p.rpc, p.W, (int)sizeof(cx<T>), true, false, C::FBUF).fbs;
   const size_t smem = sizeof(cx<T>) * (size_t)q.rpc * q.fbs;
-  k_rk<T, NX><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
+  if (q.state64 && sizeof(T) == 4) k_rk<T, NX, double><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
+  else k_rk<T, NX, T><<<blocks, C::TPR * q.rpc, smem, st>>>(q);
   return cudaGetLastError();
 }
 
@@ -1291,7 +1311,9 @@ cudaError_t launch_col_impl(int ny, const ColParams& p, cudaStream_t st) {
 // memory fits a block; 0 if even one row does not fit.
 template <typename T>
 int row_rpc_impl(int nx, int W, int nslots) {
-  const size_t budget = 227 * 1024;
+  // one block may take the whole 227 KB; blocks compiled for two per SM get
+  // half of the SM's 228 KB less the 1 KB each block reserves
+  size_t budget = 227 * 1024;
   int maxr = 0;
   size_t per = 0;
   switch (nx) {
@@ -1299,6 +1321,7 @@ int row_rpc_impl(int nx, int W, int nslots) {
   case N:                                                                   \
     maxr = RowCfg<N>::RPC_MAX;                                              \
     per = row_smem_bound<T, N>(W, nslots);                                  \
+    if (RowCfg<N>::template min_blocks<T>() == 2) budget = 113 * 1024;      \
     break;
     SBI_FOR_NX(SBI_CASE)
 #undef SBI_CASE

@@ -1,4 +1,5 @@
-// line.cuh - whole steps of one-dimensional FP32 members in one launch.
+// line.cuh - whole steps of one-dimensional FP32 members in one launch (ensembles
+// too large for it take one launch per pass: line_pays in line.h).
 //
 // A one-dimensional member is one row of 16 to 4096 points: a pass over it is
 // far below a launch in work, and a step of some 64 dependent launches took 7

@@ -76,6 +76,25 @@ struct LineParams {
 // blocks were 20 % slower than one).
 constexpr int line_cluster(int nx) { return nx >= 4096 ? 8 : (nx >= 2048 ? 4 : 1); }
 
+// Whether a group of n members of nx points takes this form.  A member fills an
+// SM (up to 1024 points; longer ones as good as), so the time is that of a
+// member for every 152 of them, while that of one launch per pass hardly grows
+// until the members fill the GPU.  Microseconds of a step, one launch and one
+// per pass:
+//   points  members  flat bottom   variable bottom
+//      256      304  214 and 332
+//      256      608  417 and 352   507 and 473
+//     1024      304  275 and 391
+//     1024      608  543 and 476   749 and 700
+//     2048      152  299 and 425   373 and 585
+//     2048      304  577 and 491   736 and 770
+//     4096      152  417 and 569   629 and 845
+//     4096      304  835 and 807   1232 and 1397
+// (2432 members of 256 points: 1633 and 432 with a flat bottom.)
+constexpr bool line_pays(int nx, int n, bool variable_bottom) {
+  return n <= 152 * (nx <= 1024 ? 3 : (variable_bottom ? 2 : 1));
+}
+
 cudaError_t prepare_line_kernels(int nx);
 cudaError_t launch_line(int nx, const LineParams& p, cudaStream_t st);
 

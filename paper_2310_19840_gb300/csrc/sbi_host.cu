@@ -162,7 +162,7 @@ struct Group {
   std::map<std::string, void*> mixed;
   std::map<std::string, void*> tables;   // multiplier tables by key
   bool packed = false;          // runs on the packed kernels (packed_kernels.cuh): FP32, two-dimensional
-  bool line = false;            // runs on k_line (line.cuh): FP32, one-dimensional
+  bool line = false;            // runs on k_line (line.cuh): FP32, one-dimensional, not too many members
   size_t phys_elems() const { return (size_t)nx * ny; }
   // stored columns of a mixed field (tiles of four in a packed group)
   int columns() const { return packed ? (W + 3) / 4 * 4 : W; }
@@ -466,7 +466,7 @@ struct Planner {
       int tpr = 0;
       return packed_row_geometry(g.nx, &tpr);
     }
-    const int r = row_rpc<double>(g.nx, g.W, nslots);
+    const int r = c->fp64 ? row_rpc<double>(g.nx, g.W, nslots) : row_rpc<float>(g.nx, g.W, nslots);
     if (r <= 0) oom = true;
     return r > 0 ? r : 1;
   }
@@ -537,8 +537,8 @@ struct Planner {
   // none from 2.7 warps per SM on.  Column passes of a step, untuned, with and
   // without: one 512^2 member 380 and 583 us, four 535 and 631, eight (3.4 warps)
   // 750 and 683.  Passes of one input and one output take two copies as well:
-  // the second sums half of the modes (four steps of one 512^2 member 1.91 ms, and
-  // 2.00 with the plain form there).
+  // the second sums half of the modes (in the plain form one 512^2 member takes
+  // 2.00 ms per four steps, 1.91 with two copies).
   int default_wide(const ColParams& p) const {
     const int most = packed_col_most_wide(p);
     int tpc = 0, group = 1;
@@ -972,10 +972,7 @@ struct Planner {
     p.rows_total = g.n * g.ny;
     p.ny = g.ny;
     p.W = g.W;
-    if (c->fp64) {
-      const int tpr = row_tpr<double>(g.nx);
-      p.rpc = std::max(1, kRkThreads / std::max(1, tpr));
-    }
+    if (!g.packed && !g.line) p.rpc = std::max(1, kRkThreads / std::max(1, row_tpr<double>(g.nx)));
     p.dt = dt;
     p.state64 = c->fp64 || !c->state_ds;
     p.dt6 = rk_scalar(dt / 6.0);
@@ -1731,9 +1728,15 @@ int launch_pass(sbi_ctx* c, const Pass& p, cudaStream_t st, bool chained = false
     if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
     return SBI_OK;
   }
-  if (p.kind == PK_ROW) e = p.row.packed ? launch_packed_row(p.nsize, p.row, st, chained) : launch_row<double>(p.nsize, p.row, st);
-  else if (p.kind == PK_COL) e = p.col.packed ? launch_packed_col(p.nsize, p.col, st, chained) : launch_col<double>(p.nsize, p.col, st);
-  else e = p.rk.packed ? launch_packed_rk(p.nsize, p.rk, st, chained) : launch_rk<double>(p.nsize, p.rk, st);
+  if (p.kind == PK_ROW)
+    e = p.row.packed ? launch_packed_row(p.nsize, p.row, st, chained)
+                     : (c->fp64 ? launch_row<double>(p.nsize, p.row, st) : launch_row<float>(p.nsize, p.row, st));
+  else if (p.kind == PK_COL)
+    e = p.col.packed ? launch_packed_col(p.nsize, p.col, st, chained)
+                     : (c->fp64 ? launch_col<double>(p.nsize, p.col, st) : launch_col<float>(p.nsize, p.col, st));
+  else
+    e = p.rk.packed ? launch_packed_rk(p.nsize, p.rk, st, chained)
+                    : (c->fp64 ? launch_rk<double>(p.nsize, p.rk, st) : launch_rk<float>(p.nsize, p.rk, st));
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
   return SBI_OK;
 }
@@ -2225,7 +2228,7 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
   } else {
     int tpc = 0, group = 1;
     const int cpb = p.col.packed ? packed_col_geometry(p.nsize, &tpc, &group)
-                               : col_geometry<double>(p.nsize, &tpc);
+                               : (c->fp64 ? col_geometry<double>(p.nsize, &tpc) : col_geometry<float>(p.nsize, &tpc));
     // the staged form of a packed group takes whole tiles of four columns
     auto base = [&](int staged) {
       const int b = p.col.cpb > 0 ? p.col.cpb : cpb;
@@ -3115,14 +3118,16 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
       g.ky_keep = std::max(g.ky_keep, 1);
       g.W = g.kx_keep;
       g.packed = g.two_d && !c->fp64;
-      g.line = !g.two_d && !c->fp64;
       c->groups.push_back(g);
     }
     Group& g = c->groups[sig[i]];
     c->where[i] = {sig[i], (int)g.members.size()};
     g.members.push_back(i);
   }
-  for (auto& g : c->groups) g.n = (int)g.members.size();
+  for (auto& g : c->groups) {
+    g.n = (int)g.members.size();
+    g.line = !g.two_d && !c->fp64 && line_pays(g.nx, g.n, g.variable);
+  }
 
   // twiddles exp(-2 pi i j / N) for N = 2..8192 in the working precision
   {
@@ -3144,10 +3149,16 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
   if (!c->d_flags) { c->err = "device allocation failed"; return bail(SBI_ENOMEM); }
 
   for (auto& g : c->groups) {
-    cudaError_t e = g.packed ? prepare_packed_row_kernels(g.nx)
-                             : (g.line ? prepare_line_kernels(g.nx) : prepare_row_kernels<double>(g.nx));
-    if (e == cudaSuccess && !g.line)
-      e = g.packed ? prepare_packed_col_kernels(g.ny) : prepare_col_kernels<double>(g.ny);
+    cudaError_t e = cudaSuccess;
+    if (g.line) {
+      e = prepare_line_kernels(g.nx);
+    } else if (g.packed) {
+      e = prepare_packed_row_kernels(g.nx);
+      if (e == cudaSuccess) e = prepare_packed_col_kernels(g.ny);
+    } else {
+      e = c->fp64 ? prepare_row_kernels<double>(g.nx) : prepare_row_kernels<float>(g.nx);
+      if (e == cudaSuccess) e = c->fp64 ? prepare_col_kernels<double>(g.ny) : prepare_col_kernels<float>(g.ny);
+    }
     if (e != cudaSuccess) { cuda_fail(c, e, "kernel setup"); return bail(SBI_ECUDA); }
     int rc = init_group(c, g);
     if (rc) return bail(rc);
