@@ -15,4 +15,9 @@ cudaError_t launch_line(int nx, const LineParams& p, cudaStream_t st) {
   SBI_SWITCH(SBI_CASE)
 #undef SBI_CASE
 }
+cudaError_t line_clusters(int nx, int cluster, int* most) {
+#define SBI_CASE(N) case N: return pk::line_clusters_n<N>(cluster, most);
+  SBI_SWITCH(SBI_CASE)
+#undef SBI_CASE
+}
 }  // namespace sbi

@@ -96,6 +96,7 @@ constexpr bool line_pays(int nx, int n, bool variable_bottom) {
 }
 
 cudaError_t prepare_line_kernels(int nx);
+cudaError_t line_clusters(int nx, int cluster, int* most);   // after prepare_line_kernels
 cudaError_t launch_line(int nx, const LineParams& p, cudaStream_t st);
 
 }  // namespace sbi

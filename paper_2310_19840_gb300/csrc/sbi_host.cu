@@ -162,6 +162,7 @@ struct Group {
   std::map<std::string, void*> mixed;
   std::map<std::string, void*> tables;   // multiplier tables by key
   bool packed = false;          // runs on the packed kernels (packed_kernels.cuh): FP32, two-dimensional
+  std::map<int, int> line_clusters;   // clusters that run at once, by their number of blocks (line_clusters)
   bool line = false;            // runs on k_line (line.cuh): FP32, one-dimensional, not too many members
   size_t phys_elems() const { return (size_t)nx * ny; }
   // stored columns of a mixed field (tiles of four in a packed group)
@@ -2072,10 +2073,12 @@ int lower_line(sbi_ctx* c, const Group& g, std::vector<Pass>& ps, int m0, int m1
     Pass p{};
     p.kind = PK_LINE;
     p.nsize = g.nx;
-    // blocks per member: as many as the size can use, while every cluster has
-    // SMs of its own
+    // blocks per member: as many as the size can use, while every cluster of the
+    // group (its units run side by side) has SMs of its own; a launch takes 128 of
+    // them at most (76 members of 2048 points: 290 us a step on a block each, 328
+    // on two)
     int cluster = line_cluster(g.nx);
-    while (cluster > 1 && (m1 - m0) * cluster > 128) cluster /= 2;
+    while (cluster > 1 && (g.n > g.line_clusters.at(cluster) || (m1 - m0) * cluster > 128)) cluster /= 2;
     p.line = lb.launch;
     p.line.program = held->second.get();
     p.line.bytes = (int)program.size();
@@ -3152,6 +3155,8 @@ int create_impl(int n, const sbi_grid* grids, double gravity, const double* cons
     cudaError_t e = cudaSuccess;
     if (g.line) {
       e = prepare_line_kernels(g.nx);
+      for (int k = 2; k <= line_cluster(g.nx) && e == cudaSuccess; k *= 2)
+        e = line_clusters(g.nx, k, &g.line_clusters[k]);
     } else if (g.packed) {
       e = prepare_packed_row_kernels(g.nx);
       if (e == cudaSuccess) e = prepare_packed_col_kernels(g.ny);

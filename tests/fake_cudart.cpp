@@ -19,6 +19,8 @@ int launches = 0;          // kernels, those of graphs not among them
 int captured = 0;          // kernels of the last capture
 int overtaken = 0;         // kernels started beside unfinished work of the library's own stream
 cudaStream_t capturing = nullptr, own = nullptr;   // own: the stream that captures
+int cluster_size = 0;      // of the last launch that has one
+std::map<unsigned, int> max_clusters;
 dim3 cfg_grid, cfg_block;
 size_t cfg_smem;
 cudaStream_t cfg_stream;
@@ -70,6 +72,8 @@ size_t fake_live_bytes() {
 int fake_launches() { return launches; }
 int fake_captured() { return captured; }
 int fake_overtaken() { return overtaken; }
+int fake_cluster_size() { return cluster_size; }
+void fake_max_clusters(int size, int most) { max_clusters[size] = most; }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
   *p = malloc(n);
@@ -154,7 +158,16 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
   return cudaSuccess;
 }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) { return launch(c->stream); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) {
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster_size = (int)c->attrs[i].val.clusterDim.x;
+  return launch(c->stream);
+}
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* c) {
+  const unsigned k = c->attrs[0].val.clusterDim.x;
+  *n = max_clusters.count(k) ? max_clusters[k] : 152 / (int)k;
+  return cudaSuccess;
+}
 cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t s) { return launch(s); }
 cudaError_t cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t s) { return launch(s); }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void*) { return handle(k); }

@@ -143,3 +143,12 @@ def test_the_wide_default_of_a_column_pass_is_among_the_timed_shapes(host):
             seen.add(share)
     assert 2 in seen and max(seen) > 2
     ctx.close()
+
+
+@pytest.mark.parametrize("eights, size", [(16, 8), (15, 4)])
+def test_clusters_of_a_batch_run_at_once(host, eights, size):
+    host.fake.fake_max_clusters(8, eights)
+    ctx = host.Context([(4096, 1, 409.6, 1.0)] * 16, 9.81, None, h0=0.7, order=3, autotune=0)
+    ctx.step(0.01, 1)
+    assert host.fake.fake_cluster_size() == size
+    ctx.close()
