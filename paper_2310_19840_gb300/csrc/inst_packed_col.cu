@@ -16,20 +16,32 @@ cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st, bool 
   SBI_SWITCH(ny, SBI_CASE, cudaErrorInvalidValue)
 #undef SBI_CASE
 }
-int packed_col_geometry(int ny, int* tpc, int* group) {
+namespace {
+template <typename G>
+int geometry(int* tpc, int* group) {
+  *tpc = G::T;
+  *group = G::CI;
+  return G::CPB;
+}
+}  // namespace
+int packed_col_geometry(const ColParams& p, int* tpc, int* group) {
+  const int ny = p.ny;
+  const bool half = pk::col_half(p);
   *tpc = *group = 0;
-#define SBI_CASE(N) case N: *tpc = pk::ColGeo<N>::T; *group = pk::ColGeo<N>::CI; return pk::ColGeo<N>::CPB;
+#define SBI_CASE(N) \
+  case N: return half ? geometry<pk::ColGeo<N, true>>(tpc, group) : geometry<pk::ColGeo<N, false>>(tpc, group);
   SBI_SWITCH(ny, SBI_CASE, 0)
 #undef SBI_CASE
 }
 bool packed_col_stageable(int ny) {
-#define SBI_CASE(N) case N: return pk::ColGeo<N>::STAGEABLE;
+#define SBI_CASE(N) case N: return pk::ColGeo<N, true>::STAGEABLE;
   SBI_SWITCH(ny, SBI_CASE, false)
 #undef SBI_CASE
 }
 int packed_col_most_wide(const ColParams& p) {
   const int ny = p.ny;
-#define SBI_CASE(N) case N: return pk::col_most_wide<N>(p);
+  const bool half = pk::col_half(p);
+#define SBI_CASE(N) case N: return half ? pk::col_most_wide<N, true>(p) : pk::col_most_wide<N, false>(p);
   SBI_SWITCH(ny, SBI_CASE, 0)
 #undef SBI_CASE
 }

@@ -9,10 +9,11 @@
 // a complex product is two.  Half of the issue slots are left to everything
 // else.
 //
-// A transform of N elements by T = N / R threads holds R elements per thread
-// (16 from N = 128 up, else up to 8): one exchange through shared memory up to
-// N = R^2, two up to 2048.  Against 8 elements per thread that halves the
-// shared-memory traffic of a 256-point transform, which bounds the row passes.
+// A transform of N elements by T = N / R threads holds R elements per thread (16
+// in rows and most columns from N = 128 up, else up to 8): one exchange through
+// shared memory up to N = R^2, two up to 8 R^2, three up to 4096 with R = 8.
+// Against 8 elements per thread, 16 halve the shared-memory traffic of a
+// 256-point transform, which bounds the row passes.
 // Elements are in the order x[r] = a[j + r T] on entry and on exit.  An element
 // is one complex number (One) or two of independent sequences that share every
 // twiddle and index (Two).
@@ -227,7 +228,7 @@ template <typename V> struct PDft<16, V> {
 // ---------------------------------------------------------------------------
 template <typename V, int N, int R, bool WARP, int CI = 1>
 struct PackedFft {
-  static_assert(N % R == 0 && (R == 4 || R == 8 || R == 16) && N <= 8 * R * R, "length");
+  static_assert(N % R == 0 && (R == 4 || R == 8 || R == 16) && (N <= 8 * R * R || (R == 8 && N <= 4096)), "length");
   using M = Mem<V>;
   using E = typename M::T;
   static constexpr int T = N / R;
@@ -256,11 +257,31 @@ struct PackedFft {
   __device__ __forceinline__ static Twiddles twiddles(const float2* t, int j) {
     return Twiddles{t + (N <= R * R ? j : j & (R - 1))};
   }
+  // v[m] *= w^m, w = table[b]
+  template <int RP>
+  __device__ __forceinline__ static void times_powers(V (&v)[RP], const float2* __restrict__ table, int b) {
+    static_assert(RP == 2 || RP == 4 || RP == 8, "later passes of radix 2, 4 and 8");
+    const float2 w1 = __ldg(table + b);
+    v[1] = cmul(v[1], w1);
+    if constexpr (RP >= 4) {
+      const float2 w2 = RP == 4 ? __ldg(table + 2 * b) : wmul(w1, w1), w3 = wmul(w1, w2);
+      v[2] = cmul(v[2], w2);
+      v[3] = cmul(v[3], w3);
+      if constexpr (RP >= 8) {
+        const float2 w4 = __ldg(table + 4 * b);
+        v[4] = cmul(v[4], w4);
+        v[5] = cmul(v[5], wmul(w4, w1));
+        v[6] = cmul(v[6], wmul(w4, w2));
+        v[7] = cmul(v[7], wmul(w4, w3));
+      }
+    }
+  }
   // Butterflies b = j + q T (q < Q) of radix RP on elements v[m] = x[q + m Q].
-  // A third pass (512 elements and more) loads w_N^b and w_N^{4b} and forms the
-  // other powers by products.  With w_N^b itself a product, w_N^j e^{-2 pi i q / R},
-  // the powers carried its error up to three times: a step of a 4096 x 2048 sea
-  // was 1.39e-7 from the 64-bit one, and is 1.24e-7.
+  // A later pass (512 elements and more with 16 per thread, 128 with 8) loads w_N^b
+  // and w_N^{4b} (radix 4: w_N^{2b}) and forms the other powers by products.  With
+  // w_N^b itself a product, w_N^j e^{-2 pi i q / R}, the powers carried its error up
+  // to three times: a step of a 4096 x 2048 sea was 1.39e-7 from the 64-bit one, and
+  // is 1.24e-7.
   template <int RP, bool SECOND>
   __device__ __forceinline__ static void last_pass(V (&x)[R], int j, Twiddles t, const float2* __restrict__ tw) {
     constexpr int Q = R / RP;
@@ -273,21 +294,7 @@ struct PackedFft {
 #pragma unroll
         for (int m = 1; m < RP; ++m) v[m] = cmul(v[m], t(m, q));
       } else {
-        const float2 w1 = __ldg(tw + tw_off(N) + j + q * T);
-        v[1] = cmul(v[1], w1);
-        if constexpr (RP >= 4) {
-          const float2 w2 = wmul(w1, w1), w3 = wmul(w1, w2);
-          v[2] = cmul(v[2], w2);
-          v[3] = cmul(v[3], w3);
-          if constexpr (RP >= 8) {
-            static_assert(RP == 8, "third passes of radix 2, 4 and 8");
-            const float2 w4 = __ldg(tw + tw_off(N) + 4 * (j + q * T));
-            v[4] = cmul(v[4], w4);
-            v[5] = cmul(v[5], wmul(w4, w1));
-            v[6] = cmul(v[6], wmul(w4, w2));
-            v[7] = cmul(v[7], wmul(w4, w3));
-          }
-        }
+        times_powers<RP>(v, tw + tw_off(N), j + q * T);
       }
       PDft<RP, V>::run(v);
 #pragma unroll
@@ -323,7 +330,21 @@ struct PackedFft {
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = M::from(s[(rb + xpad(r * T)) * CI]);
         sync();
-        last_pass<N / (R * R), false>(x, j, t, tw);
+        if constexpr (N <= 8 * R * R) {
+          last_pass<N / (R * R), false>(x, j, t, tw);
+        } else {   // a third pass of radix 8, then the last
+          const int k3 = j & (R * R - 1);
+          times_powers<R>(x, tw + tw_off(R * R * R), k3);
+          PDft<R, V>::run(x);
+          const int sb3 = xpad((j - k3) * R) + xpad(k3);   // element (j - k3) R + k3 + r R^2
+#pragma unroll
+          for (int r = 0; r < R; ++r) s[(sb3 + xpad(r * R * R)) * CI] = M::to(x[r]);
+          sync();
+#pragma unroll
+          for (int r = 0; r < R; ++r) x[r] = M::from(s[(rb + xpad(r * T)) * CI]);
+          sync();
+          last_pass<N / (R * R * R), false>(x, j, t, tw);
+        }
       }
     }
   }

@@ -19,6 +19,8 @@
 // 32 512^2 members 4.33 ms instead of 6.03.
 #pragma once
 
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "packed.cuh"
 
@@ -719,7 +721,7 @@ k_packed_rk(const __grid_constant__ RkParams p) {
 // are kept: of each pair k, k + ny2 only one can be kept, known at compile time
 // per register (r < R / 2: mode k), so only that one is formed, summed and
 // transformed back, and the sums of both accumulators stay in registers.
-// Otherwise the sums of both modes are kept in shared memory.
+// Otherwise the sums of both modes are kept, with 8 elements per thread.
 // CI adjacent columns share a group of threads (lane = j CI + c), so that a
 // warp reads whole 64-byte (CI = 4) or 32-byte (CI = 2) runs.
 // Every input is copied ahead (cp.async) into the thread's own slots of shared
@@ -727,12 +729,16 @@ k_packed_rk(const __grid_constant__ RkParams p) {
 // input are loaded before its transform: with twelve warps per SM the loads
 // would otherwise take 40 % of the time.  No barrier is needed for either.
 // ===========================================================================
-template <int NY>
+// 16 elements per thread from 256 points up, except at 1024 points and for both
+// modes' sums: 8 there, twice the threads (a step of a 2048 x 1024 sea of order 5,
+// 1.12 -> 0.93 ms; 33 members of 256^2 with three quarters of the modes 1.17 ->
+// 0.87, eight of 512^2 1.23 -> 0.91).  LONE: the threads of a column by themselves.
+template <int NY, bool HALF, bool LONE = false>
 struct ColGeo {
   static constexpr int ny2 = NY / 2;
-  static constexpr int R = ny2 >= 128 ? 16 : (ny2 >= 8 ? 8 : 4);
+  static constexpr int R = HALF && (ny2 == 128 || ny2 == 256 || ny2 == 1024) ? 16 : (ny2 >= 8 ? 8 : 4);
   static constexpr int T = ny2 / R;
-  static constexpr int CI = T == 16 || T == 64 ? 2 : 4;
+  static constexpr int CI = LONE || T == 128 ? 1 : (T == 16 || T == 64 || (T == 32 && !HALF) ? 2 : 4);
   static constexpr int GT = T * CI;                       // threads per group
   static constexpr bool WARP = GT <= 32;
   static constexpr int THREADS = 128;
@@ -744,39 +750,24 @@ struct ColGeo {
   static constexpr int XLEN = F::xlen() * CI + (GT < 8 ? GT : 0);   // exchange elements per group
   static constexpr int CTW = (F::TW + 1) / 2;             // twiddles of a block, in elements of 16 bytes
   static constexpr bool STAGEABLE = NY >= 32;
-  // whether the inputs are copied ahead: beside sums kept in shared memory the
-  // slots would cost resident blocks
-  __host__ __device__ static constexpr bool ahead(int nacc, bool half) {
-    return half;
-  }
 };
-template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem(int groups, int nacc, bool half) {
-  using G = ColGeo<NY>;
-  return sizeof(typename G::E) *
-         ((size_t)G::CTW + (size_t)groups * G::XLEN + (half ? 0 : (size_t)nacc * G::R * groups * G::GT));
+template <int NY, bool HALF>
+__host__ __device__ constexpr size_t packed_col_smem(int groups) {
+  using G = ColGeo<NY, HALF>;
+  return sizeof(typename G::E) * ((size_t)G::CTW + (size_t)groups * G::XLEN);
 }
 // the form that copies its inputs ahead
-template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem_ahead(int groups, int nacc, bool half) {
-  using G = ColGeo<NY>;
-  return packed_col_smem<NY>(groups, nacc, half) +
-         (G::ahead(nacc, half) ? sizeof(typename G::E) * (size_t)G::R * groups * G::GT : 0);
+template <int NY, bool HALF>
+__host__ __device__ constexpr size_t packed_col_smem_ahead(int groups) {
+  using G = ColGeo<NY, HALF>;
+  return packed_col_smem<NY, HALF>(groups) + sizeof(typename G::E) * (size_t)G::R * groups * G::GT;
 }
 // The staged form adds, 128-byte aligned, the block's tiles of four columns
-// and one mbarrier per tile.  Where that does not fit (2048 points, two sums
-// in shared memory) the tile lands in the exchange buffer instead, once the
-// transform of the input before it is done.
-template <int NY>
-__host__ __device__ constexpr bool col_stage_in_exchange(int nacc, bool half) {
-  using G = ColGeo<NY>;
-  return !G::WARP &&
-         (packed_col_smem<NY>(G::SG, nacc, half) + 127) / 128 * 128 + (size_t)(G::SG * G::CI / 4) * (NY * 32 + 8) > 227 * 1024;
-}
-template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem_staged(int groups, int nacc, bool half) {
-  return (packed_col_smem<NY>(groups, nacc, half) + 127) / 128 * 128 +
-         (size_t)(groups * ColGeo<NY>::CI / 4) * ((col_stage_in_exchange<NY>(nacc, half) ? 0 : (size_t)NY * 32) + 8);
+// and one mbarrier per tile.
+template <int NY, bool HALF>
+__host__ __device__ constexpr size_t packed_col_smem_staged(int groups) {
+  return (packed_col_smem<NY, HALF>(groups) + 127) / 128 * 128 +
+         (size_t)(groups * ColGeo<NY, HALF>::CI / 4) * (NY * 32 + 8);
 }
 
 // a += v f i^q
@@ -792,10 +783,10 @@ __device__ __forceinline__ F2 conj_term(F2 v, float f, int q) {
 
 
 template <int NY, int NACC, bool HALF, bool STAGED>
-__global__ void __launch_bounds__(STAGED ? ColGeo<NY>::SG* ColGeo<NY>::GT : ColGeo<NY>::THREADS,
-                                  STAGED && ColGeo<NY>::SG > ColGeo<NY>::MAXG ? 1 : 3)
+__global__ void __launch_bounds__(STAGED ? ColGeo<NY, HALF>::SG* ColGeo<NY, HALF>::GT : ColGeo<NY, HALF>::THREADS,
+                                  STAGED && ColGeo<NY, HALF>::SG > ColGeo<NY, HALF>::MAXG ? 1 : 3)
 k_packed_col(const __grid_constant__ ColParams p) {
-  using G = ColGeo<NY>;
+  using G = ColGeo<NY, HALF>;
   using E = typename G::E;
   using M = Mem<Two>;
   constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2;
@@ -805,9 +796,7 @@ k_packed_col(const __grid_constant__ ColParams p) {
   const int g = threadIdx.x / GT, l = threadIdx.x % GT, c = l % CI, j = l / CI;
   const int groups = blockDim.x / GT;
   E* xs = sm + g * G::XLEN + c;
-  E* sacc = sm + groups * G::XLEN + threadIdx.x;   // not HALF: [acc][r][thread]
-  constexpr bool AHEAD = !STAGED && G::ahead(NACC, HALF);
-  E* own = sacc + (HALF ? 0 : NACC) * R * blockDim.x;   // AHEAD: the next input, [r][thread]
+  E* own = sm + groups * G::XLEN + threadIdx.x;   // not STAGED: the next input, [r][thread]
   const float2* tw = reinterpret_cast<const float2*>(p.tw);
   const int col = p.col_begin + ((int)blockIdx.x * groups + g) * CI + c;
   const bool valid = col < p.cols_total;
@@ -833,14 +822,12 @@ k_packed_col(const __grid_constant__ ColParams p) {
     }
     cp_async_commit();
   };
-  if (AHEAD && p.nin > 0) copy_ahead(0);
+  if (!STAGED && p.nin > 0) copy_ahead(0);
 
   // staged form: tiles of four columns (one contiguous run) and barriers
   E* stg = nullptr;
   unsigned long long* bar = nullptr;
   constexpr unsigned kTileBytes = 32u * NY;
-  constexpr bool IN_EXCHANGE = STAGED && col_stage_in_exchange<NY>(NACC, HALF);
-  static_assert(!IN_EXCHANGE || sizeof(E) * G::XLEN * (4 / G::CI) >= kTileBytes, "a tile in the exchange buffer");
   bool live = act, issuer = false;
   auto issue = [&](int i) {
     const char* src = reinterpret_cast<const char*>(reinterpret_cast<const float2*>(p.buf[i].ptr) +
@@ -852,9 +839,9 @@ k_packed_col(const __grid_constant__ ColParams p) {
   };
   if constexpr (STAGED) {
     const int tile = (g * CI + c) / 4, tiles = groups * CI / 4;
-    unsigned char* st0 = smem_raw + (packed_col_smem<NY>(groups, NACC, HALF) + 127) / 128 * 128;
-    stg = IN_EXCHANGE ? sm + (size_t)(tile * 4 / CI) * G::XLEN : reinterpret_cast<E*>(st0 + (size_t)tile * kTileBytes);
-    bar = reinterpret_cast<unsigned long long*>(st0 + (IN_EXCHANGE ? 0 : (size_t)tiles * kTileBytes)) + tile;
+    unsigned char* st0 = smem_raw + (packed_col_smem<NY, HALF>(groups) + 127) / 128 * 128;
+    stg = reinterpret_cast<E*>(st0 + (size_t)tile * kTileBytes);
+    bar = reinterpret_cast<unsigned long long*>(st0 + (size_t)tiles * kTileBytes) + tile;
     if (gave_up) live = false;
     issuer = (g * CI + c) % 4 == 0 && j == 0;
     if (issuer) {
@@ -867,23 +854,23 @@ k_packed_col(const __grid_constant__ ColParams p) {
     if (issuer && live && p.nin > 0) issue(0);
   }
 
-  F2 acc[HALF ? NACC : 1][HALF ? R : 1];
-  if constexpr (HALF) {
+  std::conditional_t<HALF, F2, Two> acc[NACC][R];
 #pragma unroll
-    for (int q = 0; q < NACC; ++q)
+  for (int q = 0; q < NACC; ++q)
 #pragma unroll
-      for (int r = 0; r < R; ++r) acc[q][r] = both(0.f);
-  } else {
-    for (int q = 0; q < NACC; ++q)
-#pragma unroll
-      for (int r = 0; r < R; ++r) sacc[(q * R + r) * blockDim.x] = make_ulonglong2(0, 0);
-  }
+    for (int r = 0; r < R; ++r) {
+      if constexpr (HALF) acc[q][r] = both(0.f);
+      else acc[q][r] = Two{both(0.f), both(0.f)};
+    }
 
-  float f[HALF ? R : 1];      // multipliers of a term (HALF)
+  float f[HALF ? R : 2 * R];      // multipliers of a term
   auto load_factors = [&](const ColTerm& m) {
     const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) f[r] = __ldg(tab + r * T * 4 + (r < R / 2 ? 0 : plane));
+    for (int r = 0; r < R; ++r) {
+      f[r] = __ldg(tab + r * T * 4 + (!HALF || r < R / 2 ? 0 : plane));
+      if constexpr (!HALF) f[R + r] = __ldg(tab + r * T * 4 + plane);
+    }
   };
   // inputs, then outputs: both directions go through one transform
 #pragma unroll 1
@@ -898,21 +885,15 @@ k_packed_col(const __grid_constant__ ColParams p) {
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = M::from(live ? stg[(j + r * T) * 4 + (kx & 3)] : make_ulonglong2(0, 0));
         __syncthreads();   // the staged tiles are read
-        if (!IN_EXCHANGE && issuer && live && i + 1 < p.nin) issue(i + 1);
-      } else if constexpr (AHEAD) {
+        if (issuer && live && i + 1 < p.nin) issue(i + 1);
+      } else {
         cp_async_wait_all();
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = M::from(act ? own[r * blockDim.x] : make_ulonglong2(0, 0));
         __syncwarp();      // the slots are read before they are filled again
         if (i + 1 < p.nin) copy_ahead(i + 1);
-      } else {
-        const E* src = field(p.buf[i]);
-#pragma unroll
-        for (int r = 0; r < R; ++r) x[r] = M::from(act ? src[r * T * 4] : make_ulonglong2(0, 0));
       }
-      if constexpr (HALF) {
-        if (p.term_begin[i] < p.term_begin[i + 1]) load_factors(p.terms[p.term_begin[i]]);
-      }
+      if (p.term_begin[i] < p.term_begin[i + 1]) load_factors(p.terms[p.term_begin[i]]);
     } else {
       // even samples from the sums of the modes k and k + ny2, odd ones from
       // their differences times w*; the inverse is the conjugate of the
@@ -928,7 +909,7 @@ k_packed_col(const __grid_constant__ ColParams p) {
           const F2 e = conj_term(NACC == 1 || m.acc == 0 ? acc[0][r] : acc[NACC - 1][r], f, ph);
           x[r] = Two{e, cmul(e, r < R / 2 ? w : make_float2(-w.x, -w.y))};
         } else {
-          const Two b = M::from(sacc[((m.acc ? R : 0) + r) * blockDim.x]);
+          const Two b = NACC == 1 || m.acc == 0 ? acc[0][r] : acc[NACC - 1][r];
           const F2 y0 = conj_term(b.a, __ldg(tab + r * T * 4), ph);
           const F2 y1 = conj_term(b.b, __ldg(tab + r * T * 4 + plane), ph);
           x[r] = Two{add(y0, y1), cmul(sub(y0, y1), w)};
@@ -937,9 +918,6 @@ k_packed_col(const __grid_constant__ ColParams p) {
     }
     G::F::run(x, xs, j, t, tw);
     if (forward) {
-      if constexpr (IN_EXCHANGE) {
-        if (issuer && live && i + 1 < p.nin) issue(i + 1);
-      }
       F2 v[HALF ? R : 1];
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -950,26 +928,17 @@ k_packed_col(const __grid_constant__ ColParams p) {
       }
       for (int q = p.term_begin[i]; q < p.term_begin[i + 1]; ++q) {
         const ColTerm m = p.terms[q];
-        const float* tab = reinterpret_cast<const float*>(m.tab) + at0;
         const int ph = (m.gx + m.gy) & 3;
-        if constexpr (HALF) {
-          if (q > p.term_begin[i]) load_factors(m);
-          if (NACC == 1 || m.acc == 0) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[0][r] = acc_term(acc[0][r], v[r], f[r], ph);
-          } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[NACC - 1][r] = acc_term(acc[NACC - 1][r], v[r], f[r], ph);
-          }
-        } else {
-          E* a = sacc + (m.acc ? R : 0) * blockDim.x;
+        if (q > p.term_begin[i]) load_factors(m);
+        auto sum = [&](auto& a) {
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            const Two b = M::from(a[r * blockDim.x]);
-            a[r * blockDim.x] = M::to(Two{acc_term(b.a, x[r].a, __ldg(tab + r * T * 4), ph),
-                                          acc_term(b.b, x[r].b, __ldg(tab + r * T * 4 + plane), ph)});
+            if constexpr (HALF) a[r] = acc_term(a[r], v[r], f[r], ph);
+            else a[r] = Two{acc_term(a[r].a, x[r].a, f[r], ph), acc_term(a[r].b, x[r].b, f[R + r], ph)};
           }
-        }
+        };
+        if (NACC == 1 || m.acc == 0) sum(acc[0]);
+        else sum(acc[NACC - 1]);
       }
       continue;
     }
@@ -1006,29 +975,30 @@ __device__ __forceinline__ void copy_float_ahead(float* dst_smem, const float* s
 // A pass of eight inputs and one output then takes the time of two transforms
 // instead of nine.  Column passes of one 512^2 member: 0.38 ms a step (0.58 in
 // the plain form; 0.44 with the multipliers loaded where they are used).
-template <int NY>
+// Columns of 1024 and 2048 points stand alone here, on twice the blocks: a step of a
+// 256 x 2048 sea of order 5 0.65 -> 0.47 ms, of 256 x 1024 0.57 -> 0.39.
+template <int NY, bool HALF>
 struct WideGeo {
-  using G = ColGeo<NY>;
+  using G = ColGeo<NY, HALF, ColGeo<NY, HALF>::T == 64>;
   static constexpr int SET = G::WARP ? 32 : G::GT;      // threads of one copy
   static constexpr int COLS = G::CI * (SET / G::GT);    // columns of a block
   static constexpr int SX = G::XLEN * (SET / G::GT);    // exchange elements of one copy
 };
-template <int NY>
-__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nterms, int nacc, int npass,
-                                                          bool half) {
-  using G = ColGeo<NY>;
-  using H = WideGeo<NY>;
-  const size_t NM = (half ? 1 : 2) * G::R;
+template <int NY, bool HALF>
+__host__ __device__ constexpr size_t packed_col_smem_wide(int copies, int nin, int nterms, int nacc, int npass) {
+  using H = WideGeo<NY, HALF>;
+  using G = typename H::G;
+  const size_t NM = (HALF ? 1 : 2) * G::R;
   const size_t modes = (8 * (size_t)nin + 4 * (size_t)nterms) * NM * H::SET, pass = 16 * (size_t)npass * G::R * H::SET;
   return 16 * ((size_t)G::CTW + (size_t)copies * H::SX) + 8 * (size_t)nacc * NM * H::SET + (modes > pass ? modes : pass);
 }
 // A thread's modes: HALF the R that can be kept (j + r T, from r = R / 2 on plus
 // NY / 2), else j + r T and, from R on, those plus NY / 2.
 template <int NY, bool HALF>
-__global__ void __launch_bounds__(WideGeo<NY>::G::WARP ? 256 : 512)
+__global__ void __launch_bounds__(WideGeo<NY, HALF>::G::WARP ? 256 : 512)
 k_packed_col_wide(const __grid_constant__ ColParams p) {
-  using G = ColGeo<NY>;
-  using H = WideGeo<NY>;
+  using H = WideGeo<NY, HALF>;
+  using G = typename H::G;
   using E = typename G::E;
   using M = Mem<Two>;
   constexpr int R = G::R, T = G::T, CI = G::CI, GT = G::GT, ny2 = G::ny2, SET = H::SET;
@@ -1290,31 +1260,30 @@ inline bool col_half(const ColParams& p) {
   return half;
 }
 // largest number of copies the wide form of a pass can take (0: none)
-template <int NY>
+template <int NY, bool HALF>
 int col_most_wide(const ColParams& p) {
   if (p.staged) return 0;
-  const bool half = col_half(p);
-  const int most = (ColGeo<NY>::WARP ? 256 : 512) / WideGeo<NY>::SET;
+  const int most = (ColGeo<NY, HALF>::WARP ? 256 : 512) / WideGeo<NY, HALF>::SET;
   for (int k = most; k >= 2; k /= 2)
-    if (packed_col_smem_wide<NY>(k, p.nin, p.nterms, p.nacc, p.npass, half) <= 227 * 1024) return k;
+    if (packed_col_smem_wide<NY, HALF>(k, p.nin, p.nterms, p.nacc, p.npass) <= 227 * 1024) return k;
   return 0;
 }
 
 template <int NY, int NACC, bool HALF>
 cudaError_t launch_packed_col_a(const ColParams& p, int groups, unsigned blocks, cudaStream_t st, bool chained) {
-  using G = ColGeo<NY>;
+  using G = ColGeo<NY, HALF>;
   if (!p.staged)
     return launch(k_packed_col<NY, NACC, HALF, false>, blocks, groups * G::GT,
-                  packed_col_smem_ahead<NY>(groups, NACC, HALF), st, chained, p);
+                  packed_col_smem_ahead<NY, HALF>(groups), st, chained, p);
   if constexpr (G::STAGEABLE)
     return launch(k_packed_col<NY, NACC, HALF, true>, blocks, groups * G::GT,
-                  packed_col_smem_staged<NY>(groups, NACC, HALF), st, chained, p);
+                  packed_col_smem_staged<NY, HALF>(groups), st, chained, p);
   return cudaErrorInvalidValue;
 }
 
-template <int NY>
-cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st, bool chained) {
-  using G = ColGeo<NY>;
+template <int NY, bool HALF>
+cudaError_t launch_packed_col_h(const ColParams& p, cudaStream_t st, bool chained) {
+  using G = ColGeo<NY, HALF>;
   const int most = p.staged ? G::SG : G::MAXG;
   const int cpb = p.cpb > 0 ? p.cpb : most * G::CI;
   const int groups = cpb / G::CI;
@@ -1323,19 +1292,19 @@ cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st, bool chaine
       p.nacc > kMaxColAcc)
     return cudaErrorInvalidValue;
   const unsigned blocks = (unsigned)((p.cols_total - p.col_begin + cpb - 1) / cpb);
-  const bool half = col_half(p);
   if (p.wide > 0) {
-    using H = WideGeo<NY>;
-    const size_t smem = packed_col_smem_wide<NY>(p.wide, p.nin, p.nterms, p.nacc, p.npass, half);
+    using H = WideGeo<NY, HALF>;
+    const size_t smem = packed_col_smem_wide<NY, HALF>(p.wide, p.nin, p.nterms, p.nacc, p.npass);
     if (p.staged || p.wide * H::SET > (G::WARP ? 256 : 512) || smem > 227 * 1024) return cudaErrorInvalidValue;
     const unsigned wb = (unsigned)((p.cols_total - p.col_begin + H::COLS - 1) / H::COLS);
-    return launch(half ? k_packed_col_wide<NY, true> : k_packed_col_wide<NY, false>, wb, p.wide * H::SET, smem, st, chained, p);
+    return launch(k_packed_col_wide<NY, HALF>, wb, p.wide * H::SET, smem, st, chained, p);
   }
-  if (p.nacc == 1)
-    return half ? launch_packed_col_a<NY, 1, true>(p, groups, blocks, st, chained)
-                : launch_packed_col_a<NY, 1, false>(p, groups, blocks, st, chained);
-  return half ? launch_packed_col_a<NY, 2, true>(p, groups, blocks, st, chained)
-              : launch_packed_col_a<NY, 2, false>(p, groups, blocks, st, chained);
+  return p.nacc == 1 ? launch_packed_col_a<NY, 1, HALF>(p, groups, blocks, st, chained)
+                     : launch_packed_col_a<NY, 2, HALF>(p, groups, blocks, st, chained);
+}
+template <int NY>
+cudaError_t launch_packed_col_n(const ColParams& p, cudaStream_t st, bool chained) {
+  return col_half(p) ? launch_packed_col_h<NY, true>(p, st, chained) : launch_packed_col_h<NY, false>(p, st, chained);
 }
 
 template <typename K>
@@ -1359,11 +1328,11 @@ cudaError_t prepare_packed_row_n() {
 }
 template <int NY, int NACC, bool HALF>
 cudaError_t prepare_packed_col_a() {
-  using G = ColGeo<NY>;
-  cudaError_t e = allow_smem(k_packed_col<NY, NACC, HALF, false>, packed_col_smem_ahead<NY>(G::MAXG, NACC, HALF));
+  using G = ColGeo<NY, HALF>;
+  cudaError_t e = allow_smem(k_packed_col<NY, NACC, HALF, false>, packed_col_smem_ahead<NY, HALF>(G::MAXG));
   if constexpr (G::STAGEABLE) {
     if (e == cudaSuccess)
-      e = allow_smem(k_packed_col<NY, NACC, HALF, true>, packed_col_smem_staged<NY>(G::SG, NACC, HALF));
+      e = allow_smem(k_packed_col<NY, NACC, HALF, true>, packed_col_smem_staged<NY, HALF>(G::SG));
   }
   return e;
 }

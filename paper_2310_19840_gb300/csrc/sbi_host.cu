@@ -543,7 +543,7 @@ struct Planner {
   int default_wide(const ColParams& p) const {
     const int most = packed_col_most_wide(p);
     int tpc = 0, group = 1;
-    packed_col_geometry(g.ny, &tpc, &group);
+    packed_col_geometry(p, &tpc, &group);
     const double warps = (double)p.cols_total * tpc / 32.0;
     if (most < 2 || warps * 3 > 152.0 * 8.0) return 0;
     int k = 2;
@@ -1680,7 +1680,7 @@ bool chainable(const Pass& p) {
     packed_row_geometry(p.nsize, &t);
     threads = 2.0 * (p.rk.rows_total - p.rk.row_begin) * t;
   } else if (p.kind == PK_COL && p.col.packed) {
-    packed_col_geometry(p.nsize, &t, &group);
+    packed_col_geometry(p.col, &t, &group);
     threads = (double)(p.col.cols_total - p.col.col_begin) * t * std::max(p.col.wide, 1);
   } else {
     return false;
@@ -2230,7 +2230,7 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     if (p.row.split) cand.push_back(p.row.rpc);
   } else {
     int tpc = 0, group = 1;
-    const int cpb = p.col.packed ? packed_col_geometry(p.nsize, &tpc, &group)
+    const int cpb = p.col.packed ? packed_col_geometry(p.col, &tpc, &group)
                                : (c->fp64 ? col_geometry<double>(p.nsize, &tpc) : col_geometry<float>(p.nsize, &tpc));
     // the staged form of a packed group takes whole tiles of four columns
     auto base = [&](int staged) {

@@ -230,7 +230,7 @@ cudaError_t launch_packed_row(int nx, const RowParams& p, cudaStream_t st, bool 
 cudaError_t launch_packed_rk(int nx, const RkParams& p, cudaStream_t st, bool chained);
 cudaError_t launch_packed_col(int ny, const ColParams& p, cudaStream_t st, bool chained);
 int packed_row_geometry(int nx, int* threads);
-int packed_col_geometry(int ny, int* tpc, int* group);
+int packed_col_geometry(const ColParams& p, int* tpc, int* group);
 bool packed_col_stageable(int ny);
 int packed_col_most_wide(const ColParams& p);   // most copies of the wide form (0: not possible)
 
