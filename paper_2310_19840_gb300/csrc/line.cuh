@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line(const __grid_constant_
           }
         } else {
           One X[kKept<NX, EXACT>];
-          kept_modes<NX, EXACT>(x, X, W, j, xs, t);
+          share_modes<NX, EXACT>(x, W, j, xs);
+          kept_modes<NX, EXACT>(x, X, 0, W, j, xs, t);
           if (valid) {
             F2* out = mixed(job.buf) + j;
 #pragma unroll

@@ -145,70 +145,121 @@ __device__ __forceinline__ float2* real_row(const BufRef& b, const Row& w, int n
 // X[k] (1 + i w) for k < W, X[n - k]* (1 - i w) for k > n - W, w = e^{2 pi i k / NX}
 // (both terms where more than half of the modes are kept).  The inverse of Z
 // is taken as the conjugate of the transform of its conjugate: x = Z*.
-// EXACT: W = n / 2 (half of the modes, the default), every bound known at
-// compile time.  In that form load_modes runs ahead of the products.
-template <int NX, bool EXACT>
-inline constexpr bool kFastRow = EXACT && RowGeo<NX>::T >= 4;
+// The forms of a row by its width: half of the modes kept (W = n / 2, the default,
+// every bound known at compile time), fewer, more, or any of these.  In all but
+// the last load_modes brings each element's first term, X[k] for r < R / 2 and
+// X[n - k] above, and with more than half more_modes adds the second ones.
+enum RowForm : int { kAnyWidth = 0, kHalf = 1, kNarrow = 2, kBroad = 3 };
+template <int NX, int FORM>
+inline constexpr bool kFastRow = FORM != kAnyWidth && RowGeo<NX>::T >= 4;
+template <int NX, int FORM>
+inline constexpr bool kEveryMode = kFastRow<NX, FORM> && FORM == kHalf;   // no test against W
 
-template <int NX>
+// whether the first term of element r is a kept mode
+template <int NX, int FORM>
+__device__ __forceinline__ bool first_kept(int r, int W, int j) {
+  constexpr int R = RowGeo<NX>::R, T = RowGeo<NX>::T;
+  if (FORM == kNarrow) return (r < R / 2 ? j + r * T : T - j + (R - 1 - r) * T) < W;
+  return FORM == kBroad || r != R / 2 || j != 0;      // kHalf: mode n / 2 is not
+}
+// AHEAD: the loads of the first buffer stand by themselves
+template <int NX, int FORM, bool AHEAD>
 __device__ __forceinline__ void load_modes(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
-                                           int j) {
+                                           int W, int j) {
   constexpr int R = RowGeo<NX>::R, T = RowGeo<NX>::T;
   // k = j + r T: X[k] at lo + r step for r < R / 2; n - k = T - j + (R - 1 - r) T
   const int step = T * ny;
   const long long lo = mode_at(j, ny), hi = mode_at(T - j, ny);
-  const unsigned long long* src = mixed_row(bufs[0], w);
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    x[r].v = 0;
-    if (r < R / 2) x[r].v = src[lo + r * step];
-    else if (r > R / 2 || j != 0) x[r].v = src[hi + (R - 1 - r) * step];
-  }
-#pragma unroll 1
-  for (int q = 1; q < nb; ++q) {
-    src = mixed_row(bufs[q], w);
+  if constexpr (AHEAD) {
+    const unsigned long long* src = mixed_row(bufs[0], w);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      if (r < R / 2) x[r] = add(x[r], One{src[lo + r * step]});
-      else if (r > R / 2 || j != 0) x[r] = add(x[r], One{src[hi + (R - 1 - r) * step]});
+      x[r].v = 0;
+      if (r < R / 2 && first_kept<NX, FORM>(r, W, j)) x[r].v = src[lo + r * step];
+      else if (r >= R / 2 && first_kept<NX, FORM>(r, W, j)) x[r].v = src[hi + (R - 1 - r) * step];
     }
-  }
-}
-template <int NX>
-__device__ __forceinline__ void twist_modes(One (&x)[RowGeo<NX>::R], const RowTwiddles<NX>& t) {
-  constexpr int R = RowGeo<NX>::R;
+#pragma unroll 1
+    for (int q = 1; q < nb; ++q) {
+      src = mixed_row(bufs[q], w);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    if (r < R / 2) {   // conj(X (1 + i w)), 1 + i w = (1 + e.y, e.x) with e = w*
-      const float2 e = t.lower(r);
-      const float f = 1.f + e.y;
-      x[r] = fma(both(-e.x), swp(x[r]), mul(f2(f, -f), x[r]));
-    } else {           // X (1 - i w)*, 1 - i w = (1 - e.y, -e.x)
-      const float2 e = t.upper(r);
-      x[r] = cmul(x[r], make_float2(1.f - e.y, e.x));
+      for (int r = 0; r < R; ++r) {
+        if (r < R / 2 && first_kept<NX, FORM>(r, W, j)) x[r] = add(x[r], One{src[lo + r * step]});
+        else if (r >= R / 2 && first_kept<NX, FORM>(r, W, j)) x[r] = add(x[r], One{src[hi + (R - 1 - r) * step]});
+      }
     }
-  }
-}
-template <int NX, bool EXACT>
-__device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
-                                              int W, int j, const RowTwiddles<NX>& t) {
-  using G = RowGeo<NX>;
-  constexpr int n = G::n, R = G::R, T = G::T;
-  if constexpr (kFastRow<NX, EXACT>) {
-    const int step = T * ny;
-    const long long lo = mode_at(j, ny), hi = mode_at(T - j, ny);
+  } else {
 #pragma unroll 1
     for (int q = 0; q < nb; ++q) {
       const unsigned long long* src = mixed_row(bufs[q], w);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         One v = both(0.f);
-        if (r < R / 2) v.v = src[lo + r * step];
-        else if (r > R / 2 || j != 0) v.v = src[hi + (R - 1 - r) * step];
+        if (r < R / 2 && first_kept<NX, FORM>(r, W, j)) v.v = src[lo + r * step];
+        else if (r >= R / 2 && first_kept<NX, FORM>(r, W, j)) v.v = src[hi + (R - 1 - r) * step];
         x[r] = q == 0 ? v : add(x[r], v);
       }
     }
-    twist_modes<NX>(x, t);
+  }
+}
+// conj(X (1 + i w)), 1 + i w = (1 + e.y, e.x) with e = w*
+__device__ __forceinline__ One twist_low(One x, float2 e) {
+  const float f = 1.f + e.y;
+  return fma(both(-e.x), swp(x), mul(f2(f, -f), x));
+}
+// X (1 - i w)*, 1 - i w = (1 - e.y, -e.x)
+__device__ __forceinline__ One twist_high(One x, float2 e) { return cmul(x, make_float2(1.f - e.y, e.x)); }
+template <int NX>
+__device__ __forceinline__ void twist_modes(One (&x)[RowGeo<NX>::R], const RowTwiddles<NX>& t) {
+  constexpr int R = RowGeo<NX>::R;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (r < R / 2) x[r] = twist_low(x[r], t.lower(r));
+    else x[r] = twist_high(x[r], t.upper(r));
+  }
+}
+// The same for kBroad with the second terms, X[n - k] for r < R / 2 and X[k] above,
+// eight elements at a time, each twiddle used for both.  (With both terms of an
+// element loaded side by side the rows spilled 200 bytes per thread from 256
+// points up.)
+template <int NX>
+__device__ __forceinline__ void add_second_modes(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
+                                           int W, int j, const RowTwiddles<NX>& t) {
+  constexpr int R = RowGeo<NX>::R, T = RowGeo<NX>::T, B = 8;
+  const int step = T * ny;
+  const long long lo = mode_at(j, ny), hi = mode_at(T - j, ny);
+#pragma unroll
+  for (int r0 = 0; r0 < R; r0 += B) {
+    One v[B];
+#pragma unroll
+    for (int i = 0; i < B; ++i) v[i] = both(0.f);
+#pragma unroll 1
+    for (int q = 0; q < nb; ++q) {
+      const unsigned long long* src = mixed_row(bufs[q], w);
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        const int r = r0 + i;
+        const bool kept = (r < R / 2 ? T - j + (R - 1 - r) * T : j + r * T) < W;
+        const One u{kept ? src[r < R / 2 ? hi + (R - 1 - r) * step : lo + r * step] : 0ull};
+        v[i] = q == 0 ? u : add(v[i], u);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const int r = r0 + i;
+      const float2 e = r < R / 2 ? t.lower(r) : t.any(r);
+      x[r] = r < R / 2 ? add(twist_low(x[r], e), twist_high(v[i], e)) : add(twist_high(x[r], e), twist_low(v[i], e));
+    }
+  }
+}
+template <int NX, int FORM>
+__device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const BufRef* bufs, int nb, const Row& w, int ny,
+                                              int W, int j, const RowTwiddles<NX>& t) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
+  if constexpr (kFastRow<NX, FORM>) {
+    load_modes<NX, FORM, false>(x, bufs, nb, w, ny, W, j);
+    if constexpr (FORM == kBroad) add_second_modes<NX>(x, bufs, nb, w, ny, W, j, t);
+    else twist_modes<NX>(x, t);
   } else {
     // eight elements at a time: sixteen loads without a branch between them (one
     // after the other they made this form two to three times as slow)
@@ -250,25 +301,32 @@ __device__ __forceinline__ void inverse_input(One (&x)[RowGeo<NX>::R], const Buf
 // k = j + r T < W.  Z[n - k] sits in lane (T - j) mod T, register R - 1 - r
 // (thread 0: its own register (R - r) mod R): a shuffle, or, for rows of
 // several warps, a pass through the exchange buffer.
-template <int NX, bool EXACT>
-inline constexpr int kKept = kFastRow<NX, EXACT> ? RowGeo<NX>::R / 2 : RowGeo<NX>::R;
+// Modes first .. first + COUNT - 1 of a thread's R; where the threads of a row
+// share the exchange buffer share_modes goes before.
+template <int NX, int FORM>
+inline constexpr int kKept = kFastRow<NX, FORM> && FORM != kBroad ? RowGeo<NX>::R / 2 : RowGeo<NX>::R;
 
-template <int NX, bool EXACT>
-__device__ __forceinline__ void kept_modes(const One (&x)[RowGeo<NX>::R], One (&X)[kKept<NX, EXACT>], int W, int j,
-                                           typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
+template <int NX, int FORM>
+__device__ __forceinline__ void share_modes(const One (&x)[RowGeo<NX>::R], int W, int j, typename RowGeo<NX>::E* xs) {
   using G = RowGeo<NX>;
   constexpr int n = G::n, R = G::R, T = G::T;
-  constexpr bool FAST = kFastRow<NX, EXACT>;
   if constexpr (!G::WARP) {
     // Z[n - k] of the kept modes: the elements above n - W, and Z[0]
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      if (r == 0 || (FAST ? r >= R / 2 : (r + 1) * T > n - W)) xs[j + r * T] = x[r].v;
+      if (r == 0 || (kKept<NX, FORM> < R ? r >= R / 2 : (r + 1) * T > n - W)) xs[j + r * T] = x[r].v;
     __syncthreads();
   }
+}
+template <int NX, int FORM, int COUNT>
+__device__ __forceinline__ void kept_modes(const One (&x)[RowGeo<NX>::R], One (&X)[COUNT], int first, int W, int j,
+                                           const typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
+  using G = RowGeo<NX>;
+  constexpr int n = G::n, R = G::R, T = G::T;
 #pragma unroll
-  for (int r = 0; r < kKept<NX, EXACT>; ++r) {
-    if (!FAST && r * T >= W) break;
+  for (int i = 0; i < COUNT; ++i) {
+    const int r = first + i;
+    if (!kEveryMode<NX, FORM> && r * T >= W) break;
     const int k = j + r * T;
     One zc;
     if constexpr (!G::WARP) {
@@ -282,26 +340,32 @@ __device__ __forceinline__ void kept_modes(const One (&x)[RowGeo<NX>::R], One (&
         if (j != 0) zc = o;
       }
     }
-    const float2 e = FAST ? t.lower(r) : t.any(r);
+    const float2 e = kFastRow<NX, FORM> && r < R / 2 ? t.lower(r) : t.any(r);
     const One d = cmul(sub_conj(x[r], zc), e);
-    X[r] = scale(0.5f, subi(add_conj(x[r], zc), d));
+    X[i] = scale(0.5f, subi(add_conj(x[r], zc), d));
   }
 }
-template <int NX, bool EXACT>
+template <int NX, int FORM>
 __device__ __forceinline__ void store_modes(const One (&x)[RowGeo<NX>::R], const BufRef& dst, const Row& w, int ny,
                                             int W, int j, typename RowGeo<NX>::E* xs, const RowTwiddles<NX>& t) {
   using G = RowGeo<NX>;
-  constexpr bool FAST = kFastRow<NX, EXACT>;
-  One X[kKept<NX, EXACT>];
-  kept_modes<NX, EXACT>(x, X, W, j, xs, t);
+  constexpr bool FAST = kFastRow<NX, FORM>;
+  constexpr int KEPT = kKept<NX, FORM>, PART = G::R / 2;     // half of them at a time: registers
+  share_modes<NX, FORM>(x, W, j, xs);
   unsigned long long* out = const_cast<unsigned long long*>(mixed_row(dst, w));
   const int step = G::T * ny;
   if (FAST) out += mode_at(j, ny);
-  if (w.act) {
 #pragma unroll
-    for (int r = 0; r < kKept<NX, EXACT>; ++r) {
-      if (FAST) out[r * step] = X[r].v;
-      else if (j + r * G::T < W) out[mode_at(j + r * G::T, ny)] = X[r].v;
+  for (int first = 0; first < KEPT; first += PART) {
+    One X[PART];
+    kept_modes<NX, FORM>(x, X, first, W, j, xs, t);
+    if (w.act) {
+#pragma unroll
+      for (int i = 0; i < PART; ++i) {
+        const int r = first + i;
+        if (!kEveryMode<NX, FORM> && j + r * G::T >= W) continue;
+        out[FAST ? r * step : mode_at(j + r * G::T, ny)] = X[i].v;
+      }
     }
   }
   if constexpr (!G::WARP) __syncthreads();
@@ -322,9 +386,12 @@ __device__ __forceinline__ void times_field(One (&v)[R], const One (&f)[R], int 
 // chain (the inverse transform and the products before them are then formed
 // again without being transformed, in the same order and so with the same
 // bits), which spreads a pass over few rows across the SMs.  Both directions
-// go through the one transform of the loop (instruction cache).
-template <int NX, bool EXACT>
-__global__ void __launch_bounds__(RowGeo<NX>::THREADS, 4)
+// go through the one transform of the loop (instruction cache).  Rows of more than
+// half of the modes are compiled for three blocks per SM: with four they spill 96
+// bytes per thread (33 members of 256^2, three quarters of the modes, 950 us a step
+// of order 5; with three 854).
+template <int NX, int FORM>
+__global__ void __launch_bounds__(RowGeo<NX>::THREADS, FORM == kBroad ? 3 : 4)
 k_packed_row(const __grid_constant__ RowParams p) {
   using G = RowGeo<NX>;
   constexpr int n = G::n, R = G::R, T = G::T;
@@ -352,7 +419,7 @@ k_packed_row(const __grid_constant__ RowParams p) {
     const RowOp op = p.ops[o];
     const bool inverse = op.kind == ROP_C2R;
     if (inverse) {
-      inverse_input<NX, EXACT>(x, p.buf + op.a, op.b, w, ny, p.W, j, t);
+      inverse_input<NX, FORM>(x, p.buf + op.a, op.b, w, ny, p.W, j, t);
     } else {
       const bool running = (op.c & 2) != 0;
       if (o < first && !running) continue;
@@ -388,7 +455,7 @@ k_packed_row(const __grid_constant__ RowParams p) {
         for (int r = 0; r < R; ++r) out[r * T] = parts(run[r]);
       }
     } else {
-      store_modes<NX, EXACT>(x, p.buf[op.dst], w, ny, p.W, j, xs, t);
+      store_modes<NX, FORM>(x, p.buf[op.dst], w, ny, p.W, j, xs, t);
     }
   }
 }
@@ -410,7 +477,7 @@ __device__ __forceinline__ F2 quotient(F2 a, F2 d) {
   const float2 p = parts(a), q = parts(d);
   return f2(__fdiv_rn(p.x, q.x), __fdiv_rn(p.y, q.y));
 }
-template <int NX, bool EXACT>
+template <int NX, int FORM>
 __global__ void __launch_bounds__(RowGeo<NX>::THREADS, 3)
 k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
   using G = RowGeo<NX>;
@@ -432,10 +499,11 @@ k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
   for (int r = 0; r < R; ++r) e[r] = both(0.f);
   // steps 0..4: the inverse transforms; the forward ones follow the step that
   // forms their field.  One transform in the loop serves both.
-  constexpr bool AHEAD = kFastRow<NX, EXACT>;
+  constexpr bool AHEAD = kFastRow<NX, FORM> && FORM != kBroad;
   One next[AHEAD ? R : 1];
   auto load_ahead = [&](int step) {
-    if constexpr (AHEAD) load_modes<NX>(next, p.buf + p.ops[q.src[step]].a, p.ops[q.src[step]].b, w, ny, j);
+    if constexpr (AHEAD)
+      load_modes<NX, FORM, true>(next, p.buf + p.ops[q.src[step]].a, p.ops[q.src[step]].b, w, ny, p.W, j);
   };
   load_ahead(0);
   int s = 0, dst = -1;
@@ -451,12 +519,12 @@ k_packed_rhs(const __grid_constant__ RowParams p, const RhsOps q) {
         twist_modes<NX>(x, t);
         if (s < 4) load_ahead(s + 1);
       } else {
-        inverse_input<NX, EXACT>(x, p.buf + c.a, c.b, w, ny, p.W, j, t);
+        inverse_input<NX, FORM>(x, p.buf + c.a, c.b, w, ny, p.W, j, t);
       }
     }
     t.run(x, xs);
     if (forward) {
-      store_modes<NX, EXACT>(x, p.buf[dst], w, ny, p.W, j, xs, t);
+      store_modes<NX, FORM>(x, p.buf[dst], w, ny, p.W, j, xs, t);
       dst = -1;
       if (s == 5) return;
       continue;
@@ -543,7 +611,7 @@ __host__ __device__ constexpr size_t row_smem_wide() {
   using H = WideRow<NX>;
   return 8 * ((size_t)G::RTW + 5 * (size_t)H::ROWS * (G::XLEN + G::n));
 }
-template <int NX, bool EXACT>
+template <int NX, int FORM>
 __global__ void __launch_bounds__(5 * WideRow<NX>::SET)
 k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
   using G = RowGeo<NX>;
@@ -565,7 +633,7 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
   if (w.act && p.active) w.act = p.active[p.member0 + w.member] != 0;
   One x[R];
   const RowOp c = p.ops[q.src[copy]];
-  inverse_input<NX, EXACT>(x, p.buf + c.a, c.b, w, p.ny, p.W, j, t);
+  inverse_input<NX, FORM>(x, p.buf + c.a, c.b, w, p.ny, p.W, j, t);
   t.run(x, xs);
 #pragma unroll
   for (int r = 0; r < R; ++r) S(copy, r) = x[r] = conj(x[r]);
@@ -614,7 +682,7 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
   if (G::WARP && dst < 0) return;            // the whole warp
   t.run(x, xs);
   if (dst < 0) w.act = false;
-  store_modes<NX, EXACT>(x, p.buf[dst < 0 ? 0 : dst], w, p.ny, p.W, j, xs, t);
+  store_modes<NX, FORM>(x, p.buf[dst < 0 ? 0 : dst], w, p.ny, p.W, j, xs, t);
 }
 
 // ===========================================================================
@@ -623,7 +691,7 @@ k_packed_rhs_wide(const __grid_constant__ RowParams p, const RhsOps q) {
 // memory: a third of the crossing-sea batch of 96 members in 42 us per launch
 // (60 before), 5.4 TB/s of the bytes it cannot do without.
 // ===========================================================================
-template <int NX, bool EXACT, typename S>
+template <int NX, int FORM, typename S>
 __global__ void __launch_bounds__(RowGeo<NX>::THREADS, 5)
 k_packed_rk(const __grid_constant__ RkParams p) {
   using G = RowGeo<NX>;
@@ -650,7 +718,7 @@ k_packed_rk(const __grid_constant__ RkParams p) {
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = f2(v[r * T]);
   } else if (p.mode != RK_ENTRY) {
-    inverse_input<NX, EXACT>(x, potential && p.mode != RK_STAGE ? &p.corr_phi : &p.phit, 1, w, ny, p.W, j, t);
+    inverse_input<NX, FORM>(x, potential && p.mode != RK_STAGE ? &p.corr_phi : &p.phit, 1, w, ny, p.W, j, t);
     t.run(x, xs);
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = conj(x[r]);
@@ -710,7 +778,7 @@ k_packed_rk(const __grid_constant__ RkParams p) {
     for (int r = 0; r < R; ++r) ew[r * T] = parts(x[r]);
   }
   t.run(x, xs);
-  store_modes<NX, EXACT>(x, potential ? p.phi_hat : p.eta_hat, w, ny, p.W, j, xs, t);
+  store_modes<NX, FORM>(x, potential ? p.phi_hat : p.eta_hat, w, ny, p.W, j, xs, t);
 }
 
 // ===========================================================================
@@ -1210,6 +1278,15 @@ inline bool rhs_ops(const RowParams& p, RhsOps* q) {
   return true;
 }
 
+// calls f with the form of rows that keep W modes
+template <int NX, typename F>
+cudaError_t with_form(int W, F f) {
+  using G = RowGeo<NX>;
+  if (2 * W == G::n) return f(std::integral_constant<int, kHalf>());
+  if constexpr (G::T < 4) return f(std::integral_constant<int, kAnyWidth>());
+  else return 2 * W < G::n ? f(std::integral_constant<int, kNarrow>()) : f(std::integral_constant<int, kBroad>());
+}
+
 template <int NX>
 cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st, bool chained) {
   using G = RowGeo<NX>;
@@ -1217,40 +1294,34 @@ cudaError_t launch_packed_row_n(const RowParams& p, cudaStream_t st, bool chaine
     return cudaErrorInvalidValue;
   const unsigned blocks = (unsigned)((p.rows_total - p.row_begin + p.rpc - 1) / p.rpc);
   const int threads = p.rpc * G::T;
-  const bool exact = 2 * p.W == G::n;
   RowParams q = p;
-  if (p.nslots > 1) {
-    RhsOps r;
-    if (!rhs_ops(q, &r)) return cudaErrorInvalidValue;
-    if (p.split > 0) {
-      const unsigned wb = (unsigned)((p.rows_total - p.row_begin + WideRow<NX>::ROWS - 1) / WideRow<NX>::ROWS);
-      const int wt = 5 * WideRow<NX>::SET;
-      return launch(exact ? k_packed_rhs_wide<NX, true> : k_packed_rhs_wide<NX, false>, wb, wt, row_smem_wide<NX>(), st,
-                    chained, q, r);
+  return with_form<NX>(p.W, [&](auto form) {
+    constexpr int FORM = decltype(form)::value;
+    if (p.nslots > 1) {
+      RhsOps r;
+      if (!rhs_ops(q, &r)) return cudaErrorInvalidValue;
+      if (p.split > 0) {
+        const unsigned wb = (unsigned)((p.rows_total - p.row_begin + WideRow<NX>::ROWS - 1) / WideRow<NX>::ROWS);
+        return launch(k_packed_rhs_wide<NX, FORM>, wb, 5 * WideRow<NX>::SET, row_smem_wide<NX>(), st, chained, q, r);
+      }
+      return launch(k_packed_rhs<NX, FORM>, blocks, threads, row_smem<NX>(p.rpc, 3), st, chained, q, r);
     }
-    return launch(exact ? k_packed_rhs<NX, true> : k_packed_rhs<NX, false>, blocks, threads, row_smem<NX>(p.rpc, 3), st,
-                  chained, q, r);
-  } else {
     const int ns = q.nops > 0 && q.ops[0].kind == ROP_C2R ? make_segments(q, p.split) : 0;
     if (ns == 0) return cudaErrorInvalidValue;
-    return launch(exact ? k_packed_row<NX, true> : k_packed_row<NX, false>, dim3(blocks, (unsigned)ns), threads,
-                  row_smem<NX>(p.rpc, 0), st, chained, q);
-  }
+    return launch(k_packed_row<NX, FORM>, dim3(blocks, (unsigned)ns), threads, row_smem<NX>(p.rpc, 0), st, chained, q);
+  });
 }
 
-template <int NX, bool EXACT>
-cudaError_t launch_packed_rk_e(const RkParams& p, dim3 grid, cudaStream_t st, bool chained) {
-  using G = RowGeo<NX>;
-  return launch(p.state64 ? k_packed_rk<NX, EXACT, double> : k_packed_rk<NX, EXACT, float>, grid, G::THREADS,
-                row_smem<NX>(G::MAXR, 0), st, chained, p);
-}
 template <int NX>
 cudaError_t launch_packed_rk_n(const RkParams& p, cudaStream_t st, bool chained) {
   using G = RowGeo<NX>;
   if (p.row_begin < 0 || p.row_begin >= p.rows_total) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)((p.rows_total - p.row_begin + G::MAXR - 1) / G::MAXR), 2);
-  return 2 * p.W == G::n ? launch_packed_rk_e<NX, true>(p, grid, st, chained)
-                         : launch_packed_rk_e<NX, false>(p, grid, st, chained);
+  return with_form<NX>(p.W, [&](auto form) {
+    constexpr int FORM = decltype(form)::value;
+    return launch(p.state64 ? k_packed_rk<NX, FORM, double> : k_packed_rk<NX, FORM, float>, grid, G::THREADS,
+                  row_smem<NX>(G::MAXR, 0), st, chained, p);
+  });
 }
 
 // every output carries the dealias mask and at most half of the modes are kept
@@ -1311,20 +1382,22 @@ template <typename K>
 cudaError_t allow_smem(K k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-template <int NX, bool EXACT>
-cudaError_t prepare_packed_row_e() {
-  using G = RowGeo<NX>;
-  cudaError_t e = allow_smem(k_packed_row<NX, EXACT>, row_smem<NX>(G::MAXR, 0));
-  if (e == cudaSuccess) e = allow_smem(k_packed_rhs<NX, EXACT>, row_smem<NX>(G::MAXR, 3));
-  if (e == cudaSuccess) e = allow_smem(k_packed_rhs_wide<NX, EXACT>, row_smem_wide<NX>());
-  if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, float>, row_smem<NX>(G::MAXR, 0));
-  if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, EXACT, double>, row_smem<NX>(G::MAXR, 0));
-  return e;
-}
 template <int NX>
 cudaError_t prepare_packed_row_n() {
-  const cudaError_t e = prepare_packed_row_e<NX, true>();
-  return e == cudaSuccess ? prepare_packed_row_e<NX, false>() : e;
+  using G = RowGeo<NX>;
+  auto prepare = [](auto form) {
+    constexpr int FORM = decltype(form)::value;
+    cudaError_t e = allow_smem(k_packed_row<NX, FORM>, row_smem<NX>(G::MAXR, 0));
+    if (e == cudaSuccess) e = allow_smem(k_packed_rhs<NX, FORM>, row_smem<NX>(G::MAXR, 3));
+    if (e == cudaSuccess) e = allow_smem(k_packed_rhs_wide<NX, FORM>, row_smem_wide<NX>());
+    if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, FORM, float>, row_smem<NX>(G::MAXR, 0));
+    if (e == cudaSuccess) e = allow_smem(k_packed_rk<NX, FORM, double>, row_smem<NX>(G::MAXR, 0));
+    return e;
+  };
+  cudaError_t e = cudaSuccess;
+  for (int W : {G::n / 2, G::n / 2 - 1, G::n / 2 + 1})   // one of each form
+    if (e == cudaSuccess) e = with_form<NX>(W, prepare);
+  return e;
 }
 template <int NY, int NACC, bool HALF>
 cudaError_t prepare_packed_col_a() {
