@@ -92,7 +92,7 @@ constexpr int line_cluster(int nx) { return nx >= 4096 ? 8 : (nx >= 2048 ? 4 : 1
 //     4096      304  835 and 807   1232 and 1397
 // (2432 members of 256 points: 1633 and 432 with a flat bottom.)
 constexpr bool line_pays(int nx, int n, bool variable_bottom) {
-  return n <= 152 * (nx <= 1024 ? 3 : (variable_bottom ? 2 : 1));
+  return n <= kSMs * (nx <= 1024 ? 3 : (variable_bottom ? 2 : 1));
 }
 
 cudaError_t prepare_line_kernels(int nx);

@@ -506,7 +506,7 @@ struct Planner {
   int default_split(const RowParams& p) const {
     int tpr = 0;
     packed_row_geometry(g.nx, &tpr);
-    const double warps = (double)p.rows_total * tpr / 32.0, want = 152.0 * 12.0;
+    const double warps = (double)p.rows_total * tpr / 32.0, want = kSMs * 12.0;
     if (warps >= want) return 0;
     if (p.nslots > 1) return 1;
     for (int per : {kMaxRowOps, 3, 2, 1})
@@ -517,7 +517,7 @@ struct Planner {
   // an SM (a pass of rows alone leaves most SMs idle or unevenly loaded).
   int default_split64(const RowParams& p) const {
     const double warps = (double)p.rows_total * row_tpr<double>(g.nx) / 32.0;
-    return p.nslots == 1 && p.ops[0].kind == ROP_C2R && warps < 152.0 * 16 ? kMaxRowOps : 0;
+    return p.nslots == 1 && p.ops[0].kind == ROP_C2R && warps < kSMs * 16.0 ? kMaxRowOps : 0;
   }
   static int row_segments(const RowParams& p, int per) {
     if (per == 0) return 1;
@@ -545,9 +545,9 @@ struct Planner {
     int tpc = 0, group = 1;
     packed_col_geometry(p, &tpc, &group);
     const double warps = (double)p.cols_total * tpc / 32.0;
-    if (most < 2 || warps * 3 > 152.0 * 8.0) return 0;
+    if (most < 2 || warps * 3 > kSMs * 8.0) return 0;
     int k = 2;
-    while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < 152.0 * 8.0) k *= 2;
+    while (2 * k <= most && k < std::max(p.nin, p.nouts) && warps * k < kSMs * 8.0) k *= 2;
     return k;
   }
   struct ColIn {
@@ -1685,7 +1685,7 @@ bool chainable(const Pass& p) {
   } else {
     return false;
   }
-  return threads <= 152.0 * 16 * 32;
+  return threads <= kSMs * 16.0 * 32;
 }
 
 // chained: another pass was launched on st just before
@@ -2213,7 +2213,7 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     // split forms that differ in their number of blocks, while the rows alone
     // are less than a few waves
     std::vector<int> counts{Planner::row_segments(p.row, p.row.split)};
-    if ((double)p.row.rows_total * tpr < 32.0 * 152 * 12 * 4)
+    if ((double)p.row.rows_total * tpr < 32.0 * kSMs * 12 * 4)
       for (int per : {0, kMaxRowOps, 3, 2, 1}) {
         const int n = Planner::row_segments(p.row, per);
         if (p.row.nslots > 1 ? per < 2 && per != p.row.split
@@ -2255,7 +2255,7 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
       const int most = packed_col_most_wide(p.col);
       const double warps = (double)p.col.cols_total * tpc / 32.0;
       const int useful = std::max({2, p.col.nin, p.col.nouts});
-      for (int k = 2; k <= most && k < 2 * useful && warps * k < 152.0 * 8.0 * 4; k *= 2)
+      for (int k = 2; k <= most && k < 2 * useful && warps * k < kSMs * 8.0 * 4; k *= 2)
         if (2 * k >= p.col.wide) cand.push_back(base(0) + kWideTag * k);
     }
   }

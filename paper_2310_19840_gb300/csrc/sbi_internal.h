@@ -27,6 +27,7 @@
 
 namespace sbi {
 
+constexpr int kSMs = 152;        // SMs of the GB300 (two dies of 76); the rules that fill the GPU count them
 constexpr int kMaxRowOps = 48;
 constexpr int kMaxRowBufs = 40;
 constexpr int kMaxColTerms = 48;
