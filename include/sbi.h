@@ -30,6 +30,11 @@
  *   - Every int-returning call returns SBI_OK or one of the SBI_E* codes below
  *     and never aborts the process or traps the device; sbi_last_error() gives
  *     the message of the last failure on that context.
+ *   - A member's results do not depend on the other members, nor, with one
+ *     exception, on how many there are: in FP32 the 1-D members of one grid run
+ *     as one launch per step up to 456 of them (152 from 2048 points on, 304
+ *     there over a variable bottom) and as one launch per pass beyond, and the
+ *     two round differently.
  *   - Calls on one context are not thread-safe; different contexts are
  *     independent.  Work is enqueued on opt.cuda_stream (NULL: the legacy
  *     default stream).

@@ -16,7 +16,7 @@
 // takes 128 SM-cycles per transform instead of 312 and 336 instructions per
 // row instead of about 800; a 256-point column 137 instead of 312; the row pass
 // of a 4096 x 2048 grid 168 us per launch instead of 344; a step of 64 256^2 and
-// 32 512^2 members 4.33 ms instead of 6.03.
+// 32 512^2 members 4.40 ms instead of 6.03.
 #pragma once
 
 #include <type_traits>
@@ -467,8 +467,10 @@ k_packed_row(const __grid_constant__ RowParams p) {
 // for the one of phi~.  The modes of the next transform are loaded ahead of the
 // current one.  The quotients are IEEE divisions, correct to half a unit in the
 // last place for every operand.  Load latency bounds the pass (a quarter of the
-// issue slots used): 8192 rows of 512 points 65 us, 128 of the 168 registers
-// (four blocks per SM and no loads ahead) 66.
+// issue slots used): 8192 rows of 512 points 66 us, of which the divisions are 6.
+// It spills 40 to 140 bytes per thread from 256 points up at three blocks per SM
+// (168 registers); with four blocks, 128 registers and no loads ahead it took
+// 3 us more.
 struct RhsOps {
   int8_t src[5];      // inverse transforms in the order eta_x, phi_x, eta_y, phi_y, V (indices into ops)
   int8_t f, sx, sy;   // the operation; sponge products of phi_x and phi_y (-1: none)
