@@ -2239,7 +2239,8 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     };
     deflt = base(p.col.staged) + kStagedTag * p.col.staged + kWideTag * p.col.wide;
     // the staged form is a candidate where the option leaves the choice open
-    const bool stg = c->opt.col_staging == 0 && stageable(c, p.col);
+    // (not with tiles of 512 threads, which spill: 2048 points, both halves' sums)
+    const bool stg = c->opt.col_staging == 0 && stageable(c, p.col) && !(p.col.packed && 4 * tpc > 256);
     // few columns: the wide form beat every other block shape by a third or more
     // wherever it was the default, so only its number of copies is left open
     if (p.col.wide) cand.push_back(base(0));
@@ -2254,8 +2255,11 @@ int tune_pass(sbi_ctx* c, Pass& p, cudaStream_t st) {
     if (p.col.packed && !p.col.staged) {   // copies of the wide form
       const int most = packed_col_most_wide(p.col);
       const double warps = (double)p.col.cols_total * tpc / 32.0;
-      const int useful = std::max({2, p.col.nin, p.col.nouts});
-      for (int k = 2; k <= most && k < 2 * useful && warps * k < kSMs * 8.0 * 4; k *= 2)
+      // columns of 1024 points and more stand alone there: nothing to gain, and slow
+      // to time, once the plain form has eight warps on every SM
+      const bool wide = tpc < 64 || warps < kSMs * 8.0;
+      const int useful = std::max({p.col.wide ? 2 : 1, p.col.nin, p.col.nouts});
+      for (int k = 2; wide && k <= most && k < 2 * useful && warps * k < kSMs * 8.0 * 4; k *= 2)
         if (2 * k >= p.col.wide) cand.push_back(base(0) + kWideTag * k);
     }
   }
